@@ -15,7 +15,8 @@
 // Epilogues: plain bf16 store (QKV projection); residual add, rounded once after the add (attention output
 // and feed-forward down projections, in place on the residual stream); SwiGLU, where a tile holds w gate
 // columns and the matching w up columns (two TMA loads, one per matrix) and silu(g) * u is formed in
-// registers, so the 2F-wide intermediate never reaches memory.
+// registers, so the 2F-wide intermediate never reaches memory; RoPE for the QKV projection of many rows, whose tiles
+// then hold whole heads, so that q, k and v go from the accumulator to where the attention reads them.
 // Split K: the CTAs that share an output tile form a thread-block cluster.  After the main loop each CTA
 // sends, through distributed shared memory, the accumulator column groups it does not own into the idle
 // operand ring of the CTA that owns them; every CTA then adds the partials of its own groups in split order
@@ -66,6 +67,17 @@ struct GemmArgs {
 
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
+// v rounded to bf16 (the stack rounds the projection before it rotates q and k)
+__device__ __forceinline__ float round_bf16(float v) { return __bfloat162float(__float2bfloat16_rn(v)); }
+
+// Where head H of the fused QKV projection goes for row m = (b, i): q_out, or the K or V cache at position start + i.
+__device__ __forceinline__ __nv_bfloat16* rope_dst(const RopeArgs& r, int H, int m) {
+    if (H < r.Hq) return static_cast<__nv_bfloat16*>(r.q_out) + (static_cast<size_t>(m) * r.Hq + H) * r.d;
+    const int b = m / r.length, p = r.start + m % r.length;
+    const bool k = H < r.Hq + r.Hkv;
+    const int h = H - r.Hq - (k ? 0 : r.Hkv);
+    return static_cast<__nv_bfloat16*>(k ? r.k_cache : r.v_cache) + ((static_cast<size_t>(b) * r.Hkv + h) * r.cap + p) * r.d;
+}
 
 // Applies the epilogue to 8 accumulated columns of one row and stores them.  `res` may alias `out`.
 template <int EPI>
@@ -326,6 +338,7 @@ struct PairArgs {
     __nv_bfloat16* out;
     const __nv_bfloat16* res;
     uint32_t* dev_status;
+    RopeArgs rope;
 };
 
 // 4 x 4 transpose of 16-byte pieces inside every group of four lanes.  In: v[q] = piece q of this lane's row.
@@ -390,6 +403,25 @@ __device__ __forceinline__ void store_chunk32(float (&f)[32], int lane, int row0
         const int row = my_row0 + i;
         if (col_ok && row < n_rows_total)
             *reinterpret_cast<uint4*>(out + static_cast<size_t>(row) * ldo + my_col) = o[i];
+    }
+}
+
+// The same for 32 channels of one head, stored at dst(row) + col for each row.
+template <typename Dst>
+__device__ __forceinline__ void store_head32(const float (&f)[32], int lane, int row0, int n_rows_total, int col, const Dst& dst) {
+    uint4 o[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        o[q].x = pack_bf16(f[q * 8 + 0], f[q * 8 + 1]);
+        o[q].y = pack_bf16(f[q * 8 + 2], f[q * 8 + 3]);
+        o[q].z = pack_bf16(f[q * 8 + 4], f[q * 8 + 5]);
+        o[q].w = pack_bf16(f[q * 8 + 6], f[q * 8 + 7]);
+    }
+    quad_transpose(o, lane);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int row = row0 + (lane & ~3) + i;
+        if (row < n_rows_total) *reinterpret_cast<uint4*>(dst(row) + col + (lane & 3) * 8) = o[i];
     }
 }
 
@@ -571,9 +603,43 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
         // Without a K split the output goes 32 columns at a time through store_chunk32 (coalesced stores); the
         // last n_groups % 4 groups, and the K-split case, go 8 columns at a time with one 16-byte store per lane.
         int g_begin = set;
-        if (p.splits == 1) {             // (warp-uniform: store_chunk32 shuffles)
+        const int warp_row0 = m_pair * 2 * GM + rank * GM + lq * 32;
+        if (EPI == GEMM_EPI_ROPE) {      // whole heads per tile, no K split: 32 channels and their partners at a time
+            const RopeArgs& r = g.rope;
+            const int half = r.d / 2, per_head = half / 32, heads = p.wcols / r.d;
+            // the table is read transposed: the lanes are consecutive rows, i.e. consecutive positions of a rollout
+            const float2* t = reinterpret_cast<const float2*>(r.cs_t) + r.start + row % r.length;
+            for (int u = set; u < heads * per_head; u += 2) {
+                const int hh = u / per_head, c0 = (u % per_head) * 32;
+                const int H = n_tile * heads + hh;
+                if (H >= r.Hq + 2 * r.Hkv) break;
+                float f1[32], f2[32];
+                {
+                    uint32_t v1[32], v2[32];
+                    tmem_ld_32cols(taddr + hh * r.d + c0, v1);
+                    tmem_ld_32cols(taddr + hh * r.d + half + c0, v2);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int k = 0; k < 32; ++k) { f1[k] = __uint_as_float(v1[k]); f2[k] = __uint_as_float(v2[k]); }
+                }
+                if (H < r.Hq + r.Hkv) {
+#pragma unroll
+                    for (int k = 0; k < 32; ++k) {
+                        const float2 cs = t[static_cast<size_t>(c0 + k) * r.n_pos];
+                        const float x1 = round_bf16(f1[k]), x2 = round_bf16(f2[k]);
+                        f1[k] = x1 * cs.x - x2 * cs.y;
+                        f2[k] = x2 * cs.x + x1 * cs.y;
+                    }
+                }
+                if (live) {
+                    const auto dst = [&](int m) { return rope_dst(r, H, m); };
+                    store_head32(f1, lane, warp_row0, g.M, c0, dst);
+                    store_head32(f2, lane, warp_row0, g.M, half + c0, dst);
+                }
+            }
+            g_begin = n_groups;
+        } else if (p.splits == 1) {      // (warp-uniform: store_chunk32 shuffles)
             const int n_chunks = n_groups / 4;
-            const int warp_row0 = m_pair * 2 * GM + rank * GM + lq * 32;
             for (int ci = set; ci < n_chunks; ci += 2) {
                 float f[32];
                 if (EPI == GEMM_EPI_SWIGLU) {
@@ -711,21 +777,22 @@ int max_active_pairs(int splits = 1) {
 // per MMA plus the ~45 measured on top of that), its shared-memory traffic (the stage written by the copies plus, per MMA, 4 KB of
 // A and its half of W read by the tensor core) at 128 bytes per cycle, and the operand delivery at ~55 bytes
 // per cycle; a launch takes as many rounds as the pairs need on the device.  cost_out: the model's cycles.
-PairPlan pair_plan(int epi, int M, int N, int K, double* cost_out) {
+PairPlan pair_plan(int epi, int M, int N, int K, int head_dim, double* cost_out) {
     PairPlan best{};
     double best_cost = 1e300;
     const int nk = (K + GK - 1) / GK;
     const int m_pairs = (M + 2 * GM - 1) / (2 * GM);
     const int ring = GEMM_SMEM_BYTES - 1024 - 256;
     for (int splits = 1; splits <= 2; ++splits) {
-        if (splits > 1 && (epi == GEMM_EPI_SWIGLU || nk < 32)) break;
+        if (splits > 1 && (epi == GEMM_EPI_SWIGLU || epi == GEMM_EPI_ROPE || nk < 32)) break;
         const int resident = max_active_pairs(splits);
         if (resident < 1) continue;
         for (int nmma = 1; nmma <= 2; ++nmma) {
             for (int nchunk = 256; nchunk >= 32; nchunk -= 16) {
                 const int bn = nmma * nchunk;
                 const int wcols = epi == GEMM_EPI_SWIGLU ? bn / 2 : bn;
-                if (wcols > ((N + 7) / 8) * 8 + 15 && bn > 32) continue;      // wider than the whole output
+                if (epi == GEMM_EPI_ROPE ? wcols % head_dim != 0              // whole heads
+                                         : wcols > ((N + 7) / 8) * 8 + 15 && bn > 32) continue;   // wider than the whole output
                 const int half_rows = nchunk / 2;
                 const int stage_bytes = A_TILE_BYTES + nmma * half_rows * GK * 2;
                 int stages = ring / stage_bytes;
@@ -857,8 +924,18 @@ GemmPlan gemm_plan(int epi, int M, int N, int K, int sm_count) {
 // The pair kernel serves every problem with more than one row tile.
 bool use_pair_kernel(int M, const PairPlan& pp) { return M > GM && pp.bn != 0; }
 
+// The pair kernel is persistent: with two or more tiles of 256 x 256 per CTA pair a tile's epilogue runs beside the next
+// tile's main loop, and the rotation is hidden there (as a kernel of its own it took 64 us at 8192 rows x 12288, reading
+// and writing q, k and v once more; the prefill of 16 x 512 rows is 2 % faster without it).  With fewer it is exposed:
+// at 512 rows x 12288 (one 384-column tile per pair) the projection took 45.6 us with it, against 37.0 us plain and
+// 7.4 us for the kernel that rotates.
+bool gemm_hides_epilogue(int M, int N) {
+    const long long tiles = static_cast<long long>((M + 2 * GM - 1) / (2 * GM)) * ((N + 255) / 256);
+    return M > GM && max_active_pairs() > 0 && tiles >= 2LL * max_active_pairs();
+}
+
 int gemm_plan_describe(const dare_ctx* ctx, int epi, int M, int N, int K, int* out) {
-    const PairPlan pp = pair_plan(epi, M, N, K, nullptr);
+    const PairPlan pp = pair_plan(epi, M, N, K, 0, nullptr);
     if (use_pair_kernel(M, pp)) {
         out[0] = 2; out[1] = pp.bn; out[2] = pp.wcols; out[3] = pp.splits; out[4] = pp.stages;
         out[5] = pp.m_pairs; out[6] = pp.n_tiles; out[7] = max_active_pairs(pp.splits);
@@ -871,10 +948,10 @@ int gemm_plan_describe(const dare_ctx* ctx, int epi, int M, int N, int K, int* o
 }
 
 int launch_gemm(const dare_ctx* ctx, int epi, const void* a, int M, int K, const void* w, const void* w2, int N,
-                void* out, const void* res, int ldo, cudaStream_t stream) {
+                void* out, const void* res, int ldo, cudaStream_t stream, const RopeArgs* rope) {
     if (M < 1 || N < 8 || K < 8 || (N % 8) || (K % 8) || (ldo % 8)) return DARE_ERR_SHAPE;
-    if (epi < GEMM_EPI_STORE || epi > GEMM_EPI_SWIGLU) return DARE_ERR_RANGE;
-    const PairPlan pp = pair_plan(epi, M, N, K, nullptr);
+    if (epi < GEMM_EPI_STORE || epi > GEMM_EPI_ROPE || (epi == GEMM_EPI_ROPE) != (rope != nullptr)) return DARE_ERR_RANGE;
+    const PairPlan pp = pair_plan(epi, M, N, K, rope ? rope->d : 0, nullptr);
     if (use_pair_kernel(M, pp)) {
         PairArgs pg;
         pg.M = M; pg.N = N; pg.K = K; pg.ldo = ldo;
@@ -882,6 +959,7 @@ int launch_gemm(const dare_ctx* ctx, int epi, const void* a, int M, int K, const
         pg.out = static_cast<__nv_bfloat16*>(out);
         pg.res = static_cast<const __nv_bfloat16*>(res);
         pg.dev_status = ctx->dev_status;
+        pg.rope = rope ? *rope : RopeArgs{};
         CUtensorMap pa, pb, pb2;
         int prc = make_tmap_bf16_2d(ctx, &pa, a, static_cast<uint64_t>(M), static_cast<uint64_t>(K), GM, GK);
         if (prc != DARE_OK) return prc;
@@ -893,9 +971,11 @@ int launch_gemm(const dare_ctx* ctx, int epi, const void* a, int M, int K, const
             if (prc != DARE_OK) return prc;
             return launch_pair<GEMM_EPI_SWIGLU>(pa, pb, pb2, pg, stream, nullptr);
         }
+        if (epi == GEMM_EPI_ROPE) return launch_pair<GEMM_EPI_ROPE>(pa, pb, pb, pg, stream, nullptr);
         return epi == GEMM_EPI_STORE ? launch_pair<GEMM_EPI_STORE>(pa, pb, pb, pg, stream, nullptr)
                                      : launch_pair<GEMM_EPI_RESIDUAL>(pa, pb, pb, pg, stream, nullptr);
     }
+    if (epi == GEMM_EPI_ROPE) return DARE_ERR_SHAPE;      // (the pair kernel only: gemm_hides_epilogue)
     GemmArgs g;
     g.M = M; g.N = N; g.K = K; g.ldo = ldo;
     g.p = gemm_plan(epi, M, N, K, ctx->sm_count);

@@ -143,17 +143,28 @@ int launch_attn_varlen(const dare_ctx* ctx, int total, int n_seqs, int max_seqle
                        cudaStream_t stream);
 
 // ---- layer stack (gemm.cu, layers.cu)
-enum { GEMM_EPI_STORE = 0, GEMM_EPI_RESIDUAL = 1, GEMM_EPI_SWIGLU = 2 };
+enum { GEMM_EPI_STORE = 0, GEMM_EPI_RESIDUAL = 1, GEMM_EPI_SWIGLU = 2, GEMM_EPI_ROPE = 3 };
 // out[M, N] = epilogue(a[M, K] . w[N, K]^T), bf16 row-major, ldo = elements per output row.
 //   STORE: out = acc.  RESIDUAL: out = res + acc (res may be out).  SWIGLU: out = silu(a w^T) * (a w2^T).
+//   ROPE: the QKV projection of the stack; its columns go through rotary embedding to q_out and the K/V caches, as
+//   launch_rope_kv_write would put them, bit for bit (out, res, ldo unused; N = (Hq + 2 Hkv) d).  Only where
+//   gemm_hides_epilogue says so.
+struct RopeArgs {
+    int Hq, Hkv, d, start, length, cap;
+    const float* cs_t;                  // launch_rope_table's transposed table
+    int n_pos;
+    void *q_out, *k_cache, *v_cache;
+};
+bool gemm_hides_epilogue(int M, int N);
 int launch_gemm(const dare_ctx* ctx, int epi, const void* a, int M, int K, const void* w, const void* w2, int N,
-                void* out, const void* res, int ldo, cudaStream_t stream);
+                void* out, const void* res, int ldo, cudaStream_t stream, const RopeArgs* rope = nullptr);
 // out[8] = {row tiles per CTA, bn, output columns per tile, K splits, stages, row items, column tiles, resident clusters}
 int gemm_plan_describe(const dare_ctx* ctx, int epi, int M, int N, int K, int* out);
 int launch_embed(const void* emb, int D, int V, const int32_t* tokens, int64_t row_stride, int start, int length,
                  int n_rows, void* x, cudaStream_t stream);
 int launch_rmsnorm(const void* x, int D, int n_rows, float eps, void* y, cudaStream_t stream);
-int launch_rope_table(float* cs, int n_pos, int half, double base, cudaStream_t stream);
+// cs [n_pos][half] and cs_t [half][n_pos]: (cos, sin) pairs
+int launch_rope_table(float* cs, float* cs_t, int n_pos, int half, double base, cudaStream_t stream);
 int launch_rope_kv_write(const void* qkv, int n_rows, int Hq, int Hkv, int d, int start, int length, const float* cs,
                          void* q_out, void* k_cache, void* v_cache, int cap, cudaStream_t stream);
 

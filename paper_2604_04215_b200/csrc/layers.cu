@@ -13,6 +13,16 @@ constexpr int ROWS_PER_BLOCK = 8;   // one warp per row
 __device__ __forceinline__ float lo_f(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float hi_f(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 
+__device__ __forceinline__ float sum_squares(const uint4& v) {
+    const float a0 = lo_f(v.x), a1 = hi_f(v.x), a2 = lo_f(v.y), a3 = hi_f(v.y);
+    const float a4 = lo_f(v.z), a5 = hi_f(v.z), a6 = lo_f(v.w), a7 = hi_f(v.w);
+    return a0 * a0 + a1 * a1 + a2 * a2 + a3 * a3 + a4 * a4 + a5 * a5 + a6 * a6 + a7 * a7;
+}
+__device__ __forceinline__ uint4 scale_bf16(const uint4& v, float f) {
+    return make_uint4(pack_bf16(lo_f(v.x) * f, hi_f(v.x) * f), pack_bf16(lo_f(v.y) * f, hi_f(v.y) * f),
+                      pack_bf16(lo_f(v.z) * f, hi_f(v.z) * f), pack_bf16(lo_f(v.w) * f, hi_f(v.w) * f));
+}
+
 // x[m, :] = E[tokens[b, start + i], :] for row m = b * length + i.
 __global__ void __launch_bounds__(ROWS_PER_BLOCK * 32)
 embed_gather_kernel(const uint4* __restrict__ emb, int D8, int V, const int32_t* __restrict__ tokens, int64_t row_stride,
@@ -27,37 +37,45 @@ embed_gather_kernel(const uint4* __restrict__ emb, int D8, int V, const int32_t*
     for (int i = lane; i < D8; i += 32) dst[i] = src[i];
 }
 
-// y = x / sqrt(mean(x^2) + eps), weight 1.  Two passes over the row (the second one hits L1/L2).
-__global__ void __launch_bounds__(ROWS_PER_BLOCK * 32)
-rmsnorm_kernel(const uint4* __restrict__ x, int D8, int n_rows, float eps, uint4* __restrict__ y) {
-    const int m = blockIdx.x * ROWS_PER_BLOCK + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (m >= n_rows) return;
-    const uint4* src = x + static_cast<size_t>(m) * D8;
-    float ss = 0.f;
-    for (int i = lane; i < D8; i += 32) {
-        const uint4 v = src[i];
-        const float a0 = lo_f(v.x), a1 = hi_f(v.x), a2 = lo_f(v.y), a3 = hi_f(v.y);
-        const float a4 = lo_f(v.z), a5 = hi_f(v.z), a6 = lo_f(v.w), a7 = hi_f(v.w);
-        ss += a0 * a0 + a1 * a1 + a2 * a2 + a3 * a3 + a4 * a4 + a5 * a5 + a6 * a6 + a7 * a7;
+// y = x / sqrt(mean(x^2) + eps), weight 1.  A row's time is one trip to memory and back, so a row gets a whole CTA:
+// NORM_THREADS threads read it in one go (NORM_VECS 16-byte pieces each, all in flight together, kept in registers for
+// the scaling); longer rows are read a second time.  2.7 us at 512 rows x 4096 between two projections, where one warp
+// per row with two passes took 4.2 us.
+constexpr int NORM_THREADS = 128;
+constexpr int NORM_VECS = 4;
+__global__ void __launch_bounds__(NORM_THREADS)
+rmsnorm_kernel(const uint4* __restrict__ x, int D8, float eps, uint4* __restrict__ y) {
+    __shared__ float s_part[NORM_THREADS / 32];
+    const uint4* src = x + static_cast<size_t>(blockIdx.x) * D8;
+    uint4* dst = y + static_cast<size_t>(blockIdx.x) * D8;
+    uint4 v[NORM_VECS];
+#pragma unroll
+    for (int u = 0; u < NORM_VECS; ++u) {
+        const int i = threadIdx.x + u * NORM_THREADS;
+        v[u] = i < D8 ? src[i] : make_uint4(0, 0, 0, 0);
     }
+    float ss = 0.f;
+#pragma unroll
+    for (int u = 0; u < NORM_VECS; ++u) ss += sum_squares(v[u]);
+    for (int i = threadIdx.x + NORM_VECS * NORM_THREADS; i < D8; i += NORM_THREADS) ss += sum_squares(src[i]);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
+    if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = ss;
+    __syncthreads();
+    ss = 0.f;
+#pragma unroll
+    for (int w = 0; w < NORM_THREADS / 32; ++w) ss += s_part[w];
     const float inv = rsqrtf(ss / static_cast<float>(D8 * 8) + eps);
-    uint4* dst = y + static_cast<size_t>(m) * D8;
-    for (int i = lane; i < D8; i += 32) {
-        const uint4 v = src[i];
-        uint4 o;
-        o.x = pack_bf16(lo_f(v.x) * inv, hi_f(v.x) * inv);
-        o.y = pack_bf16(lo_f(v.y) * inv, hi_f(v.y) * inv);
-        o.z = pack_bf16(lo_f(v.z) * inv, hi_f(v.z) * inv);
-        o.w = pack_bf16(lo_f(v.w) * inv, hi_f(v.w) * inv);
-        dst[i] = o;
+#pragma unroll
+    for (int u = 0; u < NORM_VECS; ++u) {
+        const int i = threadIdx.x + u * NORM_THREADS;
+        if (i < D8) dst[i] = scale_bf16(v[u], inv);
     }
+    for (int i = threadIdx.x + NORM_VECS * NORM_THREADS; i < D8; i += NORM_THREADS) dst[i] = scale_bf16(src[i], inv);
 }
 
-// cs[p, c] = (cos, sin)(p * base^(-2c/d)), c < d/2, evaluated in double precision.
-__global__ void rope_table_kernel(float2* __restrict__ cs, int n_pos, int half, double base) {
+// cs[p, c] = (cos, sin)(p * base^(-2c/d)), c < d/2, evaluated in double precision; cs_t is its transpose.
+__global__ void rope_table_kernel(float2* __restrict__ cs, float2* __restrict__ cs_t, int n_pos, int half, double base) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n_pos * half) return;
     const int p = i / half, c = i % half;
@@ -65,6 +83,7 @@ __global__ void rope_table_kernel(float2* __restrict__ cs, int n_pos, int half, 
     double s, co;
     sincos(ang, &s, &co);
     cs[i] = make_float2(static_cast<float>(co), static_cast<float>(s));
+    cs_t[static_cast<size_t>(c) * n_pos + p] = cs[i];
 }
 
 // Row m = (b, i) of the fused QKV projection [n_rows, (Hq + 2 Hkv) d], position p = start + i:
@@ -119,14 +138,13 @@ int launch_embed(const void* emb, int D, int V, const int32_t* tokens, int64_t r
 }
 
 int launch_rmsnorm(const void* x, int D, int n_rows, float eps, void* y, cudaStream_t stream) {
-    rmsnorm_kernel<<<(n_rows + ROWS_PER_BLOCK - 1) / ROWS_PER_BLOCK, ROWS_PER_BLOCK * 32, 0, stream>>>(
-        static_cast<const uint4*>(x), D / 8, n_rows, eps, static_cast<uint4*>(y)); note_launch();
+    rmsnorm_kernel<<<n_rows, NORM_THREADS, 0, stream>>>(static_cast<const uint4*>(x), D / 8, eps, static_cast<uint4*>(y)); note_launch();
     return cudaGetLastError() == cudaSuccess ? DARE_OK : DARE_ERR_CUDA;
 }
 
-int launch_rope_table(float* cs, int n_pos, int half, double base, cudaStream_t stream) {
+int launch_rope_table(float* cs, float* cs_t, int n_pos, int half, double base, cudaStream_t stream) {
     const int n = n_pos * half;
-    rope_table_kernel<<<(n + 255) / 256, 256, 0, stream>>>(reinterpret_cast<float2*>(cs), n_pos, half, base); note_launch();
+    rope_table_kernel<<<(n + 255) / 256, 256, 0, stream>>>(reinterpret_cast<float2*>(cs), reinterpret_cast<float2*>(cs_t), n_pos, half, base); note_launch();
     return cudaGetLastError() == cudaSuccess ? DARE_OK : DARE_ERR_CUDA;
 }
 

@@ -24,7 +24,7 @@ struct dare_model {
     const void* embedding;
     const void* lm_head;
     dare_layer_weights* layers;    // host copy of the caller's array (device pointers inside)
-    float* rope_cs;                // [max_positions, d/2] (cos, sin)
+    float *rope_cs, *rope_cs_t;    // [max_positions, d/2] (cos, sin) and its transpose
     void *x, *h, *qkv, *q, *attn, *act;   // activations, max_rows each
     int32_t* host_counts;          // pinned: n_remaining of two steps in flight, [2][max_batch]
     int max_batch;
@@ -57,11 +57,18 @@ int forward_rows(dare_model* m, const int32_t* tokens, int B, int64_t row_stride
         __nv_bfloat16* vc = static_cast<__nv_bfloat16*>(v_cache) + layer_kv * l;
         rc = launch_rmsnorm(m->x, c.hidden, rows, c.rms_eps, m->h, s);
         if (rc != DARE_OK) return rc;
-        rc = launch_gemm(m->ctx, GEMM_EPI_STORE, m->h, rows, c.hidden, w.wqkv, nullptr, nq + 2 * nkv, m->qkv, nullptr,
-                         nq + 2 * nkv, s);
-        if (rc != DARE_OK) return rc;
-        rc = launch_rope_kv_write(m->qkv, rows, c.n_q_heads, c.n_kv_heads, c.head_dim, start, length, m->rope_cs, m->q,
-                                  kc, vc, cap, s);
+        if (gemm_hides_epilogue(rows, nq + 2 * nkv)) {
+            const RopeArgs rope = {c.n_q_heads, c.n_kv_heads, c.head_dim, start, length, cap, m->rope_cs_t, c.max_positions,
+                                   m->q, kc, vc};
+            rc = launch_gemm(m->ctx, GEMM_EPI_ROPE, m->h, rows, c.hidden, w.wqkv, nullptr, nq + 2 * nkv, nullptr, nullptr,
+                             nq + 2 * nkv, s, &rope);
+        } else {
+            rc = launch_gemm(m->ctx, GEMM_EPI_STORE, m->h, rows, c.hidden, w.wqkv, nullptr, nq + 2 * nkv, m->qkv, nullptr,
+                             nq + 2 * nkv, s);
+            if (rc == DARE_OK)
+                rc = launch_rope_kv_write(m->qkv, rows, c.n_q_heads, c.n_kv_heads, c.head_dim, start, length, m->rope_cs,
+                                          m->q, kc, vc, cap, s);
+        }
         if (rc != DARE_OK) return rc;
         AttnArgs a;
         a.B = B; a.L = length; a.Hq = c.n_q_heads; a.Hkv = c.n_kv_heads; a.d = c.head_dim;
@@ -160,7 +167,7 @@ int dare_model_create(dare_ctx* ctx, const dare_model_desc* desc, const void* em
     if (!m) return DARE_ERR_CUDA;
     m->ctx = ctx; m->desc = c; m->embedding = embedding; m->lm_head = lm_head; m->max_batch = c.max_batch;
     m->layers = new (std::nothrow) dare_layer_weights[c.n_layers];
-    m->rope_cs = nullptr; m->x = m->h = m->qkv = m->q = m->attn = m->act = nullptr; m->host_counts = nullptr;
+    m->rope_cs = m->rope_cs_t = nullptr; m->x = m->h = m->qkv = m->q = m->attn = m->act = nullptr; m->host_counts = nullptr;
     m->ev[0] = m->ev[1] = nullptr;
     m->work = nullptr; m->ev_in = m->ev_out = nullptr;
     m->sample_temperature = 0.f; m->sample_seed = 0; m->step_counter = nullptr;
@@ -168,7 +175,9 @@ int dare_model_create(dare_ctx* ctx, const dare_model_desc* desc, const void* em
     if (ok) for (int l = 0; l < c.n_layers; ++l) m->layers[l] = layers[l];
     const size_t rows = static_cast<size_t>(c.max_rows);
     const size_t nq = static_cast<size_t>(c.n_q_heads) * c.head_dim, nkv = static_cast<size_t>(c.n_kv_heads) * c.head_dim;
-    ok = ok && cudaMalloc(&m->rope_cs, sizeof(float) * 2 * c.max_positions * (c.head_dim / 2)) == cudaSuccess;
+    const size_t rope_bytes = sizeof(float) * 2 * static_cast<size_t>(c.max_positions) * (c.head_dim / 2);
+    ok = ok && cudaMalloc(&m->rope_cs, rope_bytes) == cudaSuccess;
+    ok = ok && cudaMalloc(&m->rope_cs_t, rope_bytes) == cudaSuccess;
     ok = ok && cudaMalloc(&m->x, rows * c.hidden * 2) == cudaSuccess;
     ok = ok && cudaMalloc(&m->h, rows * c.hidden * 2) == cudaSuccess;
     ok = ok && cudaMalloc(&m->qkv, rows * (nq + 2 * nkv) * 2) == cudaSuccess;
@@ -183,7 +192,7 @@ int dare_model_create(dare_ctx* ctx, const dare_model_desc* desc, const void* em
     ok = ok && cudaEventCreateWithFlags(&m->ev_in, cudaEventDisableTiming) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&m->ev_out, cudaEventDisableTiming) == cudaSuccess;
     ok = ok && cudaStreamCreateWithFlags(&m->work, cudaStreamNonBlocking) == cudaSuccess;
-    ok = ok && dare::launch_rope_table(m->rope_cs, c.max_positions, c.head_dim / 2, static_cast<double>(c.rope_base),
+    ok = ok && dare::launch_rope_table(m->rope_cs, m->rope_cs_t, c.max_positions, c.head_dim / 2, static_cast<double>(c.rope_base),
                                        nullptr) == DARE_OK;
     ok = ok && cudaDeviceSynchronize() == cudaSuccess;
     if (!ok) {
@@ -197,7 +206,7 @@ int dare_model_create(dare_ctx* ctx, const dare_model_desc* desc, const void* em
 int dare_model_destroy(dare_model* m) {
     if (!m) return DARE_ERR_NULL;
     dare::DeviceScope scope(m->ctx->device);
-    cudaFree(m->rope_cs); cudaFree(m->x); cudaFree(m->h); cudaFree(m->qkv); cudaFree(m->q); cudaFree(m->attn);
+    cudaFree(m->rope_cs); cudaFree(m->rope_cs_t); cudaFree(m->x); cudaFree(m->h); cudaFree(m->qkv); cudaFree(m->q); cudaFree(m->attn);
     cudaFree(m->act);
     cudaFree(m->step_counter);
     if (m->host_counts) cudaFreeHost(m->host_counts);

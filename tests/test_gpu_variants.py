@@ -1,0 +1,72 @@
+"""GPU tests of kernel variants that the dispatch picks by size, at the sizes where they begin and end."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2604_04215_b200 import binding as dare
+from paper_2604_04215_b200 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = dare.Context(0)
+    yield c
+    c.close()
+
+
+def _small_model(ctx, Hq, Hkv, d, rows, batch, positions, hidden=256, ffn=256, vocab=512):
+    n = (Hq + 2 * Hkv) * d
+    w = {"wqkv": I.normal_bf16(7, 1, (n, hidden), 0.05), "wo": I.normal_bf16(7, 2, (hidden, Hq * d), 0.05),
+         "wg": I.normal_bf16(7, 3, (ffn, hidden), 0.05), "wu": I.normal_bf16(7, 4, (ffn, hidden), 0.05),
+         "wd": I.normal_bf16(7, 5, (hidden, ffn), 0.05)}
+    emb, head = I.normal_bf16(7, 6, (vocab, hidden)), I.normal_bf16(7, 8, (vocab, hidden))
+    return dare.Model(ctx, n_layers=1, hidden=hidden, n_q_heads=Hq, n_kv_heads=Hkv, head_dim=d, ffn=ffn, vocab=vocab,
+                      mask_id=vocab - 1, embedding=emb.cuda(), layers=[{k: v.cuda() for k, v in w.items()}],
+                      lm_head=head.cuda(), max_positions=positions, max_rows=rows, max_batch=batch)
+
+
+# Enough rows for two 256 x 256 tiles of the QKV projection per CTA pair (148 tiles): there rotary embedding rides on
+# the projection.  Row counts that are no multiple of a tile, head counts that leave the last column tile part full.
+@pytest.mark.parametrize("Hq,Hkv,d,B,length", [(4, 2, 64, 37, 513), (4, 2, 128, 19, 499), (3, 1, 128, 40, 331), (2, 1, 64, 75, 260)])
+def test_rope_in_the_projection_matches_the_separate_kernel(ctx, Hq, Hkv, d, B, length):
+    start, cap = 3, length + 5
+    model = _small_model(ctx, Hq, Hkv, d, B * length, B, cap)
+    tok = I.uniform_int(7, 9, (B, cap), 0, 510).cuda()
+    hid = torch.empty(B * length, 256, dtype=torch.bfloat16, device="cuda")
+    caches = model.new_cache(B, cap)
+    dare.dare_model_forward(model, tok, start, length, *caches, hid)
+    # the same rollouts a few at a time: too few rows for that
+    one = [torch.zeros_like(c) for c in caches]
+    hid1 = torch.empty_like(hid)
+    for b in range(0, B, 3):
+        nb = min(3, B - b)
+        part = [c[:, b:b + nb].contiguous() for c in one]
+        dare.dare_model_forward(model, tok[b:b + nb].contiguous(), start, length, *part, hid1[b * length:(b + nb) * length])
+        for c, p in zip(one, part):
+            c[:, b:b + nb] = p
+    torch.cuda.synchronize()
+    assert ctx.device_status() == 0
+    # Both round q, k and v to bf16 before the rotation and once after it; the fp32 sums in front may differ in their
+    # last bits (another tile shape), which can move a value by one bf16 step (2^-8) before and one after: 2^-7 of the
+    # larger of the two channels that turn together, and v by one step.
+    k, k1, v, v1 = (t.float() for t in (caches[0], one[0], caches[1], one[1]))
+    pair = torch.maximum(k1[..., :d // 2].abs(), k1[..., d // 2:].abs())
+    assert ((k - k1).abs() <= 2.0 ** -6 * torch.cat([pair, pair], -1) + 1e-6).all()
+    assert ((v - v1).abs() <= 2.0 ** -7 * v1.abs() + 1e-6).all()
+    for c in caches:                     # nothing outside the written positions
+        assert (c[:, :, :, :start] == 0).all() and (c[:, :, :, start + length:] == 0).all()
+    rel = ((hid.float() - hid1.float()).norm() / hid1.float().norm()).item()
+    assert rel <= 5e-3                   # one layer: the bar of the stack tests per layer
+    model.close()
+
+
+# RMSNorm: a row per CTA, 4096 values in registers, longer rows read twice.
+@pytest.mark.parametrize("rows,D", [(1, 8), (5, 1032), (3, 4088), (3, 4096), (2, 4104), (2, 12296)])
+def test_rmsnorm_row_lengths(ctx, rows, D):
+    x = I.normal_bf16(3, I.TID_X, (rows, D), 3.0)
+    y = dare.dare_rmsnorm(ctx, x.cuda(), 1e-5).float().cpu().double().numpy()
+    f = x.double().numpy()
+    ref = f / np.sqrt((f * f).mean(1, keepdims=True) + 1e-5)
+    assert (np.abs(y - ref) <= 2.0 ** -8 * np.abs(ref) + 1e-6).all()      # one rounding to bf16, fp32 sums
