@@ -329,8 +329,20 @@ struct PairPlan {
     int resident;    // clusters of this shape the device holds at once
     int stages;
     int m_pairs, n_tiles;
+    int group;       // row pairs per group of the tile order (see tile_of)
     uint32_t tmem_cols;
 };
+
+// Tile `i` of the order in which the clusters take them: groups of p.group row pairs, inside a group the row index
+// fastest.  The tiles in work at one time then share a few row pairs and a few column tiles, and a group's rows of A
+// stay in L2 while W streams past.
+struct TileAt { int m_pair, n_tile; };
+__device__ __forceinline__ TileAt tile_of(const PairPlan& p, int i) {
+    const int per_group = p.group * p.n_tiles;
+    const int g = i / per_group, r = i - g * per_group;
+    const int rows = min(p.group, p.m_pairs - g * p.group);
+    return {g * p.group + r % rows, r / rows};
+}
 
 struct PairArgs {
     int M, N, K, ldo;
@@ -434,8 +446,14 @@ struct PairBarriers {
     uint32_t abort_flag;
 };
 constexpr int PAIR_EPI_WARPS = 8;
+// Rows of A that a group of tiles keeps in L2.  The L2 is two halves of 63 MB that each cache what their SMs read: with
+// the row index fastest over all of A (67 MB at 8192 x 4096) the projections of a prefill read 0.9 to 1.3 GB from HBM
+// each where 0.17 to 0.37 would do, and the weight gradient of 2048 rows (A of 518 MB) 4.2 GB, at the power cap time as
+// well as energy.  Prefill of 16 x 512 rows in ms / forward and backward of the head on 2048 rows, by MiB per group:
+// all 12.07 / 6.68, 48 11.66 / 6.54, 32 11.62 / 6.49, 24 11.66 / 6.49, 16 11.71 / 6.49; at 4048 rows 16 and 24 lose 1 %.
+constexpr long long GROUP_BYTES = 32LL << 20;
 
-// Persistent: cluster c computes tiles c, c + #clusters, ... (row index fastest).  The copies run ahead into the
+// Persistent: cluster c computes tiles c, c + #clusters, ... of tile_of's order.  The copies run ahead into the
 // next tile, and with bn <= 256 two accumulator buffers alternate, so a tile's epilogue overlaps the next tile's
 // main loop.  With a K split every cluster has exactly one tile (the exchange needs the idle ring).
 template <int EPI>
@@ -499,7 +517,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
             uint32_t phase = 0;
             bool ok = true;
             for (int tile = cluster_id; tile < total_tiles && ok; tile += n_clusters) {
-                const int m_pair = tile % p.m_pairs, n_tile = tile / p.m_pairs;
+                const auto [m_pair, n_tile] = tile_of(p, tile);
                 const int w_row0 = EPI == GEMM_EPI_SWIGLU ? n_tile * p.wcols : n_tile * p.bn + rank * half_rows;
                 for (int kb = kb_begin; kb < kb_end; ++kb) {
                     if (!mbar_wait(&bars->empty[stage], phase ^ 1, abort_flag)) { ok = false; break; }
@@ -568,7 +586,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
     int it = 0;
     bool epi_ok = true;
     for (int tile = cluster_id; tile < total_tiles; tile += n_clusters, ++it) {
-        const int m_pair = tile % p.m_pairs, n_tile = tile / p.m_pairs;
+        const auto [m_pair, n_tile] = tile_of(p, tile);
         const int acc = it % n_acc;
         const uint32_t acc_phase = (it / n_acc) & 1;
         const int row = m_pair * 2 * GM + rank * GM + row_local;
@@ -820,6 +838,9 @@ PairPlan pair_plan(int epi, int M, int N, int K, int head_dim, double* cost_out)
             }
         }
     }
+    const long long fit = GROUP_BYTES / (static_cast<long long>(2 * GM) * 2 * K);
+    const int n_groups = static_cast<int>(fit < 1 ? m_pairs : (m_pairs + fit - 1) / fit);
+    best.group = (m_pairs + n_groups - 1) / n_groups;       // groups of even size
     if (cost_out) *cost_out = best_cost;
     return best;
 }

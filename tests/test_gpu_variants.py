@@ -70,3 +70,17 @@ def test_rmsnorm_row_lengths(ctx, rows, D):
     f = x.double().numpy()
     ref = f / np.sqrt((f * f).mean(1, keepdims=True) + 1e-5)
     assert (np.abs(y - ref) <= 2.0 ** -8 * np.abs(ref) + 1e-6).all()      # one rounding to bf16, fp32 sums
+
+
+# Projections with so many rows that the tiles are taken in groups of row pairs (32 MB of A per group): one group and a
+# row more than that, an uneven last group, K so long that a group is one row pair.
+@pytest.mark.parametrize("M,K,N", [(2048, 8192, 264), (2049, 8192, 264), (5000, 8200, 520), (600, 65544, 72)])
+def test_linear_in_row_groups(ctx, M, K, N):
+    a, w = I.normal_bf16(5, I.TID_X, (M, K)).cuda(), I.normal_bf16(5, I.TID_W, (N, K), 0.05).cuda()
+    out = dare.dare_linear(ctx, dare.LINEAR_STORE, a, w).double()
+    ref = a.double() @ w.double().T
+    torch.cuda.synchronize()
+    assert ctx.device_status() == 0
+    # one rounding to bf16 (2^-8) and fp32 sums of K products: K * 2^-24 of the sum of their magnitudes at most
+    bound = 2.0 ** -8 * ref.abs() + K * 2.0 ** -24 * (a.double().abs() @ w.double().abs().T)
+    assert ((out - ref).abs() <= bound).all()
