@@ -425,7 +425,7 @@ def bench_step_workload(dare, ctx, wl, steps, warmup, rank, world, sampler, with
         sel = masked.astype(int) == m_rows
         by_rows[str(m_rows)] = round(float(lm_each[sel].mean()) * 1e3, 1)
     lm_roof = _tensor_roofline(
-        "lmhead_greedy_kernel (+ row compaction and merge kernels)", lm_flops, lm_ms, peaks, inst_seconds, inst_clocks,
+        "lmhead_head_kernel (+ row compaction and merge kernels)", lm_flops, lm_ms, peaks, inst_seconds, inst_clocks,
         DOMINANT_TRAFFIC_BYTES.get(wl.name) if wl.name == "llada8b" else None,
         {"masked_rows_avg": masked_avg, "frac_of_tensor_or_hbm_bound_time": ideal_ms / lm_ms,
          "us_by_masked_rows": by_rows, "instrumented_steps": n_inst})

@@ -311,10 +311,10 @@ static int enqueue_step(dare_ctx* ctx, const dare::AttnArgs& a, const void* hidd
         rc = dare::launch_attn(ctx, a, s);
         if (rc != DARE_OK) return rc;
     }
-    if (sample == nullptr && L <= dare::LMHEAD_SELECT_MAX_L) {      // short blocks: the selection rides on the greedy head's merge kernel
+    if (L <= dare::LMHEAD_SELECT_MAX_L) {      // short blocks: the selection rides on the head's merge kernel
         const dare::LmSelectArgs sel = {tokens + block_start, B, mode, threshold, k, n_committed, n_remaining};
         rc = dare::launch_lmhead(ctx, ctx->workspace, hidden, M, D, w, V, tokens + block_start, L, row_stride, mask_id,
-                                 exclude_mask_column, pred, conf, head, nullptr, &sel, overlap ? ctx->ev_mid : nullptr);
+                                 exclude_mask_column, pred, conf, head, sample, &sel, overlap ? ctx->ev_mid : nullptr);
     } else {
         rc = dare::launch_lmhead(ctx, ctx->workspace, hidden, M, D, w, V, tokens + block_start, L, row_stride, mask_id,
                                  exclude_mask_column, pred, conf, head, sample, nullptr, overlap ? ctx->ev_mid : nullptr);

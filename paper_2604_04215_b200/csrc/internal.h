@@ -111,7 +111,7 @@ int launch_lmhead_logprob(const dare_ctx* ctx, void* scratch, const void* hidden
 struct LmSampleArgs { float temperature; uint64_t seed; uint32_t step; uint32_t* step_dev = nullptr; };
 size_t lmhead_workspace_bytes(int M, int D, int V, int sm_count, bool with_row_tokens, bool sampling);
 // Token of LM-head row m (to skip committed rows) = row_tokens[(m / tok_L) * tok_row_stride + m % tok_L].
-// Unmask selection folded into the head's last kernel (greedy head on a block of at most LMHEAD_SELECT_MAX_L
+// Unmask selection folded into the head's last kernel (on a block of at most LMHEAD_SELECT_MAX_L
 // positions whose tokens are given by row_tokens = tokens + block_start, tok_L = L): the caller then skips
 // launch_unmask_select.  tokens_block is the same address as row_tokens, writable.
 constexpr int LMHEAD_SELECT_MAX_L = 32;

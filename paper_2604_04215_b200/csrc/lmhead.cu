@@ -34,10 +34,6 @@ constexpr int A_BYTES = BM * BK * 2;
 constexpr int B_BYTES = BN * BK * 2;
 constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
 constexpr int LM_THREADS = 192;
-// The sampling epilogue does several times the arithmetic of the greedy one per logit (a generator block and two
-// logarithms): it gets two sets of four epilogue warps that take alternate 32-column chunks of every tile.
-constexpr int LM_SAMPLE_THREADS = 320;
-__host__ __device__ constexpr int lm_threads(int mode) { return mode == 1 ? LM_SAMPLE_THREADS : LM_THREADS; }
 constexpr uint32_t TMEM_COLS = 512;
 constexpr float LOG2E = 1.4426950408889634f;
 constexpr int ARG_NONE = 0x7fffffff;
@@ -47,7 +43,6 @@ struct LmBarriers {
     uint64_t empty[STAGES];
     uint64_t tmem_full[2];
     uint64_t tmem_empty[2];
-    uint64_t exch_full, exch_empty;      // two epilogue sets: hand-over of the second set's running values
     uint32_t tmem_base;
     uint32_t abort_flag;
 };
@@ -63,7 +58,6 @@ struct LmPairBarriers {
     uint64_t empty[PSTAGES];
     uint64_t tmem_full[2];
     uint64_t tmem_empty[2];
-    uint64_t exch_full, exch_empty;
     uint32_t tmem_base;
     uint32_t abort_flag;
 };
@@ -183,6 +177,57 @@ __device__ __forceinline__ float gumbel_from_word(uint32_t w) {
     return -logf(-logf(u));
 }
 
+// One row's 32 consecutive logits z (columns cbase ..., cbase a multiple of 32; largest: column zarg) against the row's
+// best perturbed score so far.  Two logarithms per logit cost more than the MMAs hide, and almost no logit needs them:
+// y = z / T + g beats best_y only if -ln u < t = exp(z / T - best_y), and -ln u >= 1 - u, so a logit with 1 - u > t is
+// out.  That test takes one exponential, and 1 - u comes from the generator's word by its bits: f = 1.k in [1, 2) is
+// 2 - (1 - u) - 2^-24.  The logits that pass (about one in the number of columns seen) are evaluated exactly as without
+// the test, so the sampled token is the same bit for bit: the test's t is raised by 2^(2e-3 + 1e-5 |best_y|), well over
+// the rounding of the exponent (of the size of |best_y| + 17 where the test can fail at all) and of the logarithms it
+// stands in for.  Where there is no best yet, the largest logit is evaluated first, which leaves ~3 of the 32.
+// `bound`: a score of the same row that another warp has seen (or -inf): what cannot reach it need not be evaluated.
+// at(j) returns z[j] for an index that differs from lane to lane.
+// With two logarithms per logit and twice the epilogue warps the kernel executed 159 M warp instructions in 579 k SM
+// cycles at 416 rows x 126464 and 122 M in 477 k at 384; now 73 M in 501 k and 53 M in 398 k (greedy: 21 M and 369 k).
+// Two sets of epilogue warps on top of this gain nothing: these launches sit on the power cap.
+struct SampleBest { float y, z; int arg; };
+struct SampleKey { uint32_t row, step, seed_lo, seed_hi; float inv_temperature; };
+__device__ __forceinline__ void sample_one(float z, int col, const SampleKey& key, SampleBest& best) {
+    const uint4 w4 = philox4x32_10(make_uint4(static_cast<uint32_t>(col) >> 2, key.row, key.step, 0x44415245u), key.seed_lo, key.seed_hi);
+    const uint32_t w = (col & 2) ? ((col & 1) ? w4.w : w4.z) : ((col & 1) ? w4.y : w4.x);
+    const float y = fmaf(z, key.inv_temperature, gumbel_from_word(w));
+    if (y > best.y || (y == best.y && col < best.arg)) best = {y, z, col};
+}
+template <typename At>
+__device__ __forceinline__ void sample_chunk(const float (&z)[32], int cbase, float zmax, int zarg, float bound, const SampleKey& key,
+                                             SampleBest& best, const At& at) {
+    if (best.y == -INFINITY && zmax > -INFINITY) sample_one(zmax, zarg, key, best);
+    bound = fmaxf(bound, best.y);
+    const float c2 = key.inv_temperature * LOG2E;
+    const float nb = fmaf(-LOG2E, bound, fmaf(1e-5f, fabsf(bound), 2e-3f));
+    uint32_t pass = 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const uint4 w4 = philox4x32_10(make_uint4(static_cast<uint32_t>(cbase >> 2) + q, key.row, key.step, 0x44415245u), key.seed_lo,
+                                       key.seed_hi);
+        const uint32_t ww[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const float t = fast_exp2(fmaf(z[q * 4 + e], c2, nb));
+            const float f = __uint_as_float((ww[e] >> 9) + 0x3f800000u);
+            if (f + t >= 1.99999988079071044921875f) pass |= 1u << (q * 4 + e);    // 2 - 2^-23: no rounding of the sum can hide a hit
+        }
+    }
+    while (__any_sync(0xffffffffu, pass != 0)) {
+        if (pass != 0) {
+            const int j = __ffs(pass) - 1;
+            pass &= pass - 1;
+            sample_one(at(j), cbase + j, key, best);
+        }
+        __syncwarp();
+    }
+}
+
 // MODE 0: greedy (argmax token, its probability); 1: sampling epilogue; 2: log-probability of a given target
 // token per row (the partial's third slot then carries the target's logit instead of an argmax).
 // MODE 3: gradient of the log-probability with respect to the logits, g * (onehot(target) - softmax), written as
@@ -207,8 +252,6 @@ lm_rowmajor_body(const CUtensorMap& tmap_x, const CUtensorMap& tmap_w,
     constexpr bool SAMPLE = MODE == LM_SAMPLE;
     constexpr bool LOGPROB = MODE == LM_LOGPROB;
     constexpr bool GRAD = MODE == LM_GRAD;
-    constexpr int EPI_SETS = SAMPLE ? 2 : 1;                 // sets of four epilogue warps
-    __shared__ float s_exch[5][BM];                          // (max, sum, best y, its logit, its column) per row
     if (u.m_tiles <= 0) return;
     // PAIR: a work unit is a cluster of two CTAs, an item two row tiles (one per CTA) and a vocabulary group
     const int rank = PAIR ? static_cast<int>(cluster_cta_rank()) : 0;
@@ -236,10 +279,8 @@ lm_rowmajor_body(const CUtensorMap& tmap_x, const CUtensorMap& tmap_w,
         for (int a = 0; a < 2; ++a) {
             mbar_init(&bars->tmem_full[a], 1);
             // every epilogue thread arrives (PAIR: one arrival per epilogue warp of both CTAs)
-            mbar_init(&bars->tmem_empty[a], (PAIR ? 8 : 128) * EPI_SETS);
+            mbar_init(&bars->tmem_empty[a], PAIR ? 8 : 128);
         }
-        mbar_init(&bars->exch_full, 128);
-        mbar_init(&bars->exch_empty, 128);
         bars->abort_flag = 0;
         fence_barrier_init();
     }
@@ -337,23 +378,21 @@ lm_rowmajor_body(const CUtensorMap& tmap_x, const CUtensorMap& tmap_w,
     } else if (warp >= 2) {
         // epilogue: warp w may touch TMEM lanes [32 * (w % 4), +32)
         const int lq = warp & 3;
-        const int set = (warp - 2) >> 2;
         const int row_in_tile = lq * 32 + lane;
         int it = 0;
-        int items_done = 0;
         bool ok = true;
-        for (int item = unit; item < n_items && ok; item += n_units, ++items_done) {
+        for (int item = unit; item < n_items && ok; item += n_units) {
             const int m_tile = u.tile0 + (PAIR ? 2 * (item % item_rows) + rank : item % item_rows);
             const int group = item / item_rows;
             float run_max = -INFINITY;
             float run_sum = 0.f;
             int run_arg = ARG_NONE;
-            float best_y = -INFINITY, best_z = -INFINITY;       // SAMPLE: best perturbed score, raw logit there
-            uint32_t rng_row = 0, rng_step = 0;
+            SampleBest best = {-INFINITY, -INFINITY, ARG_NONE};  // SAMPLE: best perturbed score, raw logit there, column
+            SampleKey key = {0, 0, smp.seed_lo, smp.seed_hi, smp.inv_temperature};
             if (SAMPLE) {
-                rng_step = smp.step + (smp.step_dev ? *smp.step_dev : 0u);
+                key.step = smp.step + (smp.step_dev ? *smp.step_dev : 0u);
                 const int row_c = m_tile * BM + row_in_tile;
-                rng_row = static_cast<uint32_t>(row_c < Mc && smp.row_index ? smp.row_index[row_c] : row_c);
+                key.row = static_cast<uint32_t>(row_c < Mc && smp.row_index ? smp.row_index[row_c] : row_c);
             }
             int target = -1;                                     // LOGPROB: this row's target column, its logit
             float target_z = -INFINITY;
@@ -373,14 +412,14 @@ lm_rowmajor_body(const CUtensorMap& tmap_x, const CUtensorMap& tmap_w,
                 const int acc = it & 1;
                 const uint32_t acc_phase = (it >> 1) & 1;
                 ok = mbar_wait(&bars->tmem_full[acc], acc_phase, abort_flag);
-                if (PAIR) ok = __all_sync(0xffffffffu, ok);      // the warp arrives as one further down
+                if (PAIR || SAMPLE) ok = __all_sync(0xffffffffu, ok);      // the warp works and arrives as one further down
                 if (!ok) break;
                 tc_fence_after_sync();
                 const uint32_t taddr = tmem_base + (static_cast<uint32_t>(lq * 32) << 16) + acc * BN;
                 const int col0 = n_tile * BN;
                 const bool edge = (col0 + BN > V) || (mask_col >= col0 && mask_col < col0 + BN);
 #pragma unroll 1
-                for (int c = set; c < BN / 32; c += EPI_SETS) {
+                for (int c = 0; c < BN / 32; ++c) {
                     uint32_t v[32];
                     tmem_ld_32cols(taddr + c * 32, v);
                     tmem_ld_wait();
@@ -439,18 +478,21 @@ lm_rowmajor_body(const CUtensorMap& tmap_x, const CUtensorMap& tmap_w,
                             if (cbase + j == target) target_z = __uint_as_float(v[j]);   // (-inf if it is the excluded column)
                     }
                     if (SAMPLE) {
+                        float z[32];
 #pragma unroll
-                        for (int q = 0; q < 8; ++q) {
-                            const uint4 w4 = philox4x32_10(make_uint4(static_cast<uint32_t>(cbase >> 2) + q, rng_row, rng_step,
-                                                                      0x44415245u), smp.seed_lo, smp.seed_hi);
-                            const uint32_t ww[4] = {w4.x, w4.y, w4.z, w4.w};
+                        for (int j = 0; j < 32; ++j) z[j] = __uint_as_float(v[j]);
+                        const auto at = [&](int j) {      // (a thread cannot index its registers: a tree of selects)
+                            float a[16];
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                const float z = __uint_as_float(v[q * 4 + e]);
-                                const float y = fmaf(z, smp.inv_temperature, gumbel_from_word(ww[e]));
-                                if (y > best_y) { best_y = y; best_z = z; run_arg = cbase + q * 4 + e; }   // ascending columns
+                            for (int k = 0; k < 16; ++k) a[k] = (j & 16) ? z[k + 16] : z[k];
+#pragma unroll
+                            for (int h = 8; h > 0; h >>= 1) {
+#pragma unroll
+                                for (int k = 0; k < h; ++k) a[k] = (j & h) ? a[k + h] : a[k];
                             }
-                        }
+                            return a[0];
+                        };
+                        sample_chunk(z, cbase, cmax, carg, -INFINITY, key, best, at);
                     }
                     if (cmax > -INFINITY) {
                         if (cmax > run_max) {   // tiles of a group come in ascending order: '>' keeps the lowest id
@@ -473,38 +515,13 @@ lm_rowmajor_body(const CUtensorMap& tmap_x, const CUtensorMap& tmap_w,
                     mbar_arrive(&bars->tmem_empty[acc]);
                 }
             }
-            if (EPI_SETS == 2 && ok) {
-                // the second set hands its running values to the first, which folds them into its own: the larger
-                // perturbed score wins, the lower column on a tie (each set saw its columns in ascending order)
-                const uint32_t par = items_done & 1;
-                if (set == 1) {
-                    ok = mbar_wait(&bars->exch_empty, par ^ 1, abort_flag);
-                    s_exch[0][row_in_tile] = run_max; s_exch[1][row_in_tile] = run_sum;
-                    s_exch[2][row_in_tile] = best_y; s_exch[3][row_in_tile] = best_z;
-                    s_exch[4][row_in_tile] = __int_as_float(run_arg);
-                    mbar_arrive(&bars->exch_full);          // (release: the values above are visible to the waiter)
-                } else {
-                    ok = mbar_wait(&bars->exch_full, par, abort_flag);
-                    if (ok) {
-                        const float m2 = s_exch[0][row_in_tile], s2 = s_exch[1][row_in_tile];
-                        const float y2 = s_exch[2][row_in_tile], z2 = s_exch[3][row_in_tile];
-                        const int a2 = __float_as_int(s_exch[4][row_in_tile]);
-                        mbar_arrive(&bars->exch_empty);
-                        if (m2 > -INFINITY) {
-                            if (m2 > run_max) { run_sum = run_sum * fast_exp2((run_max - m2) * LOG2E) + s2; run_max = m2; }
-                            else run_sum += s2 * fast_exp2((m2 - run_max) * LOG2E);
-                        }
-                        if (y2 > best_y || (y2 == best_y && a2 < run_arg)) { best_y = y2; best_z = z2; run_arg = a2; }
-                    }
-                }
-            }
             const int row = m_tile * BM + row_in_tile;
-            if (!GRAD && ok && row < Mc && set == 0) {
+            if (!GRAD && ok && row < Mc) {
                 const size_t o = static_cast<size_t>(row) * parts_stride + group;
                 part_max[o] = run_max;
                 part_sum[o] = run_sum;
-                part_arg[o] = LOGPROB ? __float_as_int(target_z) : run_arg;
-                if (SAMPLE) { smp.part_y[o] = best_y; smp.part_zb[o] = best_z; }
+                part_arg[o] = LOGPROB ? __float_as_int(target_z) : SAMPLE ? best.arg : run_arg;
+                if (SAMPLE) { smp.part_y[o] = best.y; smp.part_zb[o] = best.z; }
             }
         }
     }
@@ -528,7 +545,7 @@ lm_rowmajor_body(const CUtensorMap& tmap_x, const CUtensorMap& tmap_w,
 }
 
 template <int MODE, bool PAIR>
-__global__ void __launch_bounds__(lm_threads(MODE), 1)
+__global__ void __launch_bounds__(LM_THREADS, 1)
 lmhead_partial_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w,
                       int M, const int32_t* __restrict__ live_rows, int D, int V, int mask_col, int n_tiles,
                       float* __restrict__ part_max, float* __restrict__ part_sum, int32_t* __restrict__ part_arg,
@@ -543,7 +560,7 @@ lmhead_partial_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
 }
 
 // ---------------------------------------------------------------------------------------------------------
-// Greedy head with the operands swapped: the VOCABULARY sits on the accumulator's lanes (W is the MMA's A operand,
+// Greedy and sampled heads with the operands swapped: the VOCABULARY sits on the accumulator's lanes (W is the MMA's A operand,
 // 128 rows per CTA, 256 per CTA pair) and the live ROWS are its columns (the compacted X is the B operand,
 // N = the number of rows, any multiple of 16 up to 256).  What that buys over the row-major kernel above:
 //   * no padding to 128-row tiles: a step with 96 masked rows issues MMAs of N = 96, not of 128 padded rows;
@@ -559,7 +576,9 @@ lmhead_partial_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
 // a thread again holds 32 consecutive vocabulary entries of ONE row, and keeps that row's running
 // (max, sum, argmax) in registers across the group's tiles: 8 column blocks x 3 values per thread.  At the end of
 // an item the four epilogue warps fold their values through the same shared memory, and one partial per (row,
-// vocabulary group, CTA of the pair) goes to the merge kernel.
+// vocabulary group, CTA of the pair) goes to the merge kernel.  The sampled head does the same with five values per row;
+// its column blocks are a rolled loop (eight copies of the generator's code are more than the instruction cache holds),
+// so the values live in shared memory, taken off the ring (6 slots become 5 above 192 rows).
 constexpr int SW_BV = 128;                               // vocabulary rows per CTA and tile
 constexpr int SW_NMAX = 256;                             // rows (accumulator columns) per chunk
 // Row counts for which the greedy head takes this path: up to one chunk, where W is streamed once and the launch is
@@ -593,7 +612,15 @@ struct SwBarriers {
     uint32_t tmem_base;
     uint32_t abort_flag;
 };
-constexpr int SW_SMEM_BYTES = SW_STAGES * SW_STAGE_BYTES + 4 * SW_XP_FLOATS * 4 + static_cast<int>(sizeof(SwBarriers)) + 1024;
+constexpr int SW_STATE_FLOATS = 5 * SW_NMAX;            // sampled head, per epilogue warp: (max, sum, y, z, column) per row
+__host__ __device__ constexpr int sw_ring_bytes(int mode) {
+    return mode == LM_SAMPLE ? (SW_STAGES * SW_STAGE_BYTES - 3072) : SW_STAGES * SW_STAGE_BYTES;
+}
+__host__ __device__ constexpr int sw_smem_bytes(int mode) {
+    return sw_ring_bytes(mode) + 4 * SW_XP_FLOATS * 4 + (mode == LM_SAMPLE ? 4 * SW_STATE_FLOATS * 4 : 0) +
+           static_cast<int>(sizeof(SwBarriers)) + 1024;
+}
+static_assert(sw_smem_bytes(LM_SAMPLE) <= 227 * 1024 && sw_smem_bytes(LM_GREEDY) <= 227 * 1024, "shared memory");
 // X tiles of 128, 64, 32, 16 and 8 rows: a CTA's share of a chunk (a multiple of 8 rows) is covered by one or two
 // of them, stacked in shared memory (each a whole number of 1 KB swizzle atoms); a few rows too many may be loaded,
 // the MMA reads only its own.  (Exact covers of up to four boxes were measured slower: 432 us for 480 rows, where
@@ -631,10 +658,12 @@ __host__ __device__ inline SwPlan sw_plan(int rows, int n_units, int n_vt) {
     return p;
 }
 
+template <int MODE>
 __device__ __forceinline__ void
 lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, int V, int mask_col, int n_vt,
                 float* __restrict__ part_max, float* __restrict__ part_sum, int32_t* __restrict__ part_arg,
-                uint32_t* __restrict__ dev_status, int parts_stride) {
+                uint32_t* __restrict__ dev_status, int parts_stride, const LmSampling& smp) {
+    constexpr bool SAMPLE = MODE == LM_SAMPLE;
     if (Mc <= 0) return;
     const int rank = static_cast<int>(cluster_cta_rank());
     const int unit = blockIdx.x >> 1;
@@ -647,8 +676,9 @@ lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, 
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    float* xpose = reinterpret_cast<float*>(tiles + SW_STAGES * SW_STAGE_BYTES);
-    SwBarriers* bars = reinterpret_cast<SwBarriers*>(xpose + 4 * SW_XP_FLOATS);
+    float* xpose = reinterpret_cast<float*>(tiles + sw_ring_bytes(MODE));
+    float* state = xpose + 4 * SW_XP_FLOATS;             // SAMPLE: [warp][value][row]
+    SwBarriers* bars = reinterpret_cast<SwBarriers*>(state + (SAMPLE ? 4 * SW_STATE_FLOATS : 0));
     volatile uint32_t* abort_flag = &bars->abort_flag;
 
     const int warp = warp_index_uniform();
@@ -659,7 +689,16 @@ lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, 
     // bandwidth (6 slots per CTA, 14 MB over the GPU, covered ~2 us of HBM latency at 6.3 TB/s and no more).
     const SwBoxes xbox = sw_boxes(rows_half);
     const int stage_bytes = SW_W_BYTES + ((xbox.rows * 128 + 1023) & ~1023);
-    const int n_stages = min(SW_MAX_STAGES, SW_STAGES * SW_STAGE_BYTES / stage_bytes);
+    const int n_stages = min(SW_MAX_STAGES, sw_ring_bytes(MODE) / stage_bytes);
+    // no logit seen yet (set here and by the fold at an item's end: the warps read one another's best scores at any time)
+    const auto clear_state = [&](int q, int r) {
+        float* s = state + q * SW_STATE_FLOATS + r;
+        s[0] = s[2 * SW_NMAX] = s[3 * SW_NMAX] = -INFINITY;
+        s[SW_NMAX] = 0.f;
+        s[4 * SW_NMAX] = __int_as_float(ARG_NONE);
+    };
+    if (SAMPLE)
+        for (int i = threadIdx.x; i < 4 * SW_NMAX; i += LM_THREADS) clear_state(i / SW_NMAX, i % SW_NMAX);
     if (threadIdx.x == 0) {
         for (int s = 0; s < n_stages; ++s) {
             mbar_init(&bars->full[s], 1);
@@ -753,6 +792,8 @@ lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, 
         // epilogue: warp w may touch TMEM lanes [32 * (w % 4), +32) = 32 consecutive vocabulary entries of the tile
         const int lq = warp & 3;
         float* xp = xpose + lq * SW_XP_FLOATS;
+        float* st = state + lq * SW_STATE_FLOATS;
+        const uint32_t rng_step = SAMPLE ? smp.step + (smp.step_dev ? *smp.step_dev : 0u) : 0u;
         int it = 0;
         uint32_t items_done = 0;
         bool ok = true;
@@ -772,43 +813,77 @@ lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, 
                 const uint32_t taddr = tmem_base + (static_cast<uint32_t>(lq * 32) << 16) + acc * SW_NMAX;
                 const int vbase = vt * (2 * SW_BV) + rank * SW_BV + lq * 32;     // first vocabulary entry of this warp's lanes
                 const bool edge = (vbase + 32 > V) || (mask_col >= vbase && mask_col < vbase + 32);
-                if (vbase < V) {
+                // column block cb: turned, so that this thread holds 32 consecutive vocabulary entries of one row; returns
+                // their maximum and its entry
+                const auto load_block = [&](int cb, float (&z)[32], float& cmax, int& carg) {
+                    uint32_t v[32];
+                    tmem_ld_32cols(taddr + cb * 32, v);
+                    tmem_ld_wait();
+                    // turn the block: in, thread = vocabulary entry with 32 rows; out, thread = row with 32 entries
+#pragma unroll
+                    for (int c = 0; c < 32; ++c) xp[lane * 33 + c] = __uint_as_float(v[c]);
+                    __syncwarp();
+#pragma unroll
+                    for (int l = 0; l < 32; ++l) z[l] = xp[l * 33 + lane];
+                    __syncwarp();
+                    if (edge) {
+#pragma unroll
+                        for (int l = 0; l < 32; ++l)
+                            if (vbase + l >= V || vbase + l == mask_col) z[l] = -INFINITY;
+                    }
+                    cmax = -INFINITY;
+                    carg = ARG_NONE;
+#pragma unroll
+                    for (int l = 0; l < 32; ++l)
+                        if (z[l] > cmax) { cmax = z[l]; carg = vbase + l; }       // strict '>' keeps the lowest id
+                };
+                // (max, sum) of a row with 32 more logits; tiles of a group come in ascending order: '>' keeps the lowest id
+                const auto add_block = [&](const float (&z)[32], float cmax, int carg, float& rmax, float& rsum, int& rarg) {
+                    if (cmax > -INFINITY) {
+                        if (cmax > rmax) {
+                            rsum *= fast_exp2((rmax - cmax) * LOG2E);   // exp2(-inf) = 0 the first time
+                            rmax = cmax;
+                            rarg = carg;
+                        }
+                        const float mb = rmax * LOG2E;
+                        float sum = 0.f;
+#pragma unroll
+                        for (int l = 0; l < 32; ++l) sum += fast_exp2(fmaf(z[l], LOG2E, -mb));
+                        rsum += sum;
+                    }
+                };
+                if (SAMPLE) {
+#pragma unroll 1
+                    for (int cb = 0; vbase < V && cb * 32 < nc; ++cb) {
+                        float z[32], cmax;
+                        int carg;
+                        load_block(cb, z, cmax, carg);
+                        const int r = cb * 32 + lane;
+                        const int row = chunk * nc + r;
+                        const uint32_t rng_row = static_cast<uint32_t>(r < nc && row < Mc && smp.row_index ? smp.row_index[row] : row);
+                        float rmax = st[r], rsum = st[SW_NMAX + r];
+                        SampleBest best = {st[2 * SW_NMAX + r], st[3 * SW_NMAX + r], __float_as_int(st[4 * SW_NMAX + r])};
+                        int ignored = 0;
+                        add_block(z, cmax, carg, rmax, rsum, ignored);
+                        float bound = -INFINITY;          // what the other warps have seen of this row (any time up to now will do)
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            bound = fmaxf(bound, *static_cast<volatile float*>(state + q * SW_STATE_FLOATS + 2 * SW_NMAX + r));
+                        const SampleKey key = {rng_row, rng_step, smp.seed_lo, smp.seed_hi, smp.inv_temperature};
+                        const auto at = [&](int j) { return vbase + j >= V || vbase + j == mask_col ? -INFINITY : xp[j * 33 + lane]; };
+                        sample_chunk(z, vbase, cmax, carg, bound, key, best, at);
+                        __syncwarp();                     // the block may be overwritten
+                        st[r] = rmax; st[SW_NMAX + r] = rsum;
+                        st[2 * SW_NMAX + r] = best.y; st[3 * SW_NMAX + r] = best.z; st[4 * SW_NMAX + r] = __int_as_float(best.arg);
+                    }
+                } else if (vbase < V) {
 #pragma unroll
                     for (int cb = 0; cb < SW_NMAX / 32; ++cb) {
                         if (cb * 32 < nc) {
-                            uint32_t v[32];
-                            tmem_ld_32cols(taddr + cb * 32, v);
-                            tmem_ld_wait();
-                            // turn the block: in, thread = vocabulary entry with 32 rows; out, thread = row with 32 entries
-#pragma unroll
-                            for (int c = 0; c < 32; ++c) xp[lane * 33 + c] = __uint_as_float(v[c]);
-                            __syncwarp();
-                            float z[32];
-#pragma unroll
-                            for (int l = 0; l < 32; ++l) z[l] = xp[l * 33 + lane];
-                            __syncwarp();
-                            if (edge) {
-#pragma unroll
-                                for (int l = 0; l < 32; ++l)
-                                    if (vbase + l >= V || vbase + l == mask_col) z[l] = -INFINITY;
-                            }
-                            float cmax = -INFINITY;
-                            int carg = ARG_NONE;
-#pragma unroll
-                            for (int l = 0; l < 32; ++l)
-                                if (z[l] > cmax) { cmax = z[l]; carg = vbase + l; }       // strict '>' keeps the lowest id
-                            if (cmax > -INFINITY) {
-                                if (cmax > run_max[cb]) {     // tiles of a group come in ascending order: '>' keeps the lowest id
-                                    run_sum[cb] *= fast_exp2((run_max[cb] - cmax) * LOG2E);   // exp2(-inf) = 0 the first time
-                                    run_max[cb] = cmax;
-                                    run_arg[cb] = carg;
-                                }
-                                const float mb = run_max[cb] * LOG2E;
-                                float sum = 0.f;
-#pragma unroll
-                                for (int l = 0; l < 32; ++l) sum += fast_exp2(fmaf(z[l], LOG2E, -mb));
-                                run_sum[cb] += sum;
-                            }
+                            float z[32], cmax;
+                            int carg;
+                            load_block(cb, z, cmax, carg);
+                            add_block(z, cmax, carg, run_max[cb], run_sum[cb], run_arg[cb]);
                         }
                     }
                 }
@@ -819,11 +894,13 @@ lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, 
             if (ok) {
                 // fold the four warps' values (each saw a quarter of every tile's vocabulary entries): every warp
                 // leaves its own in its block of shared memory, then warp q folds column blocks 2 q and 2 q + 1
+                if (!SAMPLE) {
 #pragma unroll
-                for (int cb = 0; cb < SW_NMAX / 32; ++cb) {
-                    xp[(cb * 3 + 0) * 32 + lane] = run_max[cb];
-                    xp[(cb * 3 + 1) * 32 + lane] = run_sum[cb];
-                    xp[(cb * 3 + 2) * 32 + lane] = __int_as_float(run_arg[cb]);
+                    for (int cb = 0; cb < SW_NMAX / 32; ++cb) {
+                        xp[(cb * 3 + 0) * 32 + lane] = run_max[cb];
+                        xp[(cb * 3 + 1) * 32 + lane] = run_sum[cb];
+                        xp[(cb * 3 + 2) * 32 + lane] = __int_as_float(run_arg[cb]);
+                    }
                 }
                 mbar_arrive(&bars->fold_full);            // (release: the values above are visible to the waiters)
                 ok = __all_sync(0xffffffffu, mbar_wait(&bars->fold_full, items_done & 1, abort_flag));
@@ -834,7 +911,24 @@ lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, 
                         if (col < nc && row < Mc) {
                             float m = -INFINITY, sum = 0.f;
                             int a = ARG_NONE;
-                            for (int q = 0; q < 4; ++q) {
+                            if (SAMPLE) {
+                                SampleBest best = {-INFINITY, -INFINITY, ARG_NONE};
+                                for (int q = 0; q < 4; ++q) {
+                                    const float* src = state + q * SW_STATE_FLOATS + col;
+                                    const float m2 = src[0], s2 = src[SW_NMAX], y2 = src[2 * SW_NMAX];
+                                    const int a2 = __float_as_int(src[4 * SW_NMAX]);
+                                    if (m2 > -INFINITY) {
+                                        if (m2 > m) { sum = sum * fast_exp2((m - m2) * LOG2E) + s2; m = m2; }
+                                        else sum += s2 * fast_exp2((m2 - m) * LOG2E);
+                                    }
+                                    if (y2 > best.y || (y2 == best.y && a2 < best.arg)) best = {y2, src[3 * SW_NMAX], a2};
+                                }
+                                const size_t o = static_cast<size_t>(row) * parts_stride + group * 2 + rank;
+                                smp.part_y[o] = best.y;
+                                smp.part_zb[o] = best.z;
+                                a = best.arg;
+                            }
+                            for (int q = 0; q < (SAMPLE ? 0 : 4); ++q) {
                                 const float* src = xpose + q * SW_XP_FLOATS + cb * 96 + lane;
                                 const float m2 = src[0], s2 = src[32];
                                 const int a2 = __float_as_int(src[64]);
@@ -848,6 +942,8 @@ lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, 
                             part_sum[o] = sum;
                             part_arg[o] = a;
                         }
+                        if (SAMPLE)
+                            for (int q = 0; q < 4; ++q) clear_state(q, col);
                     }
                     mbar_arrive(&bars->fold_empty);       // the blocks may be written again once all have read
                     ok = __all_sync(0xffffffffu, mbar_wait(&bars->fold_empty, items_done & 1, abort_flag));
@@ -884,52 +980,53 @@ __host__ __device__ inline int lm_mixed_pair_clusters(int n_clusters, int p) {
     return up;
 }
 
-// The greedy head, one launch on CTA pairs whatever the number of live rows (known only on the device when rows are
+// The greedy (or sampled) head, one launch on CTA pairs whatever the number of live rows (known only on the device when rows are
 // skipped): the swapped-operand path for the counts lm_greedy_swapped names (up to SW_NMAX rows, and counts that
 // cut into long chunks); otherwise row-major tiles of 128 rows, on CTA pairs when the tiles come in twos, and for
 // an odd count on pairs plus single CTAs for the last tile (see above).  The W
 // tile box is 128 rows for all of them.  A row's partials start at row * parts_stride; how many there are follows
 // from the same rules in lm_row_partials.
+template <int MODE>
 __global__ void __launch_bounds__(LM_THREADS, 1)
-lmhead_greedy_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ SwXMaps xmaps, int M,
+lmhead_head_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ SwXMaps xmaps, int M,
                      const int32_t* __restrict__ live_rows, int D, int V, int mask_col, int n_tiles,
                      float* __restrict__ part_max, float* __restrict__ part_sum, int32_t* __restrict__ part_arg,
-                     uint32_t* __restrict__ dev_status, int parts_stride) {
+                     uint32_t* __restrict__ dev_status, int parts_stride, const LmSampling smp) {
     const int Mc = live_rows ? *live_rows : M;          // rows that need logits (uniform over the grid)
     if (lm_greedy_swapped(Mc)) {
-        lm_swapped_body(tmap_w, xmaps, Mc, D, V, mask_col, n_tiles, part_max, part_sum, part_arg, dev_status, parts_stride);
+        lm_swapped_body<MODE>(tmap_w, xmaps, Mc, D, V, mask_col, n_tiles, part_max, part_sum, part_arg, dev_status, parts_stride,
+                              smp);
         return;
     }
-    const LmSampling none = {};
     const int m_tiles = (Mc + BM - 1) / BM;
     const int cluster = blockIdx.x >> 1, n_clusters = gridDim.x >> 1;
     if ((m_tiles & 1) == 0) {
         const LmUnits u = {cluster, n_clusters, 0, m_tiles, parts_stride};
-        lm_rowmajor_body<LM_GREEDY, true>(xmaps.m[0], tmap_w, Mc, D, V, mask_col, n_tiles, part_max, part_sum, part_arg,
-                                          dev_status, none, u);
+        lm_rowmajor_body<MODE, true>(xmaps.m[0], tmap_w, Mc, D, V, mask_col, n_tiles, part_max, part_sum, part_arg,
+                                          dev_status, smp, u);
     } else if (n_clusters < 2) {
         const LmUnits u = {static_cast<int>(blockIdx.x), static_cast<int>(gridDim.x), 0, m_tiles, parts_stride};
-        lm_rowmajor_body<LM_GREEDY, false, true>(xmaps.m[0], tmap_w, Mc, D, V, mask_col, n_tiles, part_max, part_sum,
-                                                 part_arg, dev_status, none, u);
+        lm_rowmajor_body<MODE, false, true>(xmaps.m[0], tmap_w, Mc, D, V, mask_col, n_tiles, part_max, part_sum,
+                                                 part_arg, dev_status, smp, u);
     } else {
         const int p = m_tiles >> 1;
         const int up = lm_mixed_pair_clusters(n_clusters, p);
         if (cluster < up) {
             const LmUnits u = {cluster, up, 0, 2 * p, parts_stride};
-            lm_rowmajor_body<LM_GREEDY, true>(xmaps.m[0], tmap_w, Mc, D, V, mask_col, n_tiles, part_max, part_sum,
-                                              part_arg, dev_status, none, u);
+            lm_rowmajor_body<MODE, true>(xmaps.m[0], tmap_w, Mc, D, V, mask_col, n_tiles, part_max, part_sum,
+                                              part_arg, dev_status, smp, u);
         } else {
             const LmUnits u = {static_cast<int>(blockIdx.x) - 2 * up, static_cast<int>(gridDim.x) - 2 * up, 2 * p, 1,
                                parts_stride};
-            lm_rowmajor_body<LM_GREEDY, false, true>(xmaps.m[0], tmap_w, Mc, D, V, mask_col, n_tiles, part_max, part_sum,
-                                                     part_arg, dev_status, none, u);
+            lm_rowmajor_body<MODE, false, true>(xmaps.m[0], tmap_w, Mc, D, V, mask_col, n_tiles, part_max, part_sum,
+                                                     part_arg, dev_status, smp, u);
         }
     }
 }
 
 // Partials of live row `row`, as the GEMM that ran wrote them (they start at row * stride).  layout 0 / 1: the
 // stand-alone row-major kernels (single CTAs only / CTA pairs where they apply), one partial per vocabulary group,
-// packed (stride = count).  layout 2: lmhead_greedy_kernel's rules.  `grid` = CTAs of the GEMM launch, n_tiles =
+// packed (stride = count).  layout 2: lmhead_head_kernel's rules.  `grid` = CTAs of the GEMM launch, n_tiles =
 // vocabulary tiles of 256.
 constexpr int LM_LAYOUT_GREEDY = 2;
 __host__ __device__ inline int lm_row_partials(int layout, int grid, int rows, int n_tiles, int row) {
@@ -944,71 +1041,72 @@ __host__ __device__ inline int lm_row_partials(int layout, int grid, int rows, i
     return row < 2 * p * BM ? lm_groups(up, p, n_tiles) : lm_groups(grid - 2 * up, 1, n_tiles);
 }
 
-// Fold of one row's partial triples by a warp: returns (argmax token, sum of exp relative to the maximum) in all
-// lanes.  Ties of the maximum go to the lowest token id.
-__device__ __forceinline__ void merge_row_partials(const float* __restrict__ part_max, const float* __restrict__ part_sum,
-                                                   const int32_t* __restrict__ part_arg, size_t base, int groups, int lane,
-                                                   int& a_out, float& s_out) {
-    float m = -INFINITY, s = 0.f;
+// Fold of one row's partials by a warp: the token and its confidence, in all lanes.  Greedy: the token of the largest
+// logit (lowest id on ties), confidence = exp(max - logsumexp) = 1 / (sum of exp relative to the maximum).  Sampled: the
+// token of the best perturbed score (lowest id on ties), confidence = exp(z_token - logsumexp z).
+struct LmParts { const float *max, *sum; const int32_t* arg; const float *y, *zb; };
+template <bool SAMPLE>
+__device__ __forceinline__ void merge_row_partials(const LmParts& p, size_t base, int groups, int lane, int& a_out, float& conf_out) {
+    float m = -INFINITY, s = 0.f, y = -INFINITY, zb = -INFINITY;
     int a = ARG_NONE;
+    const auto fold = [&](float m2, float s2, int a2, float y2, float z2) {
+        if (m2 > -INFINITY) {
+            if (m2 > m) { s = s * exp2f((m - m2) * LOG2E) + s2; m = m2; if (!SAMPLE) a = a2; }
+            else { s += s2 * exp2f((m2 - m) * LOG2E); if (!SAMPLE && m2 == m && a2 < a) a = a2; }
+        }
+        if (SAMPLE && (y2 > y || (y2 == y && a2 < a))) { y = y2; a = a2; zb = z2; }
+    };
     // the loads of a batch are issued together (five per lane cover 160 partials: one round trip to memory for the
     // usual case), then folded
     constexpr int BATCH = 5;
     for (int t0 = lane; t0 < groups; t0 += 32 * BATCH) {
-        float bm[BATCH], bs[BATCH];
+        float bm[BATCH], bs[BATCH], by[BATCH], bz[BATCH];
         int ba[BATCH];
 #pragma unroll
         for (int u = 0; u < BATCH; ++u) {
             const int t = t0 + 32 * u;
             const bool in = t < groups;
-            bm[u] = in ? part_max[base + t] : -INFINITY;
-            bs[u] = in ? part_sum[base + t] : 0.f;
-            ba[u] = in ? part_arg[base + t] : ARG_NONE;
+            bm[u] = in ? p.max[base + t] : -INFINITY;
+            bs[u] = in ? p.sum[base + t] : 0.f;
+            ba[u] = in ? p.arg[base + t] : ARG_NONE;
+            by[u] = SAMPLE && in ? p.y[base + t] : -INFINITY;
+            bz[u] = SAMPLE && in ? p.zb[base + t] : -INFINITY;
         }
 #pragma unroll
-        for (int u = 0; u < BATCH; ++u) {
-            const float m2 = bm[u], s2 = bs[u];
-            const int a2 = ba[u];
-            if (m2 > -INFINITY) {
-                if (m2 > m) { s = s * exp2f((m - m2) * LOG2E) + s2; m = m2; a = a2; }
-                else { s += s2 * exp2f((m2 - m) * LOG2E); if (m2 == m && a2 < a) a = a2; }
-            }
-        }
+        for (int u = 0; u < BATCH; ++u) fold(bm[u], bs[u], ba[u], by[u], bz[u]);
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
-        const float m2 = __shfl_xor_sync(0xffffffffu, m, off);
-        const float s2 = __shfl_xor_sync(0xffffffffu, s, off);
+        const float m2 = __shfl_xor_sync(0xffffffffu, m, off), s2 = __shfl_xor_sync(0xffffffffu, s, off);
         const int a2 = __shfl_xor_sync(0xffffffffu, a, off);
-        if (m2 > -INFINITY) {
-            if (m2 > m) { s = s * exp2f((m - m2) * LOG2E) + s2; m = m2; a = a2; }
-            else { s += s2 * exp2f((m2 - m) * LOG2E); if (m2 == m && a2 < a) a = a2; }
-        }
+        const float y2 = SAMPLE ? __shfl_xor_sync(0xffffffffu, y, off) : 0.f;
+        const float z2 = SAMPLE ? __shfl_xor_sync(0xffffffffu, zb, off) : 0.f;
+        fold(m2, s2, a2, y2, z2);
     }
     a_out = a;
-    s_out = s;
+    conf_out = SAMPLE ? exp2f((zb - m) * LOG2E) / s : 1.0f / s;
 }
 
-// One warp per live row: fold the row's partial triples (one per vocabulary group) into (token, confidence)
-// and write them at the row's original position.
-__global__ void lmhead_merge_kernel(const float* __restrict__ part_max, const float* __restrict__ part_sum,
-                                    const int32_t* __restrict__ part_arg, int grid_gemm, int n_tiles, int M,
+// One warp per live row: fold the row's partials (one or two per vocabulary group) into (token, confidence) and write
+// them at the row's original position.
+template <bool SAMPLE>
+__global__ void lmhead_merge_kernel(const LmParts parts, int grid_gemm, int n_tiles, int M,
                                     const int32_t* __restrict__ live_rows, const int32_t* __restrict__ idx,
                                     int32_t* __restrict__ pred, float* __restrict__ conf, int allow_pair,
-                                    int parts_stride) {
+                                    int parts_stride, uint32_t* __restrict__ step_dev) {
+    if (SAMPLE && step_dev && blockIdx.x == 0 && threadIdx.x == 0) *step_dev += 1;   // the GEMM kernels before this one read it
     const int c = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     const int Mc = live_rows ? *live_rows : M;
     if (c >= Mc) return;
     const int groups = lm_row_partials(allow_pair, grid_gemm, Mc, n_tiles, c);
     int a;
-    float s;
-    merge_row_partials(part_max, part_sum, part_arg, static_cast<size_t>(c) * (parts_stride < 0 ? groups : parts_stride),
-                       groups, lane, a, s);
+    float cf;
+    merge_row_partials<SAMPLE>(parts, static_cast<size_t>(c) * (parts_stride < 0 ? groups : parts_stride), groups, lane, a, cf);
     if (lane == 0) {
         const int row = idx ? idx[c] : c;
         pred[row] = a;
-        conf[row] = 1.0f / s;   // exp(max - logsumexp) with the sum taken relative to the max
+        conf[row] = cf;
     }
 }
 
@@ -1026,16 +1124,17 @@ struct LmSelect {
     int32_t* n_committed;
     int32_t* n_remaining;
 };
+template <bool SAMPLE>
 __global__ void __launch_bounds__(1024)
-lmhead_merge_select_kernel(const float* __restrict__ part_max, const float* __restrict__ part_sum,
-                           const int32_t* __restrict__ part_arg, int grid_gemm, int n_tiles, int L,
+lmhead_merge_select_kernel(const LmParts parts, int grid_gemm, int n_tiles, int L,
                            const int32_t* __restrict__ live_rows, const int32_t* __restrict__ idx, int32_t mask_id,
                            int32_t* __restrict__ pred, float* __restrict__ conf, int allow_pair, int parts_stride,
-                           const LmSelect sel) {
+                           const LmSelect sel, uint32_t* __restrict__ step_dev) {
     __shared__ int s_before;
     __shared__ int s_flag[32];
     __shared__ float s_conf[32];
     __shared__ int32_t s_pred[32];
+    if (SAMPLE && step_dev && blockIdx.x == 0 && threadIdx.x == 0) *step_dev += 1;   // (as in lmhead_merge_kernel)
     const int b = blockIdx.x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;      // warp = block position (blockDim = 32 L)
     const int Mc = *live_rows;
@@ -1057,11 +1156,9 @@ lmhead_merge_select_kernel(const float* __restrict__ part_max, const float* __re
         for (int i = 0; i < warp; ++i) c += s_flag[i];
         const int groups = lm_row_partials(allow_pair, grid_gemm, Mc, n_tiles, c);
         int a;
-        float s;
-        merge_row_partials(part_max, part_sum, part_arg, static_cast<size_t>(c) * (parts_stride < 0 ? groups : parts_stride),
-                           groups, lane, a, s);
+        float cf;
+        merge_row_partials<SAMPLE>(parts, static_cast<size_t>(c) * (parts_stride < 0 ? groups : parts_stride), groups, lane, a, cf);
         if (lane == 0) {
-            float cf = 1.0f / s;
             pred[b * L + warp] = a;
             conf[b * L + warp] = cf;
             if (cf != cf) cf = -INFINITY;
@@ -1097,53 +1194,6 @@ lmhead_merge_select_kernel(const float* __restrict__ part_max, const float* __re
     if (lane == 0) {
         if (sel.n_committed) sel.n_committed[b] = __popc(commit_set);
         if (sel.n_remaining) sel.n_remaining[b] = __popc(masked_set) - __popc(commit_set);
-    }
-}
-
-// The same fold for the sampling epilogue: log-sum-exp of the raw logits from (max, sum); the sampled token is the
-// partial with the best perturbed score (lowest token id on ties); confidence = exp(z_token - logsumexp z).
-__global__ void lmhead_merge_sample_kernel(const float* __restrict__ part_max, const float* __restrict__ part_sum,
-                                           const int32_t* __restrict__ part_arg, const float* __restrict__ part_y,
-                                           const float* __restrict__ part_zb, int grid_gemm, int n_tiles, int M,
-                                           const int32_t* __restrict__ live_rows, const int32_t* __restrict__ idx,
-                                           int32_t* __restrict__ pred, float* __restrict__ conf, int allow_pair,
-                                           uint32_t* __restrict__ step_dev) {
-    if (step_dev && blockIdx.x == 0 && threadIdx.x == 0) *step_dev += 1;   // the GEMM kernels before this one read it
-    const int c = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    const int Mc = live_rows ? *live_rows : M;
-    if (c >= Mc) return;
-    const int groups = lm_groups_mode(grid_gemm, (Mc + BM - 1) / BM, n_tiles, allow_pair);
-    float m = -INFINITY, s = 0.f, y = -INFINITY, zb = -INFINITY;
-    int a = ARG_NONE;
-    const size_t base = static_cast<size_t>(c) * groups;
-    for (int t = lane; t < groups; t += 32) {
-        const float m2 = part_max[base + t], s2 = part_sum[base + t];
-        if (m2 > -INFINITY) {
-            if (m2 > m) { s = s * exp2f((m - m2) * LOG2E) + s2; m = m2; }
-            else s += s2 * exp2f((m2 - m) * LOG2E);
-        }
-        const float y2 = part_y[base + t];
-        const int a2 = part_arg[base + t];
-        if (y2 > y || (y2 == y && a2 < a)) { y = y2; a = a2; zb = part_zb[base + t]; }
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        const float m2 = __shfl_xor_sync(0xffffffffu, m, off);
-        const float s2 = __shfl_xor_sync(0xffffffffu, s, off);
-        const float y2 = __shfl_xor_sync(0xffffffffu, y, off);
-        const float z2 = __shfl_xor_sync(0xffffffffu, zb, off);
-        const int a2 = __shfl_xor_sync(0xffffffffu, a, off);
-        if (m2 > -INFINITY) {
-            if (m2 > m) { s = s * exp2f((m - m2) * LOG2E) + s2; m = m2; }
-            else s += s2 * exp2f((m2 - m) * LOG2E);
-        }
-        if (y2 > y || (y2 == y && a2 < a)) { y = y2; a = a2; zb = z2; }
-    }
-    if (lane == 0) {
-        const int row = idx ? idx[c] : c;
-        pred[row] = a;
-        conf[row] = exp2f((zb - m) * LOG2E) / s;
     }
 }
 
@@ -1226,7 +1276,7 @@ int launch_partial(const dare_ctx* ctx, int grid, const CUtensorMap& tmap_x, con
         if (rc != DARE_OK) return rc;
         static std::atomic<uint64_t> smem_set{0};
         if (ensure_dynamic_smem(smem_set, lmhead_partial_kernel<MODE, false>, LM_SMEM_BYTES) != DARE_OK) return DARE_ERR_CUDA;
-        lmhead_partial_kernel<MODE, false><<<grid, lm_threads(MODE), LM_SMEM_BYTES, stream>>>(
+        lmhead_partial_kernel<MODE, false><<<grid, LM_THREADS, LM_SMEM_BYTES, stream>>>(
             tmap_x, tmap_w, M, live_rows, D, V, mask_col, n_tiles, part_max, part_sum, part_arg, ctx->dev_status, smp,
             allow_pair); note_launch();
         if (cudaGetLastError() != cudaSuccess) return DARE_ERR_CUDA;
@@ -1240,7 +1290,7 @@ int launch_partial(const dare_ctx* ctx, int grid, const CUtensorMap& tmap_x, con
             return DARE_ERR_CUDA;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(static_cast<unsigned>(grid & ~1), 1, 1);
-        cfg.blockDim = dim3(lm_threads(MODE), 1, 1);
+        cfg.blockDim = dim3(LM_THREADS, 1, 1);
         cfg.dynamicSmemBytes = LM_PAIR_SMEM_BYTES;
         cfg.stream = stream;
         cudaLaunchAttribute attr;
@@ -1259,25 +1309,97 @@ int launch_partial(const dare_ctx* ctx, int grid, const CUtensorMap& tmap_x, con
 }  // namespace
 
 // Scratch layout: [compacted X: M*D bf16][row indices: M int32][live-row count][partials: 3 x M x groups]
-size_t lmhead_workspace_bytes(int M, int D, int V, int sm_count, bool with_row_tokens, bool sampling) {
+static size_t lmhead_scratch_bytes(int M, int D, int V, int sm_count, bool with_row_tokens, bool sampling, int parts_per_tile) {
     const size_t n_tiles = (static_cast<size_t>(V) + BN - 1) / BN;
     size_t groups = static_cast<size_t>(sm_count);
-    if (groups > n_tiles) groups = n_tiles;
-    if (!sampling) {      // the greedy head's swapped path: two partials per vocabulary group of a CTA pair
-        groups = static_cast<size_t>(sm_count);
-        if (groups > 2 * n_tiles) groups = 2 * n_tiles;
-    }
+    if (groups > parts_per_tile * n_tiles) groups = parts_per_tile * n_tiles;
     size_t bytes = (sampling ? 5 : 3) * sizeof(float) * groups * static_cast<size_t>(M);
     if (with_row_tokens)
         bytes += round_up(static_cast<size_t>(M) * D * 2, 1024) + round_up(static_cast<size_t>(M) * 4 + 4, 1024);
     return bytes;
+}
+// (the swapped path leaves two partials per vocabulary group of a CTA pair; the sampled head can do without that path)
+size_t lmhead_workspace_bytes(int M, int D, int V, int sm_count, bool with_row_tokens, bool sampling) {
+    return lmhead_scratch_bytes(M, D, V, sm_count, with_row_tokens, sampling, sampling ? 1 : 2);
+}
+
+// The head's GEMM, its merge and, with `select`, the unmask selection, for one epilogue.
+template <int MODE>
+static int launch_head(const dare_ctx* ctx, int grid, bool pairs, const void* x_gemm, int M, int D, const void* w, int V,
+                       int mask_col, int n_tiles, const int32_t* live_rows, const int32_t* idx, float* parts, LmSampling smp,
+                       uint32_t* step_dev, int tok_L, int64_t tok_row_stride, int32_t mask_id, int32_t* pred, float* conf,
+                       const LmSelectArgs* select, cudaStream_t stream) {
+    constexpr bool SAMPLE = MODE == LM_SAMPLE;
+    size_t parts_max = pairs ? (grid & ~1) : ctx->sm_count;      // pairs: a fixed stride, at most two partials per vocabulary tile
+    const size_t tile_parts = static_cast<size_t>(pairs ? 2 : 1) * n_tiles;
+    if (parts_max > tile_parts) parts_max = tile_parts;
+    const size_t n_part = static_cast<size_t>(M) * parts_max;
+    float* part_max = parts;
+    float* part_sum = part_max + n_part;
+    int32_t* part_arg = reinterpret_cast<int32_t*>(part_sum + n_part);
+    if (SAMPLE) {
+        smp.part_y = reinterpret_cast<float*>(part_arg + n_part);
+        smp.part_zb = smp.part_y + n_part;
+    }
+    int rc = DARE_OK, layout = LM_LAYOUT_GREEDY, parts_stride = -1, grid_gemm = grid;
+    if (pairs) {
+        CUtensorMap tmap_w;
+        SwXMaps xm;
+        rc = make_tmap_bf16_2d(ctx, &tmap_w, w, static_cast<uint64_t>(V), static_cast<uint64_t>(D), SW_BV, BK);
+        for (int i = 0; i < 5 && rc == DARE_OK; ++i)
+            rc = make_tmap_bf16_2d(ctx, &xm.m[i], x_gemm, static_cast<uint64_t>(M), static_cast<uint64_t>(D), 128u >> i, BK);
+        if (rc != DARE_OK) return rc;
+        grid_gemm = grid & ~1;
+        parts_stride = static_cast<int>(parts_max);
+        constexpr int SMEM_A = sw_smem_bytes(MODE) > LM_PAIR_SMEM_BYTES ? sw_smem_bytes(MODE) : LM_PAIR_SMEM_BYTES;
+        constexpr int SMEM = SMEM_A > LM_SMEM_BYTES ? SMEM_A : LM_SMEM_BYTES;
+        static std::atomic<uint64_t> smem_set{0};
+        if (ensure_dynamic_smem(smem_set, lmhead_head_kernel<MODE>, SMEM) != DARE_OK) return DARE_ERR_CUDA;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(static_cast<unsigned>(grid_gemm), 1, 1);
+        cfg.blockDim = dim3(LM_THREADS, 1, 1);
+        cfg.dynamicSmemBytes = SMEM;
+        cfg.stream = stream;
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = 2; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        if (cudaLaunchKernelEx(&cfg, lmhead_head_kernel<MODE>, tmap_w, xm, M, live_rows, D, V, mask_col, n_tiles, part_max,
+                               part_sum, part_arg, ctx->dev_status, parts_stride, smp) != cudaSuccess)
+            return DARE_ERR_CUDA;
+        note_launch();
+    } else {
+        CUtensorMap tmap_x;
+        rc = make_tmap_bf16_2d(ctx, &tmap_x, x_gemm, static_cast<uint64_t>(M), static_cast<uint64_t>(D), BM, BK);
+        if (rc == DARE_OK)
+            rc = launch_partial<MODE>(ctx, grid, tmap_x, w, M, live_rows, D, V, mask_col, n_tiles, part_max, part_sum, part_arg,
+                                      smp, stream, &layout);
+        if (rc != DARE_OK) return rc;
+    }
+    const LmParts lp = {part_max, part_sum, part_arg, smp.part_y, smp.part_zb};
+    if (select) {
+        LmSelect sel;
+        sel.tokens_block = select->tokens_block; sel.row_stride = tok_row_stride; sel.mode = select->mode;
+        sel.threshold = select->threshold; sel.k = select->k;
+        sel.n_committed = select->n_committed; sel.n_remaining = select->n_remaining;
+        lmhead_merge_select_kernel<SAMPLE><<<select->B, 32 * tok_L, 0, stream>>>(lp, grid_gemm, n_tiles, tok_L, live_rows, idx,
+                                                                                 mask_id, pred, conf, layout, parts_stride, sel,
+                                                                                 step_dev);
+    } else {
+        constexpr int rows_per_block = 8;
+        lmhead_merge_kernel<SAMPLE><<<(M + rows_per_block - 1) / rows_per_block, rows_per_block * 32, 0, stream>>>(
+            lp, grid_gemm, n_tiles, M, live_rows, idx, pred, conf, layout, parts_stride, step_dev);
+    }
+    note_launch();
+    return cudaGetLastError() == cudaSuccess ? DARE_OK : DARE_ERR_CUDA;
 }
 
 int launch_lmhead(const dare_ctx* ctx, void* scratch, const void* hidden, int M, int D, const void* w, int V,
                   const int32_t* row_tokens, int tok_L, int64_t tok_row_stride, int32_t mask_id,
                   int exclude_mask_column, int32_t* pred, float* conf, cudaStream_t stream, const LmSampleArgs* sample,
                   const LmSelectArgs* select, cudaEvent_t after_compaction) {
-    if (select && (sample || !row_tokens || tok_L > LMHEAD_SELECT_MAX_L || tok_L < 1 || M != select->B * tok_L))
+    if (select && (!row_tokens || tok_L > LMHEAD_SELECT_MAX_L || tok_L < 1 || M != select->B * tok_L))
         return DARE_ERR_SHAPE;
     const int n_tiles = (V + BN - 1) / BN;
     const int m_tiles_max = (M + BM - 1) / BM;
@@ -1301,105 +1423,22 @@ int launch_lmhead(const dare_ctx* ctx, void* scratch, const void* hidden, int M,
         if (cudaGetLastError() != cudaSuccess) return DARE_ERR_CUDA;
     }
     if (after_compaction && cudaEventRecord(after_compaction, stream) != cudaSuccess) return DARE_ERR_CUDA;
-    size_t groups_max = static_cast<size_t>(ctx->sm_count);
-    if (groups_max > static_cast<size_t>(n_tiles)) groups_max = n_tiles;
-    const bool greedy_pairs = sample == nullptr && grid >= 2 && lm_pair_available();
-    if (greedy_pairs) {      // lmhead_greedy_kernel: a fixed stride, at most min(#CTAs, 2 per vocabulary tile) partials
-        groups_max = static_cast<size_t>(grid & ~1);
-        if (groups_max > static_cast<size_t>(2 * n_tiles)) groups_max = 2 * n_tiles;
-    }
-    const size_t n_part = static_cast<size_t>(M) * groups_max;
-    float* part_max = reinterpret_cast<float*>(cur);
-    float* part_sum = part_max + n_part;
-    int32_t* part_arg = reinterpret_cast<int32_t*>(part_sum + n_part);
-
     const int mask_col = (exclude_mask_column && mask_id >= 0 && mask_id < V) ? mask_id : -1;
-    const int rows_per_block = 8;
-    int rc = DARE_OK;
-    if (greedy_pairs) {
-        CUtensorMap tmap_w;
-        SwXMaps xm;
-        rc = make_tmap_bf16_2d(ctx, &tmap_w, w, static_cast<uint64_t>(V), static_cast<uint64_t>(D), SW_BV, BK);
-        for (int i = 0; i < 5 && rc == DARE_OK; ++i)
-            rc = make_tmap_bf16_2d(ctx, &xm.m[i], x_gemm, static_cast<uint64_t>(M), static_cast<uint64_t>(D), 128u >> i, BK);
-        if (rc != DARE_OK) return rc;
-        const int grid_pair = grid & ~1;
-        const int parts_stride = static_cast<int>(groups_max);
-        constexpr int SMEM_A = SW_SMEM_BYTES > LM_PAIR_SMEM_BYTES ? SW_SMEM_BYTES : LM_PAIR_SMEM_BYTES;
-        constexpr int SMEM = SMEM_A > LM_SMEM_BYTES ? SMEM_A : LM_SMEM_BYTES;
-        static std::atomic<uint64_t> smem_set_greedy{0};
-        if (ensure_dynamic_smem(smem_set_greedy, lmhead_greedy_kernel, SMEM) != DARE_OK) return DARE_ERR_CUDA;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(static_cast<unsigned>(grid_pair), 1, 1);
-        cfg.blockDim = dim3(LM_THREADS, 1, 1);
-        cfg.dynamicSmemBytes = SMEM;
-        cfg.stream = stream;
-        cudaLaunchAttribute attr;
-        attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = 2; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
-        cfg.attrs = &attr;
-        cfg.numAttrs = 1;
-        if (cudaLaunchKernelEx(&cfg, lmhead_greedy_kernel, tmap_w, xm, M, static_cast<const int32_t*>(live_rows), D, V,
-                               mask_col, n_tiles, part_max, part_sum, part_arg, ctx->dev_status, parts_stride) != cudaSuccess)
-            return DARE_ERR_CUDA;
-        note_launch();
-        if (select) {
-            LmSelect sel;
-            sel.tokens_block = select->tokens_block; sel.row_stride = tok_row_stride; sel.mode = select->mode;
-            sel.threshold = select->threshold; sel.k = select->k;
-            sel.n_committed = select->n_committed; sel.n_remaining = select->n_remaining;
-            lmhead_merge_select_kernel<<<select->B, 32 * tok_L, 0, stream>>>(part_max, part_sum, part_arg, grid_pair, n_tiles,
-                                                                             tok_L, live_rows, idx, mask_id, pred, conf,
-                                                                             LM_LAYOUT_GREEDY, parts_stride, sel);
-        } else {
-            lmhead_merge_kernel<<<(M + rows_per_block - 1) / rows_per_block, rows_per_block * 32, 0, stream>>>(
-                part_max, part_sum, part_arg, grid_pair, n_tiles, M, live_rows, idx, pred, conf, LM_LAYOUT_GREEDY,
-                parts_stride);
-        }
-        note_launch();
-        return cudaGetLastError() == cudaSuccess ? DARE_OK : DARE_ERR_CUDA;
-    }
-
-    CUtensorMap tmap_x;
-    rc = make_tmap_bf16_2d(ctx, &tmap_x, x_gemm, static_cast<uint64_t>(M), static_cast<uint64_t>(D), BM, BK);
-    if (rc != DARE_OK) return rc;
-
+    const bool pairs = grid >= 2 && lm_pair_available() &&
+                       lmhead_scratch_bytes(M, D, V, ctx->sm_count, row_tokens != nullptr, sample != nullptr, 2) <= ctx->workspace_bytes;
+    float* parts = reinterpret_cast<float*>(cur);
     LmSampling smp = {};
-    int allow_pair = 0;
-    if (sample == nullptr) {
-        rc = launch_partial<LM_GREEDY>(ctx, grid, tmap_x, w, M, live_rows, D, V, mask_col, n_tiles, part_max, part_sum,
-                                       part_arg, smp, stream, &allow_pair);
-        if (rc != DARE_OK) return rc;
-        if (select) {
-            LmSelect sel;
-            sel.tokens_block = select->tokens_block; sel.row_stride = tok_row_stride; sel.mode = select->mode;
-            sel.threshold = select->threshold; sel.k = select->k;
-            sel.n_committed = select->n_committed; sel.n_remaining = select->n_remaining;
-            lmhead_merge_select_kernel<<<select->B, 32 * tok_L, 0, stream>>>(part_max, part_sum, part_arg, grid, n_tiles,
-                                                                             tok_L, live_rows, idx, mask_id, pred, conf,
-                                                                             allow_pair, -1, sel); note_launch();
-        } else {
-            lmhead_merge_kernel<<<(M + rows_per_block - 1) / rows_per_block, rows_per_block * 32, 0, stream>>>(
-                part_max, part_sum, part_arg, grid, n_tiles, M, live_rows, idx, pred, conf, allow_pair, -1); note_launch();
-        }
-    } else {
-        smp.inv_temperature = 1.0f / sample->temperature;
-        smp.seed_lo = static_cast<uint32_t>(sample->seed & 0xffffffffu);
-        smp.seed_hi = static_cast<uint32_t>(sample->seed >> 32);
-        smp.step = sample->step;
-        smp.step_dev = sample->step_dev;
-        smp.row_index = idx;
-        smp.part_y = reinterpret_cast<float*>(part_arg + n_part);
-        smp.part_zb = smp.part_y + n_part;
-        rc = launch_partial<LM_SAMPLE>(ctx, grid, tmap_x, w, M, live_rows, D, V, mask_col, n_tiles, part_max, part_sum,
-                                       part_arg, smp, stream, &allow_pair);
-        if (rc != DARE_OK) return rc;
-        lmhead_merge_sample_kernel<<<(M + rows_per_block - 1) / rows_per_block, rows_per_block * 32, 0, stream>>>(
-            part_max, part_sum, part_arg, smp.part_y, smp.part_zb, grid, n_tiles, M, live_rows, idx, pred, conf,
-            allow_pair, sample->step_dev); note_launch();
-    }
-    if (cudaGetLastError() != cudaSuccess) return DARE_ERR_CUDA;
-    return DARE_OK;
+    if (sample == nullptr)
+        return launch_head<LM_GREEDY>(ctx, grid, pairs, x_gemm, M, D, w, V, mask_col, n_tiles, live_rows, idx, parts, smp,
+                                      nullptr, tok_L, tok_row_stride, mask_id, pred, conf, select, stream);
+    smp.inv_temperature = 1.0f / sample->temperature;
+    smp.seed_lo = static_cast<uint32_t>(sample->seed & 0xffffffffu);
+    smp.seed_hi = static_cast<uint32_t>(sample->seed >> 32);
+    smp.step = sample->step;
+    smp.step_dev = sample->step_dev;
+    smp.row_index = idx;
+    return launch_head<LM_SAMPLE>(ctx, grid, pairs, x_gemm, M, D, w, V, mask_col, n_tiles, live_rows, idx, parts, smp,
+                                  sample->step_dev, tok_L, tok_row_stride, mask_id, pred, conf, select, stream);
 }
 
 int launch_lmhead_logprob(const dare_ctx* ctx, void* scratch, const void* hidden, int M, int D, const void* w, int V,

@@ -112,22 +112,17 @@ int step_rows(dare_model* m, int32_t* tokens, int B, int64_t row_stride, int sta
     int rc = forward_rows(m, tokens, B, row_stride, start, L, kv_len, k_cache, v_cache, cap, nullptr, s);
     if (rc != DARE_OK) return rc;
     const int M = B * L;
-    if (m->sample_temperature > 0.f) {          // sampled head, then the separate selection kernel
-        dare::LmSampleArgs smp;
-        smp.temperature = m->sample_temperature; smp.seed = m->sample_seed; smp.step = 0; smp.step_dev = m->step_counter;
-        rc = dare::launch_lmhead(m->ctx, m->ctx->workspace, m->h, M, m->desc.hidden, m->lm_head, m->desc.vocab,
-                                 tokens + start, L, row_stride, m->desc.mask_id, 1, pred, conf, s, &smp);
-        if (rc != DARE_OK) return rc;
-        return dare::launch_unmask_select(tokens, B, row_stride, start, L, pred, conf, m->desc.mask_id, mode, threshold,
-                                          k, n_committed, n_remaining, s);
-    }
+    dare::LmSampleArgs smp;
+    const bool sampled = m->sample_temperature > 0.f;
+    smp.temperature = m->sample_temperature; smp.seed = m->sample_seed; smp.step = 0; smp.step_dev = m->step_counter;
     if (L <= dare::LMHEAD_SELECT_MAX_L) {      // short blocks: the selection rides on the head's merge kernel
         const dare::LmSelectArgs sel = {tokens + start, B, mode, threshold, k, n_committed, n_remaining};
         return dare::launch_lmhead(m->ctx, m->ctx->workspace, m->h, M, m->desc.hidden, m->lm_head, m->desc.vocab,
-                                   tokens + start, L, row_stride, m->desc.mask_id, 1, pred, conf, s, nullptr, &sel);
+                                   tokens + start, L, row_stride, m->desc.mask_id, 1, pred, conf, s, sampled ? &smp : nullptr,
+                                   &sel);
     }
     rc = dare::launch_lmhead(m->ctx, m->ctx->workspace, m->h, M, m->desc.hidden, m->lm_head, m->desc.vocab,
-                             tokens + start, L, row_stride, m->desc.mask_id, 1, pred, conf, s, nullptr);
+                             tokens + start, L, row_stride, m->desc.mask_id, 1, pred, conf, s, sampled ? &smp : nullptr);
     if (rc != DARE_OK) return rc;
     return dare::launch_unmask_select(tokens, B, row_stride, start, L, pred, conf, m->desc.mask_id, mode, threshold, k,
                                       n_committed, n_remaining, s);

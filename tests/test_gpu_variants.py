@@ -3,6 +3,7 @@ import numpy as np
 import pytest
 import torch
 
+from oracle import dare_sampling_oracle as SO
 from paper_2604_04215_b200 import binding as dare
 from paper_2604_04215_b200 import inputs as I
 
@@ -84,3 +85,37 @@ def test_linear_in_row_groups(ctx, M, K, N):
     # one rounding to bf16 (2^-8) and fp32 sums of K products: K * 2^-24 of the sum of their magnitudes at most
     bound = 2.0 ** -8 * ref.abs() + K * 2.0 ** -24 * (a.double().abs() @ w.double().abs().T)
     assert ((out - ref).abs() <= bound).all()
+
+
+# The sampled head takes the same paths as the greedy one: swapped operands up to 256 rows (five ring slots above 192)
+# and for rows that cut into chunks of 208 to 240, row-major pairs for an even number of 128-row tiles, pairs and single
+# CTAs for an odd one.  V leaves the last vocabulary tile part full.
+@pytest.mark.parametrize("M", [1, 16, 17, 33, 192, 193, 255, 256, 257, 300, 400, 420, 512, 520, 900])
+@pytest.mark.parametrize("T", [1.0, 0.35])
+def test_sampled_head_on_every_path(ctx, M, T):
+    D, V, mu, seed, step = 72, 1300, 1290, 0x9876543210 + M, 5
+    x, w = I.normal_bf16(M, I.TID_X, (M, D)), I.normal_bf16(3, I.TID_W, (V, D), 0.2)
+    ref = SO.lmhead_sample(x.double().numpy(), w.double().numpy(), None, mu, True, T, seed, step)
+    pred, conf = dare.dare_lmhead_sample(ctx, x.cuda(), w.cuda(), None, mu, True, T, seed, step)
+    torch.cuda.synchronize()
+    assert ctx.device_status() == 0
+    pred, conf = pred.cpu().numpy(), conf.cpu().double().numpy()
+    # scores are fp32 (sums of 72 products of magnitude ~2: 1e-5) over T plus noise of one ulp: well inside 1e-3
+    sure = ref["gap_y"] > 1e-3
+    assert (pred[sure] == ref["pred"][sure]).all() and sure.mean() > 0.9
+    same = pred == ref["pred"]
+    assert np.abs(np.log(conf[same]) - ref["logconf"][same]).max() <= 1e-3
+
+
+def test_sampled_head_with_a_workspace_for_one_partial_per_tile():
+    """The swapped path wants room for two partials per vocabulary tile; a context without it takes the other path."""
+    M, D, V, mu = 40, 64, 2000, 1999
+    need = 20 * M * ((V + 255) // 256)
+    c = dare.Context(0, need)
+    x, w = I.normal_bf16(1, I.TID_X, (M, D)), I.normal_bf16(2, I.TID_W, (V, D), 0.2)
+    ref = SO.lmhead_sample(x.double().numpy(), w.double().numpy(), None, mu, True, 1.0, 4, 1)
+    pred, conf = dare.dare_lmhead_sample(c, x.cuda(), w.cuda(), None, mu, True, 1.0, 4, 1)
+    torch.cuda.synchronize()
+    sure = ref["gap_y"] > 1e-3
+    assert (pred.cpu().numpy()[sure] == ref["pred"][sure]).all()
+    c.close()
