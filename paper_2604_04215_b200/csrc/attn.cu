@@ -41,7 +41,14 @@ struct AttnParams {
     float* part_o;                // [splits][B*L*Hq][D] fp32, used when splits > 1
     float* part_lse;              // [splits][B*L*Hq]
     uint32_t* dev_status;
+    int beside_head;              // inputs are ready although the kernels before this one still run (see enqueue_step)
 };
+
+// The CTA that is started last (in a step the attention waits in it for the head, so that what follows in the stream is
+// behind both; any other CTA would hold its place on the SM while it waits).
+__device__ __forceinline__ bool is_last_cta() {
+    return blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 && blockIdx.z == gridDim.z - 1;
+}
 
 struct AttBarriers {
     uint64_t full[ATT_MAX_STAGES];
@@ -112,12 +119,8 @@ attn_block_kernel(const __grid_constant__ CUtensorMap tm_kpre, const __grid_cons
     // for anything else: the row's lengths are requested first (needed only after the barrier below), the producer
     // lane sets up the barriers itself and, where the first tile's place does not depend on the lengths (in-place
     // cache: the prefix segment holds at least the block's L >= 1 keys and starts at the unit's base), sends for that
-    // tile at once; the consumers' Q rows are requested beside it.
-    int P = p.prefix_len ? p.prefix_len[b]
-                         : (p.uniform_P >= 0 ? p.uniform_P : (p.inplace ? p.prefix_cap - p.L : p.prefix_cap));
-    int S = p.has_suffix ? (p.suffix_len ? p.suffix_len[b] : p.suffix_cap) : 0;
-    // (only without a K/V split: a CTA of a split launch may own no tile at all, and a tile sent for must be waited for)
-    const bool early_tile = p.inplace && p.splits == 1;     // tile 0 of this CTA is tile 0 of the prefix segment
+    // tile at once; the consumers' Q rows are requested beside it.  All of it but the barriers comes behind pdl_wait,
+    // except in a step, where the kernels that still run do not write what this one reads.
     if (threadIdx.x == NCW * 32) {
         for (int s = 0; s < ATT_STAGES; ++s) {
             mbar_init(&bars->full[s], 1);
@@ -127,13 +130,20 @@ attn_block_kernel(const __grid_constant__ CUtensorMap tm_kpre, const __grid_cons
         fence_barrier_init();
         prefetch_tensormap(&tm_kpre);
         prefetch_tensormap(&tm_vpre);
-        if (early_tile) {
-            mbar_arrive_expect_tx(&bars->full[0], 2 * KV_BYTES);
+    }
+    if (!p.beside_head) pdl_wait();
+    pdl_trigger();
+    int P = p.prefix_len ? p.prefix_len[b]
+                         : (p.uniform_P >= 0 ? p.uniform_P : (p.inplace ? p.prefix_cap - p.L : p.prefix_cap));
+    int S = p.has_suffix ? (p.suffix_len ? p.suffix_len[b] : p.suffix_cap) : 0;
+    // (only without a K/V split: a CTA of a split launch may own no tile at all, and a tile sent for must be waited for)
+    const bool early_tile = p.inplace && p.splits == 1;     // tile 0 of this CTA is tile 0 of the prefix segment
+    if (threadIdx.x == NCW * 32 && early_tile) {
+        mbar_arrive_expect_tx(&bars->full[0], 2 * KV_BYTES);
 #pragma unroll
-            for (int h = 0; h < NHALF; ++h) {
-                tma_load_2d(tiles + h * HALF, &tm_kpre, &bars->full[0], h * 64, unit * p.prefix_cap);
-                tma_load_2d(tiles + KV_BYTES + h * HALF, &tm_vpre, &bars->full[0], h * 64, unit * p.prefix_cap);
-            }
+        for (int h = 0; h < NHALF; ++h) {
+            tma_load_2d(tiles + h * HALF, &tm_kpre, &bars->full[0], h * 64, unit * p.prefix_cap);
+            tma_load_2d(tiles + KV_BYTES + h * HALF, &tm_vpre, &bars->full[0], h * 64, unit * p.prefix_cap);
         }
     }
 
@@ -404,6 +414,7 @@ attn_block_kernel(const __grid_constant__ CUtensorMap tm_kpre, const __grid_cons
         if (threadIdx.x == 0) atomicOr(p.dev_status, DEV_WAIT_EXPIRED);
         __syncthreads();
     }
+    if (p.beside_head && is_last_cta()) pdl_wait();
 }
 
 // ---------------------------------------------------------------------------------------------------------
@@ -491,9 +502,10 @@ attn_block_tc_kernel(const __grid_constant__ CUtensorMap tm_kpre, const __grid_c
     // Packed variable-length mode: "rollout" b is sequence b of the packed token list; its tokens are both the
     // queries (a block of L_eff positions, no prefix) and, in place, the keys.  K and V are [tokens, Hkv * D].
     const bool packed = p.cu_seqlens != nullptr;
+    if (packed) pdl_wait();
     const int seq_base = packed ? p.cu_seqlens[b] : 0;
     const int L_eff = packed ? p.cu_seqlens[b + 1] - seq_base : p.L;
-    if (static_cast<int>(blockIdx.x) * QT * pos_per_tile >= L_eff) return;   // (whole CTA, before anything is set up)
+    if (static_cast<int>(blockIdx.x) * QT * pos_per_tile >= L_eff) return;   // (packed only: whole CTA, before anything is set up)
     const int kv_col0 = packed ? kvh * D : 0;      // first column of this KV head in the 2-D view of K / V
 
     // Set-up, with nothing waiting for anything else (a launch is a single wave of CTAs that live for about ten key
@@ -501,10 +513,10 @@ attn_block_tc_kernel(const __grid_constant__ CUtensorMap tm_kpre, const __grid_c
     // TMA producer, sets up the barriers and sends for key tile 0 at once where its place does not depend on the
     // lengths (packed sequences and the in-place cache: the first segment is not empty and starts at the unit's
     // base); warp 1 allocates tensor memory; the softmax threads stage their Q rows.
-    int P = p.prefix_len ? p.prefix_len[b]
-                         : (p.uniform_P >= 0 ? p.uniform_P : (p.inplace ? p.prefix_cap - p.L : p.prefix_cap));
-    int Sx = p.has_suffix ? (p.suffix_len ? p.suffix_len[b] : p.suffix_cap) : 0;
-    const bool early_tile = packed || p.inplace;
+    if (warp == 1) {
+        tmem_alloc(&bars->tmem_base, S::TMEM_COLS);
+        tmem_relinquish();
+    }
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(&bars->full[s], 1);
@@ -521,19 +533,20 @@ attn_block_tc_kernel(const __grid_constant__ CUtensorMap tm_kpre, const __grid_c
         fence_barrier_init();
         prefetch_tensormap(&tm_kpre);
         prefetch_tensormap(&tm_vpre);
-        if (early_tile) {
-            const int row0 = packed ? seq_base : unit * p.prefix_cap;
-            mbar_arrive_expect_tx(&bars->full[0], 2 * KV_BYTES);
-#pragma unroll
-            for (int h = 0; h < NHALF; ++h) {
-                tma_load_2d(kv_s + h * HALF_K, &tm_kpre, &bars->full[0], kv_col0 + h * 64, row0);
-                tma_load_2d(kv_s + KV_BYTES + h * HALF_K, &tm_vpre, &bars->full[0], kv_col0 + h * 64, row0);
-            }
-        }
     }
-    if (warp == 1) {
-        tmem_alloc(&bars->tmem_base, S::TMEM_COLS);
-        tmem_relinquish();
+    if (!packed && !p.beside_head) pdl_wait();             // (as in the warp-level kernel)
+    int P = p.prefix_len ? p.prefix_len[b]
+                         : (p.uniform_P >= 0 ? p.uniform_P : (p.inplace ? p.prefix_cap - p.L : p.prefix_cap));
+    int Sx = p.has_suffix ? (p.suffix_len ? p.suffix_len[b] : p.suffix_cap) : 0;
+    const bool early_tile = packed || p.inplace;
+    if (threadIdx.x == 0 && early_tile) {
+        const int row0 = packed ? seq_base : unit * p.prefix_cap;
+        mbar_arrive_expect_tx(&bars->full[0], 2 * KV_BYTES);
+#pragma unroll
+        for (int h = 0; h < NHALF; ++h) {
+            tma_load_2d(kv_s + h * HALF_K, &tm_kpre, &bars->full[0], kv_col0 + h * 64, row0);
+            tma_load_2d(kv_s + KV_BYTES + h * HALF_K, &tm_vpre, &bars->full[0], kv_col0 + h * 64, row0);
+        }
     }
     if (warp >= 2) {
         // Q rows -> shared memory, K-major with the 128-byte swizzle (16-byte chunk c of row r sits at c ^ (r & 7)).
@@ -563,6 +576,7 @@ attn_block_tc_kernel(const __grid_constant__ CUtensorMap tm_kpre, const __grid_c
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
+    pdl_trigger();
     const uint32_t tmem_base = bars->tmem_base;
 
     // lengths and tiles of this unit (same bookkeeping as the warp-level kernel)
@@ -840,6 +854,7 @@ attn_block_tc_kernel(const __grid_constant__ CUtensorMap tm_kpre, const __grid_c
         tc_fence_after_sync();
         tmem_dealloc(tmem_base, S::TMEM_COLS);
     }
+    if (p.beside_head && is_last_cta()) pdl_wait();
 }
 
 template <int D, int QT>
@@ -848,8 +863,8 @@ int launch_tc(const CUtensorMap* tm, const AttnParams& p, int q_tiles, cudaStrea
     static std::atomic<uint64_t> smem_set{0};
     if (ensure_dynamic_smem(smem_set, attn_block_tc_kernel<D, QT>, SMEM) != DARE_OK) return DARE_ERR_CUDA;
     dim3 grid((q_tiles + QT - 1) / QT, p.B * p.Hkv, 1);
-    attn_block_tc_kernel<D, QT><<<grid, TcShape<D, QT>::THREADS, SMEM, stream>>>(tm[0], tm[1], tm[2], tm[3], tm[4], tm[5], p); note_launch();
-    return cudaGetLastError() == cudaSuccess ? DARE_OK : DARE_ERR_CUDA;
+    return launch_kernel(attn_block_tc_kernel<D, QT>, grid, TcShape<D, QT>::THREADS, SMEM, stream, 1, tm[0], tm[1], tm[2], tm[3],
+                         tm[4], tm[5], p);
 }
 
 // The tensor-core tile is worth it when a tile's 128 rows are mostly real query rows.
@@ -868,6 +883,8 @@ __global__ void attn_combine_kernel(const float* __restrict__ part_o, const floa
                                     float* __restrict__ lse) {
     const size_t row = static_cast<size_t>(blockIdx.x) * (blockDim.x / (D / 4)) + threadIdx.x / (D / 4);
     const int c4 = threadIdx.x % (D / 4);
+    pdl_wait();
+    pdl_trigger();
     if (row >= n_rows) return;
     float mx = -INFINITY;
     for (int s = 0; s < splits; ++s) mx = fmaxf(mx, part_lse[s * n_rows + row]);
@@ -901,8 +918,8 @@ int launch_one(const CUtensorMap* tm, const AttnParams& p, int chunks, cudaStrea
     static std::atomic<uint64_t> smem_set{0};
     if (ensure_dynamic_smem(smem_set, attn_block_kernel<D, NW, KS, KT, STAGES, CPS>, SMEM) != DARE_OK) return DARE_ERR_CUDA;
     dim3 grid(chunks, p.B * p.Hkv, p.splits);
-    attn_block_kernel<D, NW, KS, KT, STAGES, CPS><<<grid, (NW * KS + 1) * 32, SMEM, stream>>>(tm[0], tm[1], tm[2], tm[3], tm[4], tm[5], p); note_launch();
-    return cudaGetLastError() == cudaSuccess ? DARE_OK : DARE_ERR_CUDA;
+    return launch_kernel(attn_block_kernel<D, NW, KS, KT, STAGES, CPS>, grid, (NW * KS + 1) * 32, SMEM, stream, 1, tm[0], tm[1],
+                         tm[2], tm[3], tm[4], tm[5], p);
 }
 
 // The warp-level kernel's variants by the number of packed query rows R per (rollout, KV head):
@@ -957,8 +974,9 @@ int launch_attn(const dare_ctx* ctx, const AttnArgs& a, cudaStream_t stream) {
     p.prefix_len = a.prefix_len; p.suffix_len = a.suffix_len;
     p.out = static_cast<__nv_bfloat16*>(a.out); p.lse = a.lse;
     p.dev_status = ctx->dev_status;
+    p.beside_head = a.beside_head;
     const size_t n_rows = static_cast<size_t>(a.B) * a.L * a.Hq;
-    p.part_o = static_cast<float*>(ctx->workspace);
+    p.part_o = static_cast<float*>(a.scratch ? a.scratch : ctx->workspace);
     p.part_lse = p.part_o + static_cast<size_t>(p.splits) * n_rows * a.d;
 
     CUtensorMap tm[6];
@@ -1007,12 +1025,8 @@ int launch_attn(const dare_ctx* ctx, const AttnArgs& a, cudaStream_t stream) {
         const int tpr = a.d / 4;                    // threads per row
         const int rows_per_block = 256 / tpr;
         const unsigned blocks = static_cast<unsigned>((n_rows + rows_per_block - 1) / rows_per_block);
-        if (a.d == 128)
-            attn_combine_kernel<128><<<blocks, 256, 0, stream>>>(p.part_o, p.part_lse, p.splits, n_rows, a.L, a.Hq, p.out, p.lse);
-        else
-            attn_combine_kernel<64><<<blocks, 256, 0, stream>>>(p.part_o, p.part_lse, p.splits, n_rows, a.L, a.Hq, p.out, p.lse);
-        note_launch();
-        if (cudaGetLastError() != cudaSuccess) return DARE_ERR_CUDA;
+        return launch_kernel(a.d == 128 ? attn_combine_kernel<128> : attn_combine_kernel<64>, dim3(blocks), 256, 0, stream, 1,
+                             p.part_o, p.part_lse, p.splits, n_rows, a.L, a.Hq, p.out, p.lse);
     }
     return DARE_OK;
 }

@@ -9,6 +9,7 @@
 #include <cuda_bf16.h>
 
 #include "internal.h"
+#include "ptx.cuh"
 
 namespace dare {
 int launch_lmhead_grad(const dare_ctx* ctx, const void* hidden, int M, int D, const void* w, int V,
@@ -24,6 +25,8 @@ transpose_bf16_kernel(const unsigned short* __restrict__ in, int rows, int cols,
     __shared__ unsigned short tile[32][34];
     const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;      // 32 x 8 threads
+    pdl_wait();
+    pdl_trigger();
     for (int i = ty; i < 32; i += 8) {
         const int r = r0 + i, c = c0 + tx;
         tile[i][tx] = (r < rows && c < cols) ? in[static_cast<size_t>(r) * cols + c] : static_cast<unsigned short>(0);
@@ -38,9 +41,8 @@ transpose_bf16_kernel(const unsigned short* __restrict__ in, int rows, int cols,
 int launch_transpose(const void* in, int rows, int cols, void* out, cudaStream_t stream) {
     dim3 grid((cols + 31) / 32, (rows + 31) / 32, 1);
     if (grid.y > 65535u) return DARE_ERR_SHAPE;
-    transpose_bf16_kernel<<<grid, 256, 0, stream>>>(static_cast<const unsigned short*>(in), rows, cols,
-                                                    static_cast<unsigned short*>(out)); note_launch();
-    return cudaGetLastError() == cudaSuccess ? DARE_OK : DARE_ERR_CUDA;
+    return launch_kernel(transpose_bf16_kernel, grid, 256, 0, stream, 1, static_cast<const unsigned short*>(in), rows, cols,
+                         static_cast<unsigned short*>(out));
 }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }

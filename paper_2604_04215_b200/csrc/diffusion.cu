@@ -7,6 +7,7 @@
 #include <math.h>
 
 #include "internal.h"
+#include "ptx.cuh"
 
 namespace dare {
 namespace {
@@ -31,6 +32,8 @@ __global__ void forward_mask_kernel(const int32_t* x0, int32_t* xt, int64_t row_
                                     uint32_t seed_hi, uint32_t sample) {
     const int b = blockIdx.y;
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
+    pdl_wait();
+    pdl_trigger();
     if (q * 4 >= length) return;
     const uint4 w4 = philox4x32_10(make_uint4(static_cast<uint32_t>(q), static_cast<uint32_t>(b), sample, MASK_TAG),
                                    seed_lo, seed_hi);
@@ -54,6 +57,8 @@ __global__ void masked_nelbo_kernel(const float* __restrict__ logprob, const int
                                     int32_t* __restrict__ n_masked) {
     const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
+    pdl_wait();
+    pdl_trigger();
     if (b >= B) return;
     const int32_t* row = xt + static_cast<int64_t>(b) * row_stride + start;
     const float* lp = logprob + static_cast<int64_t>(b) * length;
@@ -78,17 +83,14 @@ int launch_forward_mask(const int32_t* x0, int32_t* xt, int B, int64_t row_strid
                         const float* p_mask, int32_t mask_id, uint64_t seed, uint32_t sample, cudaStream_t stream) {
     const int groups = (length + 3) / 4;
     dim3 grid((groups + 127) / 128, B, 1);
-    forward_mask_kernel<<<grid, 128, 0, stream>>>(x0, xt, row_stride, start, length, p_mask, mask_id,
-                                                  static_cast<uint32_t>(seed & 0xffffffffu),
-                                                  static_cast<uint32_t>(seed >> 32), sample); note_launch();
-    return cudaGetLastError() == cudaSuccess ? DARE_OK : DARE_ERR_CUDA;
+    return launch_kernel(forward_mask_kernel, grid, 128, 0, stream, 1, x0, xt, row_stride, start, length, p_mask, mask_id,
+                         static_cast<uint32_t>(seed & 0xffffffffu), static_cast<uint32_t>(seed >> 32), sample);
 }
 
 int launch_masked_nelbo(const float* logprob, const int32_t* xt, int B, int64_t row_stride, int start, int length,
                         int32_t mask_id, const float* t, float* nelbo, int32_t* n_masked, cudaStream_t stream) {
-    masked_nelbo_kernel<<<(B + 3) / 4, 128, 0, stream>>>(logprob, xt, B, row_stride, start, length, mask_id, t, nelbo,
-                                                         n_masked); note_launch();
-    return cudaGetLastError() == cudaSuccess ? DARE_OK : DARE_ERR_CUDA;
+    return launch_kernel(masked_nelbo_kernel, dim3((B + 3) / 4), 128, 0, stream, 1, logprob, xt, B, row_stride, start, length,
+                         mask_id, t, nelbo, n_masked);
 }
 
 }  // namespace dare

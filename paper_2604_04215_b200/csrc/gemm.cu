@@ -148,6 +148,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
             if (EPI == GEMM_EPI_SWIGLU) prefetch_tensormap(&tmap_b2);
             int stage = 0;
             uint32_t phase = 0;
+            pdl_wait();
             // the weights come from HBM: ask L2 for them L2_AHEAD steps before the load that needs them
             for (int kb = kb_begin; kb < kb_end && kb < kb_begin + L2_AHEAD; ++kb) {
                 tma_prefetch_l2_2d(&tmap_b, kb * GK, n_tile * (EPI == GEMM_EPI_SWIGLU ? p.wcols : p.bn));
@@ -221,7 +222,9 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
     const int col_base = n_tile * p.wcols;
     const uint32_t taddr = tmem_base + (static_cast<uint32_t>(lq * 32) << 16) + rt * acc_stride;
     if (epi_warp) {
+        pdl_wait();
         mbar_wait(&bars->tmem_full, 0, abort_flag);     // (a wait that gave up leaves the abort flag set)
+        pdl_trigger();
         tc_fence_after_sync();
     }
     __syncwarp();
@@ -513,6 +516,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
             const CUtensorMap* tmap_w = (EPI == GEMM_EPI_SWIGLU && rank == 1) ? &tmap_b2 : &tmap_b;
             const int w_step = EPI == GEMM_EPI_SWIGLU ? half_rows : p.nchunk;   // rows from one chunk to the next
             const uint32_t full0 = cluster_map_shared(smem_u32(&bars->full[0]), rank4 & ~1);   // the even CTA's barriers
+            pdl_wait();
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true;
@@ -579,6 +583,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
     // to the pair (gi / 2) % 2; the other pair's CTA with the same rows sends its partial into slot gi of this
     // CTA's idle ring ([group][row][8 floats]).
     const bool epi_warp = warp >= 2;
+    if (epi_warp) pdl_wait();
     const int lq = warp & 3;
     const int set = epi_warp ? (warp - 2) >> 2 : 0;
     const int n_groups = p.wcols / 8;
@@ -596,6 +601,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
         const uint32_t taddr = tmem_base + (static_cast<uint32_t>(lq * 32) << 16) + acc * 256;
         if (epi_warp && epi_ok) {
             epi_ok = mbar_wait(&bars->tmem_full[acc], acc_phase, abort_flag);   // (a wait that gave up leaves the abort flag set)
+            if (tile + n_clusters >= total_tiles) pdl_trigger();                // the last tile's epilogue is all that is left
             tc_fence_after_sync();
         }
         __syncwarp();
@@ -754,25 +760,10 @@ int launch_pair(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap&
     if (g.p.splits == 1 && !max_clusters_query && clusters > g.p.resident) clusters = g.p.resident;
     const long long ctas = 2LL * g.p.splits * clusters;
     if (ctas > 0x7fffffffLL) return DARE_ERR_SHAPE;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(ctas), 1, 1);
-    cfg.blockDim = dim3(GEMM_THREADS, 1, 1);
-    cfg.dynamicSmemBytes = GEMM_SMEM_BYTES;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = static_cast<unsigned>(2 * g.p.splits);
-    attr.val.clusterDim.y = 1;
-    attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    if (max_clusters_query) {
-        cfg.gridDim = dim3(4096u, 1, 1);
-        return cudaOccupancyMaxActiveClusters(max_clusters_query, gemm_pair_kernel<EPI>, &cfg) == cudaSuccess
-                   ? DARE_OK : DARE_ERR_CUDA;
-    }
-    note_launch();
-    return cudaLaunchKernelEx(&cfg, gemm_pair_kernel<EPI>, ta, tb, tb2, g) == cudaSuccess ? DARE_OK : DARE_ERR_CUDA;
+    if (max_clusters_query)
+        return query_max_clusters(gemm_pair_kernel<EPI>, 4096u, GEMM_THREADS, GEMM_SMEM_BYTES, 2 * g.p.splits, max_clusters_query);
+    return launch_kernel(gemm_pair_kernel<EPI>, dim3(static_cast<unsigned>(ctas)), GEMM_THREADS, GEMM_SMEM_BYTES, stream,
+                         2 * g.p.splits, ta, tb, tb2, g);
 }
 
 // Clusters of `splits` CTA pairs of the pair kernel that can be resident at once (cached; 0 = they cannot run).
@@ -852,25 +843,11 @@ int launch_one(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& 
     if (ensure_dynamic_smem(smem_set, gemm_bf16_kernel<EPI>, GEMM_SMEM_BYTES) != DARE_OK) return DARE_ERR_CUDA;
     const long long ctas = static_cast<long long>(g.p.m_items) * g.p.n_tiles * g.p.splits;
     if (ctas > 0x7fffffffLL) return DARE_ERR_SHAPE;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(ctas), 1, 1);
-    cfg.blockDim = dim3(GEMM_THREADS, 1, 1);
-    cfg.dynamicSmemBytes = GEMM_SMEM_BYTES;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = static_cast<unsigned>(g.p.splits);
-    attr.val.clusterDim.y = 1;
-    attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    if (max_clusters_query) {     // how many clusters of this size the device runs at once (plan input)
-        cfg.gridDim = dim3(static_cast<unsigned>(g.p.splits) * 1024u, 1, 1);
-        return cudaOccupancyMaxActiveClusters(max_clusters_query, gemm_bf16_kernel<EPI>, &cfg) == cudaSuccess
-                   ? DARE_OK : DARE_ERR_CUDA;
-    }
-    note_launch();
-    return cudaLaunchKernelEx(&cfg, gemm_bf16_kernel<EPI>, ta, tb, tb2, g) == cudaSuccess ? DARE_OK : DARE_ERR_CUDA;
+    if (max_clusters_query)       // how many clusters of this size the device runs at once (plan input)
+        return query_max_clusters(gemm_bf16_kernel<EPI>, static_cast<unsigned>(g.p.splits) * 1024u, GEMM_THREADS,
+                                  GEMM_SMEM_BYTES, g.p.splits, max_clusters_query);
+    return launch_kernel(gemm_bf16_kernel<EPI>, dim3(static_cast<unsigned>(ctas)), GEMM_THREADS, GEMM_SMEM_BYTES, stream,
+                         g.p.splits, ta, tb, tb2, g);
 }
 
 // Clusters of `splits` CTAs of this kernel that can be resident at once (cached; 0 = such clusters cannot run).

@@ -39,14 +39,10 @@ struct dare_ctx {
     uint32_t* dev_status;   // device word, bits DARE_DEV_*
     dare_encode_tiled_fn encode_tiled;
     TmapCache* tmaps;       // host memory; NULL = encode on every call
-    // side stream of the step (dare_denoise_block, highest priority): the LM head runs on it, forked from the caller's
-    // stream (ev_fork) and joined back (ev_join); ev_mid marks the end of the head's row compaction, behind which the
-    // attention is enqueued on the caller's stream.  NULL = none (the step then runs in sequence)
-    cudaStream_t aux;
-    cudaEvent_t ev_fork, ev_mid, ev_join;
 };
 
 #include <atomic>
+#include <utility>
 
 namespace dare {
 
@@ -67,6 +63,48 @@ inline int ensure_dynamic_smem(std::atomic<uint64_t>& done, Kernel kernel, int b
         return DARE_ERR_CUDA;
     if (bit) done.fetch_or(bit, std::memory_order_release);
     return DARE_OK;
+}
+
+// Every kernel of the library is launched through this: optionally as clusters of `cluster` CTAs along x, and always as
+// a programmatic dependent of whatever precedes it in the stream.  A kernel's CTAs may therefore be set up while its
+// predecessor still runs; what keeps the stream's order are the two calls each kernel makes (pdl_wait and pdl_trigger
+// in ptx.cuh, with the rules).
+template <typename... Params, typename... Args>
+inline int launch_kernel(void (*kernel)(Params...), dim3 grid, int threads, size_t smem_bytes, cudaStream_t stream,
+                         int cluster, Args&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(static_cast<unsigned>(threads), 1, 1);
+    cfg.dynamicSmemBytes = smem_bytes;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = static_cast<unsigned>(cluster); attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    if (cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...) != cudaSuccess) {
+        (void)cudaGetLastError();      // reported through the return value
+        return DARE_ERR_CUDA;
+    }
+    note_launch();
+    return DARE_OK;
+}
+
+// How many clusters of `cluster` CTAs of a kernel the device holds at once.
+template <typename Kernel>
+inline int query_max_clusters(Kernel kernel, unsigned grid_x, int threads, size_t smem_bytes, int cluster, int* out) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid_x, 1, 1);
+    cfg.blockDim = dim3(static_cast<unsigned>(threads), 1, 1);
+    cfg.dynamicSmemBytes = smem_bytes;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = static_cast<unsigned>(cluster); attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaOccupancyMaxActiveClusters(out, kernel, &cfg) == cudaSuccess ? DARE_OK : DARE_ERR_CUDA;
 }
 
 // Makes `device` current for the lifetime of the object and puts the previous device back afterwards (the create
@@ -110,6 +148,7 @@ int launch_lmhead_logprob(const dare_ctx* ctx, void* scratch, const void* hidden
 // from a CUDA graph draws fresh noise every time.
 struct LmSampleArgs { float temperature; uint64_t seed; uint32_t step; uint32_t* step_dev = nullptr; };
 size_t lmhead_workspace_bytes(int M, int D, int V, int sm_count, bool with_row_tokens, bool sampling);
+size_t lmhead_max_scratch_bytes(int M, int D, int V, int sm_count, bool sampling);
 // Token of LM-head row m (to skip committed rows) = row_tokens[(m / tok_L) * tok_row_stride + m % tok_L].
 // Unmask selection folded into the head's last kernel (on a block of at most LMHEAD_SELECT_MAX_L
 // positions whose tokens are given by row_tokens = tokens + block_start, tok_L = L): the caller then skips
@@ -118,9 +157,7 @@ constexpr int LMHEAD_SELECT_MAX_L = 32;
 struct LmSelectArgs { int32_t* tokens_block; int B; int mode; float threshold; int k; int32_t* n_committed; int32_t* n_remaining; };
 int launch_lmhead(const dare_ctx* ctx, void* scratch, const void* hidden, int M, int D, const void* w, int V,
                   const int32_t* row_tokens, int tok_L, int64_t tok_row_stride, int32_t mask_id, int exclude_mask_column, int32_t* pred, float* conf,
-                  cudaStream_t stream, const LmSampleArgs* sample, const LmSelectArgs* select = nullptr,
-                  cudaEvent_t after_compaction = nullptr);    // non-NULL: recorded on `stream` behind the row compaction,
-                                                              // i.e. just before the head's GEMM becomes ready to run
+                  cudaStream_t stream, const LmSampleArgs* sample, const LmSelectArgs* select = nullptr);
 
 struct AttnArgs {
     int B, L, Hq, Hkv, d, prefix_cap, suffix_cap;
@@ -134,6 +171,8 @@ struct AttnArgs {
     const int32_t* suffix_len;
     void* out;
     float* lse;
+    bool beside_head = false;   // enqueued behind the LM head whose results it does not read: see enqueue_step
+    void* scratch = nullptr;    // partials of a K/V split (NULL: the start of the ctx workspace)
 };
 int attn_plan_splits(const dare_ctx* ctx, const AttnArgs& a);
 size_t attn_workspace_bytes(const AttnArgs& a, int splits);

@@ -101,6 +101,8 @@ lmhead_compact_kernel(const uint4* __restrict__ x, int M, int D8, const int32_t*
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) s_base = 0;
     __syncthreads();
+    pdl_wait();
+    pdl_trigger();
     int local = 0;
     for (int m = threadIdx.x; m < row0; m += blockDim.x) local += row_token(row_tokens, tok_L, tok_row_stride, m) == mask_id;
 #pragma unroll
@@ -292,6 +294,7 @@ lm_rowmajor_body(const CUtensorMap& tmap_x, const CUtensorMap& tmap_w,
     if (PAIR) cluster_sync_all();     // both CTAs' barriers exist before either signals the other's
     else __syncthreads();
     tc_fence_after_sync();
+    pdl_trigger();
     const uint32_t tmem_base = bars->tmem_base;
     const int num_k = (D + BK - 1) / BK;
 
@@ -550,6 +553,7 @@ lmhead_partial_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
                       int M, const int32_t* __restrict__ live_rows, int D, int V, int mask_col, int n_tiles,
                       float* __restrict__ part_max, float* __restrict__ part_sum, int32_t* __restrict__ part_arg,
                       uint32_t* __restrict__ dev_status, const LmSampling smp, int allow_pair) {
+    pdl_wait();
     const int Mc = live_rows ? *live_rows : M;          // rows that need logits (uniform over the grid)
     const int m_tiles = (Mc + BM - 1) / BM;
     if (lm_pair_mode(m_tiles, allow_pair) != PAIR) return;        // the other kernel does this launch's work
@@ -717,6 +721,7 @@ lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, 
     tc_fence_before_sync();
     cluster_sync_all();                                  // both CTAs' barriers exist before either signals the other's
     tc_fence_after_sync();
+    pdl_trigger();
     const uint32_t tmem_base = bars->tmem_base;
     const int num_k = (D + BK - 1) / BK;
 
@@ -992,6 +997,7 @@ lmhead_head_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
                      const int32_t* __restrict__ live_rows, int D, int V, int mask_col, int n_tiles,
                      float* __restrict__ part_max, float* __restrict__ part_sum, int32_t* __restrict__ part_arg,
                      uint32_t* __restrict__ dev_status, int parts_stride, const LmSampling smp) {
+    pdl_wait();
     const int Mc = live_rows ? *live_rows : M;          // rows that need logits (uniform over the grid)
     if (lm_greedy_swapped(Mc)) {
         lm_swapped_body<MODE>(tmap_w, xmaps, Mc, D, V, mask_col, n_tiles, part_max, part_sum, part_arg, dev_status, parts_stride,
@@ -1094,6 +1100,8 @@ __global__ void lmhead_merge_kernel(const LmParts parts, int grid_gemm, int n_ti
                                     const int32_t* __restrict__ live_rows, const int32_t* __restrict__ idx,
                                     int32_t* __restrict__ pred, float* __restrict__ conf, int allow_pair,
                                     int parts_stride, uint32_t* __restrict__ step_dev) {
+    pdl_trigger();      // (before the wait, as in lmhead_merge_select_kernel; a selection kernel may come in between)
+    pdl_wait();
     if (SAMPLE && step_dev && blockIdx.x == 0 && threadIdx.x == 0) *step_dev += 1;   // the GEMM kernels before this one read it
     const int c = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
@@ -1134,6 +1142,8 @@ lmhead_merge_select_kernel(const LmParts parts, int grid_gemm, int n_tiles, int 
     __shared__ int s_flag[32];
     __shared__ float s_conf[32];
     __shared__ int32_t s_pred[32];
+    pdl_trigger();      // (before the wait: the attention of the step, which may follow, does not depend on the head)
+    pdl_wait();
     if (SAMPLE && step_dev && blockIdx.x == 0 && threadIdx.x == 0) *step_dev += 1;   // (as in lmhead_merge_kernel)
     const int b = blockIdx.x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;      // warp = block position (blockDim = 32 L)
@@ -1204,6 +1214,8 @@ __global__ void lmhead_merge_logprob_kernel(const float* __restrict__ part_max, 
                                             float* __restrict__ logprob, float* __restrict__ lse_out, int allow_pair) {
     const int c = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
+    pdl_wait();
+    pdl_trigger();
     if (c >= M) return;
     const int groups = lm_groups_mode(grid_gemm, (M + BM - 1) / BM, n_tiles, allow_pair);
     float m = -INFINITY, s = 0.f, zt = -INFINITY;
@@ -1239,18 +1251,9 @@ int lm_pair_available() {
     static int cache = -1;
     if (cache < 0) {
         int n = 0;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(2048, 1, 1);
-        cfg.blockDim = dim3(LM_THREADS, 1, 1);
-        cfg.dynamicSmemBytes = LM_PAIR_SMEM_BYTES;
-        cudaLaunchAttribute attr;
-        attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = 2; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
-        cfg.attrs = &attr;
-        cfg.numAttrs = 1;
         if (cudaFuncSetAttribute(lmhead_partial_kernel<LM_GREEDY, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  LM_PAIR_SMEM_BYTES) != cudaSuccess ||
-            cudaOccupancyMaxActiveClusters(&n, lmhead_partial_kernel<LM_GREEDY, true>, &cfg) != cudaSuccess)
+            query_max_clusters(lmhead_partial_kernel<LM_GREEDY, true>, 2048u, LM_THREADS, LM_PAIR_SMEM_BYTES, 2, &n) != DARE_OK)
             n = 0;
         cache = n > 0 ? 1 : 0;
     }
@@ -1276,10 +1279,10 @@ int launch_partial(const dare_ctx* ctx, int grid, const CUtensorMap& tmap_x, con
         if (rc != DARE_OK) return rc;
         static std::atomic<uint64_t> smem_set{0};
         if (ensure_dynamic_smem(smem_set, lmhead_partial_kernel<MODE, false>, LM_SMEM_BYTES) != DARE_OK) return DARE_ERR_CUDA;
-        lmhead_partial_kernel<MODE, false><<<grid, LM_THREADS, LM_SMEM_BYTES, stream>>>(
-            tmap_x, tmap_w, M, live_rows, D, V, mask_col, n_tiles, part_max, part_sum, part_arg, ctx->dev_status, smp,
-            allow_pair); note_launch();
-        if (cudaGetLastError() != cudaSuccess) return DARE_ERR_CUDA;
+        rc = launch_kernel(lmhead_partial_kernel<MODE, false>, dim3(grid), LM_THREADS, LM_SMEM_BYTES, stream, 1, tmap_x,
+                           tmap_w, M, live_rows, D, V, mask_col, n_tiles, part_max, part_sum, part_arg, ctx->dev_status, smp,
+                           allow_pair);
+        if (rc != DARE_OK) return rc;
     }
     if (run_pair) {
         CUtensorMap tmap_wh;      // half a W tile per CTA
@@ -1288,20 +1291,10 @@ int launch_partial(const dare_ctx* ctx, int grid, const CUtensorMap& tmap_x, con
         static std::atomic<uint64_t> smem_set_pair{0};
         if (ensure_dynamic_smem(smem_set_pair, lmhead_partial_kernel<MODE, true>, LM_PAIR_SMEM_BYTES) != DARE_OK)
             return DARE_ERR_CUDA;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(static_cast<unsigned>(grid & ~1), 1, 1);
-        cfg.blockDim = dim3(LM_THREADS, 1, 1);
-        cfg.dynamicSmemBytes = LM_PAIR_SMEM_BYTES;
-        cfg.stream = stream;
-        cudaLaunchAttribute attr;
-        attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = 2; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
-        cfg.attrs = &attr;
-        cfg.numAttrs = 1;
-        if (cudaLaunchKernelEx(&cfg, lmhead_partial_kernel<MODE, true>, tmap_x, tmap_wh, M, live_rows, D, V, mask_col,
-                               n_tiles, part_max, part_sum, part_arg, ctx->dev_status, smp, allow_pair) != cudaSuccess)
-            return DARE_ERR_CUDA;
-        note_launch();
+        rc = launch_kernel(lmhead_partial_kernel<MODE, true>, dim3(static_cast<unsigned>(grid & ~1)), LM_THREADS,
+                           LM_PAIR_SMEM_BYTES, stream, 2, tmap_x, tmap_wh, M, live_rows, D, V, mask_col, n_tiles, part_max,
+                           part_sum, part_arg, ctx->dev_status, smp, allow_pair);
+        if (rc != DARE_OK) return rc;
     }
     return DARE_OK;
 }
@@ -1321,6 +1314,11 @@ static size_t lmhead_scratch_bytes(int M, int D, int V, int sm_count, bool with_
 // (the swapped path leaves two partials per vocabulary group of a CTA pair; the sampled head can do without that path)
 size_t lmhead_workspace_bytes(int M, int D, int V, int sm_count, bool with_row_tokens, bool sampling) {
     return lmhead_scratch_bytes(M, D, V, sm_count, with_row_tokens, sampling, sampling ? 1 : 2);
+}
+
+// The most that a launch with row tokens uses where the workspace allows it.
+size_t lmhead_max_scratch_bytes(int M, int D, int V, int sm_count, bool sampling) {
+    return lmhead_scratch_bytes(M, D, V, sm_count, true, sampling, 2);
 }
 
 // The head's GEMM, its merge and, with `select`, the unmask selection, for one epilogue.
@@ -1355,20 +1353,10 @@ static int launch_head(const dare_ctx* ctx, int grid, bool pairs, const void* x_
         constexpr int SMEM = SMEM_A > LM_SMEM_BYTES ? SMEM_A : LM_SMEM_BYTES;
         static std::atomic<uint64_t> smem_set{0};
         if (ensure_dynamic_smem(smem_set, lmhead_head_kernel<MODE>, SMEM) != DARE_OK) return DARE_ERR_CUDA;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(static_cast<unsigned>(grid_gemm), 1, 1);
-        cfg.blockDim = dim3(LM_THREADS, 1, 1);
-        cfg.dynamicSmemBytes = SMEM;
-        cfg.stream = stream;
-        cudaLaunchAttribute attr;
-        attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = 2; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
-        cfg.attrs = &attr;
-        cfg.numAttrs = 1;
-        if (cudaLaunchKernelEx(&cfg, lmhead_head_kernel<MODE>, tmap_w, xm, M, live_rows, D, V, mask_col, n_tiles, part_max,
-                               part_sum, part_arg, ctx->dev_status, parts_stride, smp) != cudaSuccess)
-            return DARE_ERR_CUDA;
-        note_launch();
+        rc = launch_kernel(lmhead_head_kernel<MODE>, dim3(static_cast<unsigned>(grid_gemm)), LM_THREADS, SMEM, stream, 2, tmap_w,
+                           xm, M, live_rows, D, V, mask_col, n_tiles, part_max, part_sum, part_arg, ctx->dev_status, parts_stride,
+                           smp);
+        if (rc != DARE_OK) return rc;
     } else {
         CUtensorMap tmap_x;
         rc = make_tmap_bf16_2d(ctx, &tmap_x, x_gemm, static_cast<uint64_t>(M), static_cast<uint64_t>(D), BM, BK);
@@ -1383,22 +1371,18 @@ static int launch_head(const dare_ctx* ctx, int grid, bool pairs, const void* x_
         sel.tokens_block = select->tokens_block; sel.row_stride = tok_row_stride; sel.mode = select->mode;
         sel.threshold = select->threshold; sel.k = select->k;
         sel.n_committed = select->n_committed; sel.n_remaining = select->n_remaining;
-        lmhead_merge_select_kernel<SAMPLE><<<select->B, 32 * tok_L, 0, stream>>>(lp, grid_gemm, n_tiles, tok_L, live_rows, idx,
-                                                                                 mask_id, pred, conf, layout, parts_stride, sel,
-                                                                                 step_dev);
-    } else {
-        constexpr int rows_per_block = 8;
-        lmhead_merge_kernel<SAMPLE><<<(M + rows_per_block - 1) / rows_per_block, rows_per_block * 32, 0, stream>>>(
-            lp, grid_gemm, n_tiles, M, live_rows, idx, pred, conf, layout, parts_stride, step_dev);
+        return launch_kernel(lmhead_merge_select_kernel<SAMPLE>, dim3(select->B), 32 * tok_L, 0, stream, 1, lp, grid_gemm, n_tiles,
+                             tok_L, live_rows, idx, mask_id, pred, conf, layout, parts_stride, sel, step_dev);
     }
-    note_launch();
-    return cudaGetLastError() == cudaSuccess ? DARE_OK : DARE_ERR_CUDA;
+    constexpr int rows_per_block = 8;
+    return launch_kernel(lmhead_merge_kernel<SAMPLE>, dim3((M + rows_per_block - 1) / rows_per_block), rows_per_block * 32, 0,
+                         stream, 1, lp, grid_gemm, n_tiles, M, live_rows, idx, pred, conf, layout, parts_stride, step_dev);
 }
 
 int launch_lmhead(const dare_ctx* ctx, void* scratch, const void* hidden, int M, int D, const void* w, int V,
                   const int32_t* row_tokens, int tok_L, int64_t tok_row_stride, int32_t mask_id,
                   int exclude_mask_column, int32_t* pred, float* conf, cudaStream_t stream, const LmSampleArgs* sample,
-                  const LmSelectArgs* select, cudaEvent_t after_compaction) {
+                  const LmSelectArgs* select) {
     if (select && (!row_tokens || tok_L > LMHEAD_SELECT_MAX_L || tok_L < 1 || M != select->B * tok_L))
         return DARE_ERR_SHAPE;
     const int n_tiles = (V + BN - 1) / BN;
@@ -1417,12 +1401,11 @@ int launch_lmhead(const dare_ctx* ctx, void* scratch, const void* hidden, int M,
         live_rows = idx + M;
         cur += round_up(static_cast<size_t>(M) * 4 + 4, 1024);
         x_gemm = xc;
-        lmhead_compact_kernel<<<(M + CP_ROWS - 1) / CP_ROWS, CP_ROWS * 32, 0, stream>>>(
-            static_cast<const uint4*>(hidden), M, D / 8, row_tokens, tok_L, tok_row_stride, mask_id,
-            static_cast<uint4*>(xc), idx, live_rows, pred, conf); note_launch();
-        if (cudaGetLastError() != cudaSuccess) return DARE_ERR_CUDA;
+        const int rc = launch_kernel(lmhead_compact_kernel, dim3((M + CP_ROWS - 1) / CP_ROWS), CP_ROWS * 32, 0, stream, 1,
+                                     static_cast<const uint4*>(hidden), M, D / 8, row_tokens, tok_L, tok_row_stride, mask_id,
+                                     static_cast<uint4*>(xc), idx, live_rows, pred, conf);
+        if (rc != DARE_OK) return rc;
     }
-    if (after_compaction && cudaEventRecord(after_compaction, stream) != cudaSuccess) return DARE_ERR_CUDA;
     const int mask_col = (exclude_mask_column && mask_id >= 0 && mask_id < V) ? mask_id : -1;
     const bool pairs = grid >= 2 && lm_pair_available() &&
                        lmhead_scratch_bytes(M, D, V, ctx->sm_count, row_tokens != nullptr, sample != nullptr, 2) <= ctx->workspace_bytes;
@@ -1465,9 +1448,8 @@ int launch_lmhead_logprob(const dare_ctx* ctx, void* scratch, const void* hidden
                                     smp, stream, &allow_pair);
     if (rc != DARE_OK) return rc;
     const int rows_per_block = 8;
-    lmhead_merge_logprob_kernel<<<(M + rows_per_block - 1) / rows_per_block, rows_per_block * 32, 0, stream>>>(
-        part_max, part_sum, part_zt, grid, n_tiles, M, logprob, lse_out, allow_pair); note_launch();
-    return cudaGetLastError() == cudaSuccess ? DARE_OK : DARE_ERR_CUDA;
+    return launch_kernel(lmhead_merge_logprob_kernel, dim3((M + rows_per_block - 1) / rows_per_block), rows_per_block * 32, 0,
+                         stream, 1, part_max, part_sum, part_zt, grid, n_tiles, M, logprob, lse_out, allow_pair);
 }
 
 // dz[m, v] = grad[m] * (1[v = targets[m]] - exp(z[m, v] - lse[m])) as bf16 [M, V] and transposed [V, ldm]
@@ -1585,7 +1567,6 @@ extern "C" int dare_lmhead_confidence_static(const void* hidden, int M, int D, c
     // a context-shaped view of the static state for the shared launcher; nothing here is allocated
     dare_ctx view;
     view.tmaps = nullptr;
-    view.aux = nullptr; view.ev_fork = nullptr; view.ev_mid = nullptr; view.ev_join = nullptr;
     view.device = st->device;
     view.sm_count = st->sm_count;
     view.workspace = st->scratch;

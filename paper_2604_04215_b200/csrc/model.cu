@@ -17,6 +17,7 @@
 #include <new>
 
 #include "internal.h"
+#include "ptx.cuh"
 
 struct dare_model {
     dare_ctx* ctx;
@@ -39,7 +40,10 @@ struct dare_model {
 
 namespace {
 
-__global__ void set_word_kernel(uint32_t* p, uint32_t v) { *p = v; }
+__global__ void set_word_kernel(uint32_t* p, uint32_t v) {
+    dare::pdl_wait();
+    *p = v;
+}
 
 // Keys visible to the rows: cache[0, kv_len), start + length <= kv_len <= cap.
 int forward_rows(dare_model* m, const int32_t* tokens, int B, int64_t row_stride, int start, int length, int kv_len,
@@ -221,8 +225,7 @@ int dare_model_set_sampling(dare_model* m, float temperature, uint64_t seed, uin
     if (!(temperature >= 0.f) || isinf(temperature)) return DARE_ERR_RANGE;
     m->sample_temperature = temperature;
     m->sample_seed = seed;
-    set_word_kernel<<<1, 1, 0, static_cast<cudaStream_t>(stream)>>>(m->step_counter, first_step); dare::note_launch();
-    return cudaGetLastError() == cudaSuccess ? DARE_OK : DARE_ERR_CUDA;
+    return dare::launch_kernel(set_word_kernel, dim3(1), 1, 0, static_cast<cudaStream_t>(stream), 1, m->step_counter, first_step);
 }
 
 int dare_linear(dare_ctx* ctx, int epilogue, const void* a, int M, int K, const void* w, const void* w2, int N, void* out,
@@ -412,8 +415,8 @@ int dare_generate(dare_model* m, int32_t* tokens, int B, int64_t row_stride, int
         const int start = prompt_len + b * L;
         int taken = -1;
         if (m->sample_temperature > 0.f) {     // step n of block b draws with the counter (b << 16) + n
-            set_word_kernel<<<1, 1, 0, m->work>>>(m->step_counter, static_cast<uint32_t>(b) << 16);
-            dare::note_launch();
+            rc = dare::launch_kernel(set_word_kernel, dim3(1), 1, 0, m->work, 1, m->step_counter, static_cast<uint32_t>(b) << 16);
+            if (rc != DARE_OK) break;
         }
         rc = run_block(m, tokens, B, row_stride, start, L, start + L, k_cache, v_cache, cache_cap, mode, threshold, k,
                        pred, conf, n_remaining, &old, &taken);
@@ -441,8 +444,8 @@ int dare_generate_dual(dare_model* m, int32_t* tokens, int B, int64_t row_stride
         if (rc != DARE_OK) break;
         int taken = -1;
         if (m->sample_temperature > 0.f) {
-            set_word_kernel<<<1, 1, 0, m->work>>>(m->step_counter, static_cast<uint32_t>(b) << 16);
-            dare::note_launch();
+            rc = dare::launch_kernel(set_word_kernel, dim3(1), 1, 0, m->work, 1, m->step_counter, static_cast<uint32_t>(b) << 16);
+            if (rc != DARE_OK) break;
         }
         rc = run_block(m, tokens, B, row_stride, start, L, T, k_cache, v_cache, cache_cap, mode, threshold, k, pred, conf,
                        n_remaining, &old, &taken);

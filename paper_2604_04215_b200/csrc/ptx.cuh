@@ -69,6 +69,18 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
     return true;
 }
 
+// ---------------------------------------------------------------- programmatic dependent launch
+// Waits until the kernel before this one in the stream has finished and its writes are visible.  All kernels of the
+// library are launched as programmatic dependents (launch_kernel), so each calls this before it touches anything an
+// earlier kernel may have written and before its own first global write; since at least one CTA of each kernel does so
+// before it ends, a kernel's end implies the end of all kernels before it.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Lets the next kernel's CTAs be set up in the room this kernel leaves.  Called behind pdl_wait unless a comment says
+// otherwise, so that when a kernel's first instruction runs only its direct predecessor can still be running.  A kernel
+// that takes tensor memory calls it behind the allocation: a successor that takes tensor memory on the same SM can then
+// only wait for a CTA that has its share and will give it back.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ---------------------------------------------------------------- thread-block cluster
 __device__ __forceinline__ uint32_t cluster_cta_rank() {
     uint32_t r;

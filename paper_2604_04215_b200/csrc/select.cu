@@ -5,6 +5,7 @@
 #include <math.h>
 
 #include "internal.h"
+#include "ptx.cuh"
 
 namespace dare {
 namespace {
@@ -22,6 +23,8 @@ unmask_select_kernel(int32_t* __restrict__ tokens, int64_t row_stride, int block
     int32_t* row = tokens + static_cast<int64_t>(r) * row_stride + block_start;
     if (threadIdx.x == 0) { s_masked = 0; s_above = 0; s_commit = 0; }
     __syncthreads();
+    pdl_trigger();      // (before the wait: the attention of a step, which may follow, does not depend on the head)
+    pdl_wait();
     int local_masked = 0, local_above = 0;
     for (int i = threadIdx.x; i < L; i += SEL_THREADS) {
         const bool masked = row[i] == mask_id;
@@ -73,10 +76,8 @@ int launch_unmask_select(int32_t* tokens, int B, int64_t row_stride, int block_s
                          const float* conf, int32_t mask_id, int mode, float threshold, int k, int32_t* n_committed,
                          int32_t* n_remaining, cudaStream_t stream) {
     if (L > SEL_MAX_L) return DARE_ERR_SHAPE;
-    unmask_select_kernel<<<B, SEL_THREADS, L * sizeof(float), stream>>>(tokens, row_stride, block_start, L, pred, conf,
-                                                                        mask_id, mode, threshold, k, n_committed,
-                                                                        n_remaining); note_launch();
-    return cudaGetLastError() == cudaSuccess ? DARE_OK : DARE_ERR_CUDA;
+    return launch_kernel(unmask_select_kernel, dim3(B), SEL_THREADS, L * sizeof(float), stream, 1, tokens, row_stride,
+                         block_start, L, pred, conf, mask_id, mode, threshold, k, n_committed, n_remaining);
 }
 
 }  // namespace dare
