@@ -132,7 +132,6 @@ attn_block_kernel(const __grid_constant__ CUtensorMap tm_kpre, const __grid_cons
         prefetch_tensormap(&tm_vpre);
     }
     if (!p.beside_head) pdl_wait();
-    pdl_trigger();
     int P = p.prefix_len ? p.prefix_len[b]
                          : (p.uniform_P >= 0 ? p.uniform_P : (p.inplace ? p.prefix_cap - p.L : p.prefix_cap));
     int S = p.has_suffix ? (p.suffix_len ? p.suffix_len[b] : p.suffix_cap) : 0;
@@ -340,6 +339,9 @@ attn_block_kernel(const __grid_constant__ CUtensorMap tm_kpre, const __grid_cons
     }
 
     // ---------------- merge the key slices of a row group (through the now idle tile ring), then write out
+    // (The next kernel is let in only now: set up any earlier, the CTAs of a small one pile up on the few SMs that have
+    // room beside this kernel's; the row compaction of the next step then took 11 us instead of 6.)
+    pdl_trigger();
     __syncthreads();   // every tile has been consumed (or the CTA is aborting): the ring may be reused
     const bool aborted = *abort_flag != 0;
     float* xch = reinterpret_cast<float*>(tiles);
@@ -576,7 +578,6 @@ attn_block_tc_kernel(const __grid_constant__ CUtensorMap tm_kpre, const __grid_c
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    pdl_trigger();
     const uint32_t tmem_base = bars->tmem_base;
 
     // lengths and tiles of this unit (same bookkeeping as the warp-level kernel)
@@ -798,6 +799,7 @@ attn_block_tc_kernel(const __grid_constant__ CUtensorMap tm_kpre, const __grid_c
         }
         if (ok && n_tiles > 0) ok = mbar_wait(&bars->pv_done[j][(n_tiles - 1) & 1], ((n_tiles - 1) >> 1) & 1, abort_flag);
         tc_fence_after_sync();
+        pdl_trigger();                                  // (this late for the reason given in the warp-level kernel)
         const float inv = l > 0.f ? 1.f / l : 0.f;
         // O rows leave through shared memory so that the global stores are coalesced (a thread holds one whole row,
         // and 32 lanes storing 16 bytes each to 32 different rows cost a request per lane).  The tile's Q rows are

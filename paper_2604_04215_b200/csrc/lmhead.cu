@@ -103,6 +103,12 @@ lmhead_compact_kernel(const uint4* __restrict__ x, int M, int D8, const int32_t*
     __syncthreads();
     pdl_wait();
     pdl_trigger();
+    // the first pieces of this warp's row are on their way while the tokens are counted (a committed row's are dropped)
+    constexpr int AHEAD = 8;
+    const uint4* src = x + static_cast<size_t>(min(row0 + warp, M - 1)) * D8;
+    uint4 ahead[AHEAD];
+#pragma unroll
+    for (int u = 0; u < AHEAD; ++u) ahead[u] = lane + u * 32 < D8 ? src[lane + u * 32] : make_uint4(0, 0, 0, 0);
     int local = 0;
     for (int m = threadIdx.x; m < row0; m += blockDim.x) local += row_token(row_tokens, tok_L, tok_row_stride, m) == mask_id;
 #pragma unroll
@@ -129,10 +135,23 @@ lmhead_compact_kernel(const uint4* __restrict__ x, int M, int D8, const int32_t*
         return;
     }
     if (lane == 0) idx[before] = row;
-    const uint4* src = x + static_cast<size_t>(row) * D8;
     uint4* dst = xc + static_cast<size_t>(before) * D8;
     // eight loads in flight per lane before the first store: the copy of a row is a chain of latencies otherwise
-    int i = lane;
+    int i = lane + AHEAD * 32;
+    if (i + 7 * 32 < D8) {              // (the next batch is requested before the first is stored)
+        uint4 v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = src[i + u * 32];
+#pragma unroll
+        for (int u = 0; u < AHEAD; ++u) dst[lane + u * 32] = ahead[u];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) dst[i + u * 32] = v[u];
+        i += 8 * 32;
+    } else {
+#pragma unroll
+        for (int u = 0; u < AHEAD; ++u)
+            if (lane + u * 32 < D8) dst[lane + u * 32] = ahead[u];
+    }
     for (; i + 7 * 32 < D8; i += 8 * 32) {
         uint4 v[8];
 #pragma unroll
@@ -1138,7 +1157,6 @@ lmhead_merge_select_kernel(const LmParts parts, int grid_gemm, int n_tiles, int 
                            const int32_t* __restrict__ live_rows, const int32_t* __restrict__ idx, int32_t mask_id,
                            int32_t* __restrict__ pred, float* __restrict__ conf, int allow_pair, int parts_stride,
                            const LmSelect sel, uint32_t* __restrict__ step_dev) {
-    __shared__ int s_before;
     __shared__ int s_flag[32];
     __shared__ float s_conf[32];
     __shared__ int32_t s_pred[32];
@@ -1147,22 +1165,22 @@ lmhead_merge_select_kernel(const LmParts parts, int grid_gemm, int n_tiles, int 
     if (SAMPLE && step_dev && blockIdx.x == 0 && threadIdx.x == 0) *step_dev += 1;   // (as in lmhead_merge_kernel)
     const int b = blockIdx.x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;      // warp = block position (blockDim = 32 L)
-    const int Mc = *live_rows;
-    if (threadIdx.x == 0) {
-        // compacted rows that belong to earlier rollouts = first entry of the ascending row list that is >= b * L
-        int lo = 0, hi = Mc;
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (idx[mid] < b * L) lo = mid + 1; else hi = mid;
-        }
-        s_before = lo;
-    }
+    // What a warp needs first is requested together: its token, the number of live rows, the row list.  Compacted rows
+    // that belong to earlier rollouts = entries of the ascending list below b * L.  (A binary search by one thread, nine
+    // dependent loads at 512 rows, was half of this kernel's 8 us.)
     int32_t* row = sel.tokens_block + static_cast<int64_t>(b) * sel.row_stride;
     const bool masked = row[warp] == mask_id;
+    const int Mc = *live_rows;
     if (lane == 0) s_flag[warp] = masked ? 1 : 0;
+    int before = 0;
+    for (int i0 = 0; i0 < b * L; i0 += blockDim.x) {        // (rows of earlier rollouts: at most b * L of them)
+        const int i = i0 + threadIdx.x;
+        const int32_t v = i < b * L ? idx[i] : 0;           // (entries from Mc on hold anything)
+        before += __syncthreads_count(i < b * L && i < Mc && v < b * L);
+    }
     __syncthreads();
     if (masked) {
-        int c = s_before;
+        int c = before;
         for (int i = 0; i < warp; ++i) c += s_flag[i];
         const int groups = lm_row_partials(allow_pair, grid_gemm, Mc, n_tiles, c);
         int a;

@@ -119,3 +119,44 @@ def test_sampled_head_with_a_workspace_for_one_partial_per_tile():
     sure = ref["gap_y"] > 1e-3
     assert (pred.cpu().numpy()[sure] == ref["pred"][sure]).all()
     c.close()
+
+
+# A step is a chain of kernels in which each may start before its predecessor ends.  With a K/V split the attention's
+# partials lie behind the head's scratch; a workspace that does not hold both makes the halves run in sequence.  Steps
+# follow one another closely, on inputs that ordinary kernels overwrite in between: each must equal the parts run alone.
+@pytest.mark.parametrize("B,L,Hq,Hkv,P,workspace", [(1, 32, 4, 4, 1500, 0), (1, 32, 4, 4, 1500, 800000), (2, 40, 4, 2, 700, 0),
+                                                    (40, 4, 8, 8, 300, 0), (3, 32, 28, 4, 500, 0)])
+def test_steps_back_to_back_equal_their_parts(ctx, B, L, Hq, Hkv, P, workspace):
+    d, D, V, mu = 128, 512, 3000, 2990
+    c = dare.Context(0, workspace) if workspace else ctx
+    mode, k, n_steps = dare.SELECT_TOPK, 2, 6
+    g = torch.Generator(device="cuda")
+    g.manual_seed(5)
+    rnd = lambda *s: torch.randn(s, generator=g, device="cuda").to(torch.bfloat16)  # noqa: E731
+    w = rnd(V, D) * 0.05
+    k_pre, v_pre, plen = rnd(B, Hkv, P, d), rnd(B, Hkv, P, d), torch.full((B,), P - 3, dtype=torch.int32, device="cuda")
+    acts = [(rnd(B, L, Hq, d), rnd(B, Hkv, L, d), rnd(B, Hkv, L, d), rnd(B * L, D)) for _ in range(n_steps)]
+    bufs = [torch.empty_like(t) for t in acts[0]]
+    new = lambda n, t: torch.zeros(n, dtype=t, device="cuda")  # noqa: E731
+    tok = torch.full((B, P + L), mu, dtype=torch.int32, device="cuda")
+    ref_tok = tok.clone()
+    got = []
+    for a in acts:
+        for dst, src in zip(bufs, a):
+            dst.copy_(src)
+        out, pred, conf, nc, nr = torch.empty_like(a[0]), new(B * L, torch.int32), new(B * L, torch.float32), new(B, torch.int32), new(B, torch.int32)
+        dare.dare_denoise_block(c, bufs[0], k_pre, v_pre, plen, bufs[1], bufs[2], None, None, None, out, None, bufs[3], w, mu,
+                                True, tok, P, mode, 0.0, k, pred, conf, nc, nr)
+        got.append((out, pred, conf, nc, nr))
+    for a, (out, pred, conf, nc, nr) in zip(acts, got):
+        ref_out = dare.dare_attn_block(ctx, a[0], k_pre, v_pre, plen, a[1], a[2])
+        p2, c2 = dare.dare_lmhead_confidence(ctx, a[3], w, ref_tok[:, P:].contiguous().view(-1), mu, True)
+        nc2, nr2 = new(B, torch.int32), new(B, torch.int32)
+        dare.dare_unmask_select(ctx, ref_tok, P, L, p2, c2, mu, mode, 0.0, k, nc2, nr2)
+        torch.cuda.synchronize()
+        for x, y in ((out, ref_out), (pred, p2), (conf, c2), (nc, nc2), (nr, nr2)):
+            assert torch.equal(x, y)
+    assert torch.equal(tok, ref_tok)
+    assert c.device_status() == 0
+    if workspace:
+        c.close()
