@@ -151,7 +151,18 @@ def _ptr(t: Optional[torch.Tensor], dtype=None):
     return C.c_void_p(t.data_ptr())
 
 
-def _count_ptr(t: Optional[torch.Tensor]):
+def _addr(t: Optional[torch.Tensor], dtype, device: int):
+    """The checks of _ptr for the calls of a rollout's inner loop, as few as they can be (a step of a small block is
+    shorter on the GPU than the marshalling of its 13 tensors was): `device` is the current one, asked for once per call,
+    and the address goes to ctypes as a plain integer."""
+    if t is None:
+        return None
+    if t.get_device() != device or not t.is_contiguous() or t.dtype is not dtype:      # (get_device(): -1 on the host)
+        return _ptr(t, dtype)          # says what is wrong
+    return t.data_ptr()
+
+
+def _count_ptr(t: Optional[torch.Tensor], device: Optional[int] = None):
     """The per-rollout count outputs (n_committed, n_remaining): a device tensor, or a page-locked host tensor (the
     kernel then stores its B integers straight into host memory and the caller needs no copy back)."""
     if t is not None and not t.is_cuda:
@@ -160,11 +171,17 @@ def _count_ptr(t: Optional[torch.Tensor]):
         if t.dtype != torch.int32:
             raise ValueError(f"expected dtype {torch.int32}, got {t.dtype}")
         return C.c_void_p(t.data_ptr())
-    return _ptr(t, torch.int32)
+    return _ptr(t, torch.int32) if device is None else _addr(t, torch.int32, device)
 
 
-def _stream(stream) -> C.c_void_p:
+# the handle of the current stream without a stream object around it
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
+def _stream(stream, device: Optional[int] = None) -> C.c_void_p:
     if stream is None:
+        if device is not None and _raw_stream is not None:
+            return _raw_stream(device)
         stream = torch.cuda.current_stream()
     return C.c_void_p(stream.cuda_stream)
 
@@ -220,11 +237,12 @@ def dare_attn_block(ctx: Context, q, k_pre, v_pre, prefix_len=None, k_blk=None, 
     if out is None:
         out = torch.empty_like(q)
     bf = torch.bfloat16
+    dev = torch.cuda.current_device()
     rc = load().dare_attn_block(ctx.handle, B, L, Hq, Hkv, d, prefix_cap, suffix_cap, float(scale),
-                                _ptr(q, bf), _ptr(k_pre, bf), _ptr(v_pre, bf), _ptr(prefix_len, torch.int32),
-                                _ptr(k_blk, bf), _ptr(v_blk, bf), _ptr(k_suf, bf), _ptr(v_suf, bf),
-                                _ptr(suffix_len, torch.int32), _ptr(out, bf), _ptr(lse, torch.float32),
-                                _stream(stream))
+                                _addr(q, bf, dev), _addr(k_pre, bf, dev), _addr(v_pre, bf, dev), _addr(prefix_len, torch.int32, dev),
+                                _addr(k_blk, bf, dev), _addr(v_blk, bf, dev), _addr(k_suf, bf, dev), _addr(v_suf, bf, dev),
+                                _addr(suffix_len, torch.int32, dev), _addr(out, bf, dev), _addr(lse, torch.float32, dev),
+                                _stream(stream, dev))
     if rc != 0 and check:
         raise DareError(rc, "dare_attn_block")
     return out if check else rc
@@ -237,9 +255,10 @@ def dare_attn_varlen(ctx: Context, q, k, v, cu_seqlens, max_seqlen: int, out=Non
     if out is None:
         out = torch.empty_like(q)
     bf = torch.bfloat16
+    dev = torch.cuda.current_device()
     rc = load().dare_attn_varlen(ctx.handle, total, cu_seqlens.numel() - 1, int(max_seqlen), Hq, Hkv, d, float(scale),
-                                 _ptr(q, bf), _ptr(k, bf), _ptr(v, bf), _ptr(cu_seqlens, torch.int32), _ptr(out, bf),
-                                 _ptr(lse, torch.float32), _stream(stream))
+                                 _addr(q, bf, dev), _addr(k, bf, dev), _addr(v, bf, dev), _addr(cu_seqlens, torch.int32, dev), _addr(out, bf, dev),
+                                 _addr(lse, torch.float32, dev), _stream(stream, dev))
     if rc != 0 and check:
         raise DareError(rc, "dare_attn_varlen")
     return out if check else rc
@@ -253,9 +272,10 @@ def dare_lmhead_confidence(ctx: Context, hidden, w, row_tokens=None, mask_id: in
         pred = torch.empty(M, dtype=torch.int32, device=hidden.device)
     if conf is None:
         conf = torch.empty(M, dtype=torch.float32, device=hidden.device)
-    rc = load().dare_lmhead_confidence(ctx.handle, _ptr(hidden, torch.bfloat16), M, D, _ptr(w, torch.bfloat16), V,
-                                       _ptr(row_tokens, torch.int32), int(mask_id), int(bool(exclude_mask_column)),
-                                       _ptr(pred, torch.int32), _ptr(conf, torch.float32), _stream(stream))
+    dev = torch.cuda.current_device()
+    rc = load().dare_lmhead_confidence(ctx.handle, _addr(hidden, torch.bfloat16, dev), M, D, _addr(w, torch.bfloat16, dev), V,
+                                       _addr(row_tokens, torch.int32, dev), int(mask_id), int(bool(exclude_mask_column)),
+                                       _addr(pred, torch.int32, dev), _addr(conf, torch.float32, dev), _stream(stream, dev))
     if rc != 0 and check:
         raise DareError(rc, "dare_lmhead_confidence")
     return (pred, conf) if check else rc
@@ -395,10 +415,11 @@ def dare_unmask_select(ctx: Context, tokens, block_start: int, L: int, pred, con
                        threshold: float = 0.0, k: int = 1, n_committed=None, n_remaining=None, stream=None,
                        check: bool = True):
     B, row_stride = tokens.shape
-    rc = load().dare_unmask_select(ctx.handle, _ptr(tokens, torch.int32), B, row_stride, int(block_start), int(L),
-                                   _ptr(pred, torch.int32), _ptr(conf, torch.float32), int(mask_id), int(mode),
-                                   float(threshold), int(k), _count_ptr(n_committed),
-                                   _count_ptr(n_remaining), _stream(stream))
+    dev = torch.cuda.current_device()
+    rc = load().dare_unmask_select(ctx.handle, _addr(tokens, torch.int32, dev), B, row_stride, int(block_start), int(L),
+                                   _addr(pred, torch.int32, dev), _addr(conf, torch.float32, dev), int(mask_id), int(mode),
+                                   float(threshold), int(k), _count_ptr(n_committed, dev),
+                                   _count_ptr(n_remaining, dev), _stream(stream, dev))
     if rc != 0 and check:
         raise DareError(rc, "dare_unmask_select")
     return rc
@@ -414,14 +435,15 @@ def dare_denoise_block(ctx: Context, q, k_pre, v_pre, prefix_len, k_blk, v_blk, 
     D = hidden.shape[1]
     V = w.shape[0]
     bf = torch.bfloat16
+    dev = torch.cuda.current_device()
     rc = load().dare_denoise_block(
         ctx.handle, B, L, Hq, Hkv, d, prefix_cap, suffix_cap, float(scale),
-        _ptr(q, bf), _ptr(k_pre, bf), _ptr(v_pre, bf), _ptr(prefix_len, torch.int32), _ptr(k_blk, bf), _ptr(v_blk, bf),
-        _ptr(k_suf, bf), _ptr(v_suf, bf), _ptr(suffix_len, torch.int32), _ptr(attn_out, bf), _ptr(lse, torch.float32),
-        _ptr(hidden, bf), D, _ptr(w, bf), V, int(mask_id), int(bool(exclude_mask_column)),
-        _ptr(tokens, torch.int32), tokens.shape[1], int(block_start), int(mode), float(threshold), int(k),
-        _ptr(pred, torch.int32), _ptr(conf, torch.float32), _count_ptr(n_committed),
-        _count_ptr(n_remaining), _stream(stream))
+        _addr(q, bf, dev), _addr(k_pre, bf, dev), _addr(v_pre, bf, dev), _addr(prefix_len, torch.int32, dev), _addr(k_blk, bf, dev), _addr(v_blk, bf, dev),
+        _addr(k_suf, bf, dev), _addr(v_suf, bf, dev), _addr(suffix_len, torch.int32, dev), _addr(attn_out, bf, dev), _addr(lse, torch.float32, dev),
+        _addr(hidden, bf, dev), D, _addr(w, bf, dev), V, int(mask_id), int(bool(exclude_mask_column)),
+        _addr(tokens, torch.int32, dev), tokens.shape[1], int(block_start), int(mode), float(threshold), int(k),
+        _addr(pred, torch.int32, dev), _addr(conf, torch.float32, dev), _count_ptr(n_committed, dev),
+        _count_ptr(n_remaining, dev), _stream(stream, dev))
     if rc != 0 and check:
         raise DareError(rc, "dare_denoise_block")
     return rc
@@ -438,15 +460,16 @@ def dare_denoise_block_sampled(ctx: Context, q, k_pre, v_pre, prefix_len, k_blk,
     D = hidden.shape[1]
     V = w.shape[0]
     bf = torch.bfloat16
+    dev = torch.cuda.current_device()
     rc = load().dare_denoise_block_sampled(
         ctx.handle, B, L, Hq, Hkv, d, prefix_cap, suffix_cap, float(scale),
-        _ptr(q, bf), _ptr(k_pre, bf), _ptr(v_pre, bf), _ptr(prefix_len, torch.int32), _ptr(k_blk, bf), _ptr(v_blk, bf),
-        _ptr(k_suf, bf), _ptr(v_suf, bf), _ptr(suffix_len, torch.int32), _ptr(attn_out, bf), _ptr(lse, torch.float32),
-        _ptr(hidden, bf), D, _ptr(w, bf), V, int(mask_id), int(bool(exclude_mask_column)), float(temperature),
+        _addr(q, bf, dev), _addr(k_pre, bf, dev), _addr(v_pre, bf, dev), _addr(prefix_len, torch.int32, dev), _addr(k_blk, bf, dev), _addr(v_blk, bf, dev),
+        _addr(k_suf, bf, dev), _addr(v_suf, bf, dev), _addr(suffix_len, torch.int32, dev), _addr(attn_out, bf, dev), _addr(lse, torch.float32, dev),
+        _addr(hidden, bf, dev), D, _addr(w, bf, dev), V, int(mask_id), int(bool(exclude_mask_column)), float(temperature),
         int(seed) & 0xFFFFFFFFFFFFFFFF, int(step) & 0xFFFFFFFF,
-        _ptr(tokens, torch.int32), tokens.shape[1], int(block_start), int(mode), float(threshold), int(k),
-        _ptr(pred, torch.int32), _ptr(conf, torch.float32), _count_ptr(n_committed),
-        _count_ptr(n_remaining), _stream(stream))
+        _addr(tokens, torch.int32, dev), tokens.shape[1], int(block_start), int(mode), float(threshold), int(k),
+        _addr(pred, torch.int32, dev), _addr(conf, torch.float32, dev), _count_ptr(n_committed, dev),
+        _count_ptr(n_remaining, dev), _stream(stream, dev))
     if rc != 0 and check:
         raise DareError(rc, "dare_denoise_block_sampled")
     return rc
@@ -551,10 +574,11 @@ def dare_model_step(model: Model, tokens, block_start: int, L: int, k_cache, v_c
                     k: int, pred, conf, n_committed=None, n_remaining=None, stream=None, check: bool = True):
     B, row_stride = tokens.shape
     bf = torch.bfloat16
-    rc = load().dare_model_step(model.handle, _ptr(tokens, torch.int32), B, row_stride, int(block_start), int(L),
-                                _ptr(k_cache, bf), _ptr(v_cache, bf), k_cache.shape[3], int(mode), float(threshold),
-                                int(k), _ptr(pred, torch.int32), _ptr(conf, torch.float32),
-                                _count_ptr(n_committed), _count_ptr(n_remaining), _stream(stream))
+    dev = torch.cuda.current_device()
+    rc = load().dare_model_step(model.handle, _addr(tokens, torch.int32, dev), B, row_stride, int(block_start), int(L),
+                                _addr(k_cache, bf, dev), _addr(v_cache, bf, dev), k_cache.shape[3], int(mode), float(threshold),
+                                int(k), _addr(pred, torch.int32, dev), _addr(conf, torch.float32, dev),
+                                _count_ptr(n_committed, dev), _count_ptr(n_remaining, dev), _stream(stream, dev))
     if rc != 0 and check:
         raise DareError(rc, "dare_model_step")
     return rc
@@ -593,10 +617,11 @@ def dare_model_step_window(model: Model, tokens, block_start: int, L: int, kv_le
                            check: bool = True):
     B, row_stride = tokens.shape
     bf = torch.bfloat16
-    rc = load().dare_model_step_window(model.handle, _ptr(tokens, torch.int32), B, row_stride, int(block_start), int(L),
-                                       int(kv_len), _ptr(k_cache, bf), _ptr(v_cache, bf), k_cache.shape[3], int(mode),
-                                       float(threshold), int(k), _ptr(pred, torch.int32), _ptr(conf, torch.float32),
-                                       _count_ptr(n_committed), _count_ptr(n_remaining), _stream(stream))
+    dev = torch.cuda.current_device()
+    rc = load().dare_model_step_window(model.handle, _addr(tokens, torch.int32, dev), B, row_stride, int(block_start), int(L),
+                                       int(kv_len), _addr(k_cache, bf, dev), _addr(v_cache, bf, dev), k_cache.shape[3], int(mode),
+                                       float(threshold), int(k), _addr(pred, torch.int32, dev), _addr(conf, torch.float32, dev),
+                                       _count_ptr(n_committed, dev), _count_ptr(n_remaining, dev), _stream(stream, dev))
     if rc != 0 and check:
         raise DareError(rc, "dare_model_step_window")
     return rc
