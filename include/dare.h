@@ -342,8 +342,8 @@ int dare_linear(dare_ctx* ctx, int epilogue, const void* a, int M, int K, const 
  * column tiles, clusters resident at once}.  M > 128: a work item is a PAIR of CTAs (a cluster of two) that
  * computes two row tiles with 256-row MMAs; entry 3 is the number of pairs along K (1 or 2; two pairs form a
  * cluster of four CTAs) and entry 7 the number of such clusters resident at once.
- * M <= 128: one CTA per (row tile, column tile, K slice); the K slices of a tile form a cluster and entry 7
- * is 0 without a K split. */
+ * M <= 128: one CTA per (column tile, K slice); the K slices of a tile form a cluster (entry 3: 1, 2, 4 or 8) and
+ * entry 7 is 0. */
 int dare_linear_plan(dare_ctx* ctx, int epilogue, int M, int K, int N, int* plan_out);
 int dare_rmsnorm(dare_ctx* ctx, const void* x, int n_rows, int D, float eps, void* y, void* stream);
 int dare_rope_kv_write(dare_model* model, const void* qkv, int B, int length, int start, void* q_out,

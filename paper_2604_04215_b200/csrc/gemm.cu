@@ -1,26 +1,18 @@
 // Dense bf16 projections of the layer stack on the tcgen05 tensor cores: out = epilogue(A W^T).
 //
-// A [M, K] activations and W [N, K] weights are both K-major bf16.  Problems with two or more row tiles run on
-// CTA pairs (gemm_pair_kernel, further down); the single-CTA kernel described here serves the rest and is the
-// shape the pair kernel is derived from.  One CTA computes one output tile of up to
-// two 128-row tiles by `bn` columns over a range of K:
-//   warp 0      TMA producer: one or two A tiles [128 x 64] and a W tile [bn x 64] per stage (128-byte swizzle)
-//   warp 1      UMMA issuer: 128 x bn x 16 MMAs, one fp32 accumulator in TMEM per row tile
-//   warps 2..9  epilogue: one TMEM lane = one output row per thread, 8 columns at a time
-// The tile shape is chosen per problem on the host (gemm_plan): at the few hundred rows of a denoising step a
-// projection has too few 128 x 256 tiles to fill the SMs evenly, so the column width bn (any multiple of 16)
-// and, for long K, a split of K are picked so that the CTAs make whole waves; two row tiles per CTA share
-// each W tile, which keeps the shared-memory and L2 traffic per flop low.  CTAs are numbered with the row index
-// fastest, so the CTAs that share a weight tile run at the same time and the weights leave HBM once.
+// A [M, K] activations and W [N, K] weights are both K-major bf16.  Problems of up to 128 rows are bound by reading W and
+// run in gemm_few.cu; here is the rest, on CTA pairs (gemm_pair_kernel):
+//   warp 0      TMA producer: a 128-row A tile and half of the W rows per MMA and stage (128-byte swizzle)
+//   warp 1      UMMA issuer (even CTA): MMAs of 256 rows, fp32 accumulators in TMEM
+//   warps 2..9  epilogue: one TMEM lane = one output row per thread
+// The tile shape is chosen per problem on the host (pair_plan): at the few hundred rows of a denoising step a
+// projection has too few 256 x 256 tiles to fill the SMs evenly, so the column width and, for long K, a split of K are
+// picked so that the pairs make whole rounds.
 // Epilogues: plain bf16 store (QKV projection); residual add, rounded once after the add (attention output
-// and feed-forward down projections, in place on the residual stream); SwiGLU, where a tile holds w gate
-// columns and the matching w up columns (two TMA loads, one per matrix) and silu(g) * u is formed in
+// and feed-forward down projections, in place on the residual stream); SwiGLU, where a tile holds gate
+// columns and the matching up columns and silu(g) * u is formed in
 // registers, so the 2F-wide intermediate never reaches memory; RoPE for the QKV projection of many rows, whose tiles
 // then hold whole heads, so that q, k and v go from the accumulator to where the attention reads them.
-// Split K: the CTAs that share an output tile form a thread-block cluster.  After the main loop each CTA
-// sends, through distributed shared memory, the accumulator column groups it does not own into the idle
-// operand ring of the CTA that owns them; every CTA then adds the partials of its own groups in split order
-// and applies the epilogue, so all CTAs of the cluster share the output work and nothing goes through HBM.
 #include <math.h>
 
 #include "internal.h"
@@ -35,35 +27,8 @@ constexpr int GEMM_THREADS = 320;
 constexpr int A_TILE_BYTES = GM * GK * 2;
 constexpr int MAX_STAGES = 8;
 constexpr int RING_BYTES = 226 * 1024;      // shared memory for the operand ring (the CTA has 227 KB)
-constexpr int MAX_SPLITS = 2;                // CTAs along K per output tile (pairs are always co-resident)
-constexpr int L2_AHEAD = 8;                 // pipeline steps between the L2 prefetch of a W tile and its load
 
-struct GemmBarriers {
-    uint64_t full[MAX_STAGES];
-    uint64_t empty[MAX_STAGES];
-    uint64_t tmem_full;
-    uint32_t tmem_base;
-    uint32_t abort_flag;
-};
 constexpr int GEMM_SMEM_BYTES = RING_BYTES - 1024;   // dynamic request; the ring starts at the next 1 KB boundary
-
-struct GemmPlan {
-    int nsub;        // row tiles per CTA (1 or 2)
-    int bn;          // MMA N: columns of W per tile (SwiGLU: w gate rows + w up rows)
-    int wcols;       // output columns per tile (bn, or bn / 2 for SwiGLU)
-    int splits;      // CTAs along K per output tile
-    int stages;
-    int m_items, n_tiles;
-    uint32_t tmem_cols;
-};
-
-struct GemmArgs {
-    int M, N, K, ldo;
-    GemmPlan p;
-    __nv_bfloat16* out;
-    const __nv_bfloat16* res;
-    uint32_t* dev_status;
-};
 
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
@@ -98,217 +63,6 @@ __device__ __forceinline__ void store_group(const float (&f)[8], const float (&u
     o.x = pack_bf16(r[0], r[1]); o.y = pack_bf16(r[2], r[3]);
     o.z = pack_bf16(r[4], r[5]); o.w = pack_bf16(r[6], r[7]);
     *reinterpret_cast<uint4*>(out + off) = o;
-}
-
-template <int EPI>
-__global__ void __launch_bounds__(GEMM_THREADS, 1)
-gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
-                 const __grid_constant__ CUtensorMap tmap_b2, const GemmArgs g) {
-    const GemmPlan& p = g.p;
-    const int stage_bytes = p.nsub * A_TILE_BYTES + p.bn * (GK * 2);
-
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    GemmBarriers* bars = reinterpret_cast<GemmBarriers*>(tiles + p.stages * stage_bytes);
-    volatile uint32_t* abort_flag = &bars->abort_flag;
-
-    const int warp = warp_index_uniform();
-    const int lane = threadIdx.x & 31;
-    // CTA -> (K split, row item, column tile): the splits of one output tile form a cluster, row items next
-    const int split = p.splits > 1 ? static_cast<int>(cluster_cta_rank()) : 0;
-    const int m_item = (blockIdx.x / p.splits) % p.m_items;
-    const int n_tile = blockIdx.x / (p.m_items * p.splits);
-    const int nk = (g.K + GK - 1) / GK;
-    const int kb_begin = static_cast<int>(static_cast<long long>(nk) * split / p.splits);
-    const int kb_end = static_cast<int>(static_cast<long long>(nk) * (split + 1) / p.splits);
-
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < p.stages; ++s) {
-            mbar_init(&bars->full[s], 1);
-            mbar_init(&bars->empty[s], 1);
-        }
-        mbar_init(&bars->tmem_full, 1);
-        bars->abort_flag = 0;
-        fence_barrier_init();
-    }
-    if (warp == 1) {
-        tmem_alloc(&bars->tmem_base, p.tmem_cols);
-        tmem_relinquish();
-    }
-    tc_fence_before_sync();
-    __syncthreads();
-    tc_fence_after_sync();
-    const uint32_t tmem_base = bars->tmem_base;
-    const int acc_stride = p.nsub == 2 ? 256 : 0;   // accumulator of row tile s starts at column s * 256
-
-    if (warp == 0) {
-        if (lane == 0) {
-            prefetch_tensormap(&tmap_a);
-            prefetch_tensormap(&tmap_b);
-            if (EPI == GEMM_EPI_SWIGLU) prefetch_tensormap(&tmap_b2);
-            int stage = 0;
-            uint32_t phase = 0;
-            pdl_wait();
-            // the weights come from HBM: ask L2 for them L2_AHEAD steps before the load that needs them
-            for (int kb = kb_begin; kb < kb_end && kb < kb_begin + L2_AHEAD; ++kb) {
-                tma_prefetch_l2_2d(&tmap_b, kb * GK, n_tile * (EPI == GEMM_EPI_SWIGLU ? p.wcols : p.bn));
-                if (EPI == GEMM_EPI_SWIGLU) tma_prefetch_l2_2d(&tmap_b2, kb * GK, n_tile * p.wcols);
-            }
-            for (int kb = kb_begin; kb < kb_end; ++kb) {
-                if (kb + L2_AHEAD < kb_end) {
-                    tma_prefetch_l2_2d(&tmap_b, (kb + L2_AHEAD) * GK, n_tile * (EPI == GEMM_EPI_SWIGLU ? p.wcols : p.bn));
-                    if (EPI == GEMM_EPI_SWIGLU) tma_prefetch_l2_2d(&tmap_b2, (kb + L2_AHEAD) * GK, n_tile * p.wcols);
-                }
-                if (!mbar_wait(&bars->empty[stage], phase ^ 1, abort_flag)) break;
-                uint8_t* a_dst = tiles + stage * stage_bytes;
-                uint8_t* b_dst = a_dst + p.nsub * A_TILE_BYTES;
-                mbar_arrive_expect_tx(&bars->full[stage], stage_bytes);
-                for (int s = 0; s < p.nsub; ++s)
-                    tma_load_2d(a_dst + s * A_TILE_BYTES, &tmap_a, &bars->full[stage], kb * GK, (m_item * p.nsub + s) * GM);
-                if (EPI == GEMM_EPI_SWIGLU) {
-                    tma_load_2d(b_dst, &tmap_b, &bars->full[stage], kb * GK, n_tile * p.wcols);
-                    tma_load_2d(b_dst + p.wcols * (GK * 2), &tmap_b2, &bars->full[stage], kb * GK, n_tile * p.wcols);
-                } else {
-                    tma_load_2d(b_dst, &tmap_b, &bars->full[stage], kb * GK, n_tile * p.bn);
-                }
-                if (++stage == p.stages) { stage = 0; phase ^= 1; }
-            }
-        }
-    } else if (warp == 1) {
-        // all lanes run the loop, one elected lane issues the MMAs and their commits
-        const bool leader = elect_one_sync();
-        const uint32_t idesc = umma_idesc_bf16(GM, p.bn);
-        int stage = 0;
-        uint32_t phase = 0;
-        bool ok = true;
-        for (int kb = kb_begin; kb < kb_end; ++kb) {
-            ok = __all_sync(0xffffffffu, mbar_wait(&bars->full[stage], phase, abort_flag));
-            if (!ok) break;
-            tc_fence_after_sync();
-            const uint32_t a_addr = smem_u32(tiles + stage * stage_bytes);
-            const uint64_t b_desc = umma_desc_sw128_kmajor(a_addr + p.nsub * A_TILE_BYTES);
-            const uint32_t accumulate = kb > kb_begin;
-            if (leader) {
-                for (int s = 0; s < p.nsub; ++s) {
-                    const uint64_t a_desc = umma_desc_sw128_kmajor(a_addr + s * A_TILE_BYTES);
-#pragma unroll
-                    for (int kk = 0; kk < GK / 16; ++kk)   // +32 bytes along K per step = +2 descriptor units
-                        umma_bf16(tmem_base + s * acc_stride, a_desc + 2 * kk, b_desc + 2 * kk, idesc,
-                                  accumulate | (kk != 0));
-                }
-                umma_commit(&bars->empty[stage]);
-            }
-            __syncwarp();
-            if (++stage == p.stages) { stage = 0; phase ^= 1; }
-        }
-        if (ok && leader) umma_commit(&bars->tmem_full);
-        __syncwarp();
-    }
-
-    // ---- epilogue (warps 2..9).  Warp w may touch TMEM lanes [32 * (w % 4), +32); warps 2..5 are set 0, warps
-    // 6..9 set 1.  Two row tiles: set s owns row tile s.  One row tile: the sets share it, alternating 8-column
-    // groups.  With a K split the CTAs of the cluster first hand each other the column groups they do not own.
-    const bool epi_warp = warp >= 2;
-    const int lq = warp & 3;
-    const int set = epi_warp ? (warp - 2) >> 2 : 0;
-    const int rt = p.nsub == 2 ? set : 0;
-    const int g_first = p.nsub == 2 ? 0 : set, g_step = p.nsub == 2 ? 1 : 2;
-    const int n_groups = p.wcols / 8;
-    const int tile_rows = p.nsub * GM;
-    const int row_local = rt * GM + lq * 32 + lane;
-    const int row = m_item * tile_rows + row_local;
-    const bool row_ok = row < g.M;
-    const size_t row_off = static_cast<size_t>(row) * g.ldo;
-    const int col_base = n_tile * p.wcols;
-    const uint32_t taddr = tmem_base + (static_cast<uint32_t>(lq * 32) << 16) + rt * acc_stride;
-    if (epi_warp) {
-        pdl_wait();
-        mbar_wait(&bars->tmem_full, 0, abort_flag);     // (a wait that gave up leaves the abort flag set)
-        pdl_trigger();
-        tc_fence_after_sync();
-    }
-    __syncwarp();
-    if (p.splits > 1) {
-        // Group gi belongs to the CTA of rank gi % splits.  Receiver layout in the (now idle) operand ring:
-        // [slot of the sending split, ascending, own split left out][gi / splits][row][8 floats].
-        const int per_owner = (n_groups + p.splits - 1) / p.splits;
-        cluster_sync_all();                              // every CTA of the cluster is done with its ring
-        if (epi_warp) {
-            const uint32_t ring = smem_u32(tiles);
-            for (int gi = g_first; gi < n_groups; gi += g_step) {
-                const int owner = gi % p.splits;
-                if (owner == split) continue;
-                uint32_t v[8];
-                tmem_ld_8cols(taddr + gi * 8, v);
-                tmem_ld_wait();
-                const int slot = split < owner ? split : split - 1;
-                const uint32_t local = ring + ((static_cast<uint32_t>(slot * per_owner + gi / p.splits) * tile_rows + row_local) << 5);
-                const uint32_t remote = cluster_map_shared(local, static_cast<uint32_t>(owner));
-                st_shared_cluster_v4(remote, v[0], v[1], v[2], v[3]);
-                st_shared_cluster_v4(remote + 16, v[4], v[5], v[6], v[7]);
-            }
-        }
-        cluster_sync_all();                              // the partials of the groups this CTA owns have arrived
-    }
-    if (epi_warp && !*abort_flag) {
-        for (int gi = g_first; gi < n_groups; gi += g_step) {
-            if (p.splits > 1 && gi % p.splits != split) continue;
-            uint32_t v[8];
-            float f[8], u[8];
-            tmem_ld_8cols(taddr + gi * 8, v);
-            if (EPI == GEMM_EPI_SWIGLU) {
-                uint32_t w[8];
-                tmem_ld_8cols(taddr + p.wcols + gi * 8, w);
-                tmem_ld_wait();
-#pragma unroll
-                for (int j = 0; j < 8; ++j) u[j] = __uint_as_float(w[j]);
-            } else {
-                tmem_ld_wait();
-#pragma unroll
-                for (int j = 0; j < 8; ++j) u[j] = 0.f;
-            }
-            if (p.splits > 1) {
-                // add the partials in split order; this CTA's own values take their place in it
-                const int per_owner = (n_groups + p.splits - 1) / p.splits;
-                const float* base = reinterpret_cast<const float*>(tiles) +
-                                    (static_cast<size_t>(gi / p.splits) * tile_rows + row_local) * 8;
-#pragma unroll
-                for (int j = 0; j < 8; ++j) f[j] = 0.f;
-                for (int s = 0; s < p.splits; ++s) {
-                    if (s == split) {
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) f[j] += __uint_as_float(v[j]);
-                    } else {
-                        const int slot = s < split ? s : s - 1;
-                        const float4* q = reinterpret_cast<const float4*>(base + static_cast<size_t>(slot) * per_owner * tile_rows * 8);
-                        const float4 a = q[0], c = q[1];
-                        f[0] += a.x; f[1] += a.y; f[2] += a.z; f[3] += a.w;
-                        f[4] += c.x; f[5] += c.y; f[6] += c.z; f[7] += c.w;
-                    }
-                }
-            } else {
-#pragma unroll
-                for (int j = 0; j < 8; ++j) f[j] = __uint_as_float(v[j]);
-            }
-            const int col = col_base + gi * 8;
-            if (row_ok && col < g.N)          // N is a multiple of 8: a group of 8 columns is inside or outside
-                store_group<EPI>(f, u, g.out, g.res, row_off + col);
-        }
-    }
-
-    // teardown
-    tc_fence_before_sync();
-    __syncthreads();
-    if (*abort_flag) {
-        const long long t0 = clock64();
-        while (clock64() - t0 < 2000000LL) {}   // let copies in flight land before the shared memory goes away
-        if (threadIdx.x == 0) atomicOr(g.dev_status, DEV_WAIT_EXPIRED);
-        __syncthreads();
-    }
-    if (warp == 1) {
-        tc_fence_after_sync();
-        tmem_dealloc(tmem_base, p.tmem_cols);
-    }
 }
 
 // ---------------------------------------------------------------------------------------------------------
@@ -785,8 +539,8 @@ int max_active_pairs(int splits = 1) {
 // Tile shape for the pair kernel.  Per K block a CTA's time is the largest of: its MMA time (nchunk / 2 cycles
 // per MMA plus the ~45 measured on top of that), its shared-memory traffic (the stage written by the copies plus, per MMA, 4 KB of
 // A and its half of W read by the tensor core) at 128 bytes per cycle, and the operand delivery at ~55 bytes
-// per cycle; a launch takes as many rounds as the pairs need on the device.  cost_out: the model's cycles.
-PairPlan pair_plan(int epi, int M, int N, int K, int head_dim, double* cost_out) {
+// per cycle; a launch takes as many rounds as the pairs need on the device.
+PairPlan pair_plan(int epi, int M, int N, int K, int head_dim) {
     PairPlan best{};
     double best_cost = 1e300;
     const int nk = (K + GK - 1) / GK;
@@ -832,168 +586,57 @@ PairPlan pair_plan(int epi, int M, int N, int K, int head_dim, double* cost_out)
     const long long fit = GROUP_BYTES / (static_cast<long long>(2 * GM) * 2 * K);
     const int n_groups = static_cast<int>(fit < 1 ? m_pairs : (m_pairs + fit - 1) / fit);
     best.group = (m_pairs + n_groups - 1) / n_groups;       // groups of even size
-    if (cost_out) *cost_out = best_cost;
-    return best;
-}
-
-template <int EPI>
-int launch_one(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tb2, const GemmArgs& g,
-               cudaStream_t stream, int* max_clusters_query) {
-    static std::atomic<uint64_t> smem_set{0};
-    if (ensure_dynamic_smem(smem_set, gemm_bf16_kernel<EPI>, GEMM_SMEM_BYTES) != DARE_OK) return DARE_ERR_CUDA;
-    const long long ctas = static_cast<long long>(g.p.m_items) * g.p.n_tiles * g.p.splits;
-    if (ctas > 0x7fffffffLL) return DARE_ERR_SHAPE;
-    if (max_clusters_query)       // how many clusters of this size the device runs at once (plan input)
-        return query_max_clusters(gemm_bf16_kernel<EPI>, static_cast<unsigned>(g.p.splits) * 1024u, GEMM_THREADS,
-                                  GEMM_SMEM_BYTES, g.p.splits, max_clusters_query);
-    return launch_kernel(gemm_bf16_kernel<EPI>, dim3(static_cast<unsigned>(ctas)), GEMM_THREADS, GEMM_SMEM_BYTES, stream,
-                         g.p.splits, ta, tb, tb2, g);
-}
-
-// Clusters of `splits` CTAs of this kernel that can be resident at once (cached; 0 = such clusters cannot run).
-int max_active_clusters(int splits) {
-    static int cache[MAX_SPLITS + 1] = {-1, -1, -1};
-    if (cache[splits] < 0) {
-        GemmArgs g{};
-        g.p.m_items = g.p.n_tiles = 1;
-        g.p.splits = splits;
-        CUtensorMap dummy{};
-        int n = 0;
-        if (launch_one<GEMM_EPI_STORE>(dummy, dummy, dummy, g, nullptr, &n) != DARE_OK) n = 0;
-        cache[splits] = n;
-    }
-    return cache[splits];
-}
-
-// Picks the tile shape by a small cost model: a CTA's time is the longer of its MMA issue time (bn / 2 cycles
-// per 128 x bn x 16 MMA) and its operand traffic at ~55 bytes per cycle (what L2 delivers per SM when every SM streams), plus prologue and epilogue; the launch
-// takes as many rounds of it as the CTAs (or clusters, with a K split) need on the device.
-GemmPlan gemm_plan(int epi, int M, int N, int K, int sm_count) {
-    const int nk = (K + GK - 1) / GK;
-    const int m_tiles = (M + GM - 1) / GM;
-    const int ring = GEMM_SMEM_BYTES - 1024 - 256;
-    GemmPlan best{};
-    double best_cost = 1e300;
-    for (int nsub = 1; nsub <= (m_tiles >= 2 ? 2 : 1); ++nsub) {
-        const int m_items = (m_tiles + nsub - 1) / nsub;
-        for (int bn = 256; bn >= 32; bn -= 16) {
-            const int wcols = epi == GEMM_EPI_SWIGLU ? bn / 2 : bn;
-            if (wcols > ((N + 7) / 8) * 8 + 15 && bn > 32) continue;          // wider than the whole output
-            const int n_tiles = (N + wcols - 1) / wcols;
-            const int stage_bytes = nsub * A_TILE_BYTES + bn * GK * 2;
-            int stages = ring / stage_bytes;
-            if (stages > MAX_STAGES) stages = MAX_STAGES;
-            if (stages < 2) continue;
-            for (int splits = 1; splits <= MAX_SPLITS; ++splits) {
-                const long long tiles = static_cast<long long>(m_items) * n_tiles;
-                long long rounds;
-                if (splits > 1) {
-                    if (epi == GEMM_EPI_SWIGLU || nk < 8 * splits) break;
-                    const int per_owner = (wcols / 8 + splits - 1) / splits;
-                    if (static_cast<long long>(splits - 1) * per_owner * nsub * GM * 32 > static_cast<long long>(stages) * stage_bytes)
-                        continue;                                              // partials must fit the idle ring
-                    const int resident = max_active_clusters(splits);
-                    if (resident < 1) continue;
-                    rounds = (tiles + resident - 1) / resident;
-                } else {
-                    rounds = (tiles + sm_count - 1) / sm_count;
-                }
-                const double kb = static_cast<double>((nk + splits - 1) / splits);
-                const double mma = kb * nsub * 4 * (bn / 2.0);
-                const double ld = kb * stage_bytes / 55.0;
-                const double epilogue = wcols * 14.0 + (splits > 1 ? 9000.0 : 0.0);   // two cluster barriers and the exchange
-                const double cost = rounds * ((mma > ld ? mma : ld) + 2500.0 + epilogue);
-                if (cost < best_cost) {
-                    best_cost = cost;
-                    best.nsub = nsub; best.bn = bn; best.wcols = wcols; best.splits = splits; best.stages = stages;
-                    best.m_items = m_items; best.n_tiles = n_tiles;
-                    uint32_t cols = 32;
-                    while (cols < static_cast<uint32_t>(nsub == 2 ? 256 + bn : bn)) cols <<= 1;
-                    best.tmem_cols = cols;
-                }
-            }
-        }
-    }
     return best;
 }
 
 }  // namespace
-
-// The pair kernel serves every problem with more than one row tile.
-bool use_pair_kernel(int M, const PairPlan& pp) { return M > GM && pp.bn != 0; }
 
 // The pair kernel is persistent: with two or more tiles of 256 x 256 per CTA pair a tile's epilogue runs beside the next
 // tile's main loop, and the rotation is hidden there (as a kernel of its own it took 64 us at 8192 rows x 12288, reading
 // and writing q, k and v once more; the prefill of 16 x 512 rows is 2 % faster without it).  With fewer it is exposed:
 // at 512 rows x 12288 (one 384-column tile per pair) the projection took 45.6 us with it, against 37.0 us plain and
 // 7.4 us for the kernel that rotates.
-bool gemm_hides_epilogue(int M, int N) {
+bool gemm_takes_rope(int M, int N) {
+    if (M <= GM) return true;        // few rows: the epilogue works on whole heads anyway
     const long long tiles = static_cast<long long>((M + 2 * GM - 1) / (2 * GM)) * ((N + 255) / 256);
-    return M > GM && max_active_pairs() > 0 && tiles >= 2LL * max_active_pairs();
+    return max_active_pairs() > 0 && tiles >= 2LL * max_active_pairs();
 }
 
 int gemm_plan_describe(const dare_ctx* ctx, int epi, int M, int N, int K, int* out) {
-    const PairPlan pp = pair_plan(epi, M, N, K, 0, nullptr);
-    if (use_pair_kernel(M, pp)) {
-        out[0] = 2; out[1] = pp.bn; out[2] = pp.wcols; out[3] = pp.splits; out[4] = pp.stages;
-        out[5] = pp.m_pairs; out[6] = pp.n_tiles; out[7] = max_active_pairs(pp.splits);
-        return DARE_OK;
-    }
-    const GemmPlan p = gemm_plan(epi, M, N, K, ctx->sm_count);
-    out[0] = p.nsub; out[1] = p.bn; out[2] = p.wcols; out[3] = p.splits; out[4] = p.stages;
-    out[5] = p.m_items; out[6] = p.n_tiles; out[7] = p.splits > 1 ? max_active_clusters(p.splits) : 0;
-    return p.bn ? DARE_OK : DARE_ERR_SHAPE;
+    if (M <= GM) return gemm_few_describe(epi, M, N, K, ctx->sm_count, out);
+    const PairPlan pp = pair_plan(epi, M, N, K, 0);
+    if (pp.bn == 0) return DARE_ERR_SHAPE;
+    out[0] = 2; out[1] = pp.bn; out[2] = pp.wcols; out[3] = pp.splits; out[4] = pp.stages;
+    out[5] = pp.m_pairs; out[6] = pp.n_tiles; out[7] = max_active_pairs(pp.splits);
+    return DARE_OK;
 }
 
 int launch_gemm(const dare_ctx* ctx, int epi, const void* a, int M, int K, const void* w, const void* w2, int N,
-                void* out, const void* res, int ldo, cudaStream_t stream, const RopeArgs* rope) {
+                void* out, const void* res, int ldo, cudaStream_t stream, const RopeArgs* rope, bool w_static) {
     if (M < 1 || N < 8 || K < 8 || (N % 8) || (K % 8) || (ldo % 8)) return DARE_ERR_SHAPE;
     if (epi < GEMM_EPI_STORE || epi > GEMM_EPI_ROPE || (epi == GEMM_EPI_ROPE) != (rope != nullptr)) return DARE_ERR_RANGE;
-    const PairPlan pp = pair_plan(epi, M, N, K, rope ? rope->d : 0, nullptr);
-    if (use_pair_kernel(M, pp)) {
-        PairArgs pg;
-        pg.M = M; pg.N = N; pg.K = K; pg.ldo = ldo;
-        pg.p = pp;
-        pg.out = static_cast<__nv_bfloat16*>(out);
-        pg.res = static_cast<const __nv_bfloat16*>(res);
-        pg.dev_status = ctx->dev_status;
-        pg.rope = rope ? *rope : RopeArgs{};
-        CUtensorMap pa, pb, pb2;
-        int prc = make_tmap_bf16_2d(ctx, &pa, a, static_cast<uint64_t>(M), static_cast<uint64_t>(K), GM, GK);
-        if (prc != DARE_OK) return prc;
-        const uint32_t half_rows = static_cast<uint32_t>(pp.nchunk / 2);
-        prc = make_tmap_bf16_2d(ctx, &pb, w, static_cast<uint64_t>(N), static_cast<uint64_t>(K), half_rows, GK);
-        if (prc != DARE_OK) return prc;
-        if (epi == GEMM_EPI_SWIGLU) {
-            prc = make_tmap_bf16_2d(ctx, &pb2, w2, static_cast<uint64_t>(N), static_cast<uint64_t>(K), half_rows, GK);
-            if (prc != DARE_OK) return prc;
-            return launch_pair<GEMM_EPI_SWIGLU>(pa, pb, pb2, pg, stream, nullptr);
-        }
-        if (epi == GEMM_EPI_ROPE) return launch_pair<GEMM_EPI_ROPE>(pa, pb, pb, pg, stream, nullptr);
-        return epi == GEMM_EPI_STORE ? launch_pair<GEMM_EPI_STORE>(pa, pb, pb, pg, stream, nullptr)
-                                     : launch_pair<GEMM_EPI_RESIDUAL>(pa, pb, pb, pg, stream, nullptr);
-    }
-    if (epi == GEMM_EPI_ROPE) return DARE_ERR_SHAPE;      // (the pair kernel only: gemm_hides_epilogue)
-    GemmArgs g;
-    g.M = M; g.N = N; g.K = K; g.ldo = ldo;
-    g.p = gemm_plan(epi, M, N, K, ctx->sm_count);
-    if (g.p.bn == 0) return DARE_ERR_SHAPE;
-    g.out = static_cast<__nv_bfloat16*>(out);
-    g.res = static_cast<const __nv_bfloat16*>(res);
-    g.dev_status = ctx->dev_status;
-    CUtensorMap ta, tb, tb2;
-    int rc = make_tmap_bf16_2d(ctx, &ta, a, static_cast<uint64_t>(M), static_cast<uint64_t>(K), GM, GK);
+    if (M <= GM) return launch_gemm_few(ctx, epi, a, M, K, w, w2, N, out, res, ldo, stream, rope, w_static);
+    PairArgs pg;
+    pg.p = pair_plan(epi, M, N, K, rope ? rope->d : 0);
+    if (pg.p.bn == 0) return DARE_ERR_SHAPE;
+    pg.M = M; pg.N = N; pg.K = K; pg.ldo = ldo;
+    pg.out = static_cast<__nv_bfloat16*>(out);
+    pg.res = static_cast<const __nv_bfloat16*>(res);
+    pg.dev_status = ctx->dev_status;
+    pg.rope = rope ? *rope : RopeArgs{};
+    CUtensorMap pa, pb, pb2;
+    int rc = make_tmap_bf16_2d(ctx, &pa, a, static_cast<uint64_t>(M), static_cast<uint64_t>(K), GM, GK);
+    const uint32_t half_rows = static_cast<uint32_t>(pg.p.nchunk / 2);
+    if (rc == DARE_OK) rc = make_tmap_bf16_2d(ctx, &pb, w, static_cast<uint64_t>(N), static_cast<uint64_t>(K), half_rows, GK);
+    if (rc == DARE_OK && epi == GEMM_EPI_SWIGLU)
+        rc = make_tmap_bf16_2d(ctx, &pb2, w2, static_cast<uint64_t>(N), static_cast<uint64_t>(K), half_rows, GK);
     if (rc != DARE_OK) return rc;
-    const uint32_t box_rows = static_cast<uint32_t>(epi == GEMM_EPI_SWIGLU ? g.p.wcols : g.p.bn);
-    rc = make_tmap_bf16_2d(ctx, &tb, w, static_cast<uint64_t>(N), static_cast<uint64_t>(K), box_rows, GK);
-    if (rc != DARE_OK) return rc;
-    if (epi == GEMM_EPI_SWIGLU) {
-        rc = make_tmap_bf16_2d(ctx, &tb2, w2, static_cast<uint64_t>(N), static_cast<uint64_t>(K), box_rows, GK);
-        if (rc != DARE_OK) return rc;
-        return launch_one<GEMM_EPI_SWIGLU>(ta, tb, tb2, g, stream, nullptr);
+    switch (epi) {
+        case GEMM_EPI_STORE: return launch_pair<GEMM_EPI_STORE>(pa, pb, pb, pg, stream, nullptr);
+        case GEMM_EPI_RESIDUAL: return launch_pair<GEMM_EPI_RESIDUAL>(pa, pb, pb, pg, stream, nullptr);
+        case GEMM_EPI_SWIGLU: return launch_pair<GEMM_EPI_SWIGLU>(pa, pb, pb2, pg, stream, nullptr);
+        default: return launch_pair<GEMM_EPI_ROPE>(pa, pb, pb, pg, stream, nullptr);
     }
-    return epi == GEMM_EPI_STORE ? launch_one<GEMM_EPI_STORE>(ta, tb, tb, g, stream, nullptr)
-                                 : launch_one<GEMM_EPI_RESIDUAL>(ta, tb, tb, g, stream, nullptr);
 }
 
 }  // namespace dare

@@ -187,16 +187,21 @@ enum { GEMM_EPI_STORE = 0, GEMM_EPI_RESIDUAL = 1, GEMM_EPI_SWIGLU = 2, GEMM_EPI_
 //   STORE: out = acc.  RESIDUAL: out = res + acc (res may be out).  SWIGLU: out = silu(a w^T) * (a w2^T).
 //   ROPE: the QKV projection of the stack; its columns go through rotary embedding to q_out and the K/V caches, as
 //   launch_rope_kv_write would put them, bit for bit (out, res, ldo unused; N = (Hq + 2 Hkv) d).  Only where
-//   gemm_hides_epilogue says so.
+//   gemm_takes_rope says so.
+// w_static: no kernel that may still run when this one starts writes w or w2 (model weights).
 struct RopeArgs {
     int Hq, Hkv, d, start, length, cap;
-    const float* cs_t;                  // launch_rope_table's transposed table
+    const float *cs, *cs_t;             // launch_rope_table's two tables
     int n_pos;
     void *q_out, *k_cache, *v_cache;
 };
-bool gemm_hides_epilogue(int M, int N);
+bool gemm_takes_rope(int M, int N);
 int launch_gemm(const dare_ctx* ctx, int epi, const void* a, int M, int K, const void* w, const void* w2, int N,
-                void* out, const void* res, int ldo, cudaStream_t stream, const RopeArgs* rope = nullptr);
+                void* out, const void* res, int ldo, cudaStream_t stream, const RopeArgs* rope = nullptr,
+                bool w_static = false);
+int launch_gemm_few(const dare_ctx* ctx, int epi, const void* a, int M, int K, const void* w, const void* w2, int N, void* out,
+                    const void* res, int ldo, cudaStream_t stream, const RopeArgs* rope, bool w_static);
+int gemm_few_describe(int epi, int M, int N, int K, int sm_count, int* out);
 // out[8] = {row tiles per CTA, bn, output columns per tile, K splits, stages, row items, column tiles, resident clusters}
 int gemm_plan_describe(const dare_ctx* ctx, int epi, int M, int N, int K, int* out);
 int launch_embed(const void* emb, int D, int V, const int32_t* tokens, int64_t row_stride, int start, int length,

@@ -61,14 +61,14 @@ int forward_rows(dare_model* m, const int32_t* tokens, int B, int64_t row_stride
         __nv_bfloat16* vc = static_cast<__nv_bfloat16*>(v_cache) + layer_kv * l;
         rc = launch_rmsnorm(m->x, c.hidden, rows, c.rms_eps, m->h, s);
         if (rc != DARE_OK) return rc;
-        if (gemm_hides_epilogue(rows, nq + 2 * nkv)) {
-            const RopeArgs rope = {c.n_q_heads, c.n_kv_heads, c.head_dim, start, length, cap, m->rope_cs_t, c.max_positions,
-                                   m->q, kc, vc};
+        if (gemm_takes_rope(rows, nq + 2 * nkv)) {
+            const RopeArgs rope = {c.n_q_heads, c.n_kv_heads, c.head_dim, start, length, cap, m->rope_cs, m->rope_cs_t,
+                                   c.max_positions, m->q, kc, vc};
             rc = launch_gemm(m->ctx, GEMM_EPI_ROPE, m->h, rows, c.hidden, w.wqkv, nullptr, nq + 2 * nkv, nullptr, nullptr,
-                             nq + 2 * nkv, s, &rope);
+                             nq + 2 * nkv, s, &rope, true);
         } else {
             rc = launch_gemm(m->ctx, GEMM_EPI_STORE, m->h, rows, c.hidden, w.wqkv, nullptr, nq + 2 * nkv, m->qkv, nullptr,
-                             nq + 2 * nkv, s);
+                             nq + 2 * nkv, s, nullptr, true);
             if (rc == DARE_OK)
                 rc = launch_rope_kv_write(m->qkv, rows, c.n_q_heads, c.n_kv_heads, c.head_dim, start, length, m->rope_cs,
                                           m->q, kc, vc, cap, s);
@@ -84,13 +84,13 @@ int forward_rows(dare_model* m, const int32_t* tokens, int B, int64_t row_stride
         if (attn_workspace_bytes(a, attn_plan_splits(m->ctx, a)) > m->ctx->workspace_bytes) return DARE_ERR_WORKSPACE;
         rc = launch_attn(m->ctx, a, s);
         if (rc != DARE_OK) return rc;
-        rc = launch_gemm(m->ctx, GEMM_EPI_RESIDUAL, m->attn, rows, nq, w.wo, nullptr, c.hidden, m->x, m->x, c.hidden, s);
+        rc = launch_gemm(m->ctx, GEMM_EPI_RESIDUAL, m->attn, rows, nq, w.wo, nullptr, c.hidden, m->x, m->x, c.hidden, s, nullptr, true);
         if (rc != DARE_OK) return rc;
         rc = launch_rmsnorm(m->x, c.hidden, rows, c.rms_eps, m->h, s);
         if (rc != DARE_OK) return rc;
-        rc = launch_gemm(m->ctx, GEMM_EPI_SWIGLU, m->h, rows, c.hidden, w.wg, w.wu, c.ffn, m->act, nullptr, c.ffn, s);
+        rc = launch_gemm(m->ctx, GEMM_EPI_SWIGLU, m->h, rows, c.hidden, w.wg, w.wu, c.ffn, m->act, nullptr, c.ffn, s, nullptr, true);
         if (rc != DARE_OK) return rc;
-        rc = launch_gemm(m->ctx, GEMM_EPI_RESIDUAL, m->act, rows, c.ffn, w.wd, nullptr, c.hidden, m->x, m->x, c.hidden, s);
+        rc = launch_gemm(m->ctx, GEMM_EPI_RESIDUAL, m->act, rows, c.ffn, w.wd, nullptr, c.hidden, m->x, m->x, c.hidden, s, nullptr, true);
         if (rc != DARE_OK) return rc;
     }
     return launch_rmsnorm(m->x, c.hidden, rows, c.rms_eps, hidden_out ? hidden_out : m->h, s);

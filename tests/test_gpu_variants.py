@@ -160,3 +160,48 @@ def test_steps_back_to_back_equal_their_parts(ctx, B, L, Hq, Hkv, P, workspace):
     assert c.device_status() == 0
     if workspace:
         c.close()
+
+
+# Projections of up to 128 rows: one to eight K slices (a cluster), ragged last K block, last W tile part full, every row
+# padding; all epilogues.
+@pytest.mark.parametrize("M", [1, 15, 16, 17, 47, 96, 127, 128])
+@pytest.mark.parametrize("K,N", [(8, 8), (72, 264), (520, 1000), (4096, 136), (1280, 512), (256, 40000)])
+def test_linear_of_few_rows(ctx, M, K, N):
+    a, w = I.normal_bf16(M, I.TID_X, (M, K)).cuda(), I.normal_bf16(5, I.TID_W, (N, K), 0.05).cuda()
+    w2, r = I.normal_bf16(6, I.TID_Q, (N, K), 0.05).cuda(), I.normal_bf16(7, I.TID_Q, (M, N)).cuda()
+    store = dare.dare_linear(ctx, dare.LINEAR_STORE, a, w).double()
+    resid = dare.dare_linear(ctx, dare.LINEAR_RESIDUAL, a, w, residual=r).double()
+    swiglu = dare.dare_linear(ctx, dare.LINEAR_SWIGLU, a, w, w2=w2).double()
+    ref, up = a.double() @ w.double().T, a.double() @ w2.double().T
+    torch.cuda.synchronize()
+    assert ctx.device_status() == 0
+    # one rounding to bf16 (2^-8) and fp32 sums of K products: K * 2^-24 of the sum of their magnitudes at most
+    acc = K * 2.0 ** -24 * (a.double().abs() @ w.double().abs().T)
+    acc2 = K * 2.0 ** -24 * (a.double().abs() @ w2.double().abs().T)
+    assert ((store - ref).abs() <= 2.0 ** -8 * ref.abs() + acc).all()
+    want = ref + r.double()
+    assert ((resid - want).abs() <= 2.0 ** -8 * want.abs() + acc).all()
+    want = ref * torch.sigmoid(ref) * up                 # |silu'| < 1.1; exp and division to a few ulp
+    assert ((swiglu - want).abs() <= 2.0 ** -7.9 * want.abs() + 1.1 * acc * (up.abs() + acc2) + acc2 * ref.abs() + 1e-6).all()
+
+
+@pytest.mark.parametrize("Hq,Hkv,d,B,length", [(4, 2, 64, 3, 16), (3, 1, 128, 1, 127), (5, 1, 64, 16, 8), (4, 4, 128, 2, 1)])
+def test_rope_in_a_projection_of_few_rows(ctx, Hq, Hkv, d, B, length):
+    start, cap = 3, length + 5
+    model = _small_model(ctx, Hq, Hkv, d, B * length, B, cap)
+    tok = I.uniform_int(7, 9, (B, cap), 0, 510).cuda()
+    caches = model.new_cache(B, cap)
+    dare.dare_model_forward(model, tok, start, length, *caches)
+    # the same projection and the rotation as separate calls
+    emb, layers, _ = model._keep
+    x = emb[tok[:, start:start + length].reshape(-1).long()].contiguous()
+    qkv = dare.dare_linear(ctx, dare.LINEAR_STORE, dare.dare_rmsnorm(ctx, x, 1e-5), layers[0]["wqkv"])
+    kc, vc = torch.zeros_like(caches[0]), torch.zeros_like(caches[1])
+    q = torch.empty(B * length, Hq, d, dtype=torch.bfloat16, device="cuda")
+    dare.dare_rope_kv_write(model, qkv, B, length, start, q, kc[0], vc[0])
+    torch.cuda.synchronize()
+    assert ctx.device_status() == 0
+    # the same sums, the same rounding before the rotation; a multiply-add may be contracted differently behind it
+    assert torch.equal(caches[1], vc)
+    assert ((caches[0].float() - kc.float()).abs() <= 2.0 ** -7 * kc.float().abs() + 1e-6).all()
+    model.close()
