@@ -245,10 +245,9 @@ int dare_unmask_select(dare_ctx* ctx,
  * Ordering: everything the step reads is taken as `stream` has it when the call is made, and everything it
  * writes (attn_out, lse, pred, conf, tokens, the counts) is complete for whatever is enqueued on `stream`
  * afterwards.  Inside the step the attention and the head, neither of which reads what the other writes, are
- * not kept in sequence: the head runs on a stream of the context, forked from and joined back to `stream` by
- * events, and the attention's CTAs fill the SMs that the head's GEMM leaves early.  `hidden` and attn_out must
- * therefore not overlap (nor any other input of one half with an output of the other).  The fork and the join are
- * capturable in a CUDA graph like any event fork / join.
+ * not kept in sequence: the head goes first and the attention's CTAs fill the SMs that its GEMM leaves early.
+ * `hidden` and attn_out must therefore not overlap (nor any other input of one half with an output of the other).
+ * The step is capturable in a CUDA graph.
  */
 int dare_denoise_block(dare_ctx* ctx,
                        int B, int L, int Hq, int Hkv, int d, int prefix_cap, int suffix_cap, float scale,
@@ -268,7 +267,7 @@ int dare_denoise_block(dare_ctx* ctx,
  * The same step with the sampled head (Section 4.2: several different rollouts per prompt): dare_attn_block,
  * dare_lmhead_sample on the block's rows (temperature, seed and step counter as there), then dare_unmask_select on
  * the sampled tokens and their temperature-1 probabilities.  Same buffers, rules and ordering as dare_denoise_block
- * (the head on the context's stream, the attention beside it); temperature must be finite and > 0 (DARE_ERR_RANGE
+ * (the attention beside the head); temperature must be finite and > 0 (DARE_ERR_RANGE
  * otherwise).
  */
 int dare_denoise_block_sampled(dare_ctx* ctx, int B, int L, int Hq, int Hkv, int d, int prefix_cap, int suffix_cap,

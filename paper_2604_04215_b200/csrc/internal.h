@@ -137,7 +137,8 @@ int make_tmap_bf16_2d(const dare_ctx* ctx, CUtensorMap* out, const void* base, u
 
 int launch_unmask_select(int32_t* tokens, int B, int64_t row_stride, int block_start, int L, const int32_t* pred,
                          const float* conf, int32_t mask_id, int mode, float threshold, int k, int32_t* n_committed,
-                         int32_t* n_remaining, cudaStream_t stream);
+                         int32_t* n_remaining, cudaStream_t stream,
+                         int32_t* host_remaining = nullptr);
 
 // log p(target) per row = z_target - logsumexp z (and optionally logsumexp z); logits never stored.
 int launch_lmhead_logprob(const dare_ctx* ctx, void* scratch, const void* hidden, int M, int D, const void* w, int V,
@@ -154,7 +155,15 @@ size_t lmhead_max_scratch_bytes(int M, int D, int V, int sm_count, bool sampling
 // positions whose tokens are given by row_tokens = tokens + block_start, tok_L = L): the caller then skips
 // launch_unmask_select.  tokens_block is the same address as row_tokens, writable.
 constexpr int LMHEAD_SELECT_MAX_L = 32;
-struct LmSelectArgs { int32_t* tokens_block; int B; int mode; float threshold; int k; int32_t* n_committed; int32_t* n_remaining; };
+// host_remaining (optional): page-locked host memory that also gets the remaining counts, as soon as they are known.
+struct LmSelectArgs {
+    int32_t* tokens_block;
+    int B, mode;
+    float threshold;
+    int k;
+    int32_t *n_committed, *n_remaining;
+    int32_t* host_remaining = nullptr;
+};
 int launch_lmhead(const dare_ctx* ctx, void* scratch, const void* hidden, int M, int D, const void* w, int V,
                   const int32_t* row_tokens, int tok_L, int64_t tok_row_stride, int32_t mask_id, int exclude_mask_column, int32_t* pred, float* conf,
                   cudaStream_t stream, const LmSampleArgs* sample, const LmSelectArgs* select = nullptr);

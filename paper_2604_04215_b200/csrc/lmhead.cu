@@ -1150,6 +1150,7 @@ struct LmSelect {
     int k;
     int32_t* n_committed;
     int32_t* n_remaining;
+    int32_t* host_remaining;
 };
 template <bool SAMPLE>
 __global__ void __launch_bounds__(1024)
@@ -1222,6 +1223,7 @@ lmhead_merge_select_kernel(const LmParts parts, int grid_gemm, int n_tiles, int 
     if (lane == 0) {
         if (sel.n_committed) sel.n_committed[b] = __popc(commit_set);
         if (sel.n_remaining) sel.n_remaining[b] = __popc(masked_set) - __popc(commit_set);
+        if (sel.host_remaining) st_host(sel.host_remaining + b, __popc(masked_set) - __popc(commit_set));
     }
 }
 
@@ -1389,6 +1391,7 @@ static int launch_head(const dare_ctx* ctx, int grid, bool pairs, const void* x_
         sel.tokens_block = select->tokens_block; sel.row_stride = tok_row_stride; sel.mode = select->mode;
         sel.threshold = select->threshold; sel.k = select->k;
         sel.n_committed = select->n_committed; sel.n_remaining = select->n_remaining;
+        sel.host_remaining = select->host_remaining;
         return launch_kernel(lmhead_merge_select_kernel<SAMPLE>, dim3(select->B), 32 * tok_L, 0, stream, 1, lp, grid_gemm, n_tiles,
                              tok_L, live_rows, idx, mask_id, pred, conf, layout, parts_stride, sel, step_dev);
     }

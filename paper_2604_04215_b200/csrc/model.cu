@@ -27,11 +27,8 @@ struct dare_model {
     dare_layer_weights* layers;    // host copy of the caller's array (device pointers inside)
     float *rope_cs, *rope_cs_t;    // [max_positions, d/2] (cos, sin) and its transpose
     void *x, *h, *qkv, *q, *attn, *act;   // activations, max_rows each
-    int32_t* host_counts;          // pinned: n_remaining of two steps in flight, [2][max_batch]
+    int32_t* host_counts;          // page-locked: remaining masks of the loop's last steps, [COUNT_SLOTS][max_batch]
     int max_batch;
-    cudaEvent_t ev[2];
-    cudaStream_t work;             // the loop runs here: a block's step is captured once into a CUDA graph
-    cudaEvent_t ev_in, ev_out;     // order the work stream after / before the caller's stream
     // sampled head (dare_model_set_sampling): temperature 0 = greedy; the device word counts the steps
     float sample_temperature;
     uint64_t sample_seed;
@@ -39,6 +36,8 @@ struct dare_model {
 };
 
 namespace {
+
+constexpr int COUNT_SLOTS = 4;
 
 __global__ void set_word_kernel(uint32_t* p, uint32_t v) {
     dare::pdl_wait();
@@ -112,7 +111,7 @@ int check_rows(const dare_model* m, const void* tokens, int B, int64_t row_strid
 
 int step_rows(dare_model* m, int32_t* tokens, int B, int64_t row_stride, int start, int L, int kv_len, void* k_cache,
               void* v_cache, int cap, int mode, float threshold, int k, int32_t* pred, float* conf, int32_t* n_committed,
-              int32_t* n_remaining, cudaStream_t s) {
+              int32_t* n_remaining, cudaStream_t s, int32_t* host_remaining = nullptr) {
     int rc = forward_rows(m, tokens, B, row_stride, start, L, kv_len, k_cache, v_cache, cap, nullptr, s);
     if (rc != DARE_OK) return rc;
     const int M = B * L;
@@ -120,7 +119,8 @@ int step_rows(dare_model* m, int32_t* tokens, int B, int64_t row_stride, int sta
     const bool sampled = m->sample_temperature > 0.f;
     smp.temperature = m->sample_temperature; smp.seed = m->sample_seed; smp.step = 0; smp.step_dev = m->step_counter;
     if (L <= dare::LMHEAD_SELECT_MAX_L) {      // short blocks: the selection rides on the head's merge kernel
-        const dare::LmSelectArgs sel = {tokens + start, B, mode, threshold, k, n_committed, n_remaining};
+        const dare::LmSelectArgs sel = {tokens + start, B, mode, threshold, k, n_committed, n_remaining,
+                                        host_remaining};
         return dare::launch_lmhead(m->ctx, m->ctx->workspace, m->h, M, m->desc.hidden, m->lm_head, m->desc.vocab,
                                    tokens + start, L, row_stride, m->desc.mask_id, 1, pred, conf, s, sampled ? &smp : nullptr,
                                    &sel);
@@ -129,7 +129,7 @@ int step_rows(dare_model* m, int32_t* tokens, int B, int64_t row_stride, int sta
                              tokens + start, L, row_stride, m->desc.mask_id, 1, pred, conf, s, sampled ? &smp : nullptr);
     if (rc != DARE_OK) return rc;
     return dare::launch_unmask_select(tokens, B, row_stride, start, L, pred, conf, m->desc.mask_id, mode, threshold, k,
-                                      n_committed, n_remaining, s);
+                                      n_committed, n_remaining, s, host_remaining);
 }
 
 int check_step(const dare_model* m, int B, int L, int mode, float threshold, int k, const void* pred, const void* conf) {
@@ -167,8 +167,6 @@ int dare_model_create(dare_ctx* ctx, const dare_model_desc* desc, const void* em
     m->ctx = ctx; m->desc = c; m->embedding = embedding; m->lm_head = lm_head; m->max_batch = c.max_batch;
     m->layers = new (std::nothrow) dare_layer_weights[c.n_layers];
     m->rope_cs = m->rope_cs_t = nullptr; m->x = m->h = m->qkv = m->q = m->attn = m->act = nullptr; m->host_counts = nullptr;
-    m->ev[0] = m->ev[1] = nullptr;
-    m->work = nullptr; m->ev_in = m->ev_out = nullptr;
     m->sample_temperature = 0.f; m->sample_seed = 0; m->step_counter = nullptr;
     bool ok = m->layers != nullptr;
     if (ok) for (int l = 0; l < c.n_layers; ++l) m->layers[l] = layers[l];
@@ -185,12 +183,7 @@ int dare_model_create(dare_ctx* ctx, const dare_model_desc* desc, const void* em
     ok = ok && cudaMalloc(&m->act, rows * c.ffn * 2) == cudaSuccess;
     ok = ok && cudaMalloc(reinterpret_cast<void**>(&m->step_counter), sizeof(uint32_t)) == cudaSuccess;
     ok = ok && cudaMemset(m->step_counter, 0, sizeof(uint32_t)) == cudaSuccess;
-    ok = ok && cudaMallocHost(reinterpret_cast<void**>(&m->host_counts), sizeof(int32_t) * 2 * c.max_batch) == cudaSuccess;
-    ok = ok && cudaEventCreateWithFlags(&m->ev[0], cudaEventDisableTiming) == cudaSuccess;
-    ok = ok && cudaEventCreateWithFlags(&m->ev[1], cudaEventDisableTiming) == cudaSuccess;
-    ok = ok && cudaEventCreateWithFlags(&m->ev_in, cudaEventDisableTiming) == cudaSuccess;
-    ok = ok && cudaEventCreateWithFlags(&m->ev_out, cudaEventDisableTiming) == cudaSuccess;
-    ok = ok && cudaStreamCreateWithFlags(&m->work, cudaStreamNonBlocking) == cudaSuccess;
+    ok = ok && cudaMallocHost(reinterpret_cast<void**>(&m->host_counts), sizeof(int32_t) * COUNT_SLOTS * c.max_batch) == cudaSuccess;
     ok = ok && dare::launch_rope_table(m->rope_cs, m->rope_cs_t, c.max_positions, c.head_dim / 2, static_cast<double>(c.rope_base),
                                        nullptr) == DARE_OK;
     ok = ok && cudaDeviceSynchronize() == cudaSuccess;
@@ -209,11 +202,6 @@ int dare_model_destroy(dare_model* m) {
     cudaFree(m->act);
     cudaFree(m->step_counter);
     if (m->host_counts) cudaFreeHost(m->host_counts);
-    if (m->ev[0]) cudaEventDestroy(m->ev[0]);
-    if (m->ev[1]) cudaEventDestroy(m->ev[1]);
-    if (m->ev_in) cudaEventDestroy(m->ev_in);
-    if (m->ev_out) cudaEventDestroy(m->ev_out);
-    if (m->work) cudaStreamDestroy(m->work);
     delete[] m->layers;
     delete m;
     return DARE_OK;
@@ -307,19 +295,28 @@ int dare_model_step(dare_model* m, int32_t* tokens, int B, int64_t row_stride, i
 
 namespace {
 
-// The previous block's graph: destroyed once its launches are known to have finished.
-struct BlockGraph {
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t exec = nullptr;
-    void destroy() {
-        if (exec) cudaGraphExecDestroy(exec);
-        if (graph) cudaGraphDestroy(graph);
-        exec = nullptr; graph = nullptr;
+// Waits until step `slot` has left its counts; *done: no rollout has a mask left.  The kernel that takes the decisions
+// writes them straight into page-locked memory (an event behind the step, let alone a copy, would stand between the step
+// and the next one, which is already enqueued).
+int read_counts(const dare_model* m, int slot, int B, cudaStream_t s, bool* done) {
+    const volatile int32_t* c = m->host_counts + slot * m->max_batch;
+    *done = true;
+    uint32_t spins = 0;
+    for (int r = 0; r < B; ++r) {
+        while (c[r] < 0) {
+            if ((++spins & 0xffff) == 0) {      // now and then: has the stream failed, or ended without writing them?
+                const cudaError_t q = cudaStreamQuery(s);
+                if (q != cudaErrorNotReady && (q != cudaSuccess || c[r] < 0)) return DARE_ERR_CUDA;
+            }
+        }
+        *done = *done && c[r] == 0;
     }
-};
+    return DARE_OK;
+}
 
-// All denoising steps of one block on the model's work stream.  The step (about forty launches with fixed
-// arguments) is captured once into a CUDA graph and replayed.
+// All denoising steps of one block.  The host enqueues a step (about thirty launches, 2 us each) while the one before it
+// runs; as a CUDA graph per block it cost the GPU 17 us between replays and, on a small model, the capture and the
+// instantiation besides (44 us per step of 110 us).
 //
 // A step whose block holds no mask any more does exactly what the refresh forward of the prefix-cache loop
 // must do (the LM head finds no live row, the selection changes nothing, the stack rewrites the block's K/V
@@ -329,71 +326,31 @@ struct BlockGraph {
 // same K/V.)
 int run_block(dare_model* m, int32_t* tokens, int B, int64_t row_stride, int start, int L, int kv_len, void* k_cache,
               void* v_cache, int cap, int mode, float threshold, int k, int32_t* pred, float* conf, int32_t* n_remaining,
-              BlockGraph* old, int* steps_taken) {
-    cudaStream_t s = m->work;
-    BlockGraph cur;
-    if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return DARE_ERR_CUDA;
-    const uint64_t launches_before = dare::g_kernel_launches.load();      // the capture itself launches nothing:
-    int rc = step_rows(m, tokens, B, row_stride, start, L, kv_len, k_cache, v_cache, cap, mode, threshold, k, pred, conf,
-                       nullptr, n_remaining, s);
-    const uint64_t per_replay = dare::g_kernel_launches.load() - launches_before;
-    dare::g_kernel_launches.fetch_sub(per_replay);                        // ... its kernels are counted per replay
-    const cudaError_t end = cudaStreamEndCapture(s, &cur.graph);      // always ends the capture, also after an error
-    if (rc == DARE_OK && (end != cudaSuccess || cur.graph == nullptr)) rc = DARE_ERR_CUDA;
-    if (rc == DARE_OK && cudaGraphInstantiate(&cur.exec, cur.graph, 0) != cudaSuccess) rc = DARE_ERR_CUDA;
-    int issued = 0, taken = -1;
-    while (rc == DARE_OK && taken < 0) {
-        if (issued > L + 1) { rc = DARE_ERR_CUDA; break; }   // cannot happen: every step commits a token per row
-        const int slot = issued & 1;
-        if (cudaGraphLaunch(cur.exec, s) != cudaSuccess ||
-            cudaMemcpyAsync(m->host_counts + slot * m->max_batch, n_remaining, sizeof(int32_t) * B,
-                            cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-            cudaEventRecord(m->ev[slot], s) != cudaSuccess) {
-            rc = DARE_ERR_CUDA;
-            break;
-        }
-        ++issued;
-        dare::note_launch(per_replay);
-        if (issued >= 2) {
-            const int prev = (issued - 2) & 1;
-            if (cudaEventSynchronize(m->ev[prev]) != cudaSuccess) { rc = DARE_ERR_CUDA; break; }
-            old->destroy();      // a step of this block has finished, so every launch of the previous block has
-            bool done = true;
-            for (int r = 0; r < B; ++r) done = done && m->host_counts[prev * m->max_batch + r] == 0;
-            if (done) taken = issued - 1;   // steps 0 .. issued-2 denoised; the last one issued found no mask
+              cudaStream_t s, uint32_t* step_no, int* steps_taken) {
+    for (int issued = 0;; ++issued) {
+        if (issued > L + 1) return DARE_ERR_CUDA;            // cannot happen: every step commits a token per row
+        // The slots go round over the whole loop, not per block: when a slot comes round again, a later step than the one
+        // that used it has been read, so nothing writes to it any more.
+        const uint32_t n = (*step_no)++;
+        int32_t* slot = m->host_counts + (n % COUNT_SLOTS) * m->max_batch;
+        for (int r = 0; r < B; ++r) slot[r] = -1;
+        int rc = step_rows(m, tokens, B, row_stride, start, L, kv_len, k_cache, v_cache, cap, mode, threshold, k, pred, conf,
+                           nullptr, n_remaining, s, slot);
+        if (rc != DARE_OK) return rc;
+        if (issued == 0) continue;
+        bool done = false;
+        rc = read_counts(m, (n - 1) % COUNT_SLOTS, B, s, &done);
+        if (rc != DARE_OK) return rc;
+        if (done) {      // steps 0 .. issued - 1 denoised; the last one issued finds no mask
+            *steps_taken = issued;
+            return DARE_OK;
         }
     }
-    if (old->exec) {      // (only if this block issued fewer than two steps or failed)
-        cudaStreamSynchronize(s);
-        old->destroy();
-    }
-    *old = cur;
-    *steps_taken = taken;
-    return rc;
-}
-
-// Order the model's work stream after the caller's stream (entry) / the caller's stream after it (exit).
-int enter_work_stream(dare_model* m, cudaStream_t user) {
-    if (cudaEventRecord(m->ev_in, user) != cudaSuccess || cudaStreamWaitEvent(m->work, m->ev_in, 0) != cudaSuccess)
-        return DARE_ERR_CUDA;
-    return DARE_OK;
-}
-int leave_work_stream(dare_model* m, cudaStream_t user, BlockGraph* old, int rc) {
-    const bool synced = cudaStreamSynchronize(m->work) == cudaSuccess;
-    old->destroy();
-    if (rc != DARE_OK) return rc;
-    if (!synced || cudaEventRecord(m->ev_out, m->work) != cudaSuccess ||
-        cudaStreamWaitEvent(user, m->ev_out, 0) != cudaSuccess)
-        return DARE_ERR_CUDA;
-    return DARE_OK;
 }
 
 }  // namespace
 
 extern "C" {
-
-// The loops run on the model's own stream, ordered after the caller's stream at entry and before it at exit:
-// the caller's stream (possibly the legacy default stream) may not allow a capture.
 
 int dare_generate(dare_model* m, int32_t* tokens, int B, int64_t row_stride, int prompt_len, int gen_len, int L,
                   void* k_cache, void* v_cache, int cache_cap, int mode, float threshold, int k, int32_t* pred,
@@ -407,22 +364,21 @@ int dare_generate(dare_model* m, int32_t* tokens, int B, int64_t row_stride, int
     if (rc == DARE_OK) rc = check_step(m, B, L, mode, threshold, k, pred, conf);
     if (rc != DARE_OK) return rc;
     cudaStream_t user = static_cast<cudaStream_t>(stream);
-    rc = enter_work_stream(m, user);
-    if (rc != DARE_OK) return rc;
-    rc = forward_rows(m, tokens, B, row_stride, 0, prompt_len, prompt_len, k_cache, v_cache, cache_cap, nullptr, m->work);
-    BlockGraph old;
+    rc = forward_rows(m, tokens, B, row_stride, 0, prompt_len, prompt_len, k_cache, v_cache, cache_cap, nullptr, user);
+    uint32_t step_no = 0;
     for (int b = 0; b < gen_len / L && rc == DARE_OK; ++b) {
         const int start = prompt_len + b * L;
         int taken = -1;
         if (m->sample_temperature > 0.f) {     // step n of block b draws with the counter (b << 16) + n
-            rc = dare::launch_kernel(set_word_kernel, dim3(1), 1, 0, m->work, 1, m->step_counter, static_cast<uint32_t>(b) << 16);
+            rc = dare::launch_kernel(set_word_kernel, dim3(1), 1, 0, user, 1, m->step_counter, static_cast<uint32_t>(b) << 16);
             if (rc != DARE_OK) break;
         }
         rc = run_block(m, tokens, B, row_stride, start, L, start + L, k_cache, v_cache, cache_cap, mode, threshold, k,
-                       pred, conf, n_remaining, &old, &taken);
+                       pred, conf, n_remaining, user, &step_no, &taken);
         if (rc == DARE_OK && steps_per_block) steps_per_block[b] = taken;
     }
-    return leave_work_stream(m, user, &old, rc);
+    const bool synced = cudaStreamSynchronize(user) == cudaSuccess;      // (also after an error: the counts' slots are still in use)
+    return rc != DARE_OK ? rc : synced ? DARE_OK : DARE_ERR_CUDA;
 }
 
 int dare_generate_dual(dare_model* m, int32_t* tokens, int B, int64_t row_stride, int prompt_len, int gen_len, int L,
@@ -435,23 +391,22 @@ int dare_generate_dual(dare_model* m, int32_t* tokens, int B, int64_t row_stride
     if (rc == DARE_OK) rc = check_step(m, B, L, mode, threshold, k, pred, conf);
     if (rc != DARE_OK) return rc;
     cudaStream_t user = static_cast<cudaStream_t>(stream);
-    rc = enter_work_stream(m, user);
-    if (rc != DARE_OK) return rc;
-    BlockGraph old;
+    uint32_t step_no = 0;
     for (int b = 0; b < gen_len / L && rc == DARE_OK; ++b) {
         const int start = prompt_len + b * L;
-        rc = forward_rows(m, tokens, B, row_stride, 0, T, T, k_cache, v_cache, cache_cap, nullptr, m->work);
+        rc = forward_rows(m, tokens, B, row_stride, 0, T, T, k_cache, v_cache, cache_cap, nullptr, user);
         if (rc != DARE_OK) break;
         int taken = -1;
         if (m->sample_temperature > 0.f) {
-            rc = dare::launch_kernel(set_word_kernel, dim3(1), 1, 0, m->work, 1, m->step_counter, static_cast<uint32_t>(b) << 16);
+            rc = dare::launch_kernel(set_word_kernel, dim3(1), 1, 0, user, 1, m->step_counter, static_cast<uint32_t>(b) << 16);
             if (rc != DARE_OK) break;
         }
         rc = run_block(m, tokens, B, row_stride, start, L, T, k_cache, v_cache, cache_cap, mode, threshold, k, pred, conf,
-                       n_remaining, &old, &taken);
+                       n_remaining, user, &step_no, &taken);
         if (rc == DARE_OK && steps_per_block) steps_per_block[b] = taken;
     }
-    return leave_work_stream(m, user, &old, rc);
+    const bool synced = cudaStreamSynchronize(user) == cudaSuccess;      // (also after an error: the counts' slots are still in use)
+    return rc != DARE_OK ? rc : synced ? DARE_OK : DARE_ERR_CUDA;
 }
 
 }  // extern "C"

@@ -81,6 +81,11 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 // only wait for a CTA that has its share and will give it back.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Store to memory that the host polls while the kernel runs.
+__device__ __forceinline__ void st_host(int32_t* p, int32_t v) {
+    asm volatile("st.relaxed.sys.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
 // ---------------------------------------------------------------- thread-block cluster
 __device__ __forceinline__ uint32_t cluster_cta_rank() {
     uint32_t r;

@@ -16,7 +16,8 @@ constexpr int SEL_MAX_L = 4096;
 __global__ void __launch_bounds__(SEL_THREADS)
 unmask_select_kernel(int32_t* __restrict__ tokens, int64_t row_stride, int block_start, int L,
                      const int32_t* __restrict__ pred, const float* __restrict__ conf, int32_t mask_id, int mode,
-                     float threshold, int k, int32_t* __restrict__ n_committed, int32_t* __restrict__ n_remaining) {
+                     float threshold, int k, int32_t* __restrict__ n_committed, int32_t* __restrict__ n_remaining,
+                     int32_t* host_remaining) {
     extern __shared__ float s_conf[];   // [L]; -inf for NaN; positions that are not masked hold NaN as "absent"
     __shared__ int s_masked, s_above, s_commit;
     const int r = blockIdx.x;
@@ -67,6 +68,7 @@ unmask_select_kernel(int32_t* __restrict__ tokens, int64_t row_stride, int block
     if (threadIdx.x == 0) {
         if (n_committed) n_committed[r] = s_commit;
         if (n_remaining) n_remaining[r] = n_masked - s_commit;
+        if (host_remaining) st_host(host_remaining + r, n_masked - s_commit);
     }
 }
 
@@ -74,10 +76,11 @@ unmask_select_kernel(int32_t* __restrict__ tokens, int64_t row_stride, int block
 
 int launch_unmask_select(int32_t* tokens, int B, int64_t row_stride, int block_start, int L, const int32_t* pred,
                          const float* conf, int32_t mask_id, int mode, float threshold, int k, int32_t* n_committed,
-                         int32_t* n_remaining, cudaStream_t stream) {
+                         int32_t* n_remaining, cudaStream_t stream, int32_t* host_remaining) {
     if (L > SEL_MAX_L) return DARE_ERR_SHAPE;
     return launch_kernel(unmask_select_kernel, dim3(B), SEL_THREADS, L * sizeof(float), stream, 1, tokens, row_stride,
-                         block_start, L, pred, conf, mask_id, mode, threshold, k, n_committed, n_remaining);
+                         block_start, L, pred, conf, mask_id, mode, threshold, k, n_committed, n_remaining,
+                         host_remaining);
 }
 
 }  // namespace dare
