@@ -572,7 +572,13 @@ PairPlan pair_plan(int epi, int M, int N, int K, int head_dim) {
                 double per_kb = mma > smem ? mma : smem;
                 if (ld > per_kb) per_kb = ld;
                 const double epilogue = wcols * 14.0 / splits + (splits > 1 ? 6000.0 : 0.0);   // two cluster barriers, exchange
-                const double cost = rounds * (kb * per_kb + 2500.0 + epilogue);
+                // SwiGLU's epilogue is the long one (two columns and an exponential per output): there it counts that with
+                // two accumulator buffers it runs beside the next main loop.  512 instead of 256 columns for gate and up of
+                // 8192 rows: prefill 11.73 against 11.55 ms.  For the others wider tiles' lower operand traffic weighs more
+                // (weight gradient of 126464 x 4096 x 2048 in 256 instead of 512 columns: +1.5 %; QKV of 512 rows in two
+                // rounds of 176 instead of one of 352: a generation +1.3 %).
+                const double cost = epi == GEMM_EPI_SWIGLU && bn <= 256 ? rounds * kb * per_kb + 2500.0 + epilogue
+                                                                        : rounds * (kb * per_kb + 2500.0 + epilogue);
                 if (cost < best_cost) {
                     best_cost = cost;
                     best.bn = bn; best.wcols = wcols; best.nmma = nmma; best.nchunk = nchunk; best.stages = stages;
