@@ -464,6 +464,18 @@ struct TcShape {
     static_assert(STAGES >= NBUF + 1, "K/V ring too small");
 };
 
+// The (block position, head) of packed query row r, walked in steps of `step` rows: one division up front.  (Two per row
+// made the staging of Q 3.2 k cycles before its first load was out, a tenth of a CTA's life on packed sequences.)
+struct RowWalk {
+    int i, h, g, step_i, step_h;
+    __device__ __forceinline__ RowWalk(int r, int step, int g_) : i(r / g_), h(r % g_), g(g_), step_i(step / g_), step_h(step % g_) {}
+    __device__ __forceinline__ void next() {
+        i += step_i;
+        h += step_h;
+        if (h >= g) { h -= g; ++i; }
+    }
+};
+
 template <int STAGES, int QT>
 struct TcBarriers {
     uint64_t full[STAGES];
@@ -560,13 +572,13 @@ attn_block_tc_kernel(const __grid_constant__ CUtensorMap tm_kpre, const __grid_c
         const size_t q_token = packed ? static_cast<size_t>(seq_base) : static_cast<size_t>(b) * p.L;
         uint8_t* qt = q_s + j * S::Q_BYTES;
         uint4 v[CPR];
+        RowWalk rw((warp & 3) * 32 + lane / CPR, 32 / CPR, p.g);
+        const int pos0 = (blockIdx.x * QT + j) * pos_per_tile;
+        const uint4* qsrc = reinterpret_cast<const uint4*>(p.q + ((q_token + pos0) * p.Hq + kvh * p.g) * D) + c;
 #pragma unroll
-        for (int k = 0; k < CPR; ++k) {
-            const int r = (warp & 3) * 32 + k * (32 / CPR) + lane / CPR;
-            const int i = (blockIdx.x * QT + j) * pos_per_tile + r / p.g;
-            const int h = kvh * p.g + r % p.g;
-            const bool live = r < pos_per_tile * p.g && i < L_eff;
-            v[k] = live ? reinterpret_cast<const uint4*>(p.q + ((q_token + i) * p.Hq + h) * D)[c] : make_uint4(0, 0, 0, 0);
+        for (int k = 0; k < CPR; ++k, rw.next()) {
+            const bool live = rw.i < pos_per_tile && pos0 + rw.i < L_eff;      // (a tile's rows are pos_per_tile * g)
+            v[k] = live ? qsrc[(static_cast<size_t>(rw.i) * p.Hq + rw.h) * (D / 8)] : make_uint4(0, 0, 0, 0);
         }
 #pragma unroll
         for (int k = 0; k < CPR; ++k) {
@@ -828,13 +840,14 @@ attn_block_tc_kernel(const __grid_constant__ CUtensorMap tm_kpre, const __grid_c
         {
             constexpr int CPR = D / 8;
             const int c = lane % CPR;
+            RowWalk rw((warp & 3) * 32 + lane / CPR, 32 / CPR, p.g);
+            const int pos0 = (blockIdx.x * QT + j) * pos_per_tile;
+            uint4* dst = reinterpret_cast<uint4*>(p.out + ((q_token + pos0) * p.Hq + kvh * p.g) * D) + c;
 #pragma unroll
-            for (int k = 0; k < CPR; ++k) {
+            for (int k = 0; k < CPR; ++k, rw.next()) {
                 const int r2 = (warp & 3) * 32 + k * (32 / CPR) + lane / CPR;
-                const int i2 = (blockIdx.x * QT + j) * pos_per_tile + r2 / p.g;
-                const int h2 = kvh * p.g + r2 % p.g;
-                if (ok && r2 < rows_in_tile && i2 < L_eff)
-                    reinterpret_cast<uint4*>(p.out + ((q_token + i2) * p.Hq + h2) * D)[c] =
+                if (ok && rw.i < pos_per_tile && pos0 + rw.i < L_eff)
+                    dst[(static_cast<size_t>(rw.i) * p.Hq + rw.h) * (D / 8)] =
                         *reinterpret_cast<const uint4*>(ot + (c >> 3) * HALF_Q + r2 * 128 + (((c & 7) ^ (r2 & 7)) << 4));
             }
         }
