@@ -148,7 +148,7 @@ int dare_attn_varlen(dare_ctx* ctx, int total_tokens, int n_seqs, int max_seqlen
  *   row_tokens   int32 [M] or NULL: rows whose token != mask_id are already committed and get
  *                pred = that token, conf = -inf
  *   pred         int32 [M] out      conf  fp32 [M] out
- * Only rows that are still masked are evaluated (they are compacted on the device first).
+ * Only rows that are still masked are answered by the head; above 128 rows they are compacted on the device first.
  * Supported: D % 8 == 0, D >= 8; V >= 2; M >= 1.  Needs ctx workspace of 12 * M * min(#SMs, 2 * ceil(V/256))
  * bytes (partial (max, sum, argmax) triples per row), plus 2*M*D + 4*M + 2048 bytes when row_tokens is given.
  */

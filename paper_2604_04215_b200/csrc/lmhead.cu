@@ -88,6 +88,14 @@ __device__ __forceinline__ int32_t row_token(const int32_t* row_tokens, int tok_
     return row_tokens[static_cast<int64_t>(m / tok_L) * tok_row_stride + m % tok_L];
 }
 
+// Up to this many rows the head evaluates all of them where they lie, committed ones too, and nothing is compacted: the
+// launch is bound by reading W (161 us at 32 live rows x 126464, 167 us at 128), while the compaction kernel stood in
+// front of it with 3 to 5 us.  What is left of it: the GEMM does nothing if no row is masked, and the merge kernels answer
+// committed rows.
+constexpr int LM_DIRECT_ROWS = 128;
+// Token of row m = tokens[(m / L) * stride + m % L]; tokens == NULL: no direct launch
+struct LmTokens { const int32_t* tokens; int L; int64_t stride; int32_t mask_id; };
+
 // Compacts the still-masked rows of X into xc (order preserved), records their original indices, counts
 // them, and answers committed rows (pred = their token, conf = -inf).  One warp per row.
 constexpr int CP_ROWS = 8;
@@ -1015,8 +1023,14 @@ __global__ void __launch_bounds__(LM_THREADS, 1)
 lmhead_head_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ SwXMaps xmaps, int M,
                      const int32_t* __restrict__ live_rows, int D, int V, int mask_col, int n_tiles,
                      float* __restrict__ part_max, float* __restrict__ part_sum, int32_t* __restrict__ part_arg,
-                     uint32_t* __restrict__ dev_status, int parts_stride, const LmSampling smp) {
+                     uint32_t* __restrict__ dev_status, int parts_stride, const LmSampling smp, const LmTokens direct) {
     pdl_wait();
+    if (direct.tokens) {
+        bool any = false;
+        for (int m = threadIdx.x; m < M; m += LM_THREADS)
+            any |= row_token(direct.tokens, direct.L, direct.stride, m) == direct.mask_id;
+        if (!__syncthreads_or(any)) return;              // (every CTA alike)
+    }
     const int Mc = live_rows ? *live_rows : M;          // rows that need logits (uniform over the grid)
     if (lm_greedy_swapped(Mc)) {
         lm_swapped_body<MODE>(tmap_w, xmaps, Mc, D, V, mask_col, n_tiles, part_max, part_sum, part_arg, dev_status, parts_stride,
@@ -1118,7 +1132,7 @@ template <bool SAMPLE>
 __global__ void lmhead_merge_kernel(const LmParts parts, int grid_gemm, int n_tiles, int M,
                                     const int32_t* __restrict__ live_rows, const int32_t* __restrict__ idx,
                                     int32_t* __restrict__ pred, float* __restrict__ conf, int allow_pair,
-                                    int parts_stride, uint32_t* __restrict__ step_dev) {
+                                    int parts_stride, uint32_t* __restrict__ step_dev, const LmTokens direct) {
     pdl_trigger();      // (before the wait, as in lmhead_merge_select_kernel; a selection kernel may come in between)
     pdl_wait();
     if (SAMPLE && step_dev && blockIdx.x == 0 && threadIdx.x == 0) *step_dev += 1;   // the GEMM kernels before this one read it
@@ -1126,6 +1140,13 @@ __global__ void lmhead_merge_kernel(const LmParts parts, int grid_gemm, int n_ti
     const int lane = threadIdx.x & 31;
     const int Mc = live_rows ? *live_rows : M;
     if (c >= Mc) return;
+    if (direct.tokens) {
+        const int32_t tok = row_token(direct.tokens, direct.L, direct.stride, c);
+        if (tok != direct.mask_id) {
+            if (lane == 0) { pred[c] = tok; conf[c] = -INFINITY; }
+            return;
+        }
+    }
     const int groups = lm_row_partials(allow_pair, grid_gemm, Mc, n_tiles, c);
     int a;
     float cf;
@@ -1154,7 +1175,7 @@ struct LmSelect {
 };
 template <bool SAMPLE>
 __global__ void __launch_bounds__(1024)
-lmhead_merge_select_kernel(const LmParts parts, int grid_gemm, int n_tiles, int L,
+lmhead_merge_select_kernel(const LmParts parts, int grid_gemm, int n_tiles, int L, int M,
                            const int32_t* __restrict__ live_rows, const int32_t* __restrict__ idx, int32_t mask_id,
                            int32_t* __restrict__ pred, float* __restrict__ conf, int allow_pair, int parts_stride,
                            const LmSelect sel, uint32_t* __restrict__ step_dev) {
@@ -1170,19 +1191,23 @@ lmhead_merge_select_kernel(const LmParts parts, int grid_gemm, int n_tiles, int 
     // that belong to earlier rollouts = entries of the ascending list below b * L.  (A binary search by one thread, nine
     // dependent loads at 512 rows, was half of this kernel's 8 us.)
     int32_t* row = sel.tokens_block + static_cast<int64_t>(b) * sel.row_stride;
-    const bool masked = row[warp] == mask_id;
-    const int Mc = *live_rows;
+    const int32_t tok = row[warp];
+    const bool masked = tok == mask_id;
+    const int Mc = live_rows ? *live_rows : M;              // (NULL: the rows were evaluated where they lie)
     if (lane == 0) s_flag[warp] = masked ? 1 : 0;
     int before = 0;
-    for (int i0 = 0; i0 < b * L; i0 += blockDim.x) {        // (rows of earlier rollouts: at most b * L of them)
+    for (int i0 = 0; live_rows && i0 < b * L; i0 += blockDim.x) {   // (rows of earlier rollouts: at most b * L of them)
         const int i = i0 + threadIdx.x;
         const int32_t v = i < b * L ? idx[i] : 0;           // (entries from Mc on hold anything)
         before += __syncthreads_count(i < b * L && i < Mc && v < b * L);
     }
     __syncthreads();
     if (masked) {
-        int c = before;
-        for (int i = 0; i < warp; ++i) c += s_flag[i];
+        int c = b * L + warp;
+        if (live_rows) {
+            c = before;
+            for (int i = 0; i < warp; ++i) c += s_flag[i];
+        }
         const int groups = lm_row_partials(allow_pair, grid_gemm, Mc, n_tiles, c);
         int a;
         float cf;
@@ -1196,6 +1221,7 @@ lmhead_merge_select_kernel(const LmParts parts, int grid_gemm, int n_tiles, int 
         }
     } else if (lane == 0) {
         s_conf[warp] = __int_as_float(0x7fc00000);      // absent
+        if (!live_rows) { pred[b * L + warp] = tok; conf[b * L + warp] = -INFINITY; }      // (else the compaction did)
     }
     __syncthreads();
     if (warp != 0) return;
@@ -1346,7 +1372,7 @@ template <int MODE>
 static int launch_head(const dare_ctx* ctx, int grid, bool pairs, const void* x_gemm, int M, int D, const void* w, int V,
                        int mask_col, int n_tiles, const int32_t* live_rows, const int32_t* idx, float* parts, LmSampling smp,
                        uint32_t* step_dev, int tok_L, int64_t tok_row_stride, int32_t mask_id, int32_t* pred, float* conf,
-                       const LmSelectArgs* select, cudaStream_t stream) {
+                       const LmSelectArgs* select, const LmTokens& direct, cudaStream_t stream) {
     constexpr bool SAMPLE = MODE == LM_SAMPLE;
     size_t parts_max = pairs ? (grid & ~1) : ctx->sm_count;      // pairs: a fixed stride, at most two partials per vocabulary tile
     const size_t tile_parts = static_cast<size_t>(pairs ? 2 : 1) * n_tiles;
@@ -1375,7 +1401,7 @@ static int launch_head(const dare_ctx* ctx, int grid, bool pairs, const void* x_
         if (ensure_dynamic_smem(smem_set, lmhead_head_kernel<MODE>, SMEM) != DARE_OK) return DARE_ERR_CUDA;
         rc = launch_kernel(lmhead_head_kernel<MODE>, dim3(static_cast<unsigned>(grid_gemm)), LM_THREADS, SMEM, stream, 2, tmap_w,
                            xm, M, live_rows, D, V, mask_col, n_tiles, part_max, part_sum, part_arg, ctx->dev_status, parts_stride,
-                           smp);
+                           smp, direct);
         if (rc != DARE_OK) return rc;
     } else {
         CUtensorMap tmap_x;
@@ -1393,11 +1419,11 @@ static int launch_head(const dare_ctx* ctx, int grid, bool pairs, const void* x_
         sel.n_committed = select->n_committed; sel.n_remaining = select->n_remaining;
         sel.host_remaining = select->host_remaining;
         return launch_kernel(lmhead_merge_select_kernel<SAMPLE>, dim3(select->B), 32 * tok_L, 0, stream, 1, lp, grid_gemm, n_tiles,
-                             tok_L, live_rows, idx, mask_id, pred, conf, layout, parts_stride, sel, step_dev);
+                             tok_L, M, live_rows, idx, mask_id, pred, conf, layout, parts_stride, sel, step_dev);
     }
     constexpr int rows_per_block = 8;
     return launch_kernel(lmhead_merge_kernel<SAMPLE>, dim3((M + rows_per_block - 1) / rows_per_block), rows_per_block * 32, 0,
-                         stream, 1, lp, grid_gemm, n_tiles, M, live_rows, idx, pred, conf, layout, parts_stride, step_dev);
+                         stream, 1, lp, grid_gemm, n_tiles, M, live_rows, idx, pred, conf, layout, parts_stride, step_dev, direct);
 }
 
 int launch_lmhead(const dare_ctx* ctx, void* scratch, const void* hidden, int M, int D, const void* w, int V,
@@ -1415,7 +1441,12 @@ int launch_lmhead(const dare_ctx* ctx, void* scratch, const void* hidden, int M,
     const void* x_gemm = hidden;
     int32_t* idx = nullptr;
     int32_t* live_rows = nullptr;
-    if (row_tokens != nullptr) {
+    const bool pairs = grid >= 2 && lm_pair_available() &&
+                       lmhead_scratch_bytes(M, D, V, ctx->sm_count, row_tokens != nullptr, sample != nullptr, 2) <= ctx->workspace_bytes;
+    LmTokens direct = {};
+    if (row_tokens != nullptr && pairs && M <= LM_DIRECT_ROWS) {
+        direct = {row_tokens, tok_L, tok_row_stride, mask_id};
+    } else if (row_tokens != nullptr) {
         void* xc = cur;
         cur += round_up(static_cast<size_t>(M) * D * 2, 1024);
         idx = reinterpret_cast<int32_t*>(cur);
@@ -1428,13 +1459,11 @@ int launch_lmhead(const dare_ctx* ctx, void* scratch, const void* hidden, int M,
         if (rc != DARE_OK) return rc;
     }
     const int mask_col = (exclude_mask_column && mask_id >= 0 && mask_id < V) ? mask_id : -1;
-    const bool pairs = grid >= 2 && lm_pair_available() &&
-                       lmhead_scratch_bytes(M, D, V, ctx->sm_count, row_tokens != nullptr, sample != nullptr, 2) <= ctx->workspace_bytes;
     float* parts = reinterpret_cast<float*>(cur);
     LmSampling smp = {};
     if (sample == nullptr)
         return launch_head<LM_GREEDY>(ctx, grid, pairs, x_gemm, M, D, w, V, mask_col, n_tiles, live_rows, idx, parts, smp,
-                                      nullptr, tok_L, tok_row_stride, mask_id, pred, conf, select, stream);
+                                      nullptr, tok_L, tok_row_stride, mask_id, pred, conf, select, direct, stream);
     smp.inv_temperature = 1.0f / sample->temperature;
     smp.seed_lo = static_cast<uint32_t>(sample->seed & 0xffffffffu);
     smp.seed_hi = static_cast<uint32_t>(sample->seed >> 32);
@@ -1442,7 +1471,7 @@ int launch_lmhead(const dare_ctx* ctx, void* scratch, const void* hidden, int M,
     smp.step_dev = sample->step_dev;
     smp.row_index = idx;
     return launch_head<LM_SAMPLE>(ctx, grid, pairs, x_gemm, M, D, w, V, mask_col, n_tiles, live_rows, idx, parts, smp,
-                                  sample->step_dev, tok_L, tok_row_stride, mask_id, pred, conf, select, stream);
+                                  sample->step_dev, tok_L, tok_row_stride, mask_id, pred, conf, select, direct, stream);
 }
 
 int launch_lmhead_logprob(const dare_ctx* ctx, void* scratch, const void* hidden, int M, int D, const void* w, int V,

@@ -205,3 +205,42 @@ def test_rope_in_a_projection_of_few_rows(ctx, Hq, Hkv, d, B, length):
     assert torch.equal(caches[1], vc)
     assert ((caches[0].float() - kc.float()).abs() <= 2.0 ** -7 * kc.float().abs() + 1e-6).all()
     model.close()
+
+
+# Up to 128 rows the head evaluates committed rows too and answers them in its last kernel: the largest such launch and the
+# next one, sampled and greedy, with and without the selection on the last kernel, no row and every row masked.
+@pytest.mark.parametrize("B,L", [(1, 1), (4, 32), (3, 43), (2, 64)])
+@pytest.mark.parametrize("share", [0.0, 0.3, 1.0])
+def test_head_with_committed_rows(ctx, B, L, share):
+    D, V, mu, M = 64, 1300, 7, B * L
+    x, w = I.normal_bf16(M, I.TID_X, (M, D)).cuda(), I.normal_bf16(3, I.TID_W, (V, D), 0.2).cuda()
+    tok = I.uniform_int(9, M, (B, L + 5), 8, V - 1)
+    masked = torch.rand(B, L, generator=torch.Generator().manual_seed(M)) < share
+    tok[:, 5:] = torch.where(masked, torch.full_like(tok[:, 5:], mu), tok[:, 5:])
+    tok, flat = tok.cuda(), tok[:, 5:].reshape(-1).cuda()
+    for temperature in (0.0, 0.7):
+        head = (lambda r: dare.dare_lmhead_sample(ctx, x, w, r, mu, True, temperature, 5, 3)) if temperature else \
+               (lambda r: dare.dare_lmhead_confidence(ctx, x, w, r, mu, True))
+        p_all, c_all = head(None)                          # every row evaluated
+        pred, conf = head(flat)
+        m = flat == mu
+        assert torch.equal(pred, torch.where(m, p_all, flat))
+        # (a row's sums are cut up differently with fewer rows: fp32 rounding of sums of 1300 terms)
+        assert torch.allclose(conf[m], c_all[m], rtol=1e-5, atol=0) and torch.isneginf(conf[~m]).all()
+        # the step on the same rows
+        q, kv = torch.randn(B, L, 1, 64, device="cuda").bfloat16(), torch.randn(B, 1, 40 + L, 64, device="cuda").bfloat16()
+        t2, out = tok.clone(), torch.empty_like(q)
+        p2, c2 = torch.zeros_like(pred), torch.zeros_like(conf)
+        nc, nr = torch.zeros(B, dtype=torch.int32, device="cuda"), torch.zeros(B, dtype=torch.int32, device="cuda")
+        args = (ctx, q, kv, kv, torch.full((B,), 40, dtype=torch.int32, device="cuda"), None, None, None, None, None, out, None, x, w,
+                mu, True)
+        tail = (t2, 5, dare.SELECT_TOPK, 0.0, 2, p2, c2, nc, nr)
+        if temperature:
+            dare.dare_denoise_block_sampled(*args, temperature, 5, 3, *tail)
+        else:
+            dare.dare_denoise_block(*args, *tail)
+        torch.cuda.synchronize()
+        assert torch.equal(p2, pred) and torch.equal(c2, conf)
+        n = m.view(B, L).sum(1)
+        assert torch.equal(nc.long(), n.clamp(max=2)) and torch.equal(nr.long(), n - n.clamp(max=2))
+    assert ctx.device_status() == 0
