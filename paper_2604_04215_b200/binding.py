@@ -28,6 +28,7 @@ EXPORTS = ["dare_create", "dare_destroy", "dare_status_string", "dare_device_sta
            "dare_linear", "dare_linear_plan", "dare_rmsnorm", "dare_rope_kv_write"]
 
 _lib = None
+_marshal = None
 
 
 class DareError(RuntimeError):
@@ -186,6 +187,24 @@ def _stream(stream, device: Optional[int] = None) -> C.c_void_p:
     return C.c_void_p(stream.cuda_stream)
 
 
+def _raw(stream, device: int) -> int:
+    if stream is not None:
+        return stream.cuda_stream
+    return _raw_stream(device) if _raw_stream is not None else torch.cuda.current_stream().cuda_stream
+
+
+def _native():
+    """The calls of a rollout's inner loop marshalled in C++ (csrc/marshal.cpp).  They return None where an argument is not
+    what the entry point takes; the Python path behind each of them then says what is wrong."""
+    global _marshal
+    if _marshal is None:
+        load()
+        from . import _marshal as m
+        m.bind(LIB_PATH)
+        _marshal = m
+    return _marshal
+
+
 class Context:
     """Owns a dare_ctx (workspace + device status word) on one device."""
 
@@ -250,12 +269,17 @@ def dare_attn_block(ctx: Context, q, k_pre, v_pre, prefix_len=None, k_blk=None, 
 
 def dare_attn_varlen(ctx: Context, q, k, v, cu_seqlens, max_seqlen: int, out=None, lse=None, scale: float = 0.0,
                      stream=None, check: bool = True):
-    total, Hq, d = q.shape
-    Hkv = k.shape[1]
     if out is None:
         out = torch.empty_like(q)
-    bf = torch.bfloat16
     dev = torch.cuda.current_device()
+    rc = _native().attn_varlen(ctx.handle.value, dev, _raw(stream, dev), scale, q, k, v, cu_seqlens, max_seqlen, out, lse)
+    if rc is not None:
+        if rc != 0 and check:
+            raise DareError(rc, "dare_attn_varlen")
+        return out if check else rc
+    total, Hq, d = q.shape
+    Hkv = k.shape[1]
+    bf = torch.bfloat16
     rc = load().dare_attn_varlen(ctx.handle, total, cu_seqlens.numel() - 1, int(max_seqlen), Hq, Hkv, d, float(scale),
                                  _addr(q, bf, dev), _addr(k, bf, dev), _addr(v, bf, dev), _addr(cu_seqlens, torch.int32, dev), _addr(out, bf, dev),
                                  _addr(lse, torch.float32, dev), _stream(stream, dev))
@@ -429,13 +453,21 @@ def dare_denoise_block(ctx: Context, q, k_pre, v_pre, prefix_len, k_blk, v_blk, 
                        attn_out, lse, hidden, w, mask_id: int, exclude_mask_column: bool, tokens, block_start: int,
                        mode: int, threshold: float, k: int, pred, conf, n_committed=None, n_remaining=None,
                        scale: float = 0.0, stream=None, check: bool = True):
+    dev = torch.cuda.current_device()
+    rc = _native().denoise_block(
+        ctx.handle.value, dev, _raw(stream, dev), scale, q, k_pre, v_pre, prefix_len, k_blk, v_blk, k_suf, v_suf, suffix_len,
+        attn_out, lse, hidden, w, mask_id, exclude_mask_column, tokens, block_start, mode, threshold, k, pred, conf,
+        n_committed, n_remaining)
+    if rc is not None:
+        if rc != 0 and check:
+            raise DareError(rc, "dare_denoise_block")
+        return rc
     B, L, Hq, d = q.shape
     Hkv, prefix_cap = k_pre.shape[1], k_pre.shape[2]
     suffix_cap = k_suf.shape[2] if k_suf is not None else 0
     D = hidden.shape[1]
     V = w.shape[0]
     bf = torch.bfloat16
-    dev = torch.cuda.current_device()
     rc = load().dare_denoise_block(
         ctx.handle, B, L, Hq, Hkv, d, prefix_cap, suffix_cap, float(scale),
         _addr(q, bf, dev), _addr(k_pre, bf, dev), _addr(v_pre, bf, dev), _addr(prefix_len, torch.int32, dev), _addr(k_blk, bf, dev), _addr(v_blk, bf, dev),
@@ -454,13 +486,21 @@ def dare_denoise_block_sampled(ctx: Context, q, k_pre, v_pre, prefix_len, k_blk,
                                seed: int, step: int, tokens, block_start: int, mode: int, threshold: float, k: int,
                                pred, conf, n_committed=None, n_remaining=None, scale: float = 0.0, stream=None,
                                check: bool = True):
+    dev = torch.cuda.current_device()
+    rc = _native().denoise_block_sampled(
+        ctx.handle.value, dev, _raw(stream, dev), scale, q, k_pre, v_pre, prefix_len, k_blk, v_blk, k_suf, v_suf, suffix_len,
+        attn_out, lse, hidden, w, mask_id, exclude_mask_column, temperature, seed, step, tokens, block_start, mode,
+        threshold, k, pred, conf, n_committed, n_remaining)
+    if rc is not None:
+        if rc != 0 and check:
+            raise DareError(rc, "dare_denoise_block_sampled")
+        return rc
     B, L, Hq, d = q.shape
     Hkv, prefix_cap = k_pre.shape[1], k_pre.shape[2]
     suffix_cap = k_suf.shape[2] if k_suf is not None else 0
     D = hidden.shape[1]
     V = w.shape[0]
     bf = torch.bfloat16
-    dev = torch.cuda.current_device()
     rc = load().dare_denoise_block_sampled(
         ctx.handle, B, L, Hq, Hkv, d, prefix_cap, suffix_cap, float(scale),
         _addr(q, bf, dev), _addr(k_pre, bf, dev), _addr(v_pre, bf, dev), _addr(prefix_len, torch.int32, dev), _addr(k_blk, bf, dev), _addr(v_blk, bf, dev),

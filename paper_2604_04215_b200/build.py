@@ -4,6 +4,7 @@
 
 nvcc cross-compiles without a GPU.  The library links the static CUDA runtime and resolves the one driver
 entry point it needs (tensor-map encoding) at run time, so it has no link-time dependency on libcuda.
+_marshal.so beside it is the Python module through which binding.py makes the calls of a rollout's inner loop.
 """
 from __future__ import annotations
 
@@ -11,11 +12,13 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libdare.so")
 SOURCES = ["api.cu", "lmhead.cu", "attn.cu", "select.cu", "gemm.cu", "gemm_few.cu", "layers.cu", "model.cu", "diffusion.cu", "backward.cu"]
+MARSHAL = os.path.join(HERE, "_marshal.so")
 HEADERS = ["ptx.cuh", "internal.h", os.path.join("..", "..", "include", "dare.h")]
 
 
@@ -27,11 +30,21 @@ def _nvcc() -> str:
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(MARSHAL):
         return True
-    t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, s) for s in SOURCES + HEADERS] + [os.path.abspath(__file__)]
+    t = min(os.path.getmtime(LIB), os.path.getmtime(MARSHAL))
+    deps = [os.path.join(CSRC, s) for s in SOURCES + ["marshal.cpp"] + HEADERS] + [os.path.abspath(__file__)]
     return any(os.path.getmtime(d) > t for d in deps)
+
+
+def _marshal_cmd() -> list:
+    import torch
+    root = os.path.dirname(os.path.abspath(torch.__file__))
+    inc = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
+           os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include"), sysconfig.get_paths()["include"]]
+    return ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+            *[f for d in inc for f in ("-isystem", d)], "-o", MARSHAL, os.path.join(CSRC, "marshal.cpp"),
+            "-L" + os.path.join(root, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10", "-ldl"]
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -43,11 +56,12 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if verbose:
         cmd.insert(1, "-Xptxas")
         cmd.insert(2, "-v")
-    res = subprocess.run(cmd, capture_output=True, text=True)
-    if verbose or res.returncode != 0:
-        sys.stderr.write(res.stdout + res.stderr)
-    if res.returncode != 0:
-        raise RuntimeError("nvcc failed building libdare.so")
+    for what, c in (("libdare.so", cmd), ("_marshal.so", _marshal_cmd())):
+        res = subprocess.run(c, capture_output=True, text=True)
+        if verbose or res.returncode != 0:
+            sys.stderr.write(res.stdout + res.stderr)
+        if res.returncode != 0:
+            raise RuntimeError(f"{c[0]} failed building {what}")
     return LIB
 
 
