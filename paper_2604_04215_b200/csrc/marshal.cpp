@@ -1,6 +1,6 @@
 // The calls of a rollout's inner loop without Python between the tensors and the library: checks every tensor (device,
 // contiguity, type), takes addresses and sizes and calls the C entry point.  A step of a small block is bound by the host:
-// the call cost it 17.3 us, of which the library's own 3 launches 10.  8 steps of 2 blocks of 32 rows at D = 256, V = 2048:
+// the call cost it 17.3 us, of which the library's own 3 launches 10.  8 steps of one block of 32 rows at D = 256, V = 4096:
 // 155 us with ctypes, 104 us with this.
 //
 // Each function returns the entry point's status, or None when an argument is not what it should be: the caller then
