@@ -321,14 +321,22 @@ int read_counts(const dare_model* m, int slot, int B, cudaStream_t s, bool* done
 // A step whose block holds no mask any more does exactly what the refresh forward of the prefix-cache loop
 // must do (the LM head finds no live row, the selection changes nothing, the stack rewrites the block's K/V
 // from the committed tokens).  So step t + 1 is enqueued before step t's counts are read: when step t turns
-// out to have finished the block, step t + 1 was the refresh, and the GPU never waits for the host.  (In the
-// dual-cache loop that extra step is redundant and harmless: the next whole-sequence refresh rewrites the
-// same K/V.)
+// out to have finished the block, step t + 1 was the refresh, and the GPU never waits for the host.
+//
+// refresh = false: something else is about to rewrite the block's K/V (the dual-cache loop's forward of the whole
+// sequence).  With top-k commits, ceil(L / k) steps leave no mask whatever their counts say, so the extra step is not
+// enqueued: 13 instead of 14 steps of 107 us for two blocks of 16 with k = 3 (24 small kernels each).  At one step per
+// block the counts that pace the host would never be read: the extra step stays.
 int run_block(dare_model* m, int32_t* tokens, int B, int64_t row_stride, int start, int L, int kv_len, void* k_cache,
               void* v_cache, int cap, int mode, float threshold, int k, int32_t* pred, float* conf, int32_t* n_remaining,
-              cudaStream_t s, uint32_t* step_no, int* steps_taken) {
+              cudaStream_t s, uint32_t* step_no, bool refresh, int* steps_taken) {
+    const int enough = mode == DARE_SELECT_TOPK && k < L ? (L + k - 1) / k : 0;
     for (int issued = 0;; ++issued) {
         if (issued > L + 1) return DARE_ERR_CUDA;            // cannot happen: every step commits a token per row
+        if (!refresh && enough > 0 && issued == enough) {
+            *steps_taken = issued;
+            return DARE_OK;
+        }
         // The slots go round over the whole loop, not per block: when a slot comes round again, a later step than the one
         // that used it has been read, so nothing writes to it any more.
         const uint32_t n = (*step_no)++;
@@ -374,7 +382,7 @@ int dare_generate(dare_model* m, int32_t* tokens, int B, int64_t row_stride, int
             if (rc != DARE_OK) break;
         }
         rc = run_block(m, tokens, B, row_stride, start, L, start + L, k_cache, v_cache, cache_cap, mode, threshold, k,
-                       pred, conf, n_remaining, user, &step_no, &taken);
+                       pred, conf, n_remaining, user, &step_no, true, &taken);
         if (rc == DARE_OK && steps_per_block) steps_per_block[b] = taken;
     }
     const bool synced = cudaStreamSynchronize(user) == cudaSuccess;      // (also after an error: the counts' slots are still in use)
@@ -402,7 +410,7 @@ int dare_generate_dual(dare_model* m, int32_t* tokens, int B, int64_t row_stride
             if (rc != DARE_OK) break;
         }
         rc = run_block(m, tokens, B, row_stride, start, L, T, k_cache, v_cache, cache_cap, mode, threshold, k, pred, conf,
-                       n_remaining, user, &step_no, &taken);
+                       n_remaining, user, &step_no, b + 1 == gen_len / L, &taken);
         if (rc == DARE_OK && steps_per_block) steps_per_block[b] = taken;
     }
     const bool synced = cudaStreamSynchronize(user) == cudaSuccess;      // (also after an error: the counts' slots are still in use)

@@ -244,3 +244,37 @@ def test_head_with_committed_rows(ctx, B, L, share):
         n = m.view(B, L).sum(1)
         assert torch.equal(nc.long(), n.clamp(max=2)) and torch.equal(nr.long(), n - n.clamp(max=2))
     assert ctx.device_status() == 0
+
+
+@pytest.mark.parametrize("k", [1, 3, 7, 8, 20])
+@pytest.mark.parametrize("mode", [dare.SELECT_TOPK, dare.SELECT_THRESHOLD])
+def test_dual_loop_equals_its_parts(ctx, k, mode):
+    """Blocks of 8 with some tokens given beforehand (one block whole): whatever the loop leaves out or enqueues ahead, the
+    tokens, the steps and all K/V that the last forward of each position wrote are those of the calls it is made of."""
+    B, P, L, G = 2, 5, 8, 32
+    T = P + G
+    model = _small_model(ctx, 4, 2, 64, B * T, B, T)
+    mask_id = 511
+    g = torch.Generator().manual_seed(5)
+    tok0 = torch.randint(0, 500, (B, T), generator=g, dtype=torch.int32)
+    given = torch.rand(B, G, generator=g) < 0.3
+    given[:, L:2 * L] = True
+    tok0[:, P:][~given] = mask_id
+    new = lambda: model.new_cache(B, T)
+    pred, conf = torch.empty(B * L, dtype=torch.int32, device="cuda"), torch.empty(B * L, device="cuda")
+    nr = torch.zeros(B, dtype=torch.int32, device="cuda")
+
+    tok, (kc, vc), want = tok0.cuda(), new(), []
+    for start in range(P, T, L):
+        dare.dare_model_forward_window(model, tok, 0, T, T, kc, vc)
+        n = 0
+        while n == 0 or int(nr.sum()) > 0:
+            dare.dare_model_step_window(model, tok, start, L, T, kc, vc, mode, 0.9, k, pred, conf, None, nr)
+            n += 1
+        want.append(n)
+    dare.dare_model_forward_window(model, tok, T - L, L, T, kc, vc)
+
+    tok2, (kc2, vc2) = tok0.cuda(), new()
+    steps = dare.dare_generate_dual(model, tok2, P, G, L, kc2, vc2, mode, 0.9, k, pred, conf, nr)
+    assert steps == want
+    assert torch.equal(tok2, tok) and torch.equal(kc2, kc) and torch.equal(vc2, vc)
