@@ -597,11 +597,13 @@ lmhead_partial_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
 //   * no padding to 128-row tiles: a step with 96 masked rows issues MMAs of N = 96, not of 128 padded rows;
 //   * every work item is a CTA pair whatever the row count, and the 128-row vocabulary tiles per CTA spread evenly
 //     over the SMs: with few rows left the W stream is the bound and the kernel reads it at the copy bandwidth.
-// More rows than SW_NMAX are cut into equal chunks (items = chunk x vocabulary group); lm_greedy_swapped says for
-// which counts that beats the row-major tiles.  An MMA alone takes max(N / 2, ~45) cycles whether M is 64 or 128 and
-// wherever A sits (timed in isolation), but here every MMA takes a fresh 128 x 16 slab of W as its A operand, so a
-// chunk streams all of W from L2 into the SMs whatever its N: two chunks of N = 144 cost nearly what two chunks of
-// N = 256 cost (319 us for 288 rows, 350 us for 512), and only chunks close to 256 rows are worth it.
+// More rows than SW_NMAX are cut into equal chunks, in one of two ways:
+//   * items = chunk x vocabulary group: a chunk streams all of W from L2 into the SMs whatever its N, and that stream
+//     (~12 TB/s over the GPU), not the tensor pipe, sets the pace when the chunks are short (an MMA alone takes
+//     max(N / 2, ~45) cycles): only chunks close to 256 rows are worth it;
+//   * both chunks against each W tile (JOINT): W enters the SMs once.  The price is the accumulators: two chunks take half
+//     of TMEM or more, so the next tile's MMAs wait for part of this one's epilogue (three of up to 160 columns fit: for
+//     half of it), and the running values of 512 columns move to shared memory.
 // The price is the epilogue: a thread's TMEM lane is now a vocabulary entry and the softmax runs ACROSS lanes.
 // Each epilogue warp turns its 32 x 32 block of logits through shared memory (padded rows, conflict-free) so that
 // a thread again holds 32 consecutive vocabulary entries of ONE row, and keeps that row's running
@@ -612,16 +614,18 @@ lmhead_partial_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
 // so the values live in shared memory, taken off the ring (6 slots become 5 above 192 rows).
 constexpr int SW_BV = 128;                               // vocabulary rows per CTA and tile
 constexpr int SW_NMAX = 256;                             // rows (accumulator columns) per chunk
-// Row counts for which the greedy head takes this path: up to one chunk, where W is streamed once and the launch is
-// bound by HBM; and, up to 1024 rows, counts that cut into chunks of 208 to 240 rows, i.e. whose row-major tiles
-// would carry 64 or more padded rows per pair (measured in one process, us, swapped against row-major: D = 4096,
-// V = 126464: 416 rows 333 / 380, 448 rows 415 / 462, 480 rows 410 / 428, 512 rows 425 / 421; D = 3584, V = 152064:
-// 704 rows 625 / 650, 832 rows 784 / 840, 960 rows 851 / 895).  With shorter chunks the path loses (288 to 384 rows:
-// 339 to 372 against 329 to 343): every MMA of this path takes a fresh 128 x 16 slab of W as its A operand, so a
-// chunk streams all of W from L2 into the SMs whatever its N, and at N = 144 to 192 that stream (~12 TB/s over the
-// GPU), not the tensor pipe, sets the pace.
-__host__ __device__ inline bool lm_greedy_swapped(int rows) {
-    if (rows <= SW_NMAX) return true;
+// Row counts for which a head takes this path: up to one chunk, where W is streamed once and the launch is bound by HBM;
+// up to LM_JOINT_ROWS with both chunks at a time (greedy only); and, up to 1024 rows, counts that cut into chunks of 208
+// to 240 rows, i.e. whose row-major tiles would carry 64 or more padded rows per pair (swapped against row-major, one
+// chunk at a time, us: D = 4096, V = 126464: 416 rows 333 / 380, 448 rows 415 / 462, 480 rows 410 / 428, 512 rows 425 / 421;
+// D = 3584, V = 152064: 704 rows 625 / 650, 832 rows 784 / 840, 960 rows 851 / 895).
+// Both chunks at a time against row-major tiles (256 + 128 rows), under the power cap, us, D = 4096, V = 126464: 272 rows
+// 298 / 404, 320 rows 320 / 411, 336 rows 369 / 416, 384 rows 394 / 425; above, one chunk at a time is better (448 rows 442 /
+// 411).  The sampled head's epilogue is several times as long and may not be waited for: 320 rows 457 / 383.
+constexpr int LM_JOINT_ROWS = 384;
+__host__ __device__ inline bool lm_joint(int rows, bool sampled) { return !sampled && rows > SW_NMAX && rows <= LM_JOINT_ROWS; }
+__host__ __device__ inline bool lm_swapped(int rows, bool sampled) {
+    if (rows <= SW_NMAX || lm_joint(rows, sampled)) return true;
     if (rows > 1024) return false;
     const int n_chunks = (rows + SW_NMAX - 1) / SW_NMAX;
     const int nc = ((rows + n_chunks - 1) / n_chunks + 15) & ~15;      // as in sw_plan below
@@ -637,21 +641,28 @@ constexpr int SW_PARTS_PER_GROUP = 2;                    // one per CTA of the p
 struct SwBarriers {
     uint64_t full[SW_MAX_STAGES];
     uint64_t empty[SW_MAX_STAGES];
-    uint64_t tmem_full[2];
-    uint64_t tmem_empty[2];
+    uint64_t tmem_full[3];
+    uint64_t tmem_empty[3];
     uint64_t fold_full, fold_empty;                      // the epilogue warps' exchange at the end of an item
     uint32_t tmem_base;
     uint32_t abort_flag;
 };
-constexpr int SW_STATE_FLOATS = 5 * SW_NMAX;            // sampled head, per epilogue warp: (max, sum, y, z, column) per row
-__host__ __device__ constexpr int sw_ring_bytes(int mode) {
-    return mode == LM_SAMPLE ? (SW_STAGES * SW_STAGE_BYTES - 3072) : SW_STAGES * SW_STAGE_BYTES;
+// Values per row that an epilogue warp keeps in shared memory (floats): the sampled head's (max, sum, y, z, column) and, for
+// two chunks at a time, the greedy head's (max, sum, column); in registers otherwise.
+__host__ __device__ constexpr int sw_values(int mode, bool joint) { return mode == LM_SAMPLE ? 5 : joint ? 3 : 0; }
+__host__ __device__ constexpr int sw_state_bytes(int mode, bool joint) {
+    return 4 * sw_values(mode, joint) * (joint ? 2 : 1) * SW_NMAX * 4;
 }
-__host__ __device__ constexpr int sw_smem_bytes(int mode) {
-    return sw_ring_bytes(mode) + 4 * SW_XP_FLOATS * 4 + (mode == LM_SAMPLE ? 4 * SW_STATE_FLOATS * 4 : 0) +
-           static_cast<int>(sizeof(SwBarriers)) + 1024;
+constexpr int SW_SMEM_BYTES = 227 * 1024;
+__host__ __device__ constexpr int sw_ring_bytes(int mode, bool joint) {
+    return joint ? (SW_SMEM_BYTES - 1024 - 4 * SW_XP_FLOATS * 4 - sw_state_bytes(mode, true) - static_cast<int>(sizeof(SwBarriers))) & ~1023
+                 : SW_STAGES * SW_STAGE_BYTES - (mode == LM_SAMPLE ? 3072 : 0);
 }
-static_assert(sw_smem_bytes(LM_SAMPLE) <= 227 * 1024 && sw_smem_bytes(LM_GREEDY) <= 227 * 1024, "shared memory");
+__host__ __device__ constexpr int sw_smem_bytes(int mode, bool joint) {
+    return sw_ring_bytes(mode, joint) + 4 * SW_XP_FLOATS * 4 + sw_state_bytes(mode, joint) + static_cast<int>(sizeof(SwBarriers)) + 1024;
+}
+static_assert(sw_smem_bytes(LM_SAMPLE, false) <= SW_SMEM_BYTES && sw_smem_bytes(LM_GREEDY, false) <= SW_SMEM_BYTES &&
+              sw_smem_bytes(LM_GREEDY, true) <= SW_SMEM_BYTES, "shared memory");
 // X tiles of 128, 64, 32, 16 and 8 rows: a CTA's share of a chunk (a multiple of 8 rows) is covered by one or two
 // of them, stacked in shared memory (each a whole number of 1 KB swizzle atoms); a few rows too many may be loaded,
 // the MMA reads only its own.  (Exact covers of up to four boxes were measured slower: 432 us for 480 rows, where
@@ -659,6 +670,11 @@ static_assert(sw_smem_bytes(LM_SAMPLE) <= 227 * 1024 && sw_smem_bytes(LM_GREEDY)
 struct SwXMaps { CUtensorMap m[5]; };
 struct SwBoxes { int i1, i2, rows; };      // indices into SwXMaps::m (i2 < 0: one box), rows loaded in all
 __device__ __forceinline__ SwBoxes sw_boxes(int rows_half) {
+    if (rows_half > 128) {                 // two chunks at a time
+        int second = 4;
+        while ((128 >> second) < rows_half - 128) --second;
+        return {0, second, 128 + (128 >> second)};
+    }
     int single = 0;                        // smallest box that holds the rows
     while ((128 >> single) >= 2 * rows_half && single < 4) ++single;
     int first = single + 1;                // largest box below that, plus the smallest box for the remainder
@@ -676,20 +692,21 @@ __device__ __forceinline__ SwBoxes sw_boxes(int rows_half) {
 
 // How `rows` live rows are cut up for a grid of n_units CTA pairs and n_vt vocabulary tiles of 256 (the same
 // formula on the host, in the GEMM and in the merge kernels).
-struct SwPlan { int n_chunks, nc, groups, parts; };
-__host__ __device__ inline SwPlan sw_plan(int rows, int n_units, int n_vt) {
+struct SwPlan { int n_chunks, nc, groups, parts; bool joint; };
+__host__ __device__ inline SwPlan sw_plan(int rows, int n_units, int n_vt, bool sampled) {
     SwPlan p;
     p.n_chunks = (rows + SW_NMAX - 1) / SW_NMAX;
     if (p.n_chunks < 1) p.n_chunks = 1;
     const int per = (rows + p.n_chunks - 1) / p.n_chunks;
     p.nc = (per + 15) & ~15;                             // rows per chunk: N of the pair's MMA
     if (p.nc < 16) p.nc = 16;
-    p.groups = lm_groups(n_units, p.n_chunks, n_vt);
+    p.joint = lm_joint(rows, sampled);
+    p.groups = lm_groups(n_units, p.joint ? 1 : p.n_chunks, n_vt);
     p.parts = SW_PARTS_PER_GROUP * p.groups;
     return p;
 }
 
-template <int MODE>
+template <int MODE, bool JOINT>
 __device__ __forceinline__ void
 lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, int V, int mask_col, int n_vt,
                 float* __restrict__ part_max, float* __restrict__ part_sum, int32_t* __restrict__ part_arg,
@@ -699,17 +716,27 @@ lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, 
     const int rank = static_cast<int>(cluster_cta_rank());
     const int unit = blockIdx.x >> 1;
     const int n_units = gridDim.x >> 1;
-    const SwPlan plan = sw_plan(Mc, n_units, n_vt);
-    const int n_items = plan.n_chunks * plan.groups;
+    const SwPlan plan = sw_plan(Mc, n_units, n_vt, SAMPLE);
+    constexpr int J = JOINT ? 2 : 1;                     // chunks per W tile
+    constexpr bool STATE = sw_values(MODE, JOINT) > 0;   // running values in shared memory
+    constexpr int NV = sw_values(MODE, JOINT), NS = J * SW_NMAX, WARP_STATE = NV * NS;
+    const int item_chunks = JOINT ? 1 : plan.n_chunks;
+    const int n_items = item_chunks * plan.groups;
     if (unit >= n_items) return;                         // (both CTAs of a pair alike)
     const int nc = plan.nc, groups = plan.groups;
-    const int rows_half = nc >> 1;                       // this CTA's share of a chunk's rows (multiple of 8)
+    const int rows_half = J * (nc >> 1);                 // rows this CTA loads (a multiple of 8 per chunk), consecutive ones
+    // accumulators: a ring of two, or, where three fit, three
+    const int slots = JOINT && nc <= 160 ? 3 : 2, slot_cols = JOINT && nc <= 160 ? 160 : SW_NMAX;
+    // row of column c of the item's chunk j: the even CTA's rows are the columns below nc / 2
+    const auto row_of = [&](int item, int j, int c) {
+        return JOINT ? (c < (nc >> 1) ? c : c + (nc >> 1)) + j * (nc >> 1) : (item % item_chunks) * nc + c;
+    };
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    float* xpose = reinterpret_cast<float*>(tiles + sw_ring_bytes(MODE));
-    float* state = xpose + 4 * SW_XP_FLOATS;             // SAMPLE: [warp][value][row]
-    SwBarriers* bars = reinterpret_cast<SwBarriers*>(state + (SAMPLE ? 4 * SW_STATE_FLOATS : 0));
+    float* xpose = reinterpret_cast<float*>(tiles + sw_ring_bytes(MODE, JOINT));
+    float* state = xpose + 4 * SW_XP_FLOATS;             // STATE: [warp][value][chunk][column]
+    SwBarriers* bars = reinterpret_cast<SwBarriers*>(state + 4 * WARP_STATE);
     volatile uint32_t* abort_flag = &bars->abort_flag;
 
     const int warp = warp_index_uniform();
@@ -720,22 +747,23 @@ lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, 
     // bandwidth (6 slots per CTA, 14 MB over the GPU, covered ~2 us of HBM latency at 6.3 TB/s and no more).
     const SwBoxes xbox = sw_boxes(rows_half);
     const int stage_bytes = SW_W_BYTES + ((xbox.rows * 128 + 1023) & ~1023);
-    const int n_stages = min(SW_MAX_STAGES, sw_ring_bytes(MODE) / stage_bytes);
+    const int n_stages = min(SW_MAX_STAGES, sw_ring_bytes(MODE, JOINT) / stage_bytes);
     // no logit seen yet (set here and by the fold at an item's end: the warps read one another's best scores at any time)
     const auto clear_state = [&](int q, int r) {
-        float* s = state + q * SW_STATE_FLOATS + r;
-        s[0] = s[2 * SW_NMAX] = s[3 * SW_NMAX] = -INFINITY;
-        s[SW_NMAX] = 0.f;
-        s[4 * SW_NMAX] = __int_as_float(ARG_NONE);
+        float* s = state + q * WARP_STATE + r;
+        s[0] = -INFINITY;
+        s[NS] = 0.f;
+        if (SAMPLE) s[2 * NS] = s[3 * NS] = -INFINITY;
+        s[(NV - 1) * NS] = __int_as_float(ARG_NONE);
     };
-    if (SAMPLE)
-        for (int i = threadIdx.x; i < 4 * SW_NMAX; i += LM_THREADS) clear_state(i / SW_NMAX, i % SW_NMAX);
+    if (STATE)
+        for (int i = threadIdx.x; i < 4 * NS; i += LM_THREADS) clear_state(i / NS, i % NS);
     if (threadIdx.x == 0) {
         for (int s = 0; s < n_stages; ++s) {
             mbar_init(&bars->full[s], 1);
             mbar_init(&bars->empty[s], 1);
         }
-        for (int a = 0; a < 2; ++a) {
+        for (int a = 0; a < 3; ++a) {
             mbar_init(&bars->tmem_full[a], 1);
             mbar_init(&bars->tmem_empty[a], 8);          // one arrival per epilogue warp of both CTAs
         }
@@ -765,8 +793,8 @@ lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, 
             const SwBoxes box = xbox;
             const uint32_t stage_tx = 2u * static_cast<uint32_t>(SW_W_BYTES + box.rows * 128);
             for (int item = unit; item < n_items && ok; item += n_units) {
-                const int x_row0 = (item % plan.n_chunks) * nc + rank * rows_half;
-                for (int vt = item / plan.n_chunks; vt < n_vt && ok; vt += groups) {
+                const int x_row0 = (item % item_chunks) * nc + rank * rows_half;
+                for (int vt = item / item_chunks; vt < n_vt && ok; vt += groups) {
                     const int w_row0 = vt * (2 * SW_BV) + rank * SW_BV;
                     for (int kb = 0; kb < num_k; ++kb) {
                         if (!mbar_wait(&bars->empty[stage], phase ^ 1, abort_flag)) { ok = false; break; }
@@ -793,13 +821,15 @@ lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, 
         int it = 0;
         bool ok = true;
         for (int item = unit; item < n_items && ok; item += n_units) {
-            for (int vt = item / plan.n_chunks; vt < n_vt && ok; vt += groups, ++it) {
-                const int acc = it & 1;
-                const uint32_t acc_phase = (it >> 1) & 1;
-                ok = __all_sync(0xffffffffu, mbar_wait(&bars->tmem_empty[acc], acc_phase ^ 1, abort_flag));
+            for (int vt = item / item_chunks; vt < n_vt && ok; vt += groups, ++it) {
+                int acc[J];
+#pragma unroll
+                for (int j = 0; j < J; ++j) {
+                    acc[j] = (it * J + j) % slots;
+                    ok = ok && __all_sync(0xffffffffu, mbar_wait(&bars->tmem_empty[acc[j]], (((it * J + j) / slots) & 1) ^ 1, abort_flag));
+                }
                 if (!ok) break;
                 tc_fence_after_sync();
-                const uint32_t d_tmem = tmem_base + acc * SW_NMAX;
                 for (int kb = 0; kb < num_k; ++kb) {
                     ok = __all_sync(0xffffffffu, mbar_wait(&bars->full[stage], phase, abort_flag));
                     if (!ok) break;
@@ -809,14 +839,21 @@ lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, 
                     const uint64_t b_desc = umma_desc_sw128_kmajor(w_addr + SW_W_BYTES);
                     if (leader) {
 #pragma unroll
-                        for (int kk = 0; kk < BK / 16; ++kk)
-                            umma_bf16_pair(d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, idesc, (kb | kk) != 0);
+                        for (int kk = 0; kk < BK / 16; ++kk) {
+#pragma unroll
+                            for (int j = 0; j < J; ++j)      // (chunk j's columns: nc / 2 rows of 128 bytes further on)
+                                umma_bf16_pair(tmem_base + acc[j] * slot_cols, a_desc + 2 * kk, b_desc + j * (nc * 4) + 2 * kk, idesc,
+                                               (kb | kk) != 0);
+                        }
                         umma_commit_pair(&bars->empty[stage], 3);      // frees the stage in both CTAs
                     }
                     __syncwarp();
                     if (++stage == n_stages) { stage = 0; phase ^= 1; }
                 }
-                if (ok && leader) umma_commit_pair(&bars->tmem_full[acc], 3);
+                if (ok && leader) {
+#pragma unroll
+                    for (int j = 0; j < J; ++j) umma_commit_pair(&bars->tmem_full[acc[j]], 3);
+                }
                 __syncwarp();
             }
         }
@@ -824,25 +861,25 @@ lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, 
         // epilogue: warp w may touch TMEM lanes [32 * (w % 4), +32) = 32 consecutive vocabulary entries of the tile
         const int lq = warp & 3;
         float* xp = xpose + lq * SW_XP_FLOATS;
-        float* st = state + lq * SW_STATE_FLOATS;
+        float* st = state + lq * WARP_STATE;
         const uint32_t rng_step = SAMPLE ? smp.step + (smp.step_dev ? *smp.step_dev : 0u) : 0u;
         int it = 0;
         uint32_t items_done = 0;
         bool ok = true;
         for (int item = unit; item < n_items && ok; item += n_units, ++items_done) {
-            const int chunk = item % plan.n_chunks;
-            const int group = item / plan.n_chunks;
+            const int group = item / item_chunks;
             float run_max[SW_NMAX / 32], run_sum[SW_NMAX / 32];
             int run_arg[SW_NMAX / 32];
 #pragma unroll
             for (int cb = 0; cb < SW_NMAX / 32; ++cb) { run_max[cb] = -INFINITY; run_sum[cb] = 0.f; run_arg[cb] = ARG_NONE; }
-            for (int vt = group; vt < n_vt && ok; vt += groups, ++it) {
-                const int acc = it & 1;
-                const uint32_t acc_phase = (it >> 1) & 1;
+            for (int vj = group * J; vj < n_vt * J && ok; vj += (JOINT && !(vj & 1)) ? 1 : groups * J - (J - 1), ++it) {
+                const int vt = vj / J, j = vj % J;           // vocabulary tile and chunk
+                const int acc = it % slots;
+                const uint32_t acc_phase = (it / slots) & 1;
                 ok = __all_sync(0xffffffffu, mbar_wait(&bars->tmem_full[acc], acc_phase, abort_flag));
                 if (!ok) break;
                 tc_fence_after_sync();
-                const uint32_t taddr = tmem_base + (static_cast<uint32_t>(lq * 32) << 16) + acc * SW_NMAX;
+                const uint32_t taddr = tmem_base + (static_cast<uint32_t>(lq * 32) << 16) + acc * slot_cols;
                 const int vbase = vt * (2 * SW_BV) + rank * SW_BV + lq * 32;     // first vocabulary entry of this warp's lanes
                 const bool edge = (vbase + 32 > V) || (mask_col >= vbase && mask_col < vbase + 32);
                 // column block cb: turned, so that this thread holds 32 consecutive vocabulary entries of one row; returns
@@ -891,22 +928,34 @@ lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, 
                         int carg;
                         load_block(cb, z, cmax, carg);
                         const int r = cb * 32 + lane;
-                        const int row = chunk * nc + r;
+                        const int row = row_of(item, 0, r);
                         const uint32_t rng_row = static_cast<uint32_t>(r < nc && row < Mc && smp.row_index ? smp.row_index[row] : row);
-                        float rmax = st[r], rsum = st[SW_NMAX + r];
-                        SampleBest best = {st[2 * SW_NMAX + r], st[3 * SW_NMAX + r], __float_as_int(st[4 * SW_NMAX + r])};
+                        float rmax = st[r], rsum = st[NS + r];
+                        SampleBest best = {st[2 * NS + r], st[3 * NS + r], __float_as_int(st[4 * NS + r])};
                         int ignored = 0;
                         add_block(z, cmax, carg, rmax, rsum, ignored);
                         float bound = -INFINITY;          // what the other warps have seen of this row (any time up to now will do)
 #pragma unroll
                         for (int q = 0; q < 4; ++q)
-                            bound = fmaxf(bound, *static_cast<volatile float*>(state + q * SW_STATE_FLOATS + 2 * SW_NMAX + r));
+                            bound = fmaxf(bound, *static_cast<volatile float*>(state + q * WARP_STATE + 2 * NS + r));
                         const SampleKey key = {rng_row, rng_step, smp.seed_lo, smp.seed_hi, smp.inv_temperature};
                         const auto at = [&](int j) { return vbase + j >= V || vbase + j == mask_col ? -INFINITY : xp[j * 33 + lane]; };
                         sample_chunk(z, vbase, cmax, carg, bound, key, best, at);
                         __syncwarp();                     // the block may be overwritten
-                        st[r] = rmax; st[SW_NMAX + r] = rsum;
-                        st[2 * SW_NMAX + r] = best.y; st[3 * SW_NMAX + r] = best.z; st[4 * SW_NMAX + r] = __int_as_float(best.arg);
+                        st[r] = rmax; st[NS + r] = rsum;
+                        st[2 * NS + r] = best.y; st[3 * NS + r] = best.z; st[4 * NS + r] = __int_as_float(best.arg);
+                    }
+                } else if (STATE) {
+#pragma unroll 2
+                    for (int cb = 0; vbase < V && cb * 32 < nc; ++cb) {
+                        float z[32], cmax;
+                        int carg;
+                        load_block(cb, z, cmax, carg);
+                        float* s = st + j * SW_NMAX + cb * 32 + lane;
+                        float rmax = s[0], rsum = s[NS];
+                        int rarg = __float_as_int(s[2 * NS]);
+                        add_block(z, cmax, carg, rmax, rsum, rarg);
+                        s[0] = rmax; s[NS] = rsum; s[2 * NS] = __int_as_float(rarg);
                     }
                 } else if (vbase < V) {
 #pragma unroll
@@ -926,7 +975,7 @@ lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, 
             if (ok) {
                 // fold the four warps' values (each saw a quarter of every tile's vocabulary entries): every warp
                 // leaves its own in its block of shared memory, then warp q folds column blocks 2 q and 2 q + 1
-                if (!SAMPLE) {
+                if (!STATE) {
 #pragma unroll
                     for (int cb = 0; cb < SW_NMAX / 32; ++cb) {
                         xp[(cb * 3 + 0) * 32 + lane] = run_max[cb];
@@ -937,23 +986,23 @@ lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, 
                 mbar_arrive(&bars->fold_full);            // (release: the values above are visible to the waiters)
                 ok = __all_sync(0xffffffffu, mbar_wait(&bars->fold_full, items_done & 1, abort_flag));
                 if (ok) {
-                    for (int cb = 2 * lq; cb < 2 * lq + 2; ++cb) {
-                        const int col = cb * 32 + lane;
-                        const int row = chunk * nc + col;
+                    for (int cb = 2 * J * lq; cb < 2 * J * (lq + 1); ++cb) {
+                        const int j = cb / (SW_NMAX / 32), col = cb % (SW_NMAX / 32) * 32 + lane, r = cb * 32 + lane;
+                        const int row = row_of(item, j, col);
                         if (col < nc && row < Mc) {
                             float m = -INFINITY, sum = 0.f;
                             int a = ARG_NONE;
                             if (SAMPLE) {
                                 SampleBest best = {-INFINITY, -INFINITY, ARG_NONE};
                                 for (int q = 0; q < 4; ++q) {
-                                    const float* src = state + q * SW_STATE_FLOATS + col;
-                                    const float m2 = src[0], s2 = src[SW_NMAX], y2 = src[2 * SW_NMAX];
-                                    const int a2 = __float_as_int(src[4 * SW_NMAX]);
+                                    const float* src = state + q * WARP_STATE + r;
+                                    const float m2 = src[0], s2 = src[NS], y2 = src[2 * NS];
+                                    const int a2 = __float_as_int(src[4 * NS]);
                                     if (m2 > -INFINITY) {
                                         if (m2 > m) { sum = sum * fast_exp2((m - m2) * LOG2E) + s2; m = m2; }
                                         else sum += s2 * fast_exp2((m2 - m) * LOG2E);
                                     }
-                                    if (y2 > best.y || (y2 == best.y && a2 < best.arg)) best = {y2, src[3 * SW_NMAX], a2};
+                                    if (y2 > best.y || (y2 == best.y && a2 < best.arg)) best = {y2, src[3 * NS], a2};
                                 }
                                 const size_t o = static_cast<size_t>(row) * parts_stride + group * 2 + rank;
                                 smp.part_y[o] = best.y;
@@ -961,9 +1010,9 @@ lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, 
                                 a = best.arg;
                             }
                             for (int q = 0; q < (SAMPLE ? 0 : 4); ++q) {
-                                const float* src = xpose + q * SW_XP_FLOATS + cb * 96 + lane;
-                                const float m2 = src[0], s2 = src[32];
-                                const int a2 = __float_as_int(src[64]);
+                                const float* src = STATE ? state + q * WARP_STATE + r : xpose + q * SW_XP_FLOATS + cb * 96 + lane;
+                                const float m2 = src[0], s2 = src[STATE ? NS : 32];
+                                const int a2 = __float_as_int(src[STATE ? 2 * NS : 64]);
                                 if (m2 > -INFINITY) {
                                     if (m2 > m) { sum = sum * fast_exp2((m - m2) * LOG2E) + s2; m = m2; a = a2; }
                                     else { sum += s2 * fast_exp2((m2 - m) * LOG2E); if (m2 == m && a2 < a) a = a2; }
@@ -974,8 +1023,8 @@ lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, 
                             part_sum[o] = sum;
                             part_arg[o] = a;
                         }
-                        if (SAMPLE)
-                            for (int q = 0; q < 4; ++q) clear_state(q, col);
+                        if (STATE)
+                            for (int q = 0; q < 4; ++q) clear_state(q, r);
                     }
                     mbar_arrive(&bars->fold_empty);       // the blocks may be written again once all have read
                     ok = __all_sync(0xffffffffu, mbar_wait(&bars->fold_empty, items_done & 1, abort_flag));
@@ -1013,7 +1062,7 @@ __host__ __device__ inline int lm_mixed_pair_clusters(int n_clusters, int p) {
 }
 
 // The greedy (or sampled) head, one launch on CTA pairs whatever the number of live rows (known only on the device when rows are
-// skipped): the swapped-operand path for the counts lm_greedy_swapped names (up to SW_NMAX rows, and counts that
+// skipped): the swapped-operand path for the counts lm_swapped names (up to SW_NMAX rows, and counts that
 // cut into long chunks); otherwise row-major tiles of 128 rows, on CTA pairs when the tiles come in twos, and for
 // an odd count on pairs plus single CTAs for the last tile (see above).  The W
 // tile box is 128 rows for all of them.  A row's partials start at row * parts_stride; how many there are follows
@@ -1032,9 +1081,16 @@ lmhead_head_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
         if (!__syncthreads_or(any)) return;              // (every CTA alike)
     }
     const int Mc = live_rows ? *live_rows : M;          // rows that need logits (uniform over the grid)
-    if (lm_greedy_swapped(Mc)) {
-        lm_swapped_body<MODE>(tmap_w, xmaps, Mc, D, V, mask_col, n_tiles, part_max, part_sum, part_arg, dev_status, parts_stride,
-                              smp);
+    if constexpr (MODE == LM_GREEDY) {
+        if (lm_joint(Mc, false)) {
+            lm_swapped_body<MODE, true>(tmap_w, xmaps, Mc, D, V, mask_col, n_tiles, part_max, part_sum, part_arg, dev_status,
+                                        parts_stride, smp);
+            return;
+        }
+    }
+    if (lm_swapped(Mc, MODE == LM_SAMPLE)) {
+        lm_swapped_body<MODE, false>(tmap_w, xmaps, Mc, D, V, mask_col, n_tiles, part_max, part_sum, part_arg, dev_status,
+                                     parts_stride, smp);
         return;
     }
     const int m_tiles = (Mc + BM - 1) / BM;
@@ -1068,11 +1124,11 @@ lmhead_head_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
 // packed (stride = count).  layout 2: lmhead_head_kernel's rules.  `grid` = CTAs of the GEMM launch, n_tiles =
 // vocabulary tiles of 256.
 constexpr int LM_LAYOUT_GREEDY = 2;
-__host__ __device__ inline int lm_row_partials(int layout, int grid, int rows, int n_tiles, int row) {
+__host__ __device__ inline int lm_row_partials(int layout, int grid, int rows, int n_tiles, int row, bool sampled) {
     const int m_tiles = (rows + BM - 1) / BM;
     if (layout != LM_LAYOUT_GREEDY) return lm_groups_mode(grid, m_tiles, n_tiles, layout);
     const int n_clusters = grid >> 1;
-    if (lm_greedy_swapped(rows)) return sw_plan(rows, n_clusters, n_tiles).parts;
+    if (lm_swapped(rows, sampled)) return sw_plan(rows, n_clusters, n_tiles, sampled).parts;
     if ((m_tiles & 1) == 0) return lm_groups(n_clusters, m_tiles >> 1, n_tiles);
     if (n_clusters < 2) return lm_groups(grid, m_tiles, n_tiles);
     const int p = m_tiles >> 1;
@@ -1147,7 +1203,7 @@ __global__ void lmhead_merge_kernel(const LmParts parts, int grid_gemm, int n_ti
             return;
         }
     }
-    const int groups = lm_row_partials(allow_pair, grid_gemm, Mc, n_tiles, c);
+    const int groups = lm_row_partials(allow_pair, grid_gemm, Mc, n_tiles, c, SAMPLE);
     int a;
     float cf;
     merge_row_partials<SAMPLE>(parts, static_cast<size_t>(c) * (parts_stride < 0 ? groups : parts_stride), groups, lane, a, cf);
@@ -1208,7 +1264,7 @@ lmhead_merge_select_kernel(const LmParts parts, int grid_gemm, int n_tiles, int 
             c = before;
             for (int i = 0; i < warp; ++i) c += s_flag[i];
         }
-        const int groups = lm_row_partials(allow_pair, grid_gemm, Mc, n_tiles, c);
+        const int groups = lm_row_partials(allow_pair, grid_gemm, Mc, n_tiles, c, SAMPLE);
         int a;
         float cf;
         merge_row_partials<SAMPLE>(parts, static_cast<size_t>(c) * (parts_stride < 0 ? groups : parts_stride), groups, lane, a, cf);
@@ -1395,8 +1451,8 @@ static int launch_head(const dare_ctx* ctx, int grid, bool pairs, const void* x_
         if (rc != DARE_OK) return rc;
         grid_gemm = grid & ~1;
         parts_stride = static_cast<int>(parts_max);
-        constexpr int SMEM_A = sw_smem_bytes(MODE) > LM_PAIR_SMEM_BYTES ? sw_smem_bytes(MODE) : LM_PAIR_SMEM_BYTES;
-        constexpr int SMEM = SMEM_A > LM_SMEM_BYTES ? SMEM_A : LM_SMEM_BYTES;
+        constexpr int SMEM = SW_SMEM_BYTES;
+        static_assert(SMEM >= LM_PAIR_SMEM_BYTES && SMEM >= LM_SMEM_BYTES, "shared memory");
         static std::atomic<uint64_t> smem_set{0};
         if (ensure_dynamic_smem(smem_set, lmhead_head_kernel<MODE>, SMEM) != DARE_OK) return DARE_ERR_CUDA;
         rc = launch_kernel(lmhead_head_kernel<MODE>, dim3(static_cast<unsigned>(grid_gemm)), LM_THREADS, SMEM, stream, 2, tmap_w,

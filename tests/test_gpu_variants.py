@@ -278,3 +278,22 @@ def test_dual_loop_equals_its_parts(ctx, k, mode):
     steps = dare.dare_generate_dual(model, tok2, P, G, L, kc2, vc2, mode, 0.9, k, pred, conf, nr)
     assert steps == want
     assert torch.equal(tok2, tok) and torch.equal(kc2, kc) and torch.equal(vc2, vc)
+
+
+# 257 to 384 rows: two chunks of rows against each vocabulary tile.  The range's edges, chunk widths with three and with two
+# accumulators, tiles of fewer than 256 entries, fewer tiles than CTA pairs and enough for every accumulator to come round.
+@pytest.mark.parametrize("M", [256, 257, 288, 289, 320, 321, 352, 383, 384, 385])
+@pytest.mark.parametrize("V", [100, 1300, 100_000])
+def test_greedy_head_on_two_chunks(ctx, M, V):
+    D, mu = 72, V - 3
+    x, w = I.normal_bf16(M, I.TID_X, (M, D)).cuda(), I.normal_bf16(V, I.TID_W, (V, D), 0.2).cuda()
+    pred, conf = dare.dare_lmhead_confidence(ctx, x, w, None, mu, True)
+    torch.cuda.synchronize()
+    z = x.double() @ w.double().T
+    z[:, mu] = -float("inf")
+    best = z.max(1).values
+    # an fp32 logit of 72 products is off by up to 72 * 2^-24 * sum |x w| (about 10): 5e-5; the exponentials by less
+    assert (best - z.gather(1, pred.long()[:, None])[:, 0] <= 1e-4).all()
+    want = torch.exp(best - torch.logsumexp(z, 1))
+    assert torch.allclose(conf.double(), want, rtol=2e-4, atol=0)
+    assert ctx.device_status() == 0
