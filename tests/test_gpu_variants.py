@@ -297,3 +297,29 @@ def test_greedy_head_on_two_chunks(ctx, M, V):
     want = torch.exp(best - torch.logsumexp(z, 1))
     assert torch.allclose(conf.double(), want, rtol=2e-4, atol=0)
     assert ctx.device_status() == 0
+
+
+# The rotary kernel on its own: heads that leave the last batch of a thread part full, more heads than one pass takes, and
+# fewer than the threads of a CTA.
+@pytest.mark.parametrize("Hq,Hkv,d", [(1, 1, 64), (72, 24, 128), (65, 13, 64), (33, 33, 128), (31, 31, 64)])
+def test_rope_kernel_head_counts(ctx, Hq, Hkv, d):
+    B, length, start, cap = 2, 3, 5, 11
+    model = _small_model(ctx, Hq, Hkv, d, B * length, B, cap, hidden=64, ffn=64)
+    x = I.normal_bf16(Hq, 3, (B, length, Hq + 2 * Hkv, d)).cuda()
+    q = torch.empty(B, length, Hq, d, dtype=torch.bfloat16, device="cuda")
+    kc, vc = (torch.zeros(1, B, Hkv, cap, d, dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    dare.dare_rope_kv_write(model, x.view(B * length, -1), B, length, start, q, kc, vc)
+    torch.cuda.synchronize()
+    pos = torch.arange(start, start + length, dtype=torch.float64, device="cuda")
+    ang = pos[:, None] * 10000.0 ** (-2.0 * torch.arange(d // 2, dtype=torch.float64, device="cuda") / d)
+    c, s = ang.cos()[None, :, None], ang.sin()[None, :, None]
+    r = x[:, :, :Hq + Hkv].double()
+    lo, hi = r[..., :d // 2], r[..., d // 2:]
+    want = torch.cat([lo * c - hi * s, hi * c + lo * s], -1)
+    bound = (2.0 ** -8 * want.abs() + 2.0 ** -21 * torch.cat([lo.abs() + hi.abs()] * 2, -1))     # bf16 rounding; fp32 inside
+    rows = slice(start, start + length)
+    assert ((q.double() - want[:, :, :Hq]).abs() <= bound[:, :, :Hq]).all()
+    assert ((kc[0, :, :, rows].transpose(1, 2).double() - want[:, :, Hq:]).abs() <= bound[:, :, Hq:]).all()
+    assert torch.equal(vc[0, :, :, rows].transpose(1, 2), x[:, :, Hq + Hkv:])
+    assert kc[0, :, :, :start].count_nonzero() == 0 and vc[0, :, :, start + length:].count_nonzero() == 0
+    model.close()
