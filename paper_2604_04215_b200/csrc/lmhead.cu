@@ -621,7 +621,8 @@ constexpr int SW_NMAX = 256;                             // rows (accumulator co
 // D = 3584, V = 152064: 704 rows 625 / 650, 832 rows 784 / 840, 960 rows 851 / 895).
 // Both chunks at a time against row-major tiles (256 + 128 rows), under the power cap, us, D = 4096, V = 126464: 272 rows
 // 298 / 404, 320 rows 320 / 411, 352 rows 367 / 415, 384 rows 394 / 425; as a step at D = 3584, V = 152064: 352 rows
-// 415 / 422, 384 rows 441 / 422, so the line is drawn at 352.  The sampled head's epilogue is several times as long and may not be waited for: 320 rows 457 / 383.
+// 415 / 422, 384 rows 441 / 422, so the line is drawn at 352.  The sampled head's epilogue is several times as long and may
+// not be waited for: 320 rows 457 / 383.
 constexpr int LM_JOINT_ROWS = 352;
 __host__ __device__ inline bool lm_joint(int rows, bool sampled) { return !sampled && rows > SW_NMAX && rows <= LM_JOINT_ROWS; }
 __host__ __device__ inline bool lm_swapped(int rows, bool sampled) {
