@@ -615,18 +615,19 @@ lmhead_partial_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
 constexpr int SW_BV = 128;                               // vocabulary rows per CTA and tile
 constexpr int SW_NMAX = 256;                             // rows (accumulator columns) per chunk
 // Row counts for which a head takes this path: up to one chunk, where W is streamed once and the launch is bound by HBM;
-// up to LM_JOINT_ROWS with both chunks at a time (greedy only); and, up to 1024 rows, counts that cut into chunks of 208
-// to 240 rows, i.e. whose row-major tiles would carry 64 or more padded rows per pair (swapped against row-major, one
-// chunk at a time, us: D = 4096, V = 126464: 416 rows 333 / 380, 448 rows 415 / 462, 480 rows 410 / 428, 512 rows 425 / 421;
-// D = 3584, V = 152064: 704 rows 625 / 650, 832 rows 784 / 840, 960 rows 851 / 895).
-// Both chunks at a time against row-major tiles (256 + 128 rows), under the power cap, us, D = 4096, V = 126464: 272 rows
-// 298 / 404, 320 rows 320 / 411, 352 rows 367 / 415, 384 rows 394 / 425; as a step at D = 3584, V = 152064: 352 rows
-// 415 / 422, 384 rows 441 / 422, so the line is drawn at 352.  The sampled head's epilogue is several times as long and may
-// not be waited for: 320 rows 457 / 383.
+// two chunks of up to 192 rows, whose row-major tiles would be 384 padded rows; and, up to 1024 rows, counts that cut into
+// chunks of 208 to 240 rows, i.e. whose row-major tiles would carry 64 or more padded rows per pair (swapped against
+// row-major, one chunk at a time, us: D = 4096, V = 126464: 416 rows 333 / 380, 448 rows 415 / 462, 480 rows 410 / 428, 512 rows
+// 425 / 421; D = 3584, V = 152064: 704 rows 625 / 650, 832 rows 784 / 840, 960 rows 851 / 895).
+// Two chunks of up to 192 rows, D = 4096, V = 126464, us under the power cap, where padded MMAs cost twice: greedy, both
+// chunks at a time / row-major: 272 rows 298 / 404, 320 rows 320 / 411, 352 rows 367 / 415, 384 rows 394 / 425; one chunk at a time:
+// 368 rows 383 / 422, 384 rows 386 / 421.  Sampled, one at a time (its epilogue is several times as long and may not be waited
+// for: 457 both at a time at 320 rows): 272 rows 382 / 414, 320 rows 392 / 423, 384 rows 433 / 433.
 constexpr int LM_JOINT_ROWS = 352;
+constexpr int LM_SWAPPED_ROWS = 384;
 __host__ __device__ inline bool lm_joint(int rows, bool sampled) { return !sampled && rows > SW_NMAX && rows <= LM_JOINT_ROWS; }
 __host__ __device__ inline bool lm_swapped(int rows, bool sampled) {
-    if (rows <= SW_NMAX || lm_joint(rows, sampled)) return true;
+    if (rows <= LM_SWAPPED_ROWS) return true;
     if (rows > 1024) return false;
     const int n_chunks = (rows + SW_NMAX - 1) / SW_NMAX;
     const int nc = ((rows + n_chunks - 1) / n_chunks + 15) & ~15;      // as in sw_plan below
