@@ -601,9 +601,9 @@ lmhead_partial_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
 //   * items = chunk x vocabulary group: a chunk streams all of W from L2 into the SMs whatever its N, and that stream
 //     (~12 TB/s over the GPU), not the tensor pipe, sets the pace when the chunks are short (an MMA alone takes
 //     max(N / 2, ~45) cycles): only chunks close to 256 rows are worth it;
-//   * both chunks against each W tile (JOINT): W enters the SMs once.  The price is the accumulators: two chunks take half
-//     of TMEM or more, so the next tile's MMAs wait for part of this one's epilogue (three of up to 160 columns fit: for
-//     half of it), and the running values of 512 columns move to shared memory.
+//   * both chunks against each W tile (JOINT): W enters the SMs once.  The price is the accumulators: three of 160 columns
+//     fit, so the next tile's MMAs wait for half of this one's epilogue, and the running values of 320 columns move to
+//     shared memory.
 // The price is the epilogue: a thread's TMEM lane is now a vocabulary entry and the softmax runs ACROSS lanes.
 // Each epilogue warp turns its 32 x 32 block of logits through shared memory (padded rows, conflict-free) so that
 // a thread again holds 32 consecutive vocabulary entries of ONE row, and keeps that row's running
@@ -620,10 +620,11 @@ constexpr int SW_NMAX = 256;                             // rows (accumulator co
 // row-major, one chunk at a time, us: D = 4096, V = 126464: 416 rows 333 / 380, 448 rows 415 / 462, 480 rows 410 / 428, 512 rows
 // 425 / 421; D = 3584, V = 152064: 704 rows 625 / 650, 832 rows 784 / 840, 960 rows 851 / 895).
 // Two chunks of up to 192 rows, D = 4096, V = 126464, us under the power cap, where padded MMAs cost twice: greedy, both
-// chunks at a time / row-major: 272 rows 298 / 404, 320 rows 320 / 411, 352 rows 367 / 415, 384 rows 394 / 425; one chunk at a time:
-// 368 rows 383 / 422, 384 rows 386 / 421.  Sampled, one at a time (its epilogue is several times as long and may not be waited
-// for: 457 both at a time at 320 rows): 272 rows 382 / 414, 320 rows 392 / 423, 384 rows 433 / 433.
-constexpr int LM_JOINT_ROWS = 352;
+// chunks at a time / row-major: 272 rows 298 / 404, 320 rows 320 / 411; above, where two accumulators are all that fit, one chunk at
+// a time: 368 rows 383 / 422, 384 rows 386 / 421 (both at a time: 394; D = 3584, V = 152064, from idle, 352 rows 389 / 370).
+// Sampled, one at a time (its epilogue is several times as long and may not be waited for: 457 both at a time at 320
+// rows): 272 rows 382 / 414, 320 rows 392 / 423, 384 rows 433 / 433.
+constexpr int LM_JOINT_ROWS = 320;
 constexpr int LM_SWAPPED_ROWS = 384;
 __host__ __device__ inline bool lm_joint(int rows, bool sampled) { return !sampled && rows > SW_NMAX && rows <= LM_JOINT_ROWS; }
 __host__ __device__ inline bool lm_swapped(int rows, bool sampled) {
@@ -727,8 +728,8 @@ lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, 
     if (unit >= n_items) return;                         // (both CTAs of a pair alike)
     const int nc = plan.nc, groups = plan.groups;
     const int rows_half = J * (nc >> 1);                 // rows this CTA loads (a multiple of 8 per chunk), consecutive ones
-    // accumulators: a ring of two, or, where three fit, three
-    const int slots = JOINT && nc <= 160 ? 3 : 2, slot_cols = JOINT && nc <= 160 ? 160 : SW_NMAX;
+    constexpr int slots = JOINT ? 3 : 2, slot_cols = JOINT ? LM_JOINT_ROWS / 2 : SW_NMAX;      // ring of accumulators
+    static_assert(slots * slot_cols <= static_cast<int>(TMEM_COLS), "accumulators");
     // row of column c of the item's chunk j: the even CTA's rows are the columns below nc / 2
     const auto row_of = [&](int item, int j, int c) {
         return JOINT ? (c < (nc >> 1) ? c : c + (nc >> 1)) + j * (nc >> 1) : (item % item_chunks) * nc + c;

@@ -280,8 +280,8 @@ def test_dual_loop_equals_its_parts(ctx, k, mode):
     assert torch.equal(tok2, tok) and torch.equal(kc2, kc) and torch.equal(vc2, vc)
 
 
-# 257 to 352 rows: two chunks of rows against each vocabulary tile.  The range's edges, chunk widths with three and with two
-# accumulators, tiles of fewer than 256 entries, fewer tiles than CTA pairs and enough for every accumulator to come round.
+# 257 to 320 rows: two chunks of rows against each vocabulary tile; up to 384: one after the other.  The
+# ranges' edges, tiles of fewer than 256 entries, fewer tiles than CTA pairs and enough for every accumulator to come round.
 @pytest.mark.parametrize("M", [256, 257, 288, 289, 320, 321, 335, 352, 353, 384, 385])
 @pytest.mark.parametrize("V", [100, 1300, 100_000])
 def test_greedy_head_on_two_chunks(ctx, M, V):
