@@ -4,7 +4,8 @@
 // 155 us with ctypes, 104 us with this.
 //
 // Each function returns the entry point's status, or None when an argument is not what it should be: the caller then
-// goes through the checks of binding.py, which say what is wrong.
+// goes through the checks of binding.py, which say what is wrong.  A tensor without memory of its own (a FakeTensor of a
+// trace, the batched tensor of vmap) throws where it is asked for its address: that is caught, and None as well.
 #include <Python.h>
 #include <dlfcn.h>
 #include <torch/csrc/autograd/python_variable.h>
@@ -81,7 +82,7 @@ struct Args {
 // (handle, device, stream, scale, q, k_pre, v_pre, prefix_len, k_blk, v_blk, k_suf, v_suf, suffix_len, attn_out, lse, hidden, w,
 //  mask_id, exclude, [temperature, seed, step,] tokens, block_start, mode, threshold, k, pred, conf, n_committed, n_remaining)
 template <bool SAMPLED>
-PyObject* denoise(PyObject*, PyObject* const* argv, Py_ssize_t n) {
+PyObject* denoise_checked(PyObject* const* argv, Py_ssize_t n) {
     Args a{argv, n};
     dare_ctx* ctx = static_cast<dare_ctx*>(a.address());
     a.device = static_cast<long>(a.integer());
@@ -118,27 +119,28 @@ PyObject* denoise(PyObject*, PyObject* const* argv, Py_ssize_t n) {
     const int B = static_cast<int>(q->size(0)), L = static_cast<int>(q->size(1)), Hq = static_cast<int>(q->size(2));
     const int d = static_cast<int>(q->size(3)), Hkv = static_cast<int>(k_pre->size(1));
     const int prefix_cap = static_cast<int>(k_pre->size(2)), suffix_cap = k_suf ? static_cast<int>(k_suf->size(2)) : 0;
-    void* suf = k_suf ? k_suf->data_ptr() : nullptr;
+    // (everything that may throw stands in front of the part without the interpreter's lock)
+    const void *q_ptr = q->data_ptr(), *k_ptr = k_pre->data_ptr(), *suf = k_suf ? k_suf->data_ptr() : nullptr;
+    const void *x_ptr = hidden->data_ptr(), *w_ptr = w->data_ptr();
+    const int D = static_cast<int>(hidden->size(1)), V = static_cast<int>(w->size(0));
     int32_t* tok = static_cast<int32_t*>(tokens->data_ptr());
+    const int64_t row_stride = tokens->size(1);
     int rc;
     Py_BEGIN_ALLOW_THREADS;
     if (SAMPLED)
-        rc = f_denoise_sampled(ctx, B, L, Hq, Hkv, d, prefix_cap, suffix_cap, scale, q->data_ptr(), k_pre->data_ptr(), v_pre,
-                               prefix_len, k_blk, v_blk, suf, v_suf, suffix_len, out, lse, hidden->data_ptr(),
-                               static_cast<int>(hidden->size(1)), w->data_ptr(), static_cast<int>(w->size(0)), mask_id, exclude,
-                               temperature, seed, step, tok, tokens->size(1), block_start, mode, threshold, k, pred, conf,
-                               n_committed, n_remaining, stream);
+        rc = f_denoise_sampled(ctx, B, L, Hq, Hkv, d, prefix_cap, suffix_cap, scale, q_ptr, k_ptr, v_pre, prefix_len, k_blk, v_blk,
+                               suf, v_suf, suffix_len, out, lse, x_ptr, D, w_ptr, V, mask_id, exclude, temperature, seed, step, tok,
+                               row_stride, block_start, mode, threshold, k, pred, conf, n_committed, n_remaining, stream);
     else
-        rc = f_denoise(ctx, B, L, Hq, Hkv, d, prefix_cap, suffix_cap, scale, q->data_ptr(), k_pre->data_ptr(), v_pre, prefix_len,
-                       k_blk, v_blk, suf, v_suf, suffix_len, out, lse, hidden->data_ptr(), static_cast<int>(hidden->size(1)),
-                       w->data_ptr(), static_cast<int>(w->size(0)), mask_id, exclude, tok, tokens->size(1), block_start, mode,
+        rc = f_denoise(ctx, B, L, Hq, Hkv, d, prefix_cap, suffix_cap, scale, q_ptr, k_ptr, v_pre, prefix_len, k_blk, v_blk, suf,
+                       v_suf, suffix_len, out, lse, x_ptr, D, w_ptr, V, mask_id, exclude, tok, row_stride, block_start, mode,
                        threshold, k, pred, conf, n_committed, n_remaining, stream);
     Py_END_ALLOW_THREADS;
     return PyLong_FromLong(rc);
 }
 
 // (handle, device, stream, scale, q, k, v, cu_seqlens, max_seqlen, out, lse)
-PyObject* varlen(PyObject*, PyObject* const* argv, Py_ssize_t n) {
+PyObject* varlen_checked(PyObject* const* argv, Py_ssize_t n) {
     Args a{argv, n};
     dare_ctx* ctx = static_cast<dare_ctx*>(a.address());
     a.device = static_cast<long>(a.integer());
@@ -151,13 +153,25 @@ PyObject* varlen(PyObject*, PyObject* const* argv, Py_ssize_t n) {
     void* out = a.bf16();
     float* lse = a.f32();
     if (!a.ok || a.at != n || !q || !k || !cu || q->dim() != 3 || k->dim() < 2) Py_RETURN_NONE;
+    const int total = static_cast<int>(q->size(0)), Hq = static_cast<int>(q->size(1)), d = static_cast<int>(q->size(2));
+    const int Hkv = static_cast<int>(k->size(1)), n_seqs = static_cast<int>(cu->numel()) - 1;
+    const void *q_ptr = q->data_ptr(), *k_ptr = k->data_ptr();
+    const int32_t* cu_ptr = static_cast<const int32_t*>(cu->data_ptr());
     int rc;
     Py_BEGIN_ALLOW_THREADS;
-    rc = f_varlen(ctx, static_cast<int>(q->size(0)), static_cast<int>(cu->numel()) - 1, max_seqlen, static_cast<int>(q->size(1)),
-                  static_cast<int>(k->size(1)), static_cast<int>(q->size(2)), scale, q->data_ptr(), k->data_ptr(), v,
-                  static_cast<const int32_t*>(cu->data_ptr()), out, lse, stream);
+    rc = f_varlen(ctx, total, n_seqs, max_seqlen, Hq, Hkv, d, scale, q_ptr, k_ptr, v, cu_ptr, out, lse, stream);
     Py_END_ALLOW_THREADS;
     return PyLong_FromLong(rc);
+}
+
+template <PyObject* (*CALL)(PyObject* const*, Py_ssize_t)>
+PyObject* entry(PyObject*, PyObject* const* argv, Py_ssize_t n) {
+    try {
+        return CALL(argv, n);
+    } catch (...) {      // (none comes from the library: its entry points do not throw)
+        PyErr_Clear();
+        Py_RETURN_NONE;
+    }
 }
 
 // bind(path of libdare.so): resolves the entry points in the library that binding.py has loaded
@@ -179,9 +193,9 @@ PyObject* bind(PyObject*, PyObject* arg) {
 
 PyMethodDef methods[] = {
     {"bind", bind, METH_O, nullptr},
-    {"denoise_block", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(&denoise<false>)), METH_FASTCALL, nullptr},
-    {"denoise_block_sampled", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(&denoise<true>)), METH_FASTCALL, nullptr},
-    {"attn_varlen", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(&varlen)), METH_FASTCALL, nullptr},
+    {"denoise_block", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(&entry<denoise_checked<false>>)), METH_FASTCALL, nullptr},
+    {"denoise_block_sampled", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(&entry<denoise_checked<true>>)), METH_FASTCALL, nullptr},
+    {"attn_varlen", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(&entry<varlen_checked>)), METH_FASTCALL, nullptr},
     {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_marshal", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 

@@ -1,4 +1,8 @@
 """The native marshalling of the inner loop's calls leaves every argument that does not fit to the Python checks."""
+import os
+import subprocess
+import sys
+
 import pytest
 import torch
 
@@ -26,6 +30,39 @@ def test_host_tensors_and_short_argument_lists_are_left_to_the_python_checks():
     assert m.denoise_block_sampled(0, 0, 0, 0.0, *_args("cpu").values()) is None          # three arguments short
     assert m.attn_varlen(0, 0, 0, 0.0) is None
     assert m.denoise_block(None, 0) is None
+
+
+BATCHED = """
+import torch
+from torch._subclasses import FakeTensorMode
+from paper_2604_04215_b200 import binding as dare
+m = dare._native()
+with FakeTensorMode():
+    q = torch.empty(3, 1, 8, 2, 64, dtype=torch.bfloat16, device="cuda:0")
+    x = torch.empty(3, 8, 16, dtype=torch.bfloat16, device="cuda:0")
+    i = torch.empty(2, dtype=torch.int32, device="cuda:0")
+    tok = torch.empty(1, 16, dtype=torch.int32, device="cuda:0")
+    k, w, f = q[0], x[0], torch.empty(8, device="cuda:0")
+    def varlen(a):
+        assert m.attn_varlen(0, 0, 0, 0.0, a[0], k[0], k[0], i, 8, k[0], None) is None
+        return a
+    def step(a, h):
+        for call, more in ((m.denoise_block, ()), (m.denoise_block_sampled, (1.0, 5, 2))):
+            for qq, hh in ((a, w), (k, h)):
+                assert call(0, 0, 0, 0.0, qq, k, k, None, None, None, None, None, None, k, None, hh, w, 3, True, *more, tok, 0, 0,
+                            0.5, 1, i, f, None, None) is None
+        return a
+    torch.vmap(varlen)(q)
+    torch.vmap(step)(q, x)
+print("all None")
+"""
+
+
+def test_tensors_without_memory_are_left_to_the_python_checks():
+    """Under vmap a tensor has no address: asking for it throws, which must not leave the C++ module (the process would end)."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", BATCHED], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "all None" in r.stdout, r.stderr[-2000:]
 
 
 @pytest.mark.gpu
