@@ -1,16 +1,21 @@
 """ctypes binding of libdare.so: argument marshalling only.
 
 The functions carry the names of the C entry points (include/dare.h).  Tensors are torch CUDA tensors
-used purely as device memory; every step runs inside the library's kernels.  There is no fallback: if
-the shared library is missing or a call fails, an exception is raised.
+used purely as device memory; every step runs inside the library's kernels.  There is no fallback for those: if
+the shared library is missing or a call fails, an exception is raised.  (Without the module that marshals the inner
+loop's calls in C++, ctypes marshals them: the same kernels, more host time.)
 """
 from __future__ import annotations
 
 import ctypes as C
+import importlib.util
 import os
+import warnings
 from typing import Optional
 
 import torch
+
+from . import build as _build
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libdare.so")
@@ -193,14 +198,31 @@ def _raw(stream, device: int) -> int:
     return _raw_stream(device) if _raw_stream is not None else torch.cuda.current_stream().cuda_stream
 
 
+class _NoNative:
+    """In the place of the marshalling module where that cannot be loaded: every call takes the Python path."""
+
+    @staticmethod
+    def _none(*args):
+        return None
+
+    denoise_block = denoise_block_sampled = attn_varlen = _none
+
+
 def _native():
     """The calls of a rollout's inner loop marshalled in C++ (csrc/marshal.cpp).  They return None where an argument is not
     what the entry point takes; the Python path behind each of them then says what is wrong."""
     global _marshal
     if _marshal is None:
         load()
-        from . import _marshal as m
-        m.bind(LIB_PATH)
+        try:
+            spec = importlib.util.spec_from_file_location(__package__ + "._marshal", _build.marshal_path())
+            m = importlib.util.module_from_spec(spec)
+            spec.loader.exec_module(m)
+            m.bind(LIB_PATH)
+        except (ImportError, OSError, RuntimeError) as e:
+            warnings.warn(f"no marshalling module for this Python and torch ({e}): the calls go through ctypes, which takes a "
+                          "few times as long on the host; `python -m paper_2604_04215_b200.build` builds it", RuntimeWarning)
+            m = _NoNative
         _marshal = m
     return _marshal
 

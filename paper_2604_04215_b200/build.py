@@ -4,7 +4,9 @@
 
 nvcc cross-compiles without a GPU.  The library links the static CUDA runtime and resolves the one driver
 entry point it needs (tensor-map encoding) at run time, so it has no link-time dependency on libcuda.
-_marshal.so beside it is the Python module through which binding.py makes the calls of a rollout's inner loop.
+The marshalling module beside it (marshal_path) is the Python module through which binding.py makes the calls of a
+rollout's inner loop.  It reads torch's tensor objects, so it holds for one Python and one torch: both stand in its name,
+and another torch neither loads it nor takes it for up to date.
 """
 from __future__ import annotations
 
@@ -18,8 +20,13 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libdare.so")
 SOURCES = ["api.cu", "lmhead.cu", "attn.cu", "select.cu", "gemm.cu", "gemm_few.cu", "layers.cu", "model.cu", "diffusion.cu", "backward.cu"]
-MARSHAL = os.path.join(HERE, "_marshal.so")
 HEADERS = ["ptx.cuh", "internal.h", os.path.join("..", "..", "include", "dare.h")]
+
+
+def marshal_path() -> str:
+    """Where the marshalling module for this Python and this torch is (or would be)."""
+    import torch
+    return os.path.join(HERE, f"_marshal-torch{torch.__version__}{sysconfig.get_config_var('EXT_SUFFIX')}")
 
 
 def _nvcc() -> str:
@@ -30,9 +37,10 @@ def _nvcc() -> str:
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB) or not os.path.exists(MARSHAL):
+    marshal = marshal_path()
+    if not os.path.exists(LIB) or not os.path.exists(marshal):
         return True
-    t = min(os.path.getmtime(LIB), os.path.getmtime(MARSHAL))
+    t = min(os.path.getmtime(LIB), os.path.getmtime(marshal))
     deps = [os.path.join(CSRC, s) for s in SOURCES + ["marshal.cpp"] + HEADERS] + [os.path.abspath(__file__)]
     return any(os.path.getmtime(d) > t for d in deps)
 
@@ -43,7 +51,7 @@ def _marshal_cmd() -> list:
     inc = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
            os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include"), sysconfig.get_paths()["include"]]
     return ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
-            *[f for d in inc for f in ("-isystem", d)], "-o", MARSHAL, os.path.join(CSRC, "marshal.cpp"),
+            *[f for d in inc for f in ("-isystem", d)], "-o", marshal_path(), os.path.join(CSRC, "marshal.cpp"),
             "-L" + os.path.join(root, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10", "-ldl"]
 
 
@@ -56,7 +64,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if verbose:
         cmd.insert(1, "-Xptxas")
         cmd.insert(2, "-v")
-    for what, c in (("libdare.so", cmd), ("_marshal.so", _marshal_cmd())):
+    for what, c in (("libdare.so", cmd), (os.path.basename(marshal_path()), _marshal_cmd())):
         res = subprocess.run(c, capture_output=True, text=True)
         if verbose or res.returncode != 0:
             sys.stderr.write(res.stdout + res.stderr)

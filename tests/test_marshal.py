@@ -2,6 +2,7 @@
 import os
 import subprocess
 import sys
+import sysconfig
 
 import pytest
 import torch
@@ -63,6 +64,20 @@ def test_tensors_without_memory_are_left_to_the_python_checks():
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     r = subprocess.run([sys.executable, "-c", BATCHED], cwd=root, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and "all None" in r.stdout, r.stderr[-2000:]
+
+
+def test_the_module_holds_for_one_python_and_one_torch(monkeypatch):
+    """With another torch the module that is there is neither up to date nor loaded; the calls then go through ctypes."""
+    from paper_2604_04215_b200 import build
+    here = build.marshal_path()
+    assert os.path.exists(here) and here.endswith(sysconfig.get_config_var("EXT_SUFFIX")) and torch.__version__ in here
+    monkeypatch.setattr(torch, "__version__", "0.0.0+other")
+    assert build._stale()
+    monkeypatch.setattr(dare, "_marshal", None)
+    with pytest.warns(RuntimeWarning, match="marshalling module"):
+        m = dare._native()
+    assert dare._native() is m                                        # (said once)
+    assert m.denoise_block(1, 2) is None and m.denoise_block_sampled(1) is None and m.attn_varlen() is None
 
 
 @pytest.mark.gpu
