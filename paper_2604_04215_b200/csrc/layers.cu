@@ -78,6 +78,44 @@ rmsnorm_kernel(const uint4* __restrict__ x, int D8, float eps, uint4* __restrict
     for (int i = threadIdx.x + NORM_VECS * NORM_THREADS; i < D8; i += NORM_THREADS) dst[i] = scale_bf16(src[i], inv);
 }
 
+// The same with a warp per row, ROWS_PER_BLOCK rows per CTA, for many short rows (norm_warp_rows below).  Lane l stands for
+// the threads l, l + 32, ... of the kernel above and adds in the same order: a row's result does not depend on the number
+// of rows beside it.
+template <int VECS>
+__global__ void __launch_bounds__(ROWS_PER_BLOCK * 32)
+rmsnorm_warp_kernel(const uint4* __restrict__ x, int D8, int n_rows, float eps, uint4* __restrict__ y) {
+    constexpr int WARPS = NORM_THREADS / 32;
+    const int m = blockIdx.x * ROWS_PER_BLOCK + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    pdl_wait();
+    pdl_trigger();
+    if (m >= n_rows) return;
+    const uint4* src = x + static_cast<size_t>(m) * D8;
+    uint4* dst = y + static_cast<size_t>(m) * D8;
+    uint4 v[VECS];
+#pragma unroll
+    for (int u = 0; u < VECS; ++u) {
+        const int i = lane + u * 32;
+        v[u] = i < D8 ? src[i] : make_uint4(0, 0, 0, 0);
+    }
+    float ss = 0.f;
+#pragma unroll
+    for (int w = 0; w < (VECS < WARPS ? VECS : WARPS); ++w) {
+        float part = 0.f;
+#pragma unroll
+        for (int u = w; u < VECS; u += WARPS) part += sum_squares(v[u]);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
+        ss += part;
+    }
+    const float inv = rsqrtf(ss / static_cast<float>(D8 * 8) + eps);
+#pragma unroll
+    for (int u = 0; u < VECS; ++u) {
+        const int i = lane + u * 32;
+        if (i < D8) dst[i] = scale_bf16(v[u], inv);
+    }
+}
+
 // cs[p, c] = (cos, sin)(p * base^(-2c/d)), c < d/2, evaluated in double precision; cs_t is its transpose.
 __global__ void rope_table_kernel(float2* __restrict__ cs, float2* __restrict__ cs_t, int n_pos, int half, double base) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -156,6 +194,13 @@ rope_kv_write_kernel(const __nv_bfloat16* __restrict__ qkv, int Hq, int Hkv, int
 constexpr size_t SPREAD_SMEM = 45 * 1024;
 inline size_t spread_smem(int ctas) { return ctas <= 5 * 148 ? SPREAD_SMEM : 0; }
 
+// Rows for which a warp each is the better split.  CTAs start at about one per ns over the GPU, whatever they do: 65536 rows
+// of 256 took 68 us with one each and take 9.3, 16384 of 1024 17.5 and 7.0, 4096 of 512 4.7 and 2.4.  Longer rows are bound
+// by their bytes, and few of them by one row's trip to memory, which four warps make shorter: 512 of 1024 1.4 us with a CTA
+// per row and 1.7 with a warp, 600 of 1024 1.8 and 1.6, 3072 of 2048 4.0 and 4.1, 6144 of 2048 7.1 and 6.5, 4096 of 3072 5.5 and
+// 8.2.  (Up to 512 values both take 1.1 to 1.3 us up to 512 rows.)
+inline bool norm_warp_rows(int n_rows, int D) { return D <= 2048 && n_rows > (D <= 1024 ? 512 : 4095); }
+
 }  // namespace
 
 int launch_embed(const void* emb, int D, int V, const int32_t* tokens, int64_t row_stride, int start, int length,
@@ -166,8 +211,15 @@ int launch_embed(const void* emb, int D, int V, const int32_t* tokens, int64_t r
 }
 
 int launch_rmsnorm(const void* x, int D, int n_rows, float eps, void* y, cudaStream_t stream) {
-    return launch_kernel(rmsnorm_kernel, dim3(n_rows), NORM_THREADS, spread_smem(n_rows), stream, 1,
-                         static_cast<const uint4*>(x), D / 8, eps, static_cast<uint4*>(y));
+    const uint4* src = static_cast<const uint4*>(x);
+    uint4* dst = static_cast<uint4*>(y);
+    if (norm_warp_rows(n_rows, D)) {
+        const auto kernel = D <= 256 ? rmsnorm_warp_kernel<1> : D <= 512 ? rmsnorm_warp_kernel<2> : D <= 1024 ? rmsnorm_warp_kernel<4>
+                            : rmsnorm_warp_kernel<8>;
+        return launch_kernel(kernel, dim3((n_rows + ROWS_PER_BLOCK - 1) / ROWS_PER_BLOCK), ROWS_PER_BLOCK * 32, 0, stream, 1, src, D / 8,
+                             n_rows, eps, dst);
+    }
+    return launch_kernel(rmsnorm_kernel, dim3(n_rows), NORM_THREADS, spread_smem(n_rows), stream, 1, src, D / 8, eps, dst);
 }
 
 int launch_rope_table(float* cs, float* cs_t, int n_pos, int half, double base, cudaStream_t stream) {

@@ -73,6 +73,41 @@ def test_rmsnorm_row_lengths(ctx, rows, D):
     assert (np.abs(y - ref) <= 2.0 ** -8 * np.abs(ref) + 1e-6).all()      # one rounding to bf16, fp32 sums
 
 
+# ... and a warp per row for many short ones: the edges of that rule and of the row lengths a warp holds.  A row's result is
+# the same, bit for bit, whichever kernel takes it.
+@pytest.mark.parametrize("rows,D", [(1, 256), (9, 264), (31, 504), (7, 512), (512, 520), (513, 520), (514, 1024), (4095, 1032), (4096, 1032),
+                                    (4097, 2048), (4096, 2056)])
+def test_rmsnorm_of_many_short_rows(ctx, rows, D):
+    x = I.normal_bf16(3, I.TID_X, (rows, D), 3.0)
+    y = dare.dare_rmsnorm(ctx, x.cuda(), 1e-5)
+    f = x.double()
+    ref = f / (f.pow(2).mean(1, keepdim=True) + 1e-5).sqrt()
+    assert ((y.cpu().double() - ref).abs() <= 2.0 ** -8 * ref.abs() + 1e-6).all()      # one rounding to bf16, fp32 sums
+    few = torch.cat([dare.dare_rmsnorm(ctx, x[i:i + 300].cuda(), 1e-5) for i in range(0, rows, 300)])
+    assert torch.equal(few, y)
+
+
+def _us(call, n=40):
+    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    best = float("inf")
+    for _ in range(5):
+        torch.cuda.synchronize()
+        a.record()
+        for _ in range(n):
+            call()
+        b.record()
+        b.synchronize()
+        best = min(best, a.elapsed_time(b) * 1e3 / n)
+    return best
+
+
+def test_many_short_rows_cost_their_bytes(ctx):
+    """A CTA per row would take 68 us to start here; a copy of the same bytes, and a warp per row, take about 10."""
+    x = torch.randn(65536, 256, device="cuda").bfloat16()
+    y = torch.empty_like(x)
+    assert _us(lambda: dare.dare_rmsnorm(ctx, x, 1e-5, y)) <= 2.5 * max(10.0, _us(lambda: y.copy_(x)))
+
+
 # Projections with so many rows that the tiles are taken in groups of row pairs (32 MB of A per group): one group and a
 # row more than that, an uneven last group, K so long that a group is one row pair.
 @pytest.mark.parametrize("M,K,N", [(2048, 8192, 264), (2049, 8192, 264), (5000, 8200, 520), (600, 65544, 72)])
