@@ -136,16 +136,20 @@ __global__ void rope_table_kernel(float2* __restrict__ cs, float2* __restrict__ 
 // done; what it reads of the projection, it asks for ROPE_BATCH heads at a time.  512 rows of 96 heads of 128 between the
 // projection and the attention: 5.4 us, 25 MB through L2; 8.0 with 128 threads that took one head after another and its
 // angles with it (256 such threads: 6.5).
+// A row has `row_threads` threads (rope_row_threads below; WHOLE: all ROPE_THREADS), a CTA as many rows as ROPE_THREADS hold.
 constexpr int ROPE_THREADS = 256;
 constexpr int ROPE_BATCH = 2;
+template <bool WHOLE>
 __global__ void __launch_bounds__(ROPE_THREADS)
-rope_kv_write_kernel(const __nv_bfloat16* __restrict__ qkv, int Hq, int Hkv, int d, int start, int length,
+rope_kv_write_kernel(const __nv_bfloat16* __restrict__ qkv, int n_rows, int row_threads_, int Hq, int Hkv, int d, int start, int length,
                      const float2* __restrict__ cs, __nv_bfloat16* __restrict__ q_out,
                      __nv_bfloat16* __restrict__ k_cache, __nv_bfloat16* __restrict__ v_cache, int cap) {
-    const int m = blockIdx.x;
+    const int row_threads = WHOLE ? ROPE_THREADS : row_threads_, tid = WHOLE ? threadIdx.x : threadIdx.x % row_threads;
+    const int m_any = WHOLE ? blockIdx.x : (blockIdx.x * blockDim.x + threadIdx.x) / row_threads;
+    const int m = WHOLE ? m_any : min(m_any, n_rows - 1);
     const int b = m / length, i = m % length, p = start + i;
     const int half = d / 2, cpb = half / 8;                 // 8-channel groups per half head (4 or 8)
-    const int c0 = threadIdx.x % cpb * 8, h_step = ROPE_THREADS / cpb;
+    const int c0 = tid % cpb * 8, h_step = row_threads / cpb;
     const int n_rot = Hq + Hkv, n_v = Hkv * (d / 8);
     const __nv_bfloat16* row = qkv + static_cast<size_t>(m) * (Hq + 2 * Hkv) * d;
     float2 t[8];
@@ -153,7 +157,8 @@ rope_kv_write_kernel(const __nv_bfloat16* __restrict__ qkv, int Hq, int Hkv, int
     for (int j = 0; j < 8; ++j) t[j] = cs[static_cast<size_t>(p) * half + c0 + j];
     pdl_wait();
     pdl_trigger();
-    for (int h0 = threadIdx.x / cpb; h0 < n_rot; h0 += ROPE_BATCH * h_step) {
+    if (!WHOLE && m_any >= n_rows) return;
+    for (int h0 = tid / cpb; h0 < n_rot; h0 += ROPE_BATCH * h_step) {
         uint4 lo[ROPE_BATCH], hi[ROPE_BATCH];
 #pragma unroll
         for (int u = 0; u < ROPE_BATCH; ++u) {
@@ -181,7 +186,7 @@ rope_kv_write_kernel(const __nv_bfloat16* __restrict__ qkv, int Hq, int Hkv, int
         }
     }
 #pragma unroll 2
-    for (int j = threadIdx.x; j < n_v; j += ROPE_THREADS) {
+    for (int j = tid; j < n_v; j += row_threads) {
         const int h = j / (d / 8), c = (j % (d / 8)) * 8;
         const uint4 v = *reinterpret_cast<const uint4*>(row + static_cast<size_t>(n_rot + h) * d + c);
         *reinterpret_cast<uint4*>(v_cache + ((static_cast<size_t>(b) * Hkv + h) * cap + p) * d + c) = v;
@@ -200,6 +205,15 @@ inline size_t spread_smem(int ctas) { return ctas <= 5 * 148 ? SPREAD_SMEM : 0; 
 // per row and 1.7 with a warp, 600 of 1024 1.8 and 1.6, 3072 of 2048 4.0 and 4.1, 6144 of 2048 7.1 and 6.5, 4096 of 3072 5.5 and
 // 8.2.  (Up to 512 values both take 1.1 to 1.3 us up to 512 rows.)
 inline bool norm_warp_rows(int n_rows, int D) { return D <= 2048 && n_rows > (D <= 1024 ? 512 : 4095); }
+
+// Threads per row of the rotary kernel: enough for a batch of heads each, up to a warp also for one piece of v each.  (A whole
+// CTA per row, whatever its heads, leaves most threads idle and is bound by how fast CTAs start: 32768 rows of 2 + 1 heads of
+// 64 48 us, now 6.9; 2048 rows of 4 + 2 heads of 128 6.3 and 2.8, of 32 + 8 9.0 and 7.4; 48 rows 1.7 to 2.0 either way.)
+inline int rope_row_threads(int Hq, int Hkv, int d) {
+    const int rot = (Hq + Hkv + ROPE_BATCH - 1) / ROPE_BATCH * (d / 16), v = Hkv * (d / 8);      // (multiples of d / 16)
+    const int n = rot >= 32 || rot >= v ? rot : v < 32 ? v : 32;
+    return n < ROPE_THREADS ? n : ROPE_THREADS;
+}
 
 }  // namespace
 
@@ -230,8 +244,11 @@ int launch_rope_table(float* cs, float* cs_t, int n_pos, int half, double base, 
 
 int launch_rope_kv_write(const void* qkv, int n_rows, int Hq, int Hkv, int d, int start, int length, const float* cs,
                          void* q_out, void* k_cache, void* v_cache, int cap, cudaStream_t stream) {
-    return launch_kernel(rope_kv_write_kernel, dim3(n_rows), ROPE_THREADS, spread_smem(n_rows), stream, 1,
-                         static_cast<const __nv_bfloat16*>(qkv), Hq, Hkv, d, start, length, reinterpret_cast<const float2*>(cs),
+    const int row_threads = rope_row_threads(Hq, Hkv, d), rows = ROPE_THREADS / row_threads;
+    const int ctas = (n_rows + rows - 1) / rows;
+    return launch_kernel(row_threads == ROPE_THREADS ? rope_kv_write_kernel<true> : rope_kv_write_kernel<false>, dim3(ctas),
+                         rows * row_threads, spread_smem(ctas), stream, 1, static_cast<const __nv_bfloat16*>(qkv), n_rows,
+                         row_threads, Hq, Hkv, d, start, length, reinterpret_cast<const float2*>(cs),
                          static_cast<__nv_bfloat16*>(q_out), static_cast<__nv_bfloat16*>(k_cache),
                          static_cast<__nv_bfloat16*>(v_cache), cap);
 }

@@ -358,3 +358,36 @@ def test_rope_kernel_head_counts(ctx, Hq, Hkv, d):
     assert torch.equal(vc[0, :, :, rows].transpose(1, 2), x[:, :, Hq + Hkv:])
     assert kc[0, :, :, :start].count_nonzero() == 0 and vc[0, :, :, start + length:].count_nonzero() == 0
     model.close()
+
+
+# Rows with few heads share a CTA of that kernel: a last CTA with one row, threads that are no power of two, v pieces that take
+# more than one pass.  Each row as when it is alone.
+@pytest.mark.parametrize("Hq,Hkv,d", [(2, 1, 64), (4, 4, 64), (9, 1, 64), (4, 2, 128), (8, 2, 128), (16, 16, 64), (28, 4, 128), (32, 8, 128)])
+def test_rope_kernel_rows_that_share_a_cta(ctx, Hq, Hkv, d):
+    B, length, start = 33, 9, 2
+    model = _small_model(ctx, Hq, Hkv, d, B * length, B, length + start, hidden=64, ffn=64)
+    x = I.normal_bf16(Hq, 3, (B * length, (Hq + 2 * Hkv) * d)).cuda()
+    new = lambda *s: torch.zeros(*s, dtype=torch.bfloat16, device="cuda")  # noqa: E731
+    q, q1 = new(B * length, Hq, d), new(B * length, Hq, d)
+    kc, vc, k1, v1 = (new(B, Hkv, length + start, d) for _ in range(4))
+    dare.dare_rope_kv_write(model, x, B, length, start, q, kc, vc)
+    for b in range(B):
+        for i in range(length):
+            r, at = b * length + i, start + i
+            row = (new(1, Hkv, length + start, d), new(1, Hkv, length + start, d))
+            dare.dare_rope_kv_write(model, x[r:r + 1], 1, 1, at, q1[r:r + 1], *row)
+            k1[b, :, at], v1[b, :, at] = row[0][0, :, at], row[1][0, :, at]
+    torch.cuda.synchronize()
+    assert torch.equal(q, q1) and torch.equal(kc, k1) and torch.equal(vc, v1)
+    model.close()
+
+
+def test_rope_kernel_of_few_heads_costs_its_bytes(ctx):
+    """A CTA per row would take 48 us here; a copy of the same bytes and rows that share a CTA take about 10."""
+    B, length = 64, 512
+    model = _small_model(ctx, 2, 1, 64, B * length, B, length, hidden=64, ffn=64)
+    x, y = torch.randn(2, B * length, 256, device="cuda").bfloat16()
+    q, kc, vc = torch.empty_like(x[:, :128]).contiguous(), *model.new_cache(B, length)
+    us = _us(lambda: dare.dare_rope_kv_write(model, x, B, length, 0, q, kc, vc))
+    assert us <= 2.5 * max(10.0, _us(lambda: y.copy_(x)))
+    model.close()
