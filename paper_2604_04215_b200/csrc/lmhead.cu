@@ -225,7 +225,7 @@ __device__ __forceinline__ void sample_one(float z, int col, const SampleKey& ke
     const uint4 w4 = philox4x32_10(make_uint4(static_cast<uint32_t>(col) >> 2, key.row, key.step, 0x44415245u), key.seed_lo, key.seed_hi);
     const uint32_t w = (col & 2) ? ((col & 1) ? w4.w : w4.z) : ((col & 1) ? w4.y : w4.x);
     const float y = fmaf(z, key.inv_temperature, gumbel_from_word(w));
-    if (y > best.y || (y == best.y && col < best.arg)) best = {y, z, col};
+    if (y > best.y || (y == best.y && col < best.arg && y > -INFINITY)) best = {y, z, col};
 }
 template <typename At>
 __device__ __forceinline__ void sample_chunk(const float (&z)[32], int cbase, float zmax, int zarg, float bound, const SampleKey& key,
@@ -244,7 +244,9 @@ __device__ __forceinline__ void sample_chunk(const float (&z)[32], int cbase, fl
         for (int e = 0; e < 4; ++e) {
             const float t = fast_exp2(fmaf(z[q * 4 + e], c2, nb));
             const float f = __uint_as_float((ww[e] >> 9) + 0x3f800000u);
-            if (f + t >= 1.99999988079071044921875f) pass |= 1u << (q * 4 + e);    // 2 - 2^-23: no rounding of the sum can hide a hit
+            // 2 - 2^-23: no rounding of the sum can hide a hit.  (Not >=: t is NaN against a best score of +inf, which the
+            // lower one of two such columns must still meet.)
+            if (!(f + t < 1.99999988079071044921875f)) pass |= 1u << (q * 4 + e);
         }
     }
     while (__any_sync(0xffffffffu, pass != 0)) {

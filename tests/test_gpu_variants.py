@@ -142,6 +142,23 @@ def test_sampled_head_on_every_path(ctx, M, T):
     assert np.abs(np.log(conf[same]) - ref["logconf"][same]).max() <= 1e-3
 
 
+# Scores that are infinite tie, and the lowest id wins a tie, wherever the columns lie: in one thread's 32 columns, in two
+# warps' or two tiles' columns.  (z / T of the columns named is 5e38 and more, beyond fp32; of the others -1e38.)
+@pytest.mark.parametrize("M", [1, 40, 300, 420, 700])
+@pytest.mark.parametrize("cols", [(3, 9), (3, 40), (7, 64, 999), (100, 101, 130), (515, 1290), (1291,)])
+def test_sampled_head_ties_at_infinite_scores(ctx, M, cols):
+    D, V, mu, T = 16, 1300, 2, 1e-38
+    x, w = torch.zeros(M, D), torch.zeros(V, D)
+    x[:, 0], w[:, 0] = 1.0, -1.0
+    for n, c in enumerate(cols):
+        w[c, 0] = 5.0 + 2 * n                     # (the higher ids have the larger logits)
+    pred, conf = dare.dare_lmhead_sample(ctx, x.bfloat16().cuda(), w.bfloat16().cuda(), None, mu, True, T, 11, 3)
+    assert (pred.cpu() == cols[0]).all()
+    z = w[:, 0].double()
+    z[mu] = -float("inf")
+    assert torch.allclose(conf.cpu().double(), torch.softmax(z, 0)[cols[0]].expand(M), rtol=1e-5)
+
+
 def test_sampled_head_with_a_workspace_for_one_partial_per_tile():
     """The swapped path wants room for two partials per vocabulary tile; a context without it takes the other path."""
     M, D, V, mu = 40, 64, 2000, 1999
