@@ -206,19 +206,18 @@ __device__ __forceinline__ float gumbel_from_word(uint32_t w) {
     return -logf(-logf(u));
 }
 
-// One row's 32 consecutive logits z (columns cbase ..., cbase a multiple of 32; largest: column zarg) against the row's
-// best perturbed score so far.  Two logarithms per logit cost more than the MMAs hide, and almost no logit needs them:
-// y = z / T + g beats best_y only if -ln u < t = exp(z / T - best_y), and -ln u >= 1 - u, so a logit with 1 - u > t is
-// out.  That test takes one exponential, and 1 - u comes from the generator's word by its bits: f = 1.k in [1, 2) is
-// 2 - (1 - u) - 2^-24.  The logits that pass (about one in the number of columns seen) are evaluated exactly as without
-// the test, so the sampled token is the same bit for bit: the test's t is raised by 2^(2e-3 + 1e-5 |best_y|), well over
-// the rounding of the exponent (of the size of |best_y| + 17 where the test can fail at all) and of the logarithms it
-// stands in for.  Where there is no best yet, the largest logit is evaluated first, which leaves ~3 of the 32.
+// One row's 32 consecutive logits z (columns cbase ..., cbase a multiple of 32; largest: zmax) against the row's best
+// perturbed score so far.  Two logarithms per logit cost more than the MMAs hide, and almost no logit needs them: -ln u >=
+// 1 - u, so z / T - ln(1 - u) is an upper bound of its score, which takes one hardware logarithm (1 - u by the bits of the
+// generator's word) and is close to the score where that is large.  Only where the largest bound of the 32 can beat the
+// best does the lane evaluate a logit, that one first, and then those whose bounds beat what it made of the best (seldom
+// any).  An evaluation is as without the test, and the bounds are compared with 2e-3 + 1e-5 |best| (in log2) to spare, well
+// over the rounding of either, so the sampled token is the same bit for bit.
+// What this costs shows where a thread sees few groups of a row and nothing hides its epilogue: 256 rows x 256 x 4096 takes
+// 24.6 us, 92 when a group without a best yet was begun at its largest logit and nearly all of it evaluated, 23.4 with two
+// logarithms for every logit on twice the warps; 400 rows x 4096 x 126464 396, 451 and 538 us.
 // `bound`: a score of the same row that another warp has seen (or -inf): what cannot reach it need not be evaluated.
 // at(j) returns z[j] for an index that differs from lane to lane.
-// With two logarithms per logit and twice the epilogue warps the kernel executed 159 M warp instructions in 579 k SM
-// cycles at 416 rows x 126464 and 122 M in 477 k at 384; now 73 M in 501 k and 53 M in 398 k (greedy: 21 M and 369 k).
-// Two sets of epilogue warps on top of this gain nothing: these launches sit on the power cap.
 struct SampleBest { float y, z; int arg; };
 struct SampleKey { uint32_t row, step, seed_lo, seed_hi; float inv_temperature; };
 __device__ __forceinline__ void sample_one(float z, int col, const SampleKey& key, SampleBest& best) {
@@ -228,13 +227,14 @@ __device__ __forceinline__ void sample_one(float z, int col, const SampleKey& ke
     if (y > best.y || (y == best.y && col < best.arg && y > -INFINITY)) best = {y, z, col};
 }
 template <typename At>
-__device__ __forceinline__ void sample_chunk(const float (&z)[32], int cbase, float zmax, int zarg, float bound, const SampleKey& key,
+__device__ __forceinline__ void sample_chunk(const float (&z)[32], int cbase, float zmax, float bound, const SampleKey& key,
                                              SampleBest& best, const At& at) {
-    if (best.y == -INFINITY && zmax > -INFINITY) sample_one(zmax, zarg, key, best);
-    bound = fmaxf(bound, best.y);
     const float c2 = key.inv_temperature * LOG2E;
-    const float nb = fmaf(-LOG2E, bound, fmaf(1e-5f, fabsf(bound), 2e-3f));
-    uint32_t pass = 0;
+    const auto threshold = [&]() {      // (NaN against +inf: lets everything through, see below)
+        const float b = fmaxf(bound, best.y);
+        return fmaf(LOG2E, b, -fmaf(1e-5f, fabsf(b), 2e-3f));
+    };
+    float ub[32], ub_max = -INFINITY;
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
         const uint4 w4 = philox4x32_10(make_uint4(static_cast<uint32_t>(cbase >> 2) + q, key.row, key.step, 0x44415245u), key.seed_lo,
@@ -242,12 +242,28 @@ __device__ __forceinline__ void sample_chunk(const float (&z)[32], int cbase, fl
         const uint32_t ww[4] = {w4.x, w4.y, w4.z, w4.w};
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            const float t = fast_exp2(fmaf(z[q * 4 + e], c2, nb));
-            const float f = __uint_as_float((ww[e] >> 9) + 0x3f800000u);
-            // 2 - 2^-23: no rounding of the sum can hide a hit.  (Not >=: t is NaN against a best score of +inf, which the
-            // lower one of two such columns must still meet.)
-            if (!(f + t < 1.99999988079071044921875f)) pass |= 1u << (q * 4 + e);
+            // u = (2 k + 1) / 2^24, 1 - u = (2 k' + 1) / 2^24 with k' = the complement of k's 23 bits; 1.k' - (1 - 2^-24) is exact
+            const float v = __uint_as_float((ww[e] >> 9) ^ 0x3fffffffu) - 0.999999940395355224609375f;
+            ub[q * 4 + e] = fmaf(z[q * 4 + e], c2, -__log2f(v));
+            ub_max = fmaxf(ub_max, ub[q * 4 + e]);
         }
+    }
+    // (not ub >= thr: against a best score of +inf the lower one of two such columns must still be met)
+    float thr = threshold();
+    const bool mine = zmax > -INFINITY && !(ub_max < thr);
+    if (!__any_sync(0xffffffffu, mine)) return;
+    int first = 0;
+#pragma unroll
+    for (int j = 1; j < 32; ++j)
+        if (ub[j] == ub_max) first = j;
+    uint32_t pass = 0;
+    if (mine) {
+        sample_one(at(first), cbase + first, key, best);
+        thr = threshold();
+#pragma unroll
+        for (int j = 0; j < 32; ++j)
+            if (!(ub[j] < thr)) pass |= 1u << j;
+        pass &= ~(1u << first);
     }
     while (__any_sync(0xffffffffu, pass != 0)) {
         if (pass != 0) {
@@ -524,7 +540,7 @@ lm_rowmajor_body(const CUtensorMap& tmap_x, const CUtensorMap& tmap_w,
                             }
                             return a[0];
                         };
-                        sample_chunk(z, cbase, cmax, carg, -INFINITY, key, best, at);
+                        sample_chunk(z, cbase, cmax, -INFINITY, key, best, at);
                     }
                     if (cmax > -INFINITY) {
                         if (cmax > run_max) {   // tiles of a group come in ascending order: '>' keeps the lowest id
@@ -945,7 +961,7 @@ lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, 
                             bound = fmaxf(bound, *static_cast<volatile float*>(state + q * WARP_STATE + 2 * NS + r));
                         const SampleKey key = {rng_row, rng_step, smp.seed_lo, smp.seed_hi, smp.inv_temperature};
                         const auto at = [&](int j) { return vbase + j >= V || vbase + j == mask_col ? -INFINITY : xp[j * 33 + lane]; };
-                        sample_chunk(z, vbase, cmax, carg, bound, key, best, at);
+                        sample_chunk(z, vbase, cmax, bound, key, best, at);
                         __syncwarp();                     // the block may be overwritten
                         st[r] = rmax; st[NS + r] = rsum;
                         st[2 * NS + r] = best.y; st[3 * NS + r] = best.z; st[4 * NS + r] = __int_as_float(best.arg);

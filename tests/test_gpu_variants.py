@@ -142,6 +142,31 @@ def test_sampled_head_on_every_path(ctx, M, T):
     assert np.abs(np.log(conf[same]) - ref["logconf"][same]).max() <= 1e-3
 
 
+# The test that spares most logits their logarithms must not lose the best one: logits from flat (the noise decides) to steep
+# (the logit decides), several tiles per warp, and rows whose best comes early, late or from another warp.
+@pytest.mark.parametrize("M", [33, 160, 300, 520])
+@pytest.mark.parametrize("sigma,T", [(0.01, 1.0), (0.3, 5.0), (1.0, 0.05), (4.0, 1.0), (4.0, 40.0)])
+def test_sampled_head_evaluates_the_best(ctx, M, sigma, T):
+    D, V, mu, seed, step = 64, 20_000, 0, 0x1234567890 + M, 9
+    x, w = I.normal_bf16(M, I.TID_X, (M, D)), I.normal_bf16(4, I.TID_W, (V, D), sigma / 8)
+    ref = SO.lmhead_sample(x.double().numpy(), w.double().numpy(), None, mu, True, T, seed, step)
+    pred, _ = dare.dare_lmhead_sample(ctx, x.cuda(), w.cuda(), None, mu, True, T, seed, step)
+    torch.cuda.synchronize()
+    # scores: fp32 sums of 64 products of magnitude sigma / 8 * 3 (64 * 2^-24 * 64 * that: 1e-4 sigma) over T, noise to an ulp of 20
+    sure = ref["gap_y"] > 2e-4 * sigma / T + 1e-5
+    assert (pred.cpu().numpy()[sure] == ref["pred"][sure]).all() and sure.mean() > 0.9
+
+
+# Where a warp sees one or two groups of 32 logits of each row, nothing of a row is known yet when the first group comes: the
+# lanes then have to start with their best candidate, or nearly all 32 are evaluated (58 to 95 us here, the greedy head 12 to 18).
+@pytest.mark.parametrize("M,D,V", [(128, 256, 4096), (256, 256, 4096), (300, 512, 2048), (640, 256, 2048)])
+def test_sampled_head_on_a_small_vocabulary_costs_little_more(ctx, M, D, V):
+    x, w = torch.randn(M, D, device="cuda").bfloat16(), torch.randn(V, D, device="cuda").mul(0.02).bfloat16()
+    pred, conf = torch.empty(M, dtype=torch.int32, device="cuda"), torch.empty(M, device="cuda")
+    greedy = _us(lambda: dare.dare_lmhead_confidence(ctx, x, w, None, 3, True, pred, conf))
+    assert _us(lambda: dare.dare_lmhead_sample(ctx, x, w, None, 3, True, 1.0, 7, 1, pred, conf)) <= 2.5 * greedy
+
+
 # Scores that are infinite tie, and the lowest id wins a tie, wherever the columns lie: in one thread's 32 columns, in two
 # warps' or two tiles' columns.  (z / T of the columns named is 5e38 and more, beyond fp32; of the others -1e38.)
 @pytest.mark.parametrize("M", [1, 40, 300, 420, 700])
