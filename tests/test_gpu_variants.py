@@ -167,6 +167,17 @@ def test_sampled_head_on_a_small_vocabulary_costs_little_more(ctx, M, D, V):
     assert _us(lambda: dare.dare_lmhead_sample(ctx, x, w, None, 3, True, 1.0, 7, 1, pred, conf)) <= 2.5 * greedy
 
 
+def test_sampled_head_has_a_pair_per_vocabulary_tile(ctx):
+    """128 rows are one row tile, 160 two: the launch of the former must not be the smaller one (24 against 19 us it was)."""
+    D, V = 256, 4096
+    w, us = torch.randn(V, D, device="cuda").mul(0.02).bfloat16(), []
+    for M in (128, 160):
+        x = torch.randn(M, D, device="cuda").bfloat16()
+        pred, conf = torch.empty(M, dtype=torch.int32, device="cuda"), torch.empty(M, device="cuda")
+        us.append(_us(lambda: dare.dare_lmhead_sample(ctx, x, w, None, 3, True, 1.0, 7, 1, pred, conf)))
+    assert us[0] <= 1.1 * us[1]
+
+
 # Scores that are infinite tie, and the lowest id wins a tie, wherever the columns lie: in one thread's 32 columns, in two
 # warps' or two tiles' columns.  (z / T of the columns named is 5e38 and more, beyond fp32; of the others -1e38.)
 @pytest.mark.parametrize("M", [1, 40, 300, 420, 700])
