@@ -674,16 +674,22 @@ __host__ __device__ constexpr int sw_values(int mode, bool joint) { return mode 
 __host__ __device__ constexpr int sw_state_bytes(int mode, bool joint) {
     return 4 * sw_values(mode, joint) * (joint ? 2 : 1) * SW_NMAX * 4;
 }
-constexpr int SW_SMEM_BYTES = 227 * 1024;
+// Shared memory of the kernel.  The 5 KB that are left of the SM's 228 (the system takes 1 of them per CTA) hold CTAs of the
+// merge kernel, which are then in place when the last tile is done: with all of it taken they could only be started
+// behind the GEMM's CTAs, and every head paid 2.5 us for that (512 rows x 1024 x 16000 22.1 us, 19.6 with room).  222 KB hold
+// five slots of 36 KB for two chunks at a time at 320 rows.
+constexpr int SW_SMEM_BYTES = 222 * 1024;
 __host__ __device__ constexpr int sw_ring_bytes(int mode, bool joint) {
-    return joint ? (SW_SMEM_BYTES - 1024 - 4 * SW_XP_FLOATS * 4 - sw_state_bytes(mode, true) - static_cast<int>(sizeof(SwBarriers))) & ~1023
-                 : SW_STAGES * SW_STAGE_BYTES - (mode == LM_SAMPLE ? 3072 : 0);
+    return joint || mode == LM_SAMPLE
+               ? (SW_SMEM_BYTES - 1024 - 4 * SW_XP_FLOATS * 4 - sw_state_bytes(mode, joint) - static_cast<int>(sizeof(SwBarriers))) & ~1023
+               : SW_STAGES * SW_STAGE_BYTES;
 }
 __host__ __device__ constexpr int sw_smem_bytes(int mode, bool joint) {
     return sw_ring_bytes(mode, joint) + 4 * SW_XP_FLOATS * 4 + sw_state_bytes(mode, joint) + static_cast<int>(sizeof(SwBarriers)) + 1024;
 }
 static_assert(sw_smem_bytes(LM_SAMPLE, false) <= SW_SMEM_BYTES && sw_smem_bytes(LM_GREEDY, false) <= SW_SMEM_BYTES &&
               sw_smem_bytes(LM_GREEDY, true) <= SW_SMEM_BYTES, "shared memory");
+static_assert(SW_SMEM_BYTES + 1024 + 3 * (1024 + 512) <= 228 * 1024, "room for three CTAs of a merge kernel beside the head's");
 // X tiles of 128, 64, 32, 16 and 8 rows: a CTA's share of a chunk (a multiple of 8 rows) is covered by one or two
 // of them, stacked in shared memory (each a whole number of 1 KB swizzle atoms); a few rows too many may be loaded,
 // the MMA reads only its own.  (Exact covers of up to four boxes were measured slower: 432 us for 480 rows, where
