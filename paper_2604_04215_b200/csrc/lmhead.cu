@@ -1088,6 +1088,16 @@ __host__ __device__ inline int lm_mixed_pair_clusters(int n_clusters, int p) {
     return up;
 }
 
+// Two chunks at a time, a function of its own: compiled into the kernel it made the epilogue of the other swapped path wait
+// longer between its instructions (as many of them, 62 k SM cycles as against 80 k at 256 rows x 2048 x 24000).
+__device__ __noinline__ void
+lm_joint_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, int V, int mask_col, int n_vt, float* __restrict__ part_max,
+              float* __restrict__ part_sum, int32_t* __restrict__ part_arg, uint32_t* __restrict__ dev_status, int parts_stride,
+              const LmSampling& smp) {
+    lm_swapped_body<LM_GREEDY, true>(tmap_w, xmaps, Mc, D, V, mask_col, n_vt, part_max, part_sum, part_arg, dev_status, parts_stride,
+                                     smp);
+}
+
 // The greedy (or sampled) head, one launch on CTA pairs whatever the number of live rows (known only on the device when rows are
 // skipped): the swapped-operand path for the counts lm_swapped names (up to SW_NMAX rows, and counts that
 // cut into long chunks); otherwise row-major tiles of 128 rows, on CTA pairs when the tiles come in twos, and for
@@ -1110,8 +1120,7 @@ lmhead_head_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
     const int Mc = live_rows ? *live_rows : M;          // rows that need logits (uniform over the grid)
     if constexpr (MODE == LM_GREEDY) {
         if (lm_joint(Mc, false)) {
-            lm_swapped_body<MODE, true>(tmap_w, xmaps, Mc, D, V, mask_col, n_tiles, part_max, part_sum, part_arg, dev_status,
-                                        parts_stride, smp);
+            lm_joint_body(tmap_w, xmaps, Mc, D, V, mask_col, n_tiles, part_max, part_sum, part_arg, dev_status, parts_stride, smp);
             return;
         }
     }
