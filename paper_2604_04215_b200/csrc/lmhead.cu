@@ -618,7 +618,8 @@ lmhead_partial_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
 // More rows than SW_NMAX are cut into equal chunks, in one of two ways:
 //   * items = chunk x vocabulary group: a chunk streams all of W from L2 into the SMs whatever its N, and that stream
 //     (~12 TB/s over the GPU), not the tensor pipe, sets the pace when the chunks are short (an MMA alone takes
-//     max(N / 2, ~45) cycles): only chunks close to 256 rows are worth it;
+//     max(N / 2, ~45) cycles): worth it for chunks close to 256 rows, and for shorter ones where the row-major tiles would be
+//     padded by as much as they hold (lm_swapped below);
 //   * both chunks against each W tile (JOINT): W enters the SMs once.  The price is the accumulators: three of 160 columns
 //     fit, so the next tile's MMAs wait for half of this one's epilogue, and the running values of 320 columns move to
 //     shared memory.
@@ -632,21 +633,39 @@ lmhead_partial_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
 // so the values live in shared memory, taken off the ring (6 slots become 5 above 192 rows).
 constexpr int SW_BV = 128;                               // vocabulary rows per CTA and tile
 constexpr int SW_NMAX = 256;                             // rows (accumulator columns) per chunk
-// Row counts for which a head takes this path: up to one chunk, where W is streamed once and the launch is bound by HBM;
-// two chunks of up to 192 rows, whose row-major tiles would be 384 padded rows; and, up to 1024 rows, counts that cut into
-// chunks of 208 to 240 rows, i.e. whose row-major tiles would carry 64 or more padded rows per pair (swapped against
-// row-major, one chunk at a time, us: D = 4096, V = 126464: 416 rows 333 / 380, 448 rows 415 / 462, 480 rows 410 / 428, 512 rows
-// 425 / 421; D = 3584, V = 152064: 704 rows 625 / 650, 832 rows 784 / 840, 960 rows 851 / 895).
-// Two chunks of up to 192 rows, D = 4096, V = 126464, us under the power cap, where padded MMAs cost twice: greedy, both
-// chunks at a time / row-major: 272 rows 298 / 404, 320 rows 320 / 411; above, where two accumulators are all that fit, one chunk at
-// a time: 368 rows 383 / 422, 384 rows 386 / 421 (both at a time: 394; D = 3584, V = 152064, from idle, 352 rows 389 / 370).
-// Sampled, one at a time (its epilogue is several times as long and may not be waited for: 457 both at a time at 320
-// rows): 272 rows 382 / 414, 320 rows 392 / 423, 384 rows 433 / 433.
+// Row counts for which a head takes this path, for n_vt vocabulary tiles of 256 on n_units CTA pairs (`deep`: D >= SW_DEEP):
+// up to one chunk, where W is streamed once and the launch is bound by HBM; two chunks of up to 192 rows, whose row-major
+// tiles would be 384 padded rows; and, up to 1024 rows, counts that cut into chunks of 208 to 240 rows, i.e. whose row-major
+// tiles would carry 64 or more padded rows per pair (swapped against row-major, one chunk at a time, us: D = 4096, V = 126464:
+// 416 rows 333 / 380, 448 rows 415 / 462, 480 rows 410 / 428, 512 rows 425 / 421; D = 3584, V = 152064: 704 rows 625 / 650, 832 rows
+// 784 / 840, 960 rows 851 / 895).
+// Two chunks of up to 192 rows, greedy, both chunks at a time up to 320 rows, above, where two accumulators are all that fit, one
+// at a time; us, swapped / row-major, D = 4096, V = 126464.  On the power cap, where a rollout's steps are and padded MMAs cost
+// twice: 272 rows 310 / 395, 320 rows 329 / 405, 352 rows 375 / 412, 384 rows 386 / 422.  A launch on an idle GPU: 242 / 291, 261 / 295,
+// but 307 / 295, 312 / 298.  D = 3584, V = 152064, capped 331 / 409, 361 / 430, 405 / 435, 410 / 441, idle 266 / 298, 290 / 305, 321 / 306,
+// 327 / 310: the rule is made for the cap, and above 320 rows a single launch pays 4 to 6 % for it.
+// Where the MMAs of a tile are short or tiles are few, the epilogue shows, and the cap is out of reach: 272 / 384 rows x 1024 x
+// 126464 101 / 83 and 116 / 90, x 2048 x 126464 178 / 180 and 203 / 188, 320 rows x 2048 x 64000 103 / 91, x 2048 x 32000 55 / 49, 384 rows
+// x 64 x 1300 16.4 / 10.3, 320 rows x 3072 x 80000 171 / 151: two chunks begin at SW_DEEP and at SW_MIN_TILES per pair (320 rows x 4096
+// x 32000 95.5 / 95.2, x 64000 168 / 171, x 3584 x 60000 146 / 144).
+// Sampled (four times the epilogue): one chunk at a time, capped 272 rows x 4096 x 126464 383 / 404, 320 rows 394 / 418, 384 rows
+// 418 / 435, 480 rows 463 / 459, 640 rows 611 / 621, 832 rows 760 / 788, idle 315 / 319, 322 / 324, 349 / 339, 396 / 397, 533 / 525.  Where
+// that is not hidden one row-major pair is better than a chunk from about 170 rows on: 160 rows x 2048 x 32000 46.0 / 47.1, 200 rows
+// 54.5 / 47.3, 256 rows 58.9 / 47.7, 640 rows 115 / 92, x 2048 x 64000 256 rows 97 / 79, x 4096 x 50000 160 rows 94 / 100, 200 rows
+// 110 / 105; and 97 to 128 rows where pairs need a second round and single CTAs do not (x 2048 x 24000: 96 rows 35.1 / 34.0, 112 rows
+// 38.9 / 34.2).
 constexpr int LM_JOINT_ROWS = 320;
 constexpr int LM_SWAPPED_ROWS = 384;
-__host__ __device__ inline bool lm_joint(int rows, bool sampled) { return !sampled && rows > SW_NMAX && rows <= LM_JOINT_ROWS; }
-__host__ __device__ inline bool lm_swapped(int rows, bool sampled) {
-    if (rows <= LM_SWAPPED_ROWS) return true;
+constexpr int SW_MIN_TILES = 3, SW_MIN_TILES_SAMPLED = 4;
+constexpr int SW_DEEP = 3584;
+__host__ __device__ inline bool lm_joint(int rows, int n_vt, int n_units, bool deep, bool sampled) {
+    return !sampled && rows > SW_NMAX && rows <= LM_JOINT_ROWS && deep && n_vt >= SW_MIN_TILES * n_units;
+}
+__host__ __device__ inline bool lm_swapped(int rows, int n_vt, int n_units, bool deep, bool sampled) {
+    if (sampled && (!deep || n_vt < SW_MIN_TILES_SAMPLED * n_units))
+        return rows <= 160 && !(rows > 96 && rows <= 128 && n_vt > n_units && n_vt <= 2 * n_units);
+    if (rows <= SW_NMAX) return true;
+    if (rows <= LM_SWAPPED_ROWS) return deep && n_vt >= SW_MIN_TILES * n_units;
     if (rows > 1024) return false;
     const int n_chunks = (rows + SW_NMAX - 1) / SW_NMAX;
     const int nc = ((rows + n_chunks - 1) / n_chunks + 15) & ~15;      // as in sw_plan below
@@ -720,14 +739,14 @@ __device__ __forceinline__ SwBoxes sw_boxes(int rows_half) {
 // How `rows` live rows are cut up for a grid of n_units CTA pairs and n_vt vocabulary tiles of 256 (the same
 // formula on the host, in the GEMM and in the merge kernels).
 struct SwPlan { int n_chunks, nc, groups, parts; bool joint; };
-__host__ __device__ inline SwPlan sw_plan(int rows, int n_units, int n_vt, bool sampled) {
+__host__ __device__ inline SwPlan sw_plan(int rows, int n_units, int n_vt, bool deep, bool sampled) {
     SwPlan p;
     p.n_chunks = (rows + SW_NMAX - 1) / SW_NMAX;
     if (p.n_chunks < 1) p.n_chunks = 1;
     const int per = (rows + p.n_chunks - 1) / p.n_chunks;
     p.nc = (per + 15) & ~15;                             // rows per chunk: N of the pair's MMA
     if (p.nc < 16) p.nc = 16;
-    p.joint = lm_joint(rows, sampled);
+    p.joint = lm_joint(rows, n_vt, n_units, deep, sampled);
     p.groups = lm_groups(n_units, p.joint ? 1 : p.n_chunks, n_vt);
     p.parts = SW_PARTS_PER_GROUP * p.groups;
     return p;
@@ -743,7 +762,7 @@ lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, 
     const int rank = static_cast<int>(cluster_cta_rank());
     const int unit = blockIdx.x >> 1;
     const int n_units = gridDim.x >> 1;
-    const SwPlan plan = sw_plan(Mc, n_units, n_vt, SAMPLE);
+    const SwPlan plan = sw_plan(Mc, n_units, n_vt, D >= SW_DEEP, SAMPLE);
     constexpr int J = JOINT ? 2 : 1;                     // chunks per W tile
     constexpr bool STATE = sw_values(MODE, JOINT) > 0;   // running values in shared memory
     constexpr int NV = sw_values(MODE, JOINT), NS = J * SW_NMAX, WARP_STATE = NV * NS;
@@ -1119,12 +1138,12 @@ lmhead_head_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
     }
     const int Mc = live_rows ? *live_rows : M;          // rows that need logits (uniform over the grid)
     if constexpr (MODE == LM_GREEDY) {
-        if (lm_joint(Mc, false)) {
+        if (lm_joint(Mc, n_tiles, gridDim.x >> 1, D >= SW_DEEP, false)) {
             lm_joint_body(tmap_w, xmaps, Mc, D, V, mask_col, n_tiles, part_max, part_sum, part_arg, dev_status, parts_stride, smp);
             return;
         }
     }
-    if (lm_swapped(Mc, MODE == LM_SAMPLE)) {
+    if (lm_swapped(Mc, n_tiles, gridDim.x >> 1, D >= SW_DEEP, MODE == LM_SAMPLE)) {
         lm_swapped_body<MODE, false>(tmap_w, xmaps, Mc, D, V, mask_col, n_tiles, part_max, part_sum, part_arg, dev_status,
                                      parts_stride, smp);
         return;
@@ -1157,14 +1176,15 @@ lmhead_head_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
 
 // Partials of live row `row`, as the GEMM that ran wrote them (they start at row * stride).  layout 0 / 1: the
 // stand-alone row-major kernels (single CTAs only / CTA pairs where they apply), one partial per vocabulary group,
-// packed (stride = count).  layout 2: lmhead_head_kernel's rules.  `grid` = CTAs of the GEMM launch, n_tiles =
-// vocabulary tiles of 256.
-constexpr int LM_LAYOUT_GREEDY = 2;
+// packed (stride = count).  layout 2 / 3: lmhead_head_kernel's rules for D below SW_DEEP / from there on.  `grid` = CTAs of the
+// GEMM launch, n_tiles = vocabulary tiles of 256.
+constexpr int LM_LAYOUT_HEAD = 2, LM_LAYOUT_HEAD_DEEP = 3;
 __host__ __device__ inline int lm_row_partials(int layout, int grid, int rows, int n_tiles, int row, bool sampled) {
     const int m_tiles = (rows + BM - 1) / BM;
-    if (layout != LM_LAYOUT_GREEDY) return lm_groups_mode(grid, m_tiles, n_tiles, layout);
+    if (layout < LM_LAYOUT_HEAD) return lm_groups_mode(grid, m_tiles, n_tiles, layout);
+    const bool deep = layout == LM_LAYOUT_HEAD_DEEP;
     const int n_clusters = grid >> 1;
-    if (lm_swapped(rows, sampled)) return sw_plan(rows, n_clusters, n_tiles, sampled).parts;
+    if (lm_swapped(rows, n_tiles, n_clusters, deep, sampled)) return sw_plan(rows, n_clusters, n_tiles, deep, sampled).parts;
     if ((m_tiles & 1) == 0) return lm_groups(n_clusters, m_tiles >> 1, n_tiles);
     if (n_clusters < 2) return lm_groups(grid, m_tiles, n_tiles);
     const int p = m_tiles >> 1;
@@ -1477,7 +1497,7 @@ static int launch_head(const dare_ctx* ctx, int grid, bool pairs, const void* x_
         smp.part_y = reinterpret_cast<float*>(part_arg + n_part);
         smp.part_zb = smp.part_y + n_part;
     }
-    int rc = DARE_OK, layout = LM_LAYOUT_GREEDY, parts_stride = -1, grid_gemm = grid;
+    int rc = DARE_OK, layout = D >= SW_DEEP ? LM_LAYOUT_HEAD_DEEP : LM_LAYOUT_HEAD, parts_stride = -1, grid_gemm = grid;
     if (pairs) {
         CUtensorMap tmap_w;
         SwXMaps xm;

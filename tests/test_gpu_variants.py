@@ -368,23 +368,66 @@ def test_dual_loop_equals_its_parts(ctx, k, mode):
     assert torch.equal(tok2, tok) and torch.equal(kc2, kc) and torch.equal(vc2, vc)
 
 
-# 257 to 320 rows: two chunks of rows against each vocabulary tile; up to 384: one after the other.  The
-# ranges' edges, tiles of fewer than 256 entries, fewer tiles than CTA pairs and enough for every accumulator to come round.
+# 257 to 384 rows on row-major tiles and, with D = 3584 and 57000 entries, in two chunks: up to 320 rows both against each
+# vocabulary tile, above one after the other.  The ranges' edges, tiles of fewer than 256 entries, fewer tiles than CTA
+# pairs and enough for every accumulator to come round.
 @pytest.mark.parametrize("M", [256, 257, 288, 289, 320, 321, 335, 352, 353, 384, 385])
-@pytest.mark.parametrize("V", [100, 1300, 100_000])
-def test_greedy_head_on_two_chunks(ctx, M, V):
-    D, mu = 72, V - 3
-    x, w = I.normal_bf16(M, I.TID_X, (M, D)).cuda(), I.normal_bf16(V, I.TID_W, (V, D), 0.2).cuda()
+@pytest.mark.parametrize("D,V", [(72, 100), (72, 1300), (72, 100_000), (3584, 57_001)])
+def test_greedy_head_of_two_chunks_of_rows(ctx, M, D, V):
+    mu = V - 3
+    x, w = I.normal_bf16(M, I.TID_X, (M, D)).cuda(), I.normal_bf16(V, I.TID_W, (V, D), 1.7 / D ** 0.5).cuda()
     pred, conf = dare.dare_lmhead_confidence(ctx, x, w, None, mu, True)
     torch.cuda.synchronize()
     z = x.double() @ w.double().T
     z[:, mu] = -float("inf")
     best = z.max(1).values
-    # an fp32 logit of 72 products is off by up to 72 * 2^-24 * sum |x w| (about 10): 5e-5; the exponentials by less
+    # an fp32 logit of 72 products is off by up to 72 * 2^-24 * sum |x w| (about 10): 5e-5; of 3584, added 16 at a time to partial
+    # sums of a few units, by 224 * 2^-22: 6e-5; the exponentials by less
     assert (best - z.gather(1, pred.long()[:, None])[:, 0] <= 1e-4).all()
     want = torch.exp(best - torch.logsumexp(z, 1))
     assert torch.allclose(conf.double(), want, rtol=2e-4, atol=0)
     assert ctx.device_status() == 0
+
+
+# Two chunks of rows only at D >= 3584 and three vocabulary tiles of 256 per CTA pair (222 on 148 SMs), four for the sampled head:
+# both sides of these lines, at the edges of the row ranges.  A row's answer does not depend on the path: the rows a few at
+# a time (row_tokens picks them, the generator is keyed by a row's place) give the same tokens.
+@pytest.mark.parametrize("D,V", [(3576, 57_000), (3584, 221 * 256), (3584, 221 * 256 + 1), (3584, 295 * 256), (3584, 295 * 256 + 40)])
+def test_heads_at_the_edges_of_the_two_chunk_rules(ctx, D, V):
+    mu, big = 5, 512
+    g = torch.Generator(device="cuda").manual_seed(V)
+    w = torch.randn(V, D, generator=g, device="cuda").mul_(0.05).bfloat16()
+    x = torch.randn(big, D, generator=g, device="cuda").bfloat16()
+    for M in (97, 112, 128, 160, 161, 256, 257, 272, 320, 321, 352, 384, 385, 400, 480):
+        for temperature in (0.0, 0.8):
+            head = (lambda r: dare.dare_lmhead_sample(ctx, x[:M], w, r, mu, True, temperature, 5, 3)) if temperature else \
+                   (lambda r: dare.dare_lmhead_confidence(ctx, x[:M], w, r, mu, True))
+            pred, conf = head(None)
+            for lo in range(0, M, 90):
+                row = torch.full((M,), 7, dtype=torch.int32, device="cuda")
+                row[lo:lo + 90] = mu
+                p, c = head(row)
+                assert torch.equal(p[lo:lo + 90], pred[lo:lo + 90])
+                assert torch.allclose(c[lo:lo + 90], conf[lo:lo + 90], rtol=2e-5, atol=0)      # (sums of 57000 exponentials, cut differently)
+        z = x[:M].float() @ w.float().T
+        z[:, mu] = -float("inf")
+        greedy, conf = dare.dare_lmhead_confidence(ctx, x[:M], w, None, mu, True)
+        # fp32 sums of 3584 products of size 0.05: 3584 * 2^-24 * 3584 * 0.03 at the worst, far less in fact
+        assert (z.max(1).values - z.gather(1, greedy.long()[:, None])[:, 0] <= 1e-3).all()
+        assert torch.allclose(conf, torch.softmax(z, 1).max(1).values, rtol=2e-3, atol=0)
+    assert ctx.device_status() == 0
+
+
+# Where little hides the epilogue, 300 and 384 rows run as three row-major tiles, and cost what 512 rows as four do (18 against 12 us
+# here in two chunks).
+@pytest.mark.parametrize("D,V", [(512, 2048), (64, 1300)])
+def test_greedy_head_of_three_tiles_costs_no_more_than_of_four(ctx, D, V):
+    w, us = torch.randn(V, D, device="cuda").mul(0.02).bfloat16(), {}
+    for M in (300, 384, 512):
+        x = torch.randn(M, D, device="cuda").bfloat16()
+        pred, conf = torch.empty(M, dtype=torch.int32, device="cuda"), torch.empty(M, device="cuda")
+        us[M] = _us(lambda: dare.dare_lmhead_confidence(ctx, x, w, None, 3, True, pred, conf))
+    assert us[300] <= 1.2 * us[512] and us[384] <= 1.2 * us[512]
 
 
 # The rotary kernel on its own: heads that leave the last batch of a thread part full, more heads than one pass takes, and
