@@ -215,10 +215,10 @@ int gemm_few_describe(int epi, int M, int N, int K, int sm_count, int* out);
 int gemm_plan_describe(const dare_ctx* ctx, int epi, int M, int N, int K, int* out);
 int launch_embed(const void* emb, int D, int V, const int32_t* tokens, int64_t row_stride, int start, int length,
                  int n_rows, void* x, cudaStream_t stream);
-int launch_rmsnorm(const void* x, int D, int n_rows, float eps, void* y, cudaStream_t stream);
+int launch_rmsnorm(const void* x, int D, int n_rows, float eps, void* y, int sm_count, cudaStream_t stream);
 // cs [n_pos][half] and cs_t [half][n_pos]: (cos, sin) pairs
 int launch_rope_table(float* cs, float* cs_t, int n_pos, int half, double base, cudaStream_t stream);
 int launch_rope_kv_write(const void* qkv, int n_rows, int Hq, int Hkv, int d, int start, int length, const float* cs,
-                         void* q_out, void* k_cache, void* v_cache, int cap, cudaStream_t stream);
+                         void* q_out, void* k_cache, void* v_cache, int cap, int sm_count, cudaStream_t stream);
 
 }  // namespace dare

@@ -195,9 +195,12 @@ rope_kv_write_kernel(const __nv_bfloat16* __restrict__ qkv, int n_rows, int row_
 
 // Shared memory (unused) that a small kernel of `ctas` short CTAs asks for: set up while a projection still runs, its
 // CTAs would pile up on the few SMs that the projection leaves idle (sixteen per SM on 8 of 148 at 512 x 12288: the RoPE
-// kernel then took 19 us instead of 7.4).  With 45 KB each none fits beside a projection's CTA and five fill an SM.
-constexpr size_t SPREAD_SMEM = 45 * 1024;
-inline size_t spread_smem(int ctas) { return ctas <= 5 * 148 ? SPREAD_SMEM : 0; }
+// kernel then took 19 us instead of 7.4).  With 44 KB each none fits beside a CTA of the pair kernel, two beside one of the
+// few-row kernel's, and SPREAD_CTAS on an SM of their own; more CTAs than that ask for none, all are resident at once then.
+constexpr size_t SPREAD_SMEM = 44 * 1024;
+constexpr int SPREAD_CTAS = 5;
+static_assert(SPREAD_CTAS * (SPREAD_SMEM + 1024 + 128) <= 228 * 1024, "the system takes 1 KB per CTA, RMSNorm 16 bytes");
+inline size_t spread_smem(int ctas, int sm_count) { return ctas <= SPREAD_CTAS * sm_count ? SPREAD_SMEM : 0; }
 
 // Rows for which a warp each is the better split.  CTAs start at about one per ns over the GPU, whatever they do: 65536 rows
 // of 256 took 68 us with one each and take 9.3, 16384 of 1024 17.5 and 7.0, 4096 of 512 4.7 and 2.4.  Longer rows are bound
@@ -224,7 +227,7 @@ int launch_embed(const void* emb, int D, int V, const int32_t* tokens, int64_t r
                          static_cast<uint4*>(x));
 }
 
-int launch_rmsnorm(const void* x, int D, int n_rows, float eps, void* y, cudaStream_t stream) {
+int launch_rmsnorm(const void* x, int D, int n_rows, float eps, void* y, int sm_count, cudaStream_t stream) {
     const uint4* src = static_cast<const uint4*>(x);
     uint4* dst = static_cast<uint4*>(y);
     if (norm_warp_rows(n_rows, D)) {
@@ -233,7 +236,7 @@ int launch_rmsnorm(const void* x, int D, int n_rows, float eps, void* y, cudaStr
         return launch_kernel(kernel, dim3((n_rows + ROWS_PER_BLOCK - 1) / ROWS_PER_BLOCK), ROWS_PER_BLOCK * 32, 0, stream, 1, src, D / 8,
                              n_rows, eps, dst);
     }
-    return launch_kernel(rmsnorm_kernel, dim3(n_rows), NORM_THREADS, spread_smem(n_rows), stream, 1, src, D / 8, eps, dst);
+    return launch_kernel(rmsnorm_kernel, dim3(n_rows), NORM_THREADS, spread_smem(n_rows, sm_count), stream, 1, src, D / 8, eps, dst);
 }
 
 int launch_rope_table(float* cs, float* cs_t, int n_pos, int half, double base, cudaStream_t stream) {
@@ -243,11 +246,11 @@ int launch_rope_table(float* cs, float* cs_t, int n_pos, int half, double base, 
 }
 
 int launch_rope_kv_write(const void* qkv, int n_rows, int Hq, int Hkv, int d, int start, int length, const float* cs,
-                         void* q_out, void* k_cache, void* v_cache, int cap, cudaStream_t stream) {
+                         void* q_out, void* k_cache, void* v_cache, int cap, int sm_count, cudaStream_t stream) {
     const int row_threads = rope_row_threads(Hq, Hkv, d), rows = ROPE_THREADS / row_threads;
     const int ctas = (n_rows + rows - 1) / rows;
     return launch_kernel(row_threads == ROPE_THREADS ? rope_kv_write_kernel<true> : rope_kv_write_kernel<false>, dim3(ctas),
-                         rows * row_threads, spread_smem(ctas), stream, 1, static_cast<const __nv_bfloat16*>(qkv), n_rows,
+                         rows * row_threads, spread_smem(ctas, sm_count), stream, 1, static_cast<const __nv_bfloat16*>(qkv), n_rows,
                          row_threads, Hq, Hkv, d, start, length, reinterpret_cast<const float2*>(cs),
                          static_cast<__nv_bfloat16*>(q_out), static_cast<__nv_bfloat16*>(k_cache),
                          static_cast<__nv_bfloat16*>(v_cache), cap);

@@ -58,7 +58,7 @@ int forward_rows(dare_model* m, const int32_t* tokens, int B, int64_t row_stride
         const dare_layer_weights& w = m->layers[l];
         __nv_bfloat16* kc = static_cast<__nv_bfloat16*>(k_cache) + layer_kv * l;
         __nv_bfloat16* vc = static_cast<__nv_bfloat16*>(v_cache) + layer_kv * l;
-        rc = launch_rmsnorm(m->x, c.hidden, rows, c.rms_eps, m->h, s);
+        rc = launch_rmsnorm(m->x, c.hidden, rows, c.rms_eps, m->h, m->ctx->sm_count, s);
         if (rc != DARE_OK) return rc;
         if (gemm_takes_rope(rows, nq + 2 * nkv)) {
             const RopeArgs rope = {c.n_q_heads, c.n_kv_heads, c.head_dim, start, length, cap, m->rope_cs, m->rope_cs_t,
@@ -70,7 +70,7 @@ int forward_rows(dare_model* m, const int32_t* tokens, int B, int64_t row_stride
                              nq + 2 * nkv, s, nullptr, true);
             if (rc == DARE_OK)
                 rc = launch_rope_kv_write(m->qkv, rows, c.n_q_heads, c.n_kv_heads, c.head_dim, start, length, m->rope_cs,
-                                          m->q, kc, vc, cap, s);
+                                          m->q, kc, vc, cap, m->ctx->sm_count, s);
         }
         if (rc != DARE_OK) return rc;
         AttnArgs a;
@@ -85,14 +85,14 @@ int forward_rows(dare_model* m, const int32_t* tokens, int B, int64_t row_stride
         if (rc != DARE_OK) return rc;
         rc = launch_gemm(m->ctx, GEMM_EPI_RESIDUAL, m->attn, rows, nq, w.wo, nullptr, c.hidden, m->x, m->x, c.hidden, s, nullptr, true);
         if (rc != DARE_OK) return rc;
-        rc = launch_rmsnorm(m->x, c.hidden, rows, c.rms_eps, m->h, s);
+        rc = launch_rmsnorm(m->x, c.hidden, rows, c.rms_eps, m->h, m->ctx->sm_count, s);
         if (rc != DARE_OK) return rc;
         rc = launch_gemm(m->ctx, GEMM_EPI_SWIGLU, m->h, rows, c.hidden, w.wg, w.wu, c.ffn, m->act, nullptr, c.ffn, s, nullptr, true);
         if (rc != DARE_OK) return rc;
         rc = launch_gemm(m->ctx, GEMM_EPI_RESIDUAL, m->act, rows, c.ffn, w.wd, nullptr, c.hidden, m->x, m->x, c.hidden, s, nullptr, true);
         if (rc != DARE_OK) return rc;
     }
-    return launch_rmsnorm(m->x, c.hidden, rows, c.rms_eps, hidden_out ? hidden_out : m->h, s);
+    return launch_rmsnorm(m->x, c.hidden, rows, c.rms_eps, hidden_out ? hidden_out : m->h, m->ctx->sm_count, s);
 }
 
 int check_rows(const dare_model* m, const void* tokens, int B, int64_t row_stride, int start, int length, int kv_len,
@@ -242,7 +242,7 @@ int dare_rmsnorm(dare_ctx* ctx, const void* x, int n_rows, int D, float eps, voi
     if (n_rows < 1 || D < 8 || D % 8) return DARE_ERR_SHAPE;
     if (!(eps >= 0.f)) return DARE_ERR_RANGE;
     if ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y)) & 15u) return DARE_ERR_ALIGN;
-    return dare::launch_rmsnorm(x, D, n_rows, eps, y, static_cast<cudaStream_t>(stream));
+    return dare::launch_rmsnorm(x, D, n_rows, eps, y, ctx->sm_count, static_cast<cudaStream_t>(stream));
 }
 
 int dare_rope_kv_write(dare_model* m, const void* qkv, int B, int length, int start, void* q_out, void* k_cache,
@@ -256,7 +256,7 @@ int dare_rope_kv_write(dare_model* m, const void* qkv, int B, int length, int st
                            reinterpret_cast<uintptr_t>(k_cache) | reinterpret_cast<uintptr_t>(v_cache);
     if (bits & 15u) return DARE_ERR_ALIGN;
     return dare::launch_rope_kv_write(qkv, B * length, m->desc.n_q_heads, m->desc.n_kv_heads, m->desc.head_dim, start,
-                                      length, m->rope_cs, q_out, k_cache, v_cache, cache_cap,
+                                      length, m->rope_cs, q_out, k_cache, v_cache, cache_cap, m->ctx->sm_count,
                                       static_cast<cudaStream_t>(stream));
 }
 
