@@ -1,13 +1,14 @@
 // Projections of up to 128 rows: out = epilogue(A W^T), A [M, K], W [N, K] bf16, fp32 accumulation.
 //
 // With so few rows the work is reading W once, so everything serves that stream (one rollout's block of 32 rows against
-// the layers of the LLaDA shape, us per launch, this kernel / row-major tiles of 128 padded rows: QKV 12288 x 4096 21.3 / 29.6,
-// attention-out 4096 x 4096 12.2 / 19.0, gate and up 2 x 12288 x 4096 38.9 / 43.4, down 4096 x 12288 17.8 / 38.9; W alone takes
-// 15.4, 5.1, 30.7 and 15.4 at the measured copy bandwidth):
+// the layers of the LLaDA shape, us per launch, this kernel / row-major tiles of 128 padded rows, weights from HBM: 12288 x 4096
+// 19.6 / 29.6, attention-out 4096 x 4096 10.8 / 18.2, gate and up 2 x 12288 x 4096 35.1 / 42.5, down 4096 x 12288 20.9 / 38.9; W alone
+// takes 15.4, 5.1, 30.7 and 15.4 at the measured copy bandwidth; of 128 rows 25.7 / 31.0, 16.8 / 18.6, 41.6 / 43.0, 27.3 / 39.9):
 //   * operands swapped: 128 W rows are the MMA's A operand (the accumulator's lanes), the rows of A its N columns, so no
 //     padded rows are loaded or multiplied and a ring slot is mostly W;
-//   * 128-row W tiles are cut along K until the CTAs fill the SMs twice over: two CTAs per SM keep up to 150 KB of W in
-//     flight, and one CTA's first and last microseconds lie under the other's stream;
+//   * 128-row W tiles are cut along K until the CTAs fill the SMs twice over: two CTAs per SM keep 192 KB of W in flight at 16
+//     rows (six slots of 16 KB each), 160 KB at 17 to 48, 96 KB at 128, and one CTA's first and last microseconds lie under
+//     the other's stream;
 //   * the first ring of W is requested before the kernel waits for its predecessor (w_static: weights, which no kernel
 //     of the library writes), so the stream does not stop between kernels;
 //   * the CTAs of a tile's K slices form a cluster; each sends the accumulator columns (rows of A) it does not own to their
@@ -54,8 +55,10 @@ FewPlan few_plan(int epi, int M, int N, int K, int sm_count) {
     p.tiles = (N + p.wcols - 1) / p.wcols;
     const int nk = (K + FK - 1) / FK;
     p.splits = 1;
-    // as many K slices as the SMs take with two CTAs each, of at least two K blocks
-    while (p.splits < 8 && 2LL * p.splits * p.tiles <= 2LL * sm_count && nk >= 4 * p.splits) p.splits *= 2;
+    // as many K slices as the SMs take with two CTAs each, of at least two K blocks, and of more with more than 64 rows, whose
+    // exchange takes longer (128 rows, K = 1024, N = 4096: eight slices 13.0 us, two 9.6; K = 512, N = 1280: 6.7 either way)
+    const int least = p.nr > 64 ? p.nr / 16 : 2;
+    while (p.splits < 8 && 2LL * p.splits * p.tiles <= 2LL * sm_count && nk >= 2 * least * p.splits) p.splits *= 2;
     const int stages = FEW_RING / (FEW_W_BYTES + p.nr * FK * 2);
     p.stages = stages > FEW_MAX_STAGES ? FEW_MAX_STAGES : stages;
     return p;
@@ -77,6 +80,9 @@ __device__ __forceinline__ uint4 pack8(const float (&f)[8]) {
     return make_uint4(pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]), pack_bf16(f[4], f[5]), pack_bf16(f[6], f[7]));
 }
 __device__ __forceinline__ float round_bf16(float v) { return __bfloat162float(__float2bfloat16_rn(v)); }
+__device__ __forceinline__ void st_shared_f32(uint32_t addr, uint32_t v) {
+    asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
 __device__ __forceinline__ void st_shared_cluster_f32(uint32_t addr, uint32_t v) {
     asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
@@ -184,26 +190,46 @@ gemm_few_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
     if (p.splits > 1) cluster_sync_all();
     else __syncthreads();
     if (warp >= 2) {
+        // (owner and row are counted, not divided out, and 16 columns are read at a time: with two divisions per column and
+        // every 8 columns waited for, each row cost 68 ns, 128 rows 8.6 us)
         const int f = (warp & 3) * 32 + lane;            // W row of the tile = TMEM lane
         const uint32_t taddr = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16);
         const uint32_t slab = smem_u32(tiles) + (static_cast<uint32_t>(split) * per_owner * FW + f) * 4;
-        for (int c0 = 0; c0 < p.nr; c0 += 8) {
-            uint32_t v[8];
-            tmem_ld_8cols(taddr + c0, v);
+        const auto read16 = [&](int c0, uint32_t (&lo)[8], uint32_t (&hi)[8]) {
+            tmem_ld_8cols(taddr + c0, lo);
+            tmem_ld_8cols(taddr + c0 + 8, hi);
             tmem_ld_wait();
+        };
+        uint32_t lo[8], hi[8];
+        if (p.splits == 1) {
+            for (int c0 = 0; c0 < g.M; c0 += 16) {       // (columns from M on are padding rows: stored, not read)
+                read16(c0, lo, hi);
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                const int owner = (c0 + c) / per_owner, r = (c0 + c) - owner * per_owner;
-                const uint32_t local = slab + static_cast<uint32_t>(r) * (FW * 4);
-                if (c0 + c < g.M)
-                    st_shared_cluster_f32(p.splits > 1 ? cluster_map_shared(local, static_cast<uint32_t>(owner)) : local, v[c]);
+                for (int c = 0; c < 16; ++c) st_shared_f32(slab + static_cast<uint32_t>(c0 + c) * (FW * 4), c < 8 ? lo[c & 7] : hi[c & 7]);
+            }
+        } else {
+            int owner = 0, r = 0;
+            uint32_t addr = cluster_map_shared(slab, 0u);
+            for (int c0 = 0; c0 < g.M; c0 += 16) {
+                read16(c0, lo, hi);
+#pragma unroll
+                for (int c = 0; c < 16; ++c) {
+                    if (c0 + c < g.M) st_shared_cluster_f32(addr, c < 8 ? lo[c & 7] : hi[c & 7]);
+                    addr += FW * 4;
+                    if (++r == per_owner) {
+                        r = 0;
+                        if (++owner < p.splits) addr = cluster_map_shared(slab, static_cast<uint32_t>(owner));
+                    }
+                }
             }
         }
     }
     if (p.splits > 1) cluster_sync_all();
     else __syncthreads();
 
-    if (warp >= 2 && !*abort_flag) {
+    // the last part is for all warps (the first two have not waited for the predecessor with all their lanes yet)
+    if (warp < 2) pdl_wait();
+    if (!*abort_flag) {
         const float* slab = reinterpret_cast<const float*>(tiles);
         // 8 features from feature c of row r, the K slices added in order
         const auto sum8 = [&](int r, int c, float (&s)[8]) {
@@ -216,13 +242,13 @@ gemm_few_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
                 s[4] += b.x; s[5] += b.y; s[6] += b.z; s[7] += b.w;
             }
         };
-        const int t = threadIdx.x - 64;
+        const int t = threadIdx.x;
         const int row0 = split * per_owner;
         const int n_rows = min(per_owner, g.M - row0);   // (may be negative: nothing to do)
         if (EPI == GEMM_EPI_ROPE) {
             const RopeArgs& r = g.rope;
             const int gph = r.d / 16;                    // 8-channel groups of half a head
-            for (int i = t; i < n_rows * (FW / 16); i += 128) {
+            for (int i = t; i < n_rows * (FW / 16); i += FEW_THREADS) {
                 const int rr = i / (FW / 16), q = i % (FW / 16);
                 const int hh = q / gph, c = (q % gph) * 8;
                 const int H = tile * (FW / r.d) + hh, m = row0 + rr;
@@ -254,25 +280,36 @@ gemm_few_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
                 *reinterpret_cast<uint4*>(dst + r.d / 2 + c) = pack8(b);
             }
         } else {
-            const int groups = p.wcols / 8;
-            for (int i = t; i < n_rows * groups; i += 128) {
-                const int rr = i / groups, c = (i % groups) * 8;
-                const int col = tile * p.wcols + c;
-                if (col >= g.N) continue;                // (N is a multiple of 8)
-                float a[8];
-                sum8(rr, c, a);
-                const size_t off = static_cast<size_t>(row0 + rr) * g.ldo + col;
-                if (EPI == GEMM_EPI_SWIGLU) {
-                    float u[8];
-                    sum8(rr, FW / 2 + c, u);
+            constexpr int groups = (EPI == GEMM_EPI_SWIGLU ? FW / 2 : FW) / 8;
+            constexpr int BATCH = EPI == GEMM_EPI_RESIDUAL ? 4 : 2;      // items in work at a time (residuals: on their way together)
+            for (int i0 = t; i0 < n_rows * groups; i0 += FEW_THREADS * BATCH) {
+                uint4 x[BATCH];
+                if (EPI == GEMM_EPI_RESIDUAL) {
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) a[j] = __fdividef(a[j], 1.0f + __expf(-a[j])) * u[j];    // silu(gate) * up
-                } else if (EPI == GEMM_EPI_RESIDUAL) {
-                    const uint4 x = *reinterpret_cast<const uint4*>(g.res + off);
-                    a[0] += lo_f(x.x); a[1] += hi_f(x.x); a[2] += lo_f(x.y); a[3] += hi_f(x.y);
-                    a[4] += lo_f(x.z); a[5] += hi_f(x.z); a[6] += lo_f(x.w); a[7] += hi_f(x.w);
+                    for (int u = 0; u < BATCH; ++u) {
+                        const int i = i0 + u * FEW_THREADS, col = tile * p.wcols + (i % groups) * 8;
+                        if (i < n_rows * groups && col < g.N)
+                            x[u] = *reinterpret_cast<const uint4*>(g.res + static_cast<size_t>(row0 + i / groups) * g.ldo + col);
+                    }
                 }
-                *reinterpret_cast<uint4*>(g.out + off) = pack8(a);
+#pragma unroll
+                for (int u = 0; u < BATCH; ++u) {
+                    const int i = i0 + u * FEW_THREADS, rr = i / groups, c = (i % groups) * 8;
+                    const int col = tile * p.wcols + c;
+                    if (i >= n_rows * groups || col >= g.N) continue;      // (N is a multiple of 8)
+                    float a[8];
+                    sum8(rr, c, a);
+                    if (EPI == GEMM_EPI_SWIGLU) {
+                        float up[8];
+                        sum8(rr, FW / 2 + c, up);
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) a[j] = __fdividef(a[j], 1.0f + __expf(-a[j])) * up[j];    // silu(gate) * up
+                    } else if (EPI == GEMM_EPI_RESIDUAL) {
+                        a[0] += lo_f(x[u].x); a[1] += hi_f(x[u].x); a[2] += lo_f(x[u].y); a[3] += hi_f(x[u].y);
+                        a[4] += lo_f(x[u].z); a[5] += hi_f(x[u].z); a[6] += lo_f(x[u].w); a[7] += hi_f(x[u].w);
+                    }
+                    *reinterpret_cast<uint4*>(g.out + static_cast<size_t>(row0 + rr) * g.ldo + col) = pack8(a);
+                }
             }
         }
     }
