@@ -576,9 +576,11 @@ PairPlan pair_plan(int epi, int M, int N, int K, int head_dim) {
                 // two accumulator buffers it runs beside the next main loop.  512 instead of 256 columns for gate and up of
                 // 8192 rows: prefill 11.73 against 11.55 ms.  For the others wider tiles' lower operand traffic weighs more
                 // (weight gradient of 126464 x 4096 x 2048 in 256 instead of 512 columns: +1.5 %; QKV of 512 rows in two
-                // rounds of 176 instead of one of 352: a generation +1.3 %).
-                const double cost = epi == GEMM_EPI_SWIGLU && bn <= 256 ? rounds * kb * per_kb + 2500.0 + epilogue
-                                                                        : rounds * (kb * per_kb + 2500.0 + epilogue);
+                // rounds of 176 instead of one of 352: a generation +1.3 %), and so it does for SwiGLU below 208 columns: two
+                // rounds against one of twice the width 57.7 / 54.7 us at 176 (256 rows, 2 x 12288 x 4096), 140 / 119 (768 rows,
+                // 2 x 4096 x 12288), 78 / 76 at 192, but 57.8 / 60.6 at 208, 31.6 / 35.2 at 224, 66.8 / 73.4 at 256.
+                const bool hidden = epi == GEMM_EPI_SWIGLU && bn >= 208 && bn <= 256;
+                const double cost = hidden ? rounds * kb * per_kb + 2500.0 + epilogue : rounds * (kb * per_kb + 2500.0 + epilogue);
                 if (cost < best_cost) {
                     best_cost = cost;
                     best.bn = bn; best.wcols = wcols; best.nmma = nmma; best.nchunk = nchunk; best.stages = stages;

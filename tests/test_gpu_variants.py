@@ -250,6 +250,16 @@ def test_steps_back_to_back_equal_their_parts(ctx, B, L, Hq, Hkv, P, workspace):
         c.close()
 
 
+# SwiGLU in two rounds of tiles only where they are 208 columns or wider: one round of 352 for gate and up of 256 rows (two of 176
+# take 5 to 9 % more), two of 208 and of 256 where one would be 416 or 512.
+@pytest.mark.parametrize("M,K,N,w_rows", [(256, 4096, 12288, 352), (768, 12288, 4096, 352), (256, 4096, 14336, 208), (256, 3584, 18944, 256)])
+def test_swiglu_tile_width(ctx, M, K, N, w_rows):
+    plan = dare.dare_linear_plan(ctx, dare.LINEAR_SWIGLU, M, K, N)
+    if plan["resident_clusters"] != 74:
+        pytest.skip("the widths are those of 148 SMs")
+    assert plan["w_rows"] == w_rows
+
+
 # Projections of up to 128 rows: one to eight K slices (a cluster), ragged last K block, last W tile part full, every row
 # padding; all epilogues.
 @pytest.mark.parametrize("M", [1, 15, 16, 17, 47, 96, 127, 128])
