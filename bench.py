@@ -45,8 +45,8 @@ NPOOL = 4   # distinct activation sets cycled through the steps
 NOMINAL_TFLOPS = 2250.0
 NOMINAL_HBM_GBS = 8000.0
 # dram__bytes_read.sum + dram__bytes_write.sum of one launch of the workload's dominant kernel, from the ncu
-# captures summarised under profiles/ (LM head: W leaves HBM once; dual-cache attention: the quarter-batch capture
-# scaled by the batch, traffic grows in proportion to the rollouts)
+# captures summarised under profiles/ (LM head: lmhead_head_kernel at 512 live rows, W leaves HBM once; dual-cache
+# attention: the quarter-batch capture scaled by the batch, traffic grows in proportion to the rollouts)
 DOMINANT_TRAFFIC_BYTES = {"llada8b": 1.0681e9, "dualcache": 4 * (1.3595e9 + 4.8e6)}
 EXTRA_WORKLOADS = ("dream7b", "dualcache", "llada_loop")
 

@@ -66,11 +66,10 @@ __device__ __forceinline__ void store_group(const float (&f)[8], const float (&u
 }
 
 // ---------------------------------------------------------------------------------------------------------
-// CTA-pair variant (cta_group::2), used when the problem has at least two row tiles.  The two CTAs of a cluster
-// compute one 256-row x bn-column tile with MMAs of M = 256: each CTA loads its own 128 rows of A and only HALF
-// of the W rows of every MMA (the tensor cores exchange the halves), and holds 128 rows x bn columns of the
-// accumulator.  Per flop a CTA writes and reads a third less shared memory than a single CTA computing a
-// 128-row tile, which is what limits the single-CTA kernel.  bn may exceed 256: the tile is then made of two
+// CTA pairs (cta_group::2), for more than 128 rows.  The two CTAs of a cluster compute one 256-row x bn-column tile with MMAs
+// of M = 256: each CTA loads its own 128 rows of A and only HALF of the W rows of every MMA (the tensor cores exchange the
+// halves), and holds 128 rows x bn columns of the accumulator.  Per flop a CTA writes and reads a third less shared memory
+// than a single CTA would for a 128-row tile.  bn may exceed 256: the tile is then made of two
 // MMAs of bn / 2 columns per K step.  SwiGLU: the even CTA loads the gate rows, the odd CTA the matching up rows,
 // so that every accumulator row holds [gate | up] column pairs.
 // K split (long K, few output tiles): two pairs form a cluster of four CTAs (ranks 0, 1 = first half of K, ranks 2,

@@ -145,8 +145,8 @@ int launch_lmhead_logprob(const dare_ctx* ctx, void* scratch, const void* hidden
                           const int32_t* targets, int32_t mask_id, int exclude_mask_column, float* logprob, float* lse_out,
                           cudaStream_t stream);
 // Sampling epilogue of the LM head (NULL = greedy): temperature, 64-bit seed and step counter of the generator.
-// step_dev (optional, device): added to `step`; the head's last kernel then increments it, so that a step replayed
-// from a CUDA graph draws fresh noise every time.
+// step_dev (optional, device): added to `step`; the head's last kernel then increments it, so that the steps of a loop, which
+// is enqueued ahead of the host, and replays of a captured step each draw fresh noise.
 struct LmSampleArgs { float temperature; uint64_t seed; uint32_t step; uint32_t* step_dev = nullptr; };
 size_t lmhead_workspace_bytes(int M, int D, int V, int sm_count, bool with_row_tokens, bool sampling);
 size_t lmhead_max_scratch_bytes(int M, int D, int V, int sm_count, bool sampling);

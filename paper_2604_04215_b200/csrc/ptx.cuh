@@ -75,10 +75,15 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
 // earlier kernel may have written and before its own first global write; since at least one CTA of each kernel does so
 // before it ends, a kernel's end implies the end of all kernels before it.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-// Lets the next kernel's CTAs be set up in the room this kernel leaves.  Called behind pdl_wait unless a comment says
-// otherwise, so that when a kernel's first instruction runs only its direct predecessor can still be running.  A kernel
-// that takes tensor memory calls it behind the allocation: a successor that takes tensor memory on the same SM can then
-// only wait for a CTA that has its share and will give it back.
+// Lets the next kernel's CTAs be set up in the room this kernel leaves.  Four kernels call it before they have waited:
+// lmhead_merge_kernel, lmhead_merge_select_kernel and unmask_select_kernel, whose successor may be the step's attention,
+// and that attention itself (AttnParams::beside_head), which waits in its last CTA only.  All others call it behind
+// pdl_wait.  So in front of its own pdl_wait a kernel may find everything still running back to the last kernel that
+// triggers behind its wait (that one included: behind a merge, its head; behind a step, its head, merge, selection and
+// attention), and may touch only what no kernel of the library writes: launch parameters, the rotary table, weights the caller
+// declares constant (w_static); the step's attention also its inputs, which the head, the merge and the selection do not
+// write.  A kernel that takes tensor memory calls pdl_trigger behind the allocation: a successor that takes tensor memory
+// on the same SM can then only wait for a CTA that has its share and will give it back.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Store to memory that the host polls while the kernel runs.

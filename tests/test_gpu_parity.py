@@ -274,8 +274,8 @@ def test_tiny_workload_eight_iterations(ctx):
 
 
 def test_step_replays_from_a_cuda_graph(ctx):
-    """The step forks its LM head onto a stream of the context and joins it back by events: captured into a CUDA graph
-    on the caller's stream, a replay must give what the eager call gives (tokens, counts, attention output)."""
+    """The step is a chain of kernels on the caller's stream, each of which may start before its predecessor ends: captured
+    into a CUDA graph, a replay must give what the eager call gives (tokens, counts, attention output)."""
     wl = I.WORKLOADS["tiny"]
     w = I.make_weights(wl)
     caches = I.make_caches(wl)

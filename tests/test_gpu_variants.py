@@ -50,8 +50,8 @@ def test_rope_in_the_projection_matches_the_separate_kernel(ctx, Hq, Hkv, d, B, 
     torch.cuda.synchronize()
     assert ctx.device_status() == 0
     # Both round q, k and v to bf16 before the rotation and once after it; the fp32 sums in front may differ in their
-    # last bits (another tile shape), which can move a value by one bf16 step (2^-8) before and one after: 2^-7 of the
-    # larger of the two channels that turn together, and v by one step.
+    # last bits (another tile shape), which can move a value by one bf16 step (up to 2^-7 of it) before and one after: 2^-6 of
+    # the larger of the two channels that turn together, and v by one step, 2^-7.
     k, k1, v, v1 = (t.float() for t in (caches[0], one[0], caches[1], one[1]))
     pair = torch.maximum(k1[..., :d // 2].abs(), k1[..., d // 2:].abs())
     assert ((k - k1).abs() <= 2.0 ** -6 * torch.cat([pair, pair], -1) + 1e-6).all()
@@ -369,12 +369,29 @@ def test_head_with_committed_rows(ctx, B, L, share):
     assert ctx.device_status() == 0
 
 
-@pytest.mark.parametrize("k", [1, 3, 7, 8, 20])
+# Blocks of 8, whose selection rides on the head's last kernel, and of 40, where a kernel of its own takes the decisions and
+# writes the counts that pace the host.
+LOOP_CASES = [(8, 1), (8, 3), (8, 7), (8, 8), (8, 20), (40, 3), (40, 17), (40, 40)]
+
+
+@pytest.mark.parametrize("L,k", LOOP_CASES)
 @pytest.mark.parametrize("mode", [dare.SELECT_TOPK, dare.SELECT_THRESHOLD])
-def test_dual_loop_equals_its_parts(ctx, k, mode):
-    """Blocks of 8 with some tokens given beforehand (one block whole): whatever the loop leaves out or enqueues ahead, the
+@pytest.mark.parametrize("temperature", [0.0, 0.7])
+def test_dual_loop_equals_its_parts(ctx, temperature, mode, L, k):
+    _loop_equals_its_parts(ctx, True, temperature, mode, L, k)
+
+
+@pytest.mark.parametrize("L,k", LOOP_CASES)
+@pytest.mark.parametrize("mode", [dare.SELECT_TOPK, dare.SELECT_THRESHOLD])
+@pytest.mark.parametrize("temperature", [0.0, 0.7])
+def test_prefix_loop_equals_its_parts(ctx, temperature, mode, L, k):
+    _loop_equals_its_parts(ctx, False, temperature, mode, L, k)
+
+
+def _loop_equals_its_parts(ctx, dual, temperature, mode, L, k):
+    """Blocks with some tokens given beforehand (one block whole): whatever the loop leaves out or enqueues ahead, the
     tokens, the steps and all K/V that the last forward of each position wrote are those of the calls it is made of."""
-    B, P, L, G = 2, 5, 8, 32
+    B, P, G = 2, 5, 4 * L if L == 8 else 2 * L
     T = P + G
     model = _small_model(ctx, 4, 2, 64, B * T, B, T)
     mask_id = 511
@@ -388,19 +405,71 @@ def test_dual_loop_equals_its_parts(ctx, k, mode):
     nr = torch.zeros(B, dtype=torch.int32, device="cuda")
 
     tok, (kc, vc), want = tok0.cuda(), new(), []
-    for start in range(P, T, L):
-        dare.dare_model_forward_window(model, tok, 0, T, T, kc, vc)
-        n = 0
+    if not dual:
+        dare.dare_model_forward(model, tok, 0, P, kc, vc)
+    for block, start in enumerate(range(P, T, L)):
+        if dual:
+            dare.dare_model_forward_window(model, tok, 0, T, T, kc, vc)
+        dare.dare_model_set_sampling(model, temperature, 99, block << 16)
+        n, seen = 0, T if dual else start + L
         while n == 0 or int(nr.sum()) > 0:
-            dare.dare_model_step_window(model, tok, start, L, T, kc, vc, mode, 0.9, k, pred, conf, None, nr)
+            dare.dare_model_step_window(model, tok, start, L, seen, kc, vc, mode, 0.9, k, pred, conf, None, nr)
             n += 1
         want.append(n)
-    dare.dare_model_forward_window(model, tok, T - L, L, T, kc, vc)
+        if not dual:
+            dare.dare_model_forward(model, tok, start, L, kc, vc)
+    if dual:
+        dare.dare_model_forward_window(model, tok, T - L, L, T, kc, vc)
 
     tok2, (kc2, vc2) = tok0.cuda(), new()
-    steps = dare.dare_generate_dual(model, tok2, P, G, L, kc2, vc2, mode, 0.9, k, pred, conf, nr)
+    dare.dare_model_set_sampling(model, temperature, 99, 0)
+    loop = dare.dare_generate_dual if dual else dare.dare_generate
+    steps = loop(model, tok2, P, G, L, kc2, vc2, mode, 0.9, k, pred, conf, nr)
     assert steps == want
     assert torch.equal(tok2, tok) and torch.equal(kc2, kc) and torch.equal(vc2, vc)
+    model.close()
+
+
+# The step's chain of programmatic launches in a CUDA graph: with the row compaction (more than 128 rows), with a selection kernel
+# of its own (blocks of more than 32), with a K/V split and its combination, sampled.  Replayed twice, as the eager call.
+@pytest.mark.parametrize("B,L,Hq,Hkv,P", [(5, 32, 4, 4, 300), (2, 40, 4, 2, 300), (5, 40, 28, 4, 100), (1, 32, 4, 4, 1500)])
+@pytest.mark.parametrize("temperature", [0.0, 0.7])
+def test_step_graphs_equal_the_eager_step(ctx, B, L, Hq, Hkv, P, temperature):
+    d, D, V, mu = 128, 512, 3000, 2990
+    g = torch.Generator(device="cuda").manual_seed(5)
+    rnd = lambda *s: torch.randn(s, generator=g, device="cuda").to(torch.bfloat16)  # noqa: E731
+    w, x, q = rnd(V, D) * 0.05, rnd(B * L, D), rnd(B, L, Hq, d)
+    k_pre, v_pre, plen = rnd(B, Hkv, P, d), rnd(B, Hkv, P, d), torch.full((B,), P - 3, dtype=torch.int32, device="cuda")
+    kb, vb = rnd(B, Hkv, L, d), rnd(B, Hkv, L, d)
+    new = lambda n, t: torch.zeros(n, dtype=t, device="cuda")  # noqa: E731
+    tok0 = torch.full((B, P + L), mu, dtype=torch.int32, device="cuda")
+    tok0[:, P::3] = 7
+    out = torch.zeros_like(q)
+    bufs = [tok0.clone(), out, new(B * L, torch.int32), new(B * L, torch.float32), new(B, torch.int32), new(B, torch.int32)]
+
+    def step():
+        tok, out, pred, conf, nc, nr = bufs
+        args = (ctx, q, k_pre, v_pre, plen, kb, vb, None, None, None, out, None, x, w, mu, True)
+        tail = (tok, P, dare.SELECT_TOPK, 0.0, 2, pred, conf, nc, nr)
+        if temperature:
+            dare.dare_denoise_block_sampled(*args, temperature, 5, 3, *tail)
+        else:
+            dare.dare_denoise_block(*args, *tail)
+
+    step()
+    torch.cuda.synchronize()
+    want = [t.clone() for t in bufs]
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        step()
+    for _ in range(2):
+        for t in bufs[1:]:
+            t.zero_()
+        bufs[0].copy_(tok0)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(bufs, want))
+    assert int(want[4].sum()) == 2 * B and ctx.device_status() == 0
 
 
 # 257 to 384 rows on row-major tiles and, with D = 3584 and 57000 entries, in two chunks: up to 320 rows both against each
@@ -408,7 +477,7 @@ def test_dual_loop_equals_its_parts(ctx, k, mode):
 # pairs and enough for every accumulator to come round.
 @pytest.mark.parametrize("M", [256, 257, 288, 289, 320, 321, 335, 352, 353, 384, 385])
 @pytest.mark.parametrize("D,V", [(72, 100), (72, 1300), (72, 100_000), (3584, 57_001)])
-def test_greedy_head_of_two_chunks_of_rows(ctx, M, D, V):
+def test_greedy_head_on_two_chunks(ctx, M, D, V):
     mu = V - 3
     x, w = I.normal_bf16(M, I.TID_X, (M, D)).cuda(), I.normal_bf16(V, I.TID_W, (V, D), 1.7 / D ** 0.5).cuda()
     pred, conf = dare.dare_lmhead_confidence(ctx, x, w, None, mu, True)
