@@ -105,7 +105,7 @@ def test_many_short_rows_cost_their_bytes(ctx):
     """A CTA per row would take 68 us to start here; a copy of the same bytes, and a warp per row, take about 10."""
     x = torch.randn(65536, 256, device="cuda").bfloat16()
     y = torch.empty_like(x)
-    assert _us(lambda: dare.dare_rmsnorm(ctx, x, 1e-5, y)) <= 2.5 * max(10.0, _us(lambda: y.copy_(x)))
+    assert _device_us(lambda: dare.dare_rmsnorm(ctx, x, 1e-5, y)) <= 2.5 * max(10.0, _device_us(lambda: y.copy_(x)))
 
 
 # Projections with so many rows that the tiles are taken in groups of row pairs (32 MB of A per group): one group and a
@@ -163,8 +163,8 @@ def test_sampled_head_evaluates_the_best(ctx, M, sigma, T):
 def test_sampled_head_on_a_small_vocabulary_costs_little_more(ctx, M, D, V):
     x, w = torch.randn(M, D, device="cuda").bfloat16(), torch.randn(V, D, device="cuda").mul(0.02).bfloat16()
     pred, conf = torch.empty(M, dtype=torch.int32, device="cuda"), torch.empty(M, device="cuda")
-    greedy = _us(lambda: dare.dare_lmhead_confidence(ctx, x, w, None, 3, True, pred, conf))
-    assert _us(lambda: dare.dare_lmhead_sample(ctx, x, w, None, 3, True, 1.0, 7, 1, pred, conf)) <= 2.5 * greedy
+    greedy = _device_us(lambda: dare.dare_lmhead_confidence(ctx, x, w, None, 3, True, pred, conf))
+    assert _device_us(lambda: dare.dare_lmhead_sample(ctx, x, w, None, 3, True, 1.0, 7, 1, pred, conf)) <= 2.5 * greedy
 
 
 def test_sampled_head_has_a_pair_per_vocabulary_tile(ctx):
@@ -174,7 +174,7 @@ def test_sampled_head_has_a_pair_per_vocabulary_tile(ctx):
     for M in (128, 160):
         x = torch.randn(M, D, device="cuda").bfloat16()
         pred, conf = torch.empty(M, dtype=torch.int32, device="cuda"), torch.empty(M, device="cuda")
-        us.append(_us(lambda: dare.dare_lmhead_sample(ctx, x, w, None, 3, True, 1.0, 7, 1, pred, conf)))
+        us.append(_device_us(lambda: dare.dare_lmhead_sample(ctx, x, w, None, 3, True, 1.0, 7, 1, pred, conf)))
     assert us[0] <= 1.1 * us[1]
 
 
@@ -530,7 +530,7 @@ def test_greedy_head_of_three_tiles_costs_no_more_than_of_four(ctx, D, V):
     for M in (300, 384, 512):
         x = torch.randn(M, D, device="cuda").bfloat16()
         pred, conf = torch.empty(M, dtype=torch.int32, device="cuda"), torch.empty(M, device="cuda")
-        us[M] = _us(lambda: dare.dare_lmhead_confidence(ctx, x, w, None, 3, True, pred, conf))
+        us[M] = _device_us(lambda: dare.dare_lmhead_confidence(ctx, x, w, None, 3, True, pred, conf))
     assert us[300] <= 1.2 * us[512] and us[384] <= 1.2 * us[512]
 
 
@@ -588,6 +588,6 @@ def test_rope_kernel_of_few_heads_costs_its_bytes(ctx):
     model = _small_model(ctx, 2, 1, 64, B * length, B, length, hidden=64, ffn=64)
     x, y = torch.randn(2, B * length, 256, device="cuda").bfloat16()
     q, kc, vc = torch.empty_like(x[:, :128]).contiguous(), *model.new_cache(B, length)
-    us = _us(lambda: dare.dare_rope_kv_write(model, x, B, length, 0, q, kc, vc))
-    assert us <= 2.5 * max(10.0, _us(lambda: y.copy_(x)))
+    us = _device_us(lambda: dare.dare_rope_kv_write(model, x, B, length, 0, q, kc, vc))
+    assert us <= 2.5 * max(10.0, _device_us(lambda: y.copy_(x)))
     model.close()
