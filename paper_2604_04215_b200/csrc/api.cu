@@ -12,12 +12,17 @@ std::atomic<uint64_t> g_kernel_launches{0};
 
 int make_tmap_bf16_2d(const dare_ctx* ctx, CUtensorMap* out, const void* base, uint64_t rows, uint64_t cols,
                       uint32_t box_rows, uint32_t box_cols) {
+    return make_tmap_bf16_3d(ctx, out, base, rows, 0, cols, box_rows, 0, box_cols);
+}
+
+int make_tmap_bf16_3d(const dare_ctx* ctx, CUtensorMap* out, const void* base, uint64_t rows, uint64_t mid, uint64_t cols,
+                      uint32_t box_rows, uint32_t box_mid, uint32_t box_cols) {
     TmapCache::Slot* slot = nullptr;
     if (ctx->tmaps) {
         // 64-bit finaliser over the whole key (allocations are aligned to hundreds of bytes, shapes are round numbers:
         // the raw low bits carry almost nothing)
         uint64_t h = reinterpret_cast<uintptr_t>(base) ^ (rows * 0x9E3779B97F4A7C15ull) ^ (cols * 0xC2B2AE3D27D4EB4Full) ^
-                     (static_cast<uint64_t>(box_rows) << 40) ^ (static_cast<uint64_t>(box_cols) << 52);
+                     (mid * 0x165667B19E3779F9ull) ^ (static_cast<uint64_t>(box_mid) << 32) ^ (static_cast<uint64_t>(box_rows) << 40) ^ (static_cast<uint64_t>(box_cols) << 52);
         h ^= h >> 30; h *= 0xBF58476D1CE4E5B9ull;
         h ^= h >> 27; h *= 0x94D049BB133111EBull;
         h ^= h >> 31;
@@ -25,8 +30,8 @@ int make_tmap_bf16_2d(const dare_ctx* ctx, CUtensorMap* out, const void* base, u
         TmapCache::Slot* ways = &ctx->tmaps->slot[set * TmapCache::WAYS];
         for (int i = 0; i < TmapCache::WAYS; ++i) {
             TmapCache::Slot& s = ways[i];
-            if (s.valid && s.base == base && s.rows == rows && s.cols == cols && s.box_rows == box_rows &&
-                s.box_cols == box_cols) {
+            if (s.valid && s.base == base && s.rows == rows && s.mid == mid && s.cols == cols && s.box_rows == box_rows &&
+                s.box_mid == box_mid && s.box_cols == box_cols) {
                 *out = s.map;
                 ++ctx->tmaps->hits;
                 return DARE_OK;
@@ -38,16 +43,18 @@ int make_tmap_bf16_2d(const dare_ctx* ctx, CUtensorMap* out, const void* base, u
             if (!ways[i].valid) { slot = &ways[i]; break; }
         if (slot->valid) ctx->tmaps->next_way[set] = static_cast<uint8_t>((ctx->tmaps->next_way[set] + 1) % TmapCache::WAYS);
     }
-    cuuint64_t dims[2] = {cols, rows};
-    cuuint64_t strides[1] = {cols * 2};   // bytes, dimension 1
-    cuuint32_t box[2] = {box_cols, box_rows};
-    cuuint32_t estr[2] = {1, 1};
-    CUresult r = ctx->encode_tiled(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides,
+    const bool flat = mid == 0;
+    cuuint64_t dims[3] = {cols, flat ? rows : mid, rows};
+    cuuint64_t strides[2] = {cols * 2, cols * mid * 2};   // bytes, dimensions 1 and 2
+    cuuint32_t box[3] = {box_cols, flat ? box_rows : box_mid, box_rows};
+    cuuint32_t estr[3] = {1, 1, 1};
+    CUresult r = ctx->encode_tiled(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, flat ? 2 : 3, const_cast<void*>(base), dims, strides,
                                    box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return DARE_ERR_CUDA;
     if (slot) {
-        slot->base = base; slot->rows = rows; slot->cols = cols; slot->box_rows = box_rows; slot->box_cols = box_cols;
+        slot->base = base; slot->rows = rows; slot->mid = mid; slot->cols = cols;
+        slot->box_rows = box_rows; slot->box_mid = box_mid; slot->box_cols = box_cols;
         slot->map = *out;
         slot->valid = true;
     }

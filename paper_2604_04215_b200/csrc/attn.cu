@@ -421,51 +421,53 @@ attn_block_kernel(const __grid_constant__ CUtensorMap tm_kpre, const __grid_cons
 
 // ---------------------------------------------------------------------------------------------------------
 // tcgen05 path: used when the query rows that share a KV head fill 128-row tensor-core tiles well (GQA
-// groups, long blocks such as the prefill).  One CTA per (one or two tiles of packed query rows, rollout x
-// KV head); the two query tiles share every K/V tile:
-//   warp 0        TMA producer: 128-key K and V tiles through a shared-memory ring (as above)
-//   warp 1        UMMA issuer (one thread, so that the order of its MMAs is the order they run in):
-//                 S = Q K^T (128 x 128, K-major operands from shared memory) into tensor memory, then
+// groups, long blocks such as the prefill).  A unit of work is one or two tiles of packed query rows of one
+// rollout x KV head; the two query tiles share every K/V tile:
+//   warp 0        TMA producer: Q tiles, and 64-key K and V tiles through a shared-memory ring; takes the units
+//   warps 1, 2    UMMA issuer of query tile 0, 1 (one thread each, so that the order of a tile's MMAs is the order they
+//                 run in): S = Q K^T (128 x 64, K-major operands from shared memory) into tensor memory, then
 //                 O += P V (128 x D) with P, the A operand, read from TENSOR memory and V, the MN-major B operand,
 //                 straight from the TMA tile; O stays in tensor memory over the whole key range
-//   warps 2..5    softmax of query tile 0 (warps 6..9: tile 1): one TMEM lane = one query row per thread;
-//                 reads S twice (tile max, then exponentials), keeps the row's reference max and sum, and writes
+//   warps 4..7    softmax of query tile 0 (warps 8..11: tile 1): one TMEM lane = one query row per thread;
+//                 holds a row's 64 scores in registers, keeps the row's reference max and sum, and writes
 //                 P as packed bf16 over the columns S came from: P never touches shared memory
-// An MMA whose A operand sits in shared memory costs ~80 to 120 cycles whatever its N (the 128 x 16 A slab is
-// read at ~32 bytes per cycle); with P in tensor memory the second product runs at its N / 2 cycles, and with
-// 128-key tiles the first product's MMAs have N = 128 instead of 64: per 64 keys and query tile ~740 cycles of
-// tensor pipe instead of ~1120.
-// With two query tiles each has ONE S/P buffer and the issuer interleaves them: while the softmax warps of one
-// tile work, the pipe runs the other tile's products (S_a(t), S_b(t), then per tile P V(t) and S(t + 1), which may
-// overwrite P(t) because the pipe runs the issuer's MMAs in order).  With one query tile there are two S/P buffers.
+// Each query tile has TWO S / P buffers of 64 columns, and S(t + 2) is issued behind P V(t) (it may overwrite P(t)
+// because the pipe runs an issuer's MMAs in order), so that a softmax warp finds its next scores ready instead of
+// waiting for the chain softmax -> P V -> S.  Two issuers, because one thread takes ~90 cycles for each of the 24 MMAs
+// of a step (both query tiles x 64 keys; one issuer 2140 cycles a step, two 1880).
+// The kernel is persistent: a CTA that has sent for its unit's last key tile takes over the next unit whose CTA has not
+// been started yet (cluster launch control), and the copies of that unit's Q, K and V are under way while the last
+// tiles of the current one are worked on; only the write-back of O lies between two units (2.4 k cycles; a CTA per unit
+// spent 12 k around its loop).
+// What bounds it: on packed batches the power cap (0.97 PFLOP/s at 1.65 GHz and 985 W; 0.63 at 1.91 GHz before), on an
+// unthrottled GPU the exponential unit and the waits around it (the unit is busy 55 % of the time).
+// Before -> after, us: packed 28 + 4 heads of 128, 32 sequences of 256 to 1024 tokens 333 -> 234 (on the power cap 343 ->
+// 270), 16 x 2048 1047 -> 940; 16 x 512 queries x 32 heads 116 -> 80; Dream-shaped step (32 rollouts, 1280 keys) 34.2 -> 30.1.
+// 128-key tiles with one S / P buffer, P handed over in halves: 16 x 2048 904 and 16 x 512 77, but 282 on the packed batch
+// (its ragged ends) and 30.8 on the step.
 // O stays in TMEM, so it cannot be rescaled for free when a row's max grows.  The exponentials are therefore
 // taken relative to a reference max that is only moved when the true max has run more than 2^8 ahead of it;
 // then (rarely, mostly in the first tiles) the warp waits for the MMAs in flight, multiplies its rows of O by
 // the correction factor in place and moves the reference.  The sum uses the same reference, so O / l is exact.
 // A tile holds floor(128 / g) block positions x g heads so that a position's heads never straddle two tiles.
-constexpr int TC_KT = 128;                // keys per tile
+constexpr int TC_KT = 64;                 // keys per tile
 constexpr float TC_RESCALE_GAP = 8.0f;    // log2 units the true max may run ahead of the reference
 
 template <int D, int QT>
 struct TcShape {
     static constexpr int Q_BYTES = 128 * D * 2;                        // per query tile
     static constexpr int KV_STAGE = 2 * TC_KT * D * 2;                 // K tile + V tile
-    static constexpr int NBUF = QT == 2 ? 1 : 2;                       // S / P buffers per query tile
-    static constexpr int FIXED = QT * Q_BYTES;
-    static constexpr int FIT = (226 * 1024 - 2048 - FIXED) / KV_STAGE;
-    static constexpr int STAGES = FIT > 4 ? 4 : FIT;
-    static constexpr int SMEM = FIXED + STAGES * KV_STAGE + 1024 + 512;
-    static constexpr int THREADS = (2 + 4 * QT) * 32;                  // TMA warp, MMA warp, softmax warps
-    static constexpr uint32_t TMEM_COLS = 512;
-    // tensor-memory columns: two query tiles: tile j has S/P at j * 256 and O at j * 256 + 128;
-    // one query tile: S/P buffers at 0 and 128, O at 256
-    __host__ __device__ static constexpr uint32_t s_col(int j, int b) { return QT == 2 ? j * 256 : b * 128; }
-    __host__ __device__ static constexpr uint32_t o_col(int j) { return QT == 2 ? j * 256 + 128 : 256; }
-    static_assert(STAGES >= NBUF + 1, "K/V ring too small");
+    static constexpr int STAGES = D == 128 ? 4 : 8;                    // (a power of two: 128 KB of K/V in flight)
+    static constexpr int OUT_BYTES = 32 * 128;                         // per softmax warp: 32 rows x 64 columns of O
+    static constexpr int SMEM = QT * Q_BYTES + STAGES * KV_STAGE + 4 * QT * OUT_BYTES + 1024 + 512;
+    static constexpr int THREADS = (4 + 4 * QT) * 32;                  // TMA warp, issuing warps (and idle ones), then the softmax warps
+    static constexpr uint32_t TMEM_COLS = QT == 2 ? 512 : 256;
+    // tensor-memory columns of query tile j: S / P buffers at j * 256 and j * 256 + 64, O at j * 256 + 128
+    __host__ __device__ static constexpr uint32_t s_col(int j, int b) { return j * 256 + b * 64; }
+    __host__ __device__ static constexpr uint32_t o_col(int j) { return j * 256 + 128; }
 };
 
-// The (block position, head) of packed query row r, walked in steps of `step` rows: one division up front.  (Two per row
-// made the staging of Q 3.2 k cycles before its first load was out, a tenth of a CTA's life on packed sequences.)
+// The (block position, head) of packed query row r, walked in steps of `step` rows: one division up front.
 struct RowWalk {
     int i, h, g, step_i, step_h;
     __device__ __forceinline__ RowWalk(int r, int step, int g_) : i(r / g_), h(r % g_), g(g_), step_i(step / g_), step_h(step % g_) {}
@@ -476,57 +478,63 @@ struct RowWalk {
     }
 };
 
+// A unit of work, as the producer hands it to the other warps.
+struct TcUnit {
+    int n_tiles;             // key tiles (0: there is no further unit)
+    int n_q;                 // query tiles with live rows
+    int pos0;                // first block position of the unit
+    int token0;              // first token of the rollout / sequence in q and out
+    int L_eff;               // block positions of the rollout / sequence
+    int b, kvh;
+    int len_pre, len_blk, len_suf;
+};
+
 template <int STAGES, int QT>
 struct TcBarriers {
     uint64_t full[STAGES];
     uint64_t empty[STAGES];
-    uint64_t q_ready;
-    uint64_t s_full[QT][2], p_full[QT][2], pv_done[QT][2];     // indexed by the key tile's parity
+    uint64_t q_full[QT], q_empty[QT];
+    uint64_t s_full[QT][2], p_full[QT][2], pv_done[QT][2];     // indexed by the S / P buffer
+    uint64_t unit_full[2], unit_empty[2];
+    uint64_t turn[2][4];                                       // [query tile][quadrant of tensor-memory lanes]
+    uint64_t next_unit;
+    TcUnit unit[2];
+    alignas(16) uint4 cancelled;                               // cluster launch control's answer
     uint32_t tmem_base;
     uint32_t abort_flag;
 };
 
 template <int D, int QT>
 __global__ void __launch_bounds__(TcShape<D, QT>::THREADS, 1)
-attn_block_tc_kernel(const __grid_constant__ CUtensorMap tm_kpre, const __grid_constant__ CUtensorMap tm_vpre,
-                     const __grid_constant__ CUtensorMap tm_kblk, const __grid_constant__ CUtensorMap tm_vblk,
-                     const __grid_constant__ CUtensorMap tm_ksuf, const __grid_constant__ CUtensorMap tm_vsuf,
-                     const AttnParams p) {
+attn_block_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_kpre,
+                     const __grid_constant__ CUtensorMap tm_vpre, const __grid_constant__ CUtensorMap tm_kblk,
+                     const __grid_constant__ CUtensorMap tm_vblk, const __grid_constant__ CUtensorMap tm_ksuf,
+                     const __grid_constant__ CUtensorMap tm_vsuf, const AttnParams p) {
     using S = TcShape<D, QT>;
     constexpr int STAGES = S::STAGES;
-    constexpr int NBUF = S::NBUF;
     constexpr int NHALF = D / 64;
-    constexpr int HALF_K = TC_KT * 128;            // one 64-column half of a K or V tile: 128 rows x 128 bytes
+    constexpr int HALF_K = TC_KT * 128;            // one 64-column half of a K or V tile: 64 rows x 128 bytes
     constexpr int KV_BYTES = TC_KT * D * 2;
     constexpr int HALF_Q = 128 * 128;              // one 64-column half of a Q tile: 128 rows x 128 bytes
+    static_assert(sizeof(TcBarriers<STAGES, QT>) <= 512, "shared-memory layout");
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t* q_s = base;                                   // [QT][Q_BYTES]
     uint8_t* kv_s = q_s + QT * S::Q_BYTES;                 // [STAGES][KV_STAGE]
-    TcBarriers<STAGES, QT>* bars = reinterpret_cast<TcBarriers<STAGES, QT>*>(kv_s + STAGES * S::KV_STAGE);
+    uint8_t* out_s = kv_s + STAGES * S::KV_STAGE;          // [4 * QT][OUT_BYTES]
+    TcBarriers<STAGES, QT>* bars = reinterpret_cast<TcBarriers<STAGES, QT>*>(out_s + 4 * QT * S::OUT_BYTES);
     volatile uint32_t* abort_flag = &bars->abort_flag;
 
-    const int warp = threadIdx.x >> 5;
+    const int warp = warp_index_uniform();
     const int lane = threadIdx.x & 31;
-    const int unit = blockIdx.y;
-    const int b = unit / p.Hkv;
-    const int kvh = unit % p.Hkv;
     const int pos_per_tile = 128 / p.g;            // block positions per query tile
+    const int rows_in_tile = pos_per_tile * p.g;
     // Packed variable-length mode: "rollout" b is sequence b of the packed token list; its tokens are both the
     // queries (a block of L_eff positions, no prefix) and, in place, the keys.  K and V are [tokens, Hkv * D].
     const bool packed = p.cu_seqlens != nullptr;
-    if (packed) pdl_wait();
-    const int seq_base = packed ? p.cu_seqlens[b] : 0;
-    const int L_eff = packed ? p.cu_seqlens[b + 1] - seq_base : p.L;
-    if (static_cast<int>(blockIdx.x) * QT * pos_per_tile >= L_eff) return;   // (packed only: whole CTA, before anything is set up)
-    const int kv_col0 = packed ? kvh * D : 0;      // first column of this KV head in the 2-D view of K / V
+    bool has_last = false;                         // this CTA ran the last unit (thread 0 knows)
 
-    // Set-up, with nothing waiting for anything else (a launch is a single wave of CTAs that live for about ten key
-    // tiles, so the time to the first product counts): the lengths are requested first; thread 0, which is also the
-    // TMA producer, sets up the barriers and sends for key tile 0 at once where its place does not depend on the
-    // lengths (packed sequences and the in-place cache: the first segment is not empty and starts at the unit's
-    // base); warp 1 allocates tensor memory; the softmax threads stage their Q rows.
     if (warp == 1) {
         tmem_alloc(&bars->tmem_base, S::TMEM_COLS);
         tmem_relinquish();
@@ -534,326 +542,400 @@ attn_block_tc_kernel(const __grid_constant__ CUtensorMap tm_kpre, const __grid_c
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(&bars->full[s], 1);
-            mbar_init(&bars->empty[s], 1);                 // released by the issuer once both query tiles are done with it
+            mbar_init(&bars->empty[s], QT);                // released by each query tile's issuer
         }
-        mbar_init(&bars->q_ready, 128 * QT);
-        for (int j = 0; j < QT; ++j)
+        for (int j = 0; j < QT; ++j) {
+            mbar_init(&bars->q_full[j], 1);
+            mbar_init(&bars->q_empty[j], 1);
             for (int i = 0; i < 2; ++i) {
                 mbar_init(&bars->s_full[j][i], 1);
                 mbar_init(&bars->p_full[j][i], 128);
                 mbar_init(&bars->pv_done[j][i], 1);
             }
+        }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&bars->unit_full[i], 1);
+            mbar_init(&bars->unit_empty[i], 5 * QT);       // the issuing warps and the softmax warps
+        }
+        mbar_init(&bars->next_unit, 1);
+        for (int i = 0; i < 8; ++i) mbar_init(&bars->turn[i >> 2][i & 3], 1);
         bars->abort_flag = 0;
         fence_barrier_init();
+        prefetch_tensormap(&tm_q);
         prefetch_tensormap(&tm_kpre);
         prefetch_tensormap(&tm_vpre);
     }
-    if (!packed && !p.beside_head) pdl_wait();             // (as in the warp-level kernel)
-    int P = p.prefix_len ? p.prefix_len[b]
-                         : (p.uniform_P >= 0 ? p.uniform_P : (p.inplace ? p.prefix_cap - p.L : p.prefix_cap));
-    int Sx = p.has_suffix ? (p.suffix_len ? p.suffix_len[b] : p.suffix_cap) : 0;
-    const bool early_tile = packed || p.inplace;
-    if (threadIdx.x == 0 && early_tile) {
-        const int row0 = packed ? seq_base : unit * p.prefix_cap;
-        mbar_arrive_expect_tx(&bars->full[0], 2 * KV_BYTES);
-#pragma unroll
-        for (int h = 0; h < NHALF; ++h) {
-            tma_load_2d(kv_s + h * HALF_K, &tm_kpre, &bars->full[0], kv_col0 + h * 64, row0);
-            tma_load_2d(kv_s + KV_BYTES + h * HALF_K, &tm_vpre, &bars->full[0], kv_col0 + h * 64, row0);
-        }
+    // rows of the Q tiles that no copy writes (128 is not a multiple of every g): zero, once
+    for (int o = threadIdx.x; o < (128 - rows_in_tile) * 8 * NHALF * QT; o += S::THREADS) {
+        const int piece = o & 7, row = rows_in_tile + (o >> 3) % (128 - rows_in_tile), half = (o >> 3) / (128 - rows_in_tile);
+        *reinterpret_cast<uint4*>(q_s + half * HALF_Q + row * 128 + piece * 16) = make_uint4(0, 0, 0, 0);
     }
-    if (warp >= 2) {
-        // Q rows -> shared memory, K-major with the 128-byte swizzle (16-byte chunk c of row r sits at c ^ (r & 7)).
-        // A warp copies the 32 rows whose softmax it runs, coalesced: one instruction reads 32 / CPR whole rows
-        // (a lane per 16-byte chunk), so that a request touches 2 to 4 cache lines, not one per lane.
-        constexpr int CPR = D / 8;                     // 16-byte chunks per row
-        const int j = (warp - 2) >> 2;
-        const int c = lane % CPR;
-        const size_t q_token = packed ? static_cast<size_t>(seq_base) : static_cast<size_t>(b) * p.L;
-        uint8_t* qt = q_s + j * S::Q_BYTES;
-        uint4 v[CPR];
-        RowWalk rw((warp & 3) * 32 + lane / CPR, 32 / CPR, p.g);
-        const int pos0 = (blockIdx.x * QT + j) * pos_per_tile;
-        const uint4* qsrc = reinterpret_cast<const uint4*>(p.q + ((q_token + pos0) * p.Hq + kvh * p.g) * D) + c;
-#pragma unroll
-        for (int k = 0; k < CPR; ++k, rw.next()) {
-            const bool live = rw.i < pos_per_tile && pos0 + rw.i < L_eff;      // (a tile's rows are pos_per_tile * g)
-            v[k] = live ? qsrc[(static_cast<size_t>(rw.i) * p.Hq + rw.h) * (D / 8)] : make_uint4(0, 0, 0, 0);
-        }
-#pragma unroll
-        for (int k = 0; k < CPR; ++k) {
-            const int r = (warp & 3) * 32 + k * (32 / CPR) + lane / CPR;
-            *reinterpret_cast<uint4*>(qt + (c >> 3) * HALF_Q + r * 128 + (((c & 7) ^ (r & 7)) << 4)) = v[k];
-        }
-        fence_proxy_async_smem();
-    }
+    fence_proxy_async_smem();
+    if (!p.beside_head) pdl_wait();                        // (as in the warp-level kernel)
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem_base = bars->tmem_base;
 
-    // lengths and tiles of this unit (same bookkeeping as the warp-level kernel)
-    const int p_max = p.inplace ? p.prefix_cap - p.L : p.prefix_cap;
-    if (!packed && (P < 0 || P > p_max || Sx < 0 || Sx > p.suffix_cap)) {
-        P = max(0, min(P, p_max));
-        Sx = max(0, min(Sx, p.suffix_cap));
-        if (threadIdx.x == 0) atomicOr(p.dev_status, DEV_LEN_CLAMPED);
+    if constexpr (QT == 2) {        // 384 threads are launched with 168 registers each = 128 x (56 + 2 x 224)
+        if (warp < 4) set_max_regs_dec<56>();
+        else set_max_regs_inc<224>();
     }
-    const int len_pre = packed ? L_eff : (p.inplace ? P + p.L : P);
-    const int len_blk = (packed || p.inplace) ? 0 : p.L;
-    const int n_pre = (len_pre + TC_KT - 1) / TC_KT;
-    const int n_blk = (len_blk + TC_KT - 1) / TC_KT;
-    const int n_suf = (Sx + TC_KT - 1) / TC_KT;
-    const int n_tiles = n_pre + n_blk + n_suf;
-    const int base_pre = packed ? seq_base : unit * p.prefix_cap;
-    const int base_blk = unit * p.L;
-    const int base_suf = unit * p.suffix_cap;
-
     if (warp == 0) {
         if (lane == 0) {
-            int stage = 0;
-            uint32_t phase = 0;
-            int t = 0;
-            if (early_tile) {                               // key tile 0 is on its way already (n_tiles >= 1 here)
-                ++t;
-                if (++stage == STAGES) { stage = 0; phase ^= 1; }
-            }
-            for (; t < n_tiles; ++t) {
-                const TileInfo ti = tile_info<TC_KT>(t, n_pre, n_blk, len_pre, len_blk, Sx, base_pre, base_blk, base_suf);
-                const CUtensorMap* mk = ti.seg == 0 ? &tm_kpre : (ti.seg == 1 ? &tm_kblk : &tm_ksuf);
-                const CUtensorMap* mv = ti.seg == 0 ? &tm_vpre : (ti.seg == 1 ? &tm_vblk : &tm_vsuf);
-                if (!mbar_wait(&bars->empty[stage], phase ^ 1, abort_flag)) break;
-                uint8_t* kdst = kv_s + stage * S::KV_STAGE;
-                uint8_t* vdst = kdst + KV_BYTES;
-                mbar_arrive_expect_tx(&bars->full[stage], 2 * KV_BYTES);
+            const int p_max = p.inplace ? p.prefix_cap - p.L : p.prefix_cap;
+            uint32_t chunk = blockIdx.x, y = blockIdx.y;
+            uint32_t n_kv = 0, n_qload[QT] = {}, n_units = 0, n_taken = 0;
+            bool ok = true;
+            while (ok) {
+                has_last = has_last || (chunk == gridDim.x - 1 && y == gridDim.y - 1);
+                TcUnit w;
+                w.b = static_cast<int>(y) / p.Hkv;
+                w.kvh = static_cast<int>(y) % p.Hkv;
+                w.pos0 = static_cast<int>(chunk) * QT * pos_per_tile;
+                w.token0 = packed ? p.cu_seqlens[w.b] : w.b * p.L;
+                w.L_eff = packed ? p.cu_seqlens[w.b + 1] - w.token0 : p.L;
+                if (w.pos0 < w.L_eff) {                    // (packed: the grid is cut for the longest sequence)
+                    int P = p.prefix_len ? p.prefix_len[w.b]
+                                         : (p.uniform_P >= 0 ? p.uniform_P : (p.inplace ? p.prefix_cap - p.L : p.prefix_cap));
+                    int Sx = p.has_suffix ? (p.suffix_len ? p.suffix_len[w.b] : p.suffix_cap) : 0;
+                    if (!packed && (P < 0 || P > p_max || Sx < 0 || Sx > p.suffix_cap)) {
+                        P = max(0, min(P, p_max));
+                        Sx = max(0, min(Sx, p.suffix_cap));
+                        atomicOr(p.dev_status, DEV_LEN_CLAMPED);
+                    }
+                    w.len_pre = packed ? w.L_eff : (p.inplace ? P + p.L : P);
+                    w.len_blk = (packed || p.inplace) ? 0 : p.L;
+                    w.len_suf = Sx;
+                    const int n_pre = (w.len_pre + TC_KT - 1) / TC_KT, n_blk = (w.len_blk + TC_KT - 1) / TC_KT;
+                    w.n_tiles = n_pre + n_blk + (Sx + TC_KT - 1) / TC_KT;
+                    w.n_q = min(QT, (w.L_eff - w.pos0 + pos_per_tile - 1) / pos_per_tile);
+                    const int slot = n_units & 1;
+                    if (!mbar_wait(&bars->unit_empty[slot], ((n_units >> 1) & 1) ^ 1, abort_flag)) break;
+                    bars->unit[slot] = w;
+                    mbar_arrive(&bars->unit_full[slot]);
+                    ++n_units;
+                    const int base_pre = packed ? w.token0 : static_cast<int>(y) * p.prefix_cap;
+                    const int base_blk = static_cast<int>(y) * p.L;
+                    const int base_suf = static_cast<int>(y) * p.suffix_cap;
+                    const int kv_col0 = packed ? w.kvh * D : 0;      // first column of this KV head in the 2-D view of K / V
+                    for (int t = 0; t < w.n_tiles; ++t, ++n_kv) {
+                        const TileInfo ti = tile_info<TC_KT>(t, n_pre, n_blk, w.len_pre, w.len_blk, Sx, base_pre, base_blk, base_suf);
+                        const CUtensorMap* mk = ti.seg == 0 ? &tm_kpre : (ti.seg == 1 ? &tm_kblk : &tm_ksuf);
+                        const CUtensorMap* mv = ti.seg == 0 ? &tm_vpre : (ti.seg == 1 ? &tm_vblk : &tm_vsuf);
+                        const int stage = n_kv % STAGES;
+                        if (!mbar_wait(&bars->empty[stage], ((n_kv / STAGES) & 1) ^ 1, abort_flag)) { ok = false; break; }
+                        uint8_t* kdst = kv_s + stage * S::KV_STAGE;
+                        uint8_t* vdst = kdst + KV_BYTES;
+                        mbar_arrive_expect_tx(&bars->full[stage], 2 * KV_BYTES);
 #pragma unroll
-                for (int h = 0; h < NHALF; ++h) {
-                    tma_load_2d(kdst + h * HALF_K, mk, &bars->full[stage], kv_col0 + h * 64, ti.row0);
-                    tma_load_2d(vdst + h * HALF_K, mv, &bars->full[stage], kv_col0 + h * 64, ti.row0);
+                        for (int h = 0; h < NHALF; ++h) {
+                            tma_load_2d(kdst + h * HALF_K, mk, &bars->full[stage], kv_col0 + h * 64, ti.row0);
+                            tma_load_2d(vdst + h * HALF_K, mv, &bars->full[stage], kv_col0 + h * 64, ti.row0);
+                        }
+                        if (t != 0) continue;
+                        // The Q tiles: rows (position, head of the group), in that order, as one box.  (Positions behind
+                        // the rollout's or the sequence's last bring in other rows or zeros; they are not stored.)
+#pragma unroll
+                        for (int j = 0; j < QT; ++j) {
+                            if (j >= w.n_q || !ok) continue;
+                            ok = mbar_wait(&bars->q_empty[j], (n_qload[j] & 1) ^ 1, abort_flag);
+                            if (!ok) continue;
+                            ++n_qload[j];
+                            mbar_arrive_expect_tx(&bars->q_full[j], static_cast<uint32_t>(rows_in_tile) * D * 2);
+#pragma unroll
+                            for (int h = 0; h < NHALF; ++h)
+                                tma_load_3d(q_s + j * S::Q_BYTES + h * HALF_Q, &tm_q, &bars->q_full[j], h * 64, w.kvh * p.g,
+                                            w.token0 + w.pos0 + j * pos_per_tile);
+                        }
+                        if (!ok) break;
+                    }
+                    if (!ok) break;
                 }
-                if (++stage == STAGES) { stage = 0; phase ^= 1; }
+                // every copy of this unit is under way: take the next one (no earlier, or one CTA would sit on a unit
+                // that an idle SM could run)
+                mbar_arrive_expect_tx(&bars->next_unit, 16);
+                clc_try_cancel(&bars->cancelled, &bars->next_unit);
+                if (!mbar_wait(&bars->next_unit, n_taken & 1, abort_flag)) break;
+                ++n_taken;
+                const bool got = clc_query(&bars->cancelled, chunk, y);
+                fence_proxy_async_smem();                  // (read here before the next answer is written there)
+                if (!got) {
+                    const int slot = n_units & 1;
+                    if (!mbar_wait(&bars->unit_empty[slot], ((n_units >> 1) & 1) ^ 1, abort_flag)) break;
+                    bars->unit[slot].n_tiles = 0;
+                    mbar_arrive(&bars->unit_full[slot]);
+                    break;
+                }
             }
         }
-    } else if (warp == 1) {
-        // All 32 lanes run the loops (waits, counters and descriptors stay warp-uniform, in the registers the MMA
-        // instruction takes its operands from); one elected lane issues the MMAs and their commits.
+        __syncwarp();
+    } else if (warp < 4) {
+      if (warp <= QT) {
+        // One issuing warp per query tile.  All 32 lanes run the loops (waits, counters and descriptors stay warp-uniform, in
+        // the registers the MMA instruction takes its operands from); one elected lane issues the MMAs and their commits.
+        const int j = warp - 1;
         const bool leader = elect_one_sync();
         constexpr uint32_t idesc_s = umma_idesc_bf16(128, TC_KT);
         constexpr uint32_t idesc_o = umma_idesc_bf16(128, D) | UMMA_B_MN_MAJOR;
         // descriptor lower words (address >> 4 [| leading byte offset]); the upper word is a constant
-        const uint32_t q_lo = smem_u32(q_s) >> 4, kv_lo = smem_u32(kv_s) >> 4;
+        const uint32_t q_lo = (smem_u32(q_s) + j * S::Q_BYTES) >> 4, kv_lo = smem_u32(kv_s) >> 4;
         const uint32_t v_lbo = static_cast<uint32_t>(HALF_K >> 4) << 16;   // second 64 head-dim columns: one half tile on
-        bool ok = __all_sync(0xffffffffu, mbar_wait(&bars->q_ready, 0, abort_flag));
-        // S_j(t) = Q_j K_t^T into tile j's buffer t % NBUF (whatever that buffer held has been consumed: the P V
-        // product that read it was issued before this, and the pipe keeps the issue order)
-        auto issue_s = [&](int j, int t) -> bool {
-            const int stage = t % STAGES;
-            if (!__all_sync(0xffffffffu, mbar_wait(&bars->full[stage], (t / STAGES) & 1, abort_flag))) return false;
-            tc_fence_after_sync();
-            const uint32_t k_lo = kv_lo + stage * (S::KV_STAGE >> 4), qj = q_lo + j * (S::Q_BYTES >> 4);
-            const uint32_t sd = tmem_base + S::s_col(j, t % NBUF);
-            if (leader) {
-                umma_bf16_lo<false>(sd, qj, k_lo, idesc_s);
-#pragma unroll
-                for (int kk = 1; kk < D / 16; ++kk)     // 16 channels = 32 bytes along the swizzled row: +2
-                    umma_bf16_lo<true>(sd, qj + (kk >> 2) * (HALF_Q >> 4) + 2 * (kk & 3),
-                                       k_lo + (kk >> 2) * (HALF_K >> 4) + 2 * (kk & 3), idesc_s);
-                umma_commit(&bars->s_full[j][t & 1]);
-            }
+        const uint32_t od = tmem_base + S::o_col(j);
+        uint32_t n_kv = 0, n_unit = 0, n_q = 0, n_s = 0;   // key tiles of the ring, units, Q tiles and key tiles of query tile j so far
+        bool ok = true;
+        while (true) {
+            const int slot = n_unit & 1;
+            if (!__all_sync(0xffffffffu, mbar_wait(&bars->unit_full[slot], (n_unit >> 1) & 1, abort_flag))) break;
+            ++n_unit;
+            // (through a reduction, whose result the compiler knows to be the same in all lanes)
+            const int n_tiles = __reduce_max_sync(0xffffffffu, bars->unit[slot].n_tiles);
+            const bool idle = __reduce_max_sync(0xffffffffu, bars->unit[slot].n_q) <= j;
+            if (leader) mbar_arrive(&bars->unit_empty[slot]);
             __syncwarp();
-            return true;
-        };
-        for (int t = 0; t < NBUF && t < n_tiles && ok; ++t)
-            for (int j = 0; j < QT && ok; ++j) ok = issue_s(j, t);
-        for (int t = 0; t < n_tiles && ok; ++t) {
-            const int stage = t % STAGES;
-            const uint32_t v_lo = (kv_lo + stage * (S::KV_STAGE >> 4) + (KV_BYTES >> 4)) | v_lbo;
-            for (int j = 0; j < QT && ok; ++j) {
-                if (!__all_sync(0xffffffffu, mbar_wait(&bars->p_full[j][t & 1], (t >> 1) & 1, abort_flag))) { ok = false; break; }
+            if (n_tiles == 0) break;
+            if (idle) {                                    // (no live row in this query tile: the K/V tiles pass by)
+                for (int t = 0; t < n_tiles && ok; ++t, ++n_kv) {
+                    ok = __all_sync(0xffffffffu, mbar_wait(&bars->full[n_kv % STAGES], (n_kv / STAGES) & 1, abort_flag));
+                    if (ok && leader) mbar_arrive(&bars->empty[n_kv % STAGES]);
+                    __syncwarp();
+                }
+                if (!ok) break;
+                continue;
+            }
+            // S(t) = Q K_t^T into the buffer of t's parity (whatever that buffer held has been consumed: the P V
+            // product that read it was issued before this, and the pipe keeps the issue order)
+            auto issue_s = [&](int t) -> bool {
+                const uint32_t n = n_kv + t;
+                const int stage = n % STAGES, buf = (n_s + t) & 1;
+                if (!__all_sync(0xffffffffu, mbar_wait(&bars->full[stage], (n / STAGES) & 1, abort_flag))) return false;
+                tc_fence_after_sync();
+                const uint32_t k_lo = kv_lo + stage * (S::KV_STAGE >> 4);
+                const uint32_t sd = tmem_base + S::s_col(j, buf);
+                if (leader) {
+                    umma_bf16_lo<false>(sd, q_lo, k_lo, idesc_s);
+#pragma unroll
+                    for (int kk = 1; kk < D / 16; ++kk)     // 16 channels = 32 bytes along the swizzled row: +2
+                        umma_bf16_lo<true>(sd, q_lo + (kk >> 2) * (HALF_Q >> 4) + 2 * (kk & 3),
+                                           k_lo + (kk >> 2) * (HALF_K >> 4) + 2 * (kk & 3), idesc_s);
+                    umma_commit(&bars->s_full[j][buf]);
+                    if (t == n_tiles - 1) umma_commit(&bars->q_empty[j]);     // the next unit's Q may come
+                }
+                __syncwarp();
+                return true;
+            };
+            ok = __all_sync(0xffffffffu, mbar_wait(&bars->q_full[j], n_q & 1, abort_flag));
+            ++n_q;
+            if (ok) ok = issue_s(0);
+            if (ok && n_tiles > 1) ok = issue_s(1);
+            for (int t = 0; t < n_tiles && ok; ++t) {
+                const int stage = (n_kv + t) % STAGES;
+                const uint32_t v_lo = (kv_lo + stage * (S::KV_STAGE >> 4) + (KV_BYTES >> 4)) | v_lbo;
+                const uint32_t n = n_s + t;
+                const int buf = n & 1;
+                ok = __all_sync(0xffffffffu, mbar_wait(&bars->p_full[j][buf], (n >> 1) & 1, abort_flag));
+                if (!ok) break;
                 tc_fence_after_sync();
                 // A: P in tensor memory, 16 keys = 8 columns per MMA; B: 16 key rows (2 KB) further down V
-                const uint32_t pa = tmem_base + S::s_col(j, t % NBUF), od = tmem_base + S::o_col(j);
+                const uint32_t pa = tmem_base + S::s_col(j, buf);
                 if (leader) {
                     if (t == 0) umma_bf16_ts_lo<false>(od, pa, v_lo, idesc_o);
                     else umma_bf16_ts_lo<true>(od, pa, v_lo, idesc_o);
 #pragma unroll
                     for (int kk = 1; kk < TC_KT / 16; ++kk)
                         umma_bf16_ts_lo<true>(od, pa + 8 * kk, v_lo + kk * (2048 >> 4), idesc_o);
-                    umma_commit(&bars->pv_done[j][t & 1]);     // O holds tiles 0..t
+                    umma_commit(&bars->pv_done[j][buf]);       // O holds tiles 0..t
+                    umma_commit(&bars->empty[stage]);          // (this query tile is done with this K/V tile)
                 }
                 __syncwarp();
-                if (t + NBUF < n_tiles) ok = issue_s(j, t + NBUF);
+                if (t + 2 < n_tiles) ok = issue_s(t + 2);
             }
-            if (ok && leader) umma_commit(&bars->empty[stage]);      // every product that reads this K/V tile has been issued
-            __syncwarp();
+            if (!ok) break;
+            n_kv += n_tiles;
+            n_s += n_tiles;
         }
+        pdl_trigger();                                  // (this late for the reason given in the warp-level kernel)
+      }
     } else {
         // ---------------- softmax warps: set j = query tile, thread = packed query row r of that tile = TMEM lane r
-        const int j = (warp - 2) >> 2;
+        const int j = (warp >> 2) - 1;
         const int r = (warp & 3) * 32 + lane;          // warp w may touch TMEM lanes [32 * (w % 4), +32)
-        const int rows_in_tile = pos_per_tile * p.g;
-        const int i = (blockIdx.x * QT + j) * pos_per_tile + r / p.g;   // block position
-        const int h = kvh * p.g + r % p.g;                              // query head
-        const bool live = r < rows_in_tile && i < L_eff;
-        const size_t q_token = packed ? static_cast<size_t>(seq_base) : static_cast<size_t>(b) * p.L;   // first token of b
-        mbar_arrive(&bars->q_ready);                   // (the warp's Q rows were staged before the barrier above)
-        float m_ref = -INFINITY, l = 0.f;              // reference max (log2 domain) and sum of exp2(s - m_ref)
+        const int ri = r / p.g, rh = r % p.g;          // block position and head within the tile and the group
         const uint32_t lane_off = static_cast<uint32_t>((warp & 3) * 32) << 16;
         const uint32_t tm_o = tmem_base + S::o_col(j) + lane_off;
         const float c2 = p.scale_log2;
-        bool ok = true;
-        for (int t = 0; t < n_tiles; ++t) {
-            const TileInfo ti = tile_info<TC_KT>(t, n_pre, n_blk, len_pre, len_blk, Sx, base_pre, base_blk, base_suf);
-            const int buf = t & 1, stage = t % STAGES;
-            if (!mbar_wait(&bars->s_full[j][buf], (t >> 1) & 1, abort_flag)) { ok = false; break; }
+        uint8_t* ot = out_s + (warp - 4) * S::OUT_BYTES;
+        uint32_t n_kv = 0, n_unit = 0, n_s = 0, n_turn = 0;
+        const int quadrant = warp & 3;
+        RowWalk out_walk((warp & 3) * 32 + (lane >> 3), 4, p.g);
+        while (true) {
+            const int slot = n_unit & 1;
+            if (!__all_sync(0xffffffffu, mbar_wait(&bars->unit_full[slot], (n_unit >> 1) & 1, abort_flag))) break;
+            ++n_unit;
+            const TcUnit w = bars->unit[slot];
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bars->unit_empty[slot]);
+            if (w.n_tiles == 0) break;
+            if (j >= w.n_q) { n_kv += w.n_tiles; continue; }
+            const int n_pre = (w.len_pre + TC_KT - 1) / TC_KT, n_blk = (w.len_blk + TC_KT - 1) / TC_KT;
+            float m_ref = -INFINITY, l = 0.f;              // reference max (log2 domain) and sum of exp2(s - m_ref)
+            bool ok = true;
+            for (int t = 0; t < w.n_tiles; ++t) {
+                const int valid = tile_info<TC_KT>(t, n_pre, n_blk, w.len_pre, w.len_blk, w.len_suf, 0, 0, 0).valid;
+                const uint32_t n = n_s + t;
+                const int buf = n & 1;
+                if (!mbar_wait(&bars->s_full[j][buf], (n >> 1) & 1, abort_flag)) { ok = false; break; }
+                tc_fence_after_sync();
+                const uint32_t tm_s = tmem_base + S::s_col(j, buf) + lane_off;
+                uint32_t s0[32], s1[32];
+                tmem_ld_32cols(tm_s, s0);
+                tmem_ld_32cols(tm_s + 32, s1);
+                tmem_ld_wait();
+                if (valid < TC_KT) {                       // (keys past the segment's end do not count)
+#pragma unroll
+                    for (int k = 0; k < 32; ++k) {
+                        if (k >= valid) s0[k] = 0xff800000u;
+                        if (k + 32 >= valid) s1[k] = 0xff800000u;
+                    }
+                }
+                float t0 = max3(s0[0], s0[1], s0[2]), t1 = max3(s1[0], s1[1], s1[2]);
+                float t2 = max3(s0[3], s0[4], s0[5]), t3 = max3(s1[3], s1[4], s1[5]);
+#pragma unroll
+                for (int k = 6; k < 30; k += 4) {
+                    t0 = max3(__float_as_uint(t0), s0[k], s0[k + 1]);
+                    t1 = max3(__float_as_uint(t1), s1[k], s1[k + 1]);
+                    t2 = max3(__float_as_uint(t2), s0[k + 2], s0[k + 3]);
+                    t3 = max3(__float_as_uint(t3), s1[k + 2], s1[k + 3]);
+                }
+                t0 = max3(__float_as_uint(t0), s0[30], s0[31]);
+                t1 = max3(__float_as_uint(t1), s1[30], s1[31]);
+                t0 = fmaxf(t0, t2);
+                t1 = fmaxf(t1, t3);
+                const float tmax = fmaxf(t0, t1) * c2;     // log2 domain (the scale is > 0); finite: every tile has a key
+                // move the reference only when the true max has run away from it (decided per warp, so that the
+                // TMEM loads and stores below are executed by whole warps)
+                if (__any_sync(0xffffffffu, tmax > m_ref + TC_RESCALE_GAP)) {
+                    const float m_new = fmaxf(m_ref, tmax);
+                    const float factor = fast_exp2(m_ref - m_new);   // exp2(-inf) = 0 on the first tile
+                    m_ref = m_new;
+                    l *= factor;
+                    if (t >= 1) {
+                        // every MMA that adds to O must have landed before O is rescaled in place: tile t - 1 is the last
+                        if (!mbar_wait(&bars->pv_done[j][(n - 1) & 1], ((n - 1) >> 1) & 1, abort_flag)) { ok = false; break; }
+                        tc_fence_after_sync();
+#pragma unroll
+                        for (int c = 0; c < D / 16; ++c) {
+                            uint32_t ov[16];
+                            tmem_ld_16cols(tm_o + c * 16, ov);
+                            tmem_ld_wait();
+#pragma unroll
+                            for (int k = 0; k < 16; ++k) ov[k] = __float_as_uint(__uint_as_float(ov[k]) * factor);
+                            tmem_st_16cols(tm_o + c * 16, ov);
+                        }
+                    }
+                }
+                // The two query tiles' warps of a scheduler take turns at the exponential unit: when both are at it, both
+                // take twice as long and then wait for their next scores together, while the unit idles (16 sequences of
+                // 2048 tokens 953 -> 908 us; with 64 channels the products are short and turns cost 268 -> 301 us instead).
+                const bool turns = QT == 2 && D == 128 && w.n_q == 2;
+                if (turns) {
+                    if (!mbar_wait(&bars->turn[j][quadrant], (n_turn & 1) ^ (j == 0 ? 1 : 0), abort_flag)) { ok = false; break; }
+                    ++n_turn;
+                }
+                // P = exp2(s - m_ref) as packed bf16 over the columns S came from (all of S is in registers)
+                const float nm = m_ref == -INFINITY ? 0.f : -m_ref;      // (every score so far is -inf: all weights 0, not NaN)
+                const uint64_t c2c2 = pack_f32x2(c2, c2), nmnm = pack_f32x2(nm, nm);
+                uint64_t psum = 0;                           // two partial sums
+                uint32_t pk[32];
+                uint64_t e[2][4];
+#pragma unroll
+                for (int g8 = 0; g8 < 9; ++g8) {
+                    if (g8 < 8) {
+                        const uint32_t (&sv)[32] = g8 < 4 ? s0 : s1;
+                        const int k0 = (g8 & 3) * 8;
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            e[g8 & 1][k] = exp2_f32x2(fma_f32x2(pack_b32x2(sv[k0 + 2 * k], sv[k0 + 2 * k + 1]), c2c2, nmnm));
+                    }
+                    if (g8 > 0) {
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const uint64_t v = e[(g8 - 1) & 1][k];
+                            psum = add_f32x2(psum, v);
+                            pk[(g8 - 1) * 4 + k] = pack_bf16(__uint_as_float(static_cast<uint32_t>(v)), __uint_as_float(static_cast<uint32_t>(v >> 32)));
+                        }
+                    }
+                }
+                if (turns) {
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&bars->turn[j ^ 1][quadrant]);
+                }
+                tmem_st_32cols(tm_s, pk);
+                tmem_st_wait();
+                const float psum0 = __uint_as_float(static_cast<uint32_t>(psum)), psum1 = __uint_as_float(static_cast<uint32_t>(psum >> 32));
+                l += psum0 + psum1;
+                if (valid < TC_KT) {
+                    // V rows past the segment's end hold whatever lies behind it in memory: zero them so that
+                    // probability 0 times garbage cannot make a NaN (thread r clears 16-byte pieces of those rows;
+                    // both query tiles' warps do it, each before it releases its own second MMA)
+                    uint8_t* vt = kv_s + (n_kv + t) % STAGES * S::KV_STAGE + KV_BYTES;
+                    const int n_bad = (TC_KT - valid) * 8;          // 16-byte pieces per 64-column half
+                    for (int h2 = 0; h2 < NHALF; ++h2)
+                        for (int q = r; q < n_bad; q += 128)
+                            *reinterpret_cast<uint4*>(vt + h2 * HALF_K + valid * 128 + q * 16) = make_uint4(0, 0, 0, 0);
+                    fence_proxy_async_smem();
+                }
+                tc_fence_before_sync();
+                mbar_arrive(&bars->p_full[j][buf]);
+            }
+            n_kv += w.n_tiles;
+            n_s += w.n_tiles;
+            if (ok) ok = mbar_wait(&bars->pv_done[j][(n_s - 1) & 1], ((n_s - 1) >> 1) & 1, abort_flag);
+            if (!__all_sync(0xffffffffu, ok)) break;
             tc_fence_after_sync();
-            const uint32_t tm_s = tmem_base + S::s_col(j, t % NBUF) + lane_off;
-            // first pass over S: the tile's largest score (keys past the segment's end do not count).  The load of
-            // the next 32 columns is in flight while the current ones are looked at.  (A single pass that keeps P in
-            // registers until the reference is known to hold was measured no faster: 37.2 against 35.4 us.)
-            float tmax = -INFINITY;
-            {
-                uint32_t sa[32], sb[32];
-                tmem_ld_32cols(tm_s, sa);
+            const float inv = l > 0.f ? 1.f / l : 0.f;
+            // O rows leave through shared memory so that the global stores are coalesced (a thread holds one whole row,
+            // and 32 lanes storing 16 bytes each to 32 different rows cost a request per lane): 64 columns at a time,
+            // 16-byte chunk c of row r at c ^ (r & 7).
+            const int pos0 = w.pos0 + j * pos_per_tile;
+#pragma unroll
+            for (int h2 = 0; h2 < NHALF; ++h2) {
+                uint32_t oa[32], ob[32];
+                tmem_ld_32cols(tm_o + h2 * 64, oa);          // (whole warp, also for rows that are not stored)
+                tmem_ld_32cols(tm_o + h2 * 64 + 32, ob);
                 tmem_ld_wait();
+                if (h2 > 0) __syncwarp();                    // (the first half has been read out of `ot`)
 #pragma unroll
-                for (int c = 0; c < TC_KT / 32; ++c) {
-                    uint32_t (&cur)[32] = (c & 1) ? sb : sa;
-                    uint32_t (&nxt)[32] = (c & 1) ? sa : sb;
-                    if (c + 1 < TC_KT / 32) tmem_ld_32cols(tm_s + (c + 1) * 32, nxt);
-                    if (ti.valid >= (c + 1) * 32) {
+                for (int k = 0; k < 8; ++k) {
+                    const uint32_t (&ov)[32] = k < 4 ? oa : ob;
+                    const int k8 = (k & 3) * 8;
+                    uint4 o;
+                    o.x = pack_bf16(__uint_as_float(ov[k8 + 0]) * inv, __uint_as_float(ov[k8 + 1]) * inv);
+                    o.y = pack_bf16(__uint_as_float(ov[k8 + 2]) * inv, __uint_as_float(ov[k8 + 3]) * inv);
+                    o.z = pack_bf16(__uint_as_float(ov[k8 + 4]) * inv, __uint_as_float(ov[k8 + 5]) * inv);
+                    o.w = pack_bf16(__uint_as_float(ov[k8 + 6]) * inv, __uint_as_float(ov[k8 + 7]) * inv);
+                    *reinterpret_cast<uint4*>(ot + lane * 128 + ((k ^ (lane & 7)) << 4)) = o;
+                }
+                __syncwarp();
+                const int c = lane & 7;
+                RowWalk rw = out_walk;
+                uint4* dst = reinterpret_cast<uint4*>(p.out + ((static_cast<size_t>(w.token0) + pos0) * p.Hq + w.kvh * p.g) * D + h2 * 64) + c;
 #pragma unroll
-                        for (int k = 0; k < 32; ++k) tmax = fmaxf(tmax, __uint_as_float(cur[k]));
-                    } else {
-#pragma unroll
-                        for (int k = 0; k < 32; ++k)
-                            if (c * 32 + k < ti.valid) tmax = fmaxf(tmax, __uint_as_float(cur[k]));
-                    }
-                    if (c + 1 < TC_KT / 32) tmem_ld_wait();
+                for (int k = 0; k < 8; ++k, rw.next()) {
+                    const int rr = k * 4 + (lane >> 3);
+                    if (rw.i < pos_per_tile && pos0 + rw.i < w.L_eff)
+                        dst[(static_cast<size_t>(rw.i) * p.Hq + rw.h) * (D / 8)] =
+                            *reinterpret_cast<const uint4*>(ot + rr * 128 + ((c ^ (rr & 7)) << 4));
                 }
             }
-            tmax *= c2;                                 // log2 domain (the scale is > 0); finite: every tile has a key
-            // move the reference only when the true max has run away from it (decided per warp, so that the
-            // TMEM loads and stores below are executed by whole warps)
-            const bool move = __any_sync(0xffffffffu, tmax > m_ref + TC_RESCALE_GAP);
-            if (move) {
-                const float m_new = fmaxf(m_ref, tmax);
-                const float factor = fast_exp2(m_ref - m_new);   // exp2(-inf) = 0 on the first tile
-                m_ref = m_new;
-                l *= factor;
-                if (t >= 1) {
-                    // every MMA that adds to O must have landed before O is rescaled in place: tile t - 1 is the last
-                    if (!mbar_wait(&bars->pv_done[j][(t - 1) & 1], ((t - 1) >> 1) & 1, abort_flag)) { ok = false; break; }
-                    tc_fence_after_sync();
-#pragma unroll
-                    for (int c = 0; c < D / 32; ++c) {
-                        uint32_t ov[32];
-                        tmem_ld_32cols(tm_o + c * 32, ov);
-                        tmem_ld_wait();
-#pragma unroll
-                        for (int k = 0; k < 32; ++k) ov[k] = __float_as_uint(__uint_as_float(ov[k]) * factor);
-                        tmem_st_32cols(tm_o + c * 32, ov);
-                    }
-                }
-            }
-            // second pass: P = exp2(s - m_ref) as packed bf16 over the columns S came from.  The 16 columns written
-            // for keys [32 c, 32 c + 32) lie below column 16 c + 16, which this pass has already read.
-            const float nm = -m_ref;
-            float psum = 0.f;
-            {
-                uint32_t sa[32], sb[32];
-                tmem_ld_32cols(tm_s, sa);
-                tmem_ld_wait();
-#pragma unroll
-                for (int c = 0; c < TC_KT / 32; ++c) {
-                    uint32_t (&cur)[32] = (c & 1) ? sb : sa;
-                    uint32_t (&nxt)[32] = (c & 1) ? sa : sb;
-                    if (c + 1 < TC_KT / 32) tmem_ld_32cols(tm_s + (c + 1) * 32, nxt);
-                    uint32_t pk[16];
-                    if (ti.valid >= (c + 1) * 32) {
-#pragma unroll
-                        for (int k = 0; k < 32; k += 2) {
-                            const float e0 = fast_exp2(fmaf(__uint_as_float(cur[k]), c2, nm));
-                            const float e1 = fast_exp2(fmaf(__uint_as_float(cur[k + 1]), c2, nm));
-                            psum += e0 + e1;
-                            pk[k >> 1] = pack_bf16(e0, e1);
-                        }
-                    } else {
-#pragma unroll
-                        for (int k = 0; k < 32; k += 2) {
-                            float e0 = fast_exp2(fmaf(__uint_as_float(cur[k]), c2, nm));
-                            float e1 = fast_exp2(fmaf(__uint_as_float(cur[k + 1]), c2, nm));
-                            if (c * 32 + k >= ti.valid) e0 = 0.f;
-                            if (c * 32 + k + 1 >= ti.valid) e1 = 0.f;
-                            psum += e0 + e1;
-                            pk[k >> 1] = pack_bf16(e0, e1);
-                        }
-                    }
-                    if (c + 1 < TC_KT / 32) tmem_ld_wait();      // (the next columns, [32 c + 32, +32), lie above the store below)
-                    tmem_st_16cols(tm_s + c * 16, pk);
-                }
-            }
-            tmem_st_wait();
-            l += psum;
-            if (ti.valid < TC_KT) {
-                // V rows past the segment's end hold whatever lies behind it in memory: zero them so that
-                // probability 0 times garbage cannot make a NaN (thread r clears 16-byte pieces of those rows;
-                // both query tiles' warps do it, each before it releases its own second MMA)
-                uint8_t* vt = kv_s + stage * S::KV_STAGE + KV_BYTES;
-                const int n_bad = (TC_KT - ti.valid) * 8;       // 16-byte pieces per 64-column half
-                for (int h2 = 0; h2 < NHALF; ++h2)
-                    for (int q = r; q < n_bad; q += 128)
-                        *reinterpret_cast<uint4*>(vt + h2 * HALF_K + ti.valid * 128 + q * 16) = make_uint4(0, 0, 0, 0);
-                fence_proxy_async_smem();
-            }
-            tc_fence_before_sync();
-            mbar_arrive(&bars->p_full[j][buf]);
-        }
-        if (ok && n_tiles > 0) ok = mbar_wait(&bars->pv_done[j][(n_tiles - 1) & 1], ((n_tiles - 1) >> 1) & 1, abort_flag);
-        tc_fence_after_sync();
-        pdl_trigger();                                  // (this late for the reason given in the warp-level kernel)
-        const float inv = l > 0.f ? 1.f / l : 0.f;
-        // O rows leave through shared memory so that the global stores are coalesced (a thread holds one whole row,
-        // and 32 lanes storing 16 bytes each to 32 different rows cost a request per lane).  The tile's Q rows are
-        // no longer read (every S product has completed: the pipe runs the issuer's MMAs in order and the last P V
-        // has landed), so each warp turns its 32 rows in the place its Q rows had, in the same swizzled layout.
-        uint8_t* ot = q_s + j * S::Q_BYTES;
-#pragma unroll
-        for (int c2 = 0; c2 < D / 64; ++c2) {
-            uint32_t oa[32], ob[32];
-            tmem_ld_32cols(tm_o + c2 * 64, oa);          // (whole warp, also for rows that are not stored)
-            tmem_ld_32cols(tm_o + c2 * 64 + 32, ob);
-            tmem_ld_wait();
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const uint32_t (&ov)[32] = k < 4 ? oa : ob;
-                const int k8 = (k & 3) * 8, cc = c2 * 8 + k;
-                uint4 o;
-                o.x = pack_bf16(__uint_as_float(ov[k8 + 0]) * inv, __uint_as_float(ov[k8 + 1]) * inv);
-                o.y = pack_bf16(__uint_as_float(ov[k8 + 2]) * inv, __uint_as_float(ov[k8 + 3]) * inv);
-                o.z = pack_bf16(__uint_as_float(ov[k8 + 4]) * inv, __uint_as_float(ov[k8 + 5]) * inv);
-                o.w = pack_bf16(__uint_as_float(ov[k8 + 6]) * inv, __uint_as_float(ov[k8 + 7]) * inv);
-                *reinterpret_cast<uint4*>(ot + (cc >> 3) * HALF_Q + r * 128 + (((cc & 7) ^ (r & 7)) << 4)) = o;
+            __syncwarp();
+            tc_fence_before_sync();                          // (O has been read: the next unit's first P V may overwrite it)
+            if (p.lse != nullptr && r < rows_in_tile && pos0 + ri < w.L_eff) {
+                const int i = pos0 + ri, h = w.kvh * p.g + rh;
+                p.lse[packed ? static_cast<size_t>(h) * p.total_tokens + w.token0 + i
+                             : (static_cast<size_t>(w.b) * p.Hq + h) * p.L + i] = l > 0.f ? (m_ref + log2f(l)) * LN2_F : -INFINITY;
             }
         }
-        __syncwarp();
-        {
-            constexpr int CPR = D / 8;
-            const int c = lane % CPR;
-            RowWalk rw((warp & 3) * 32 + lane / CPR, 32 / CPR, p.g);
-            const int pos0 = (blockIdx.x * QT + j) * pos_per_tile;
-            uint4* dst = reinterpret_cast<uint4*>(p.out + ((q_token + pos0) * p.Hq + kvh * p.g) * D) + c;
-#pragma unroll
-            for (int k = 0; k < CPR; ++k, rw.next()) {
-                const int r2 = (warp & 3) * 32 + k * (32 / CPR) + lane / CPR;
-                if (ok && rw.i < pos_per_tile && pos0 + rw.i < L_eff)
-                    dst[(static_cast<size_t>(rw.i) * p.Hq + rw.h) * (D / 8)] =
-                        *reinterpret_cast<const uint4*>(ot + (c >> 3) * HALF_Q + r2 * 128 + (((c & 7) ^ (r2 & 7)) << 4));
-            }
-        }
-        if (ok && live && p.lse != nullptr)
-            p.lse[packed ? static_cast<size_t>(h) * p.total_tokens + seq_base + i
-                         : (static_cast<size_t>(b) * p.Hq + h) * p.L + i] = l > 0.f ? (m_ref + log2f(l)) * LN2_F : -INFINITY;
     }
 
     // teardown
@@ -869,17 +951,17 @@ attn_block_tc_kernel(const __grid_constant__ CUtensorMap tm_kpre, const __grid_c
         tc_fence_after_sync();
         tmem_dealloc(tmem_base, S::TMEM_COLS);
     }
-    if (p.beside_head && is_last_cta()) pdl_wait();
+    if (p.beside_head && has_last) pdl_wait();
 }
 
 template <int D, int QT>
-int launch_tc(const CUtensorMap* tm, const AttnParams& p, int q_tiles, cudaStream_t stream) {
+int launch_tc(const CUtensorMap& tm_q, const CUtensorMap* tm, const AttnParams& p, int q_tiles, cudaStream_t stream) {
     constexpr int SMEM = TcShape<D, QT>::SMEM;
     static std::atomic<uint64_t> smem_set{0};
     if (ensure_dynamic_smem(smem_set, attn_block_tc_kernel<D, QT>, SMEM) != DARE_OK) return DARE_ERR_CUDA;
     dim3 grid((q_tiles + QT - 1) / QT, p.B * p.Hkv, 1);
-    return launch_kernel(attn_block_tc_kernel<D, QT>, grid, TcShape<D, QT>::THREADS, SMEM, stream, 1, tm[0], tm[1], tm[2], tm[3],
-                         tm[4], tm[5], p);
+    return launch_kernel(attn_block_tc_kernel<D, QT>, grid, TcShape<D, QT>::THREADS, SMEM, stream, 1, tm_q, tm[0], tm[1], tm[2],
+                         tm[3], tm[4], tm[5], p);
 }
 
 // The tensor-core tile is worth it when a tile's 128 rows are mostly real query rows.
@@ -1019,10 +1101,13 @@ int launch_attn(const dare_ctx* ctx, const AttnArgs& a, cudaStream_t stream) {
         // two query tiles per CTA halve the K/V traffic, but only pay when the CTAs still fill the SMs
         const int pos_per_tile = 128 / p.g;
         const int q_tiles = (p.L + pos_per_tile - 1) / pos_per_tile;
+        CUtensorMap tm_q;
+        rc = make_tmap_bf16_3d(ctx, &tm_q, a.q, static_cast<uint64_t>(a.B) * a.L, a.Hq, a.d, pos_per_tile, p.g, 64);
+        if (rc != DARE_OK) return rc;
         const long long pairs = static_cast<long long>((q_tiles + 1) / 2) * p.B * p.Hkv;
         if (q_tiles >= 2 && 4 * pairs >= 3LL * ctx->sm_count)
-            return a.d == 128 ? launch_tc<128, 2>(tm, p, q_tiles, stream) : launch_tc<64, 2>(tm, p, q_tiles, stream);
-        return a.d == 128 ? launch_tc<128, 1>(tm, p, q_tiles, stream) : launch_tc<64, 1>(tm, p, q_tiles, stream);
+            return a.d == 128 ? launch_tc<128, 2>(tm_q, tm, p, q_tiles, stream) : launch_tc<64, 2>(tm_q, tm, p, q_tiles, stream);
+        return a.d == 128 ? launch_tc<128, 1>(tm_q, tm, p, q_tiles, stream) : launch_tc<64, 1>(tm_q, tm, p, q_tiles, stream);
     }
     const int nw = pick_variant(p.R).nw;
     const int chunks = (p.R + nw * 16 - 1) / (nw * 16);
@@ -1068,8 +1153,11 @@ int launch_attn_varlen(const dare_ctx* ctx, int total, int n_seqs, int max_seqle
     tm[2] = tm[0]; tm[3] = tm[1]; tm[4] = tm[0]; tm[5] = tm[1];
     const int pos_per_tile = 128 / p.g;
     const int q_tiles = (max_seqlen + pos_per_tile - 1) / pos_per_tile;
-    if (q_tiles >= 2) return d == 128 ? launch_tc<128, 2>(tm, p, q_tiles, stream) : launch_tc<64, 2>(tm, p, q_tiles, stream);
-    return d == 128 ? launch_tc<128, 1>(tm, p, q_tiles, stream) : launch_tc<64, 1>(tm, p, q_tiles, stream);
+    CUtensorMap tm_q;
+    rc = make_tmap_bf16_3d(ctx, &tm_q, q, static_cast<uint64_t>(total), Hq, d, pos_per_tile, p.g, 64);
+    if (rc != DARE_OK) return rc;
+    if (q_tiles >= 2) return d == 128 ? launch_tc<128, 2>(tm_q, tm, p, q_tiles, stream) : launch_tc<64, 2>(tm_q, tm, p, q_tiles, stream);
+    return d == 128 ? launch_tc<128, 1>(tm_q, tm, p, q_tiles, stream) : launch_tc<64, 1>(tm_q, tm, p, q_tiles, stream);
 }
 
 }  // namespace dare

@@ -21,8 +21,8 @@ struct TmapCache {
     static constexpr int SETS = 256, WAYS = 4, SLOTS = SETS * WAYS;
     struct Slot {
         const void* base;
-        uint64_t rows, cols;
-        uint32_t box_rows, box_cols;
+        uint64_t rows, mid, cols;              // mid = 0: two dimensions
+        uint32_t box_rows, box_mid, box_cols;
         bool valid;
         CUtensorMap map;
     };
@@ -134,6 +134,9 @@ inline int check_current_device(const dare_ctx* ctx) {
 // bf16 2-D row-major tensor [rows, cols] -> tensor map with a [box_rows, 64] box and 128-byte swizzle.
 int make_tmap_bf16_2d(const dare_ctx* ctx, CUtensorMap* out, const void* base, uint64_t rows, uint64_t cols,
                       uint32_t box_rows, uint32_t box_cols);
+// The same for [rows, mid, cols] with a [box_rows, box_mid, box_cols] box.
+int make_tmap_bf16_3d(const dare_ctx* ctx, CUtensorMap* out, const void* base, uint64_t rows, uint64_t mid, uint64_t cols,
+                      uint32_t box_rows, uint32_t box_mid, uint32_t box_cols);
 
 int launch_unmask_select(int32_t* tokens, int B, int64_t row_stride, int block_start, int L, const int32_t* pred,
                          const float* conf, int32_t mask_id, int mode, float threshold, int k, int32_t* n_committed,

@@ -91,6 +91,35 @@ __device__ __forceinline__ void st_host(int32_t* p, int32_t v) {
     asm volatile("st.relaxed.sys.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
+// ---------------------------------------------------------------- cluster launch control
+// Asks for the place of a CTA of this grid that has not been started yet: a 16-byte answer, counted on `bar`.  Not to be
+// asked again after an answer that holds none.
+__device__ __forceinline__ void clc_try_cancel(void* answer, uint64_t* bar) {
+    asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(
+                     smem_u32(answer)),
+                 "r"(smem_u32(bar))
+                 : "memory");
+}
+// The answer: whether there was one, and its index (x, y), which the caller now runs.
+__device__ __forceinline__ bool clc_query(const void* answer, uint32_t& x, uint32_t& y) {
+    uint32_t got;
+    asm volatile(
+        "{\n"
+        ".reg .b128 h;\n"
+        ".reg .pred p;\n"
+        "ld.shared.b128 h, [%3];\n"
+        "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, h;\n"
+        "selp.u32 %0, 1, 0, p;\n"
+        "mov.u32 %1, 0;\n"
+        "mov.u32 %2, 0;\n"
+        "@p clusterlaunchcontrol.query_cancel.get_first_ctaid.v4.b32.b128 {%1, %2, _, _}, h;\n"
+        "}\n"
+        : "=&r"(got), "=&r"(x), "=&r"(y)
+        : "r"(smem_u32(answer))
+        : "memory");
+    return got != 0;
+}
+
 // ---------------------------------------------------------------- thread-block cluster
 __device__ __forceinline__ uint32_t cluster_cta_rank() {
     uint32_t r;
@@ -136,6 +165,13 @@ __device__ __forceinline__ void tma_load_2d(void* smem_dst, const CUtensorMap* m
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
         ::"r"(smem_u32(smem_dst)), "l"(reinterpret_cast<uint64_t>(m)), "r"(smem_u32(bar)), "r"(c0), "r"(c1)
+        : "memory");
+}
+// 3-D tiled load (as above; the box's rows arrive one after the other, the middle dimension running faster).
+__device__ __forceinline__ void tma_load_3d(void* smem_dst, const CUtensorMap* m, uint64_t* bar, int c0, int c1, int c2) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
+        ::"r"(smem_u32(smem_dst)), "l"(reinterpret_cast<uint64_t>(m)), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2)
         : "memory");
 }
 // Asks for a tile to be brought into L2 (no shared-memory destination, nothing to wait for): issued a few
@@ -277,6 +313,15 @@ __device__ __forceinline__ void tmem_ld_32cols(uint32_t taddr, uint32_t (&v)[32]
         : "r"(taddr)
         : "memory");
 }
+// Load 16 consecutive fp32 columns of this thread's TMEM lane.  Whole warp.
+__device__ __forceinline__ void tmem_ld_16cols(uint32_t taddr, uint32_t (&v)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
+          "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+        : "r"(taddr)
+        : "memory");
+}
 // Load 8 consecutive fp32 columns of this thread's TMEM lane.  Whole warp.
 __device__ __forceinline__ void tmem_ld_8cols(uint32_t taddr, uint32_t (&v)[8]) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
@@ -284,6 +329,12 @@ __device__ __forceinline__ void tmem_ld_8cols(uint32_t taddr, uint32_t (&v)[8]) 
                  : "r"(taddr)
                  : "memory");
 }
+// Moves registers between the warpgroups of a CTA (all four warps of each must call it; the shares may not add up to more
+// than the launch's threads x registers).
+template <int REGS>
+__device__ __forceinline__ void set_max_regs_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS)); }
+template <int REGS>
+__device__ __forceinline__ void set_max_regs_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS)); }
 // Barrier among `count` threads of the CTA (a multiple of 32) on hardware barrier `id` (1..15; 0 is __syncthreads).
 __device__ __forceinline__ void named_barrier_sync(uint32_t id, uint32_t count) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
@@ -420,6 +471,32 @@ __device__ __forceinline__ float fast_exp2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
+}
+// Two fp32 values in a 64-bit register: one instruction works on both.
+__device__ __forceinline__ uint64_t pack_b32x2(uint32_t lo, uint32_t hi) {
+    uint64_t v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "r"(lo), "r"(hi));
+    return v;
+}
+__device__ __forceinline__ uint64_t pack_f32x2(float lo, float hi) { return pack_b32x2(__float_as_uint(lo), __float_as_uint(hi)); }
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t exp2_f32x2(uint64_t x) {
+    return pack_f32x2(fast_exp2(__uint_as_float(static_cast<uint32_t>(x))), fast_exp2(__uint_as_float(static_cast<uint32_t>(x >> 32))));
+}
+// The largest of three (a NaN loses).
+__device__ __forceinline__ float max3(uint32_t a, uint32_t b, uint32_t c) {
+    float d;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(__uint_as_float(a)), "f"(__uint_as_float(b)), "f"(__uint_as_float(c)));
+    return d;
 }
 
 }  // namespace dare

@@ -1,0 +1,77 @@
+"""The persistent tcgen05 attention kernel at the edges of its key tiles (64), query tiles (128 rows) and units, and with more
+units than CTAs, against the fp64 oracle.  Bars as in the other attention tests (one bf16 result: max-abs 2e-2, rel-L2 5e-3)."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import dare_oracle as O
+from paper_2604_04215_b200 import binding as dare
+from paper_2604_04215_b200 import inputs as I
+
+from _util import check_attn, f64
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = dare.Context(0)
+    yield c
+    c.close()
+
+
+@pytest.mark.parametrize("lens,Hq,Hkv,d", [
+    ([1, 63, 64, 65, 127, 128, 129, 255, 256, 257], 2, 2, 128),       # ends of key tiles; one and two live query tiles
+    ([191, 192, 193, 320, 449], 2, 1, 64),
+    ([35, 36, 37, 54, 55, 72, 73], 7, 1, 128),                        # 18 positions a tile: 126 of 128 rows, 36 a unit
+    ([int(n) for n in np.random.default_rng(5).integers(0, 150, 120)], 4, 4, 64),    # 480 units and more: CTAs take over units,
+    ([int(n) for n in np.random.default_rng(6).integers(0, 90, 90)], 6, 2, 128),     # empty sequences among them
+])
+def test_packed_units(ctx, lens, Hq, Hkv, d):
+    cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    T = int(cu[-1])
+    q, k, v = (I.normal_bf16(len(lens) + d, t, (T, h, d)) for t, h in ((I.TID_Q, Hq), (I.TID_KPRE, Hkv), (I.TID_VPRE, Hkv)))
+    ref, lse_ref = O.attn_varlen(f64(q), f64(k), f64(v), cu)
+    lse = torch.full((Hq, T), float("nan"), dtype=torch.float32, device="cuda")
+    out = torch.full_like(q, float("nan"), device="cuda")
+    dare.dare_attn_varlen(ctx, q.cuda(), k.cuda(), v.cuda(), torch.from_numpy(cu).cuda(), max(lens), out, lse)
+    torch.cuda.synchronize()
+    assert ctx.device_status() == 0
+    check_attn(out, ref)
+    assert np.abs(lse.cpu().double().numpy() - lse_ref).max() < 2e-2
+
+
+@pytest.mark.parametrize("B,L,Hq,Hkv,d,plens,slens", [
+    (3, 32, 14, 2, 128, [1, 64, 129], None),                # GQA group of 7, block apart from the cache
+    (2, 100, 2, 2, 128, [0, 65], [63, 1]),                  # no prefix; three segments, each with a ragged end
+    (5, 130, 64, 64, 64, [3, 64, 1, 100, 128], None),       # 320 units of two query tiles, the second with two rows
+    (90, 20, 14, 2, 128, None, None),                       # 180 units; 20 positions are two query tiles of 18
+])
+@pytest.mark.parametrize("inplace", [False, True])
+def test_block_units(ctx, B, L, Hq, Hkv, d, plens, slens, inplace):
+    plens = plens or [int(n) for n in np.random.default_rng(B).integers(0, 140, B)]
+    cap = max(plens) + L + 5
+    scap = max(slens) + 3 if slens else 0
+    q = I.normal_bf16(B, I.TID_Q, (B, L, Hq, d))
+    k, v = I.normal_bf16(B, I.TID_KPRE, (B, Hkv, cap, d)), I.normal_bf16(B, I.TID_VPRE, (B, Hkv, cap, d))
+    kb, vb = I.normal_bf16(B, I.TID_KBLK, (B, Hkv, L, d)), I.normal_bf16(B, I.TID_VBLK, (B, Hkv, L, d))
+    ks = I.normal_bf16(B + 1, I.TID_KPRE, (B, Hkv, scap, d)) if slens else None
+    vs = I.normal_bf16(B + 1, I.TID_VPRE, (B, Hkv, scap, d)) if slens else None
+    for b, n in enumerate(plens):                             # what lies behind the visible keys must not matter
+        if inplace:
+            k[b, :, n:n + L], v[b, :, n:n + L] = kb[b], vb[b]
+        end = n + L if inplace else n
+        k[b, :, end:], v[b, :, end:] = float("nan"), float("nan")
+    for b, n in enumerate(slens or []):
+        ks[b, :, n:], vs[b, :, n:] = float("nan"), float("nan")
+    g = lambda t: None if t is None else t.cuda()  # noqa: E731
+    pl = torch.tensor(plens, dtype=torch.int32)
+    sl = torch.tensor(slens, dtype=torch.int32) if slens else None
+    out = torch.full_like(q, float("nan"), device="cuda")
+    dare.dare_attn_block(ctx, g(q), g(k), g(v), g(pl), None if inplace else g(kb), None if inplace else g(vb), g(ks), g(vs),
+                         g(sl), out)
+    torch.cuda.synchronize()
+    assert ctx.device_status() == 0
+    c = lambda t: None if t is None else torch.nan_to_num(t.double(), nan=0.0).numpy()  # noqa: E731
+    res = O.attn_block(c(q), c(k), c(v), np.array(plens), c(kb), c(vb), c(ks), c(vs), None if sl is None else np.array(slens))
+    check_attn(out, res[0] if isinstance(res, tuple) else res)
