@@ -96,6 +96,17 @@ constexpr int LM_DIRECT_ROWS = 128;
 // Token of row m = tokens[(m / L) * stride + m % L]; tokens == NULL: no direct launch
 struct LmTokens { const int32_t* tokens; int L; int64_t stride; int32_t mask_id; };
 
+// Whether any of the rows is masked (a warp; all lanes get the answer).
+__device__ __forceinline__ bool any_masked(const LmTokens& t, int M, int lane) {
+    bool any = false;
+#pragma unroll
+    for (int u = 0; u < LM_DIRECT_ROWS / 32; ++u) {
+        const int m = lane + u * 32;
+        any |= m < M && row_token(t.tokens, t.L, t.stride, m) == t.mask_id;
+    }
+    return __any_sync(0xffffffffu, any);
+}
+
 // Compacts the still-masked rows of X into xc (order preserved), records their original indices, counts
 // them, and answers committed rows (pred = their token, conf = -inf).  One warp per row.
 constexpr int CP_ROWS = 8;
@@ -713,6 +724,7 @@ static_assert(SW_SMEM_BYTES + 1024 + 3 * (1024 + 512) <= 228 * 1024, "room for t
 // of them, stacked in shared memory (each a whole number of 1 KB swizzle atoms); a few rows too many may be loaded,
 // the MMA reads only its own.  (Exact covers of up to four boxes were measured slower: 432 us for 480 rows, where
 // each CTA loaded 64 + 32 + 16 + 8 rows per stage, against 350 us for 512 rows with one box.)
+constexpr int SW_UNSEEN = 4;                             // stages requested before it is known that a row is masked
 struct SwXMaps { CUtensorMap m[5]; };
 struct SwBoxes { int i1, i2, rows; };      // indices into SwXMaps::m (i2 < 0: one box), rows loaded in all
 __device__ __forceinline__ SwBoxes sw_boxes(int rows_half) {
@@ -752,11 +764,12 @@ __host__ __device__ inline SwPlan sw_plan(int rows, int n_units, int n_vt, bool 
     return p;
 }
 
-template <int MODE, bool JOINT>
+// LATE: nothing has been waited for yet, and only if a row is masked there is anything to do.
+template <int MODE, bool JOINT, bool LATE>
 __device__ __forceinline__ void
 lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, int V, int mask_col, int n_vt,
                 float* __restrict__ part_max, float* __restrict__ part_sum, int32_t* __restrict__ part_arg,
-                uint32_t* __restrict__ dev_status, int parts_stride, const LmSampling& smp) {
+                uint32_t* __restrict__ dev_status, int parts_stride, const LmSampling& smp, const LmTokens& tokens) {
     constexpr bool SAMPLE = MODE == LM_SAMPLE;
     if (Mc <= 0) return;
     const int rank = static_cast<int>(cluster_cta_rank());
@@ -822,37 +835,61 @@ lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, 
     tc_fence_before_sync();
     cluster_sync_all();                                  // both CTAs' barriers exist before either signals the other's
     tc_fence_after_sync();
-    pdl_trigger();
     const uint32_t tmem_base = bars->tmem_base;
     const int num_k = (D + BK - 1) / BK;
+    bool any = true;                                     // is any row masked?
+    const bool late = LATE && tokens.tokens != nullptr;      // (a run-time value: as a constant W came 1 % slower, 168.9 / 167.1 us)
+    if (late) {
+        pdl_wait();
+        pdl_trigger();
+        if (warp != 0) any = any_masked(tokens, Mc, lane);
+    } else {
+        pdl_trigger();
+    }
 
     // item w -> chunk w % n_chunks, vocabulary group w / n_chunks; the group's tiles are g, g + groups, ...
     if (warp == 0) {
+        const uint32_t full0 = cluster_map_shared(smem_u32(&bars->full[0]), 0);   // the even CTA's barriers count both CTAs' bytes
+        const SwBoxes box = xbox;
+        const auto load = [&](int item, int vt, int kb, int stage) {
+            const int x_row0 = (item % item_chunks) * nc + rank * rows_half, w_row0 = vt * (2 * SW_BV) + rank * SW_BV;
+            uint8_t* w_dst = tiles + stage * stage_bytes;
+            uint8_t* x_dst = w_dst + SW_W_BYTES;
+            const uint32_t full = full0 + stage * static_cast<uint32_t>(sizeof(uint64_t));
+            if (rank == 0) mbar_arrive_expect_tx(&bars->full[stage], 2u * static_cast<uint32_t>(SW_W_BYTES + box.rows * 128));
+            tma_load_2d_pair(w_dst, &tmap_w, full, kb * BK, w_row0);
+            tma_load_2d_pair(x_dst, &xmaps.m[box.i1], full, kb * BK, x_row0);
+            if (box.i2 >= 0)
+                tma_load_2d_pair(x_dst + (128 >> box.i1) * 128, &xmaps.m[box.i2], full, kb * BK, x_row0 + (128 >> box.i1));
+        };
         if (lane == 0) {
             prefetch_tensormap(&tmap_w);
 #pragma unroll
             for (int i = 0; i < 5; ++i) prefetch_tensormap(&xmaps.m[i]);
+        }
+        // LATE: the first stages are on their way while the tokens are looked at; if no row is masked after all, they are waited for.
+        int ahead = late ? min(SW_UNSEEN, num_k) : 0;
+        if (late) {
+            if (lane == 0)
+                for (int kb = 0; kb < ahead; ++kb) load(unit, unit / item_chunks, kb, kb);
+            __syncwarp();
+            any = any_masked(tokens, Mc, lane);
+            if (!any && lane == 0 && rank == 0)
+                for (int st = 0; st < ahead; ++st) mbar_wait(&bars->full[st], 0, abort_flag);
+        }
+        if (lane == 0 && any) {
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true;
-            const uint32_t full0 = cluster_map_shared(smem_u32(&bars->full[0]), 0);   // the even CTA's barriers count both CTAs' bytes
-            const SwBoxes box = xbox;
-            const uint32_t stage_tx = 2u * static_cast<uint32_t>(SW_W_BYTES + box.rows * 128);
             for (int item = unit; item < n_items && ok; item += n_units) {
-                const int x_row0 = (item % item_chunks) * nc + rank * rows_half;
                 for (int vt = item / item_chunks; vt < n_vt && ok; vt += groups) {
-                    const int w_row0 = vt * (2 * SW_BV) + rank * SW_BV;
                     for (int kb = 0; kb < num_k; ++kb) {
-                        if (!mbar_wait(&bars->empty[stage], phase ^ 1, abort_flag)) { ok = false; break; }
-                        uint8_t* w_dst = tiles + stage * stage_bytes;
-                        uint8_t* x_dst = w_dst + SW_W_BYTES;
-                        const uint32_t full = full0 + stage * static_cast<uint32_t>(sizeof(uint64_t));
-                        if (rank == 0) mbar_arrive_expect_tx(&bars->full[stage], stage_tx);
-                        tma_load_2d_pair(w_dst, &tmap_w, full, kb * BK, w_row0);
-                        tma_load_2d_pair(x_dst, &xmaps.m[box.i1], full, kb * BK, x_row0);
-                        if (box.i2 >= 0)
-                            tma_load_2d_pair(x_dst + (128 >> box.i1) * 128, &xmaps.m[box.i2], full, kb * BK,
-                                             x_row0 + (128 >> box.i1));
+                        if (ahead > 0) {
+                            --ahead;
+                        } else {
+                            if (!mbar_wait(&bars->empty[stage], phase ^ 1, abort_flag)) { ok = false; break; }
+                            load(item, vt, kb, stage);
+                        }
                         if (++stage == n_stages) { stage = 0; phase ^= 1; }
                     }
                 }
@@ -865,7 +902,7 @@ lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, 
         int stage = 0;
         uint32_t phase = 0;
         int it = 0;
-        bool ok = true;
+        bool ok = any;
         for (int item = unit; item < n_items && ok; item += n_units) {
             for (int vt = item / item_chunks; vt < n_vt && ok; vt += groups, ++it) {
                 int acc[J];
@@ -911,7 +948,7 @@ lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, 
         const uint32_t rng_step = SAMPLE ? smp.step + (smp.step_dev ? *smp.step_dev : 0u) : 0u;
         int it = 0;
         uint32_t items_done = 0;
-        bool ok = true;
+        bool ok = any;
         for (int item = unit; item < n_items && ok; item += n_units, ++items_done) {
             const int group = item / item_chunks;
             float run_max[SW_NMAX / 32], run_sum[SW_NMAX / 32];
@@ -1113,8 +1150,8 @@ __device__ __noinline__ void
 lm_joint_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, int V, int mask_col, int n_vt, float* __restrict__ part_max,
               float* __restrict__ part_sum, int32_t* __restrict__ part_arg, uint32_t* __restrict__ dev_status, int parts_stride,
               const LmSampling& smp) {
-    lm_swapped_body<LM_GREEDY, true>(tmap_w, xmaps, Mc, D, V, mask_col, n_vt, part_max, part_sum, part_arg, dev_status, parts_stride,
-                                     smp);
+    lm_swapped_body<LM_GREEDY, true, false>(tmap_w, xmaps, Mc, D, V, mask_col, n_vt, part_max, part_sum, part_arg, dev_status,
+                                            parts_stride, smp, LmTokens{});
 }
 
 // The greedy (or sampled) head, one launch on CTA pairs whatever the number of live rows (known only on the device when rows are
@@ -1123,30 +1160,39 @@ lm_joint_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, in
 // an odd count on pairs plus single CTAs for the last tile (see above).  The W
 // tile box is 128 rows for all of them.  A row's partials start at row * parts_stride; how many there are follows
 // from the same rules in lm_row_partials.
-template <int MODE>
+template <int MODE, bool DIRECT>
 __global__ void __launch_bounds__(LM_THREADS, 1)
 lmhead_head_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ SwXMaps xmaps, int M,
                      const int32_t* __restrict__ live_rows, int D, int V, int mask_col, int n_tiles,
                      float* __restrict__ part_max, float* __restrict__ part_sum, int32_t* __restrict__ part_arg,
                      uint32_t* __restrict__ dev_status, int parts_stride, const LmSampling smp, const LmTokens direct) {
-    pdl_wait();
-    if (direct.tokens) {
-        bool any = false;
-        for (int m = threadIdx.x; m < M; m += LM_THREADS)
-            any |= row_token(direct.tokens, direct.L, direct.stride, m) == direct.mask_id;
-        if (!__syncthreads_or(any)) return;              // (every CTA alike)
+    // DIRECT: rows evaluated where they lie.  How many is known before the predecessor is done, so the swapped path sets itself
+    // up beside it and waits in its place.  With what lmhead_merge_select_kernel does in front of its wait, a replayed step of 32
+    // rows x 512 x 4096 takes 12.0 us for 14.0, 128 rows x 256 x 1000 14.9 for 16.6, 32 rows x 4096 x 126464 165.6 for 167.5; one
+    // that finds no masked row 1 us more (its SW_UNSEEN stages).  (In one kernel with the other launches it slowed the sampled
+    // head of 416 rows by 1.4 %.)
+    if constexpr (DIRECT) {
+        if (lm_swapped(M, n_tiles, gridDim.x >> 1, D >= SW_DEEP, MODE == LM_SAMPLE)) {
+            lm_swapped_body<MODE, false, true>(tmap_w, xmaps, M, D, V, mask_col, n_tiles, part_max, part_sum, part_arg, dev_status,
+                                               parts_stride, smp, direct);
+            return;
+        }
     }
+    pdl_wait();
+    if (DIRECT && !any_masked(direct, M, threadIdx.x & 31)) return;      // (every warp of every CTA alike)
     const int Mc = live_rows ? *live_rows : M;          // rows that need logits (uniform over the grid)
-    if constexpr (MODE == LM_GREEDY) {
+    if constexpr (MODE == LM_GREEDY && !DIRECT) {
         if (lm_joint(Mc, n_tiles, gridDim.x >> 1, D >= SW_DEEP, false)) {
             lm_joint_body(tmap_w, xmaps, Mc, D, V, mask_col, n_tiles, part_max, part_sum, part_arg, dev_status, parts_stride, smp);
             return;
         }
     }
-    if (lm_swapped(Mc, n_tiles, gridDim.x >> 1, D >= SW_DEEP, MODE == LM_SAMPLE)) {
-        lm_swapped_body<MODE, false>(tmap_w, xmaps, Mc, D, V, mask_col, n_tiles, part_max, part_sum, part_arg, dev_status,
-                                     parts_stride, smp);
-        return;
+    if constexpr (!DIRECT) {
+        if (lm_swapped(Mc, n_tiles, gridDim.x >> 1, D >= SW_DEEP, MODE == LM_SAMPLE)) {
+            lm_swapped_body<MODE, false, false>(tmap_w, xmaps, Mc, D, V, mask_col, n_tiles, part_max, part_sum, part_arg, dev_status,
+                                                parts_stride, smp, direct);
+            return;
+        }
     }
     const int m_tiles = (Mc + BM - 1) / BM;
     const int cluster = blockIdx.x >> 1, n_clusters = gridDim.x >> 1;
@@ -1295,32 +1341,34 @@ lmhead_merge_select_kernel(const LmParts parts, int grid_gemm, int n_tiles, int 
     __shared__ float s_conf[32];
     __shared__ int32_t s_pred[32];
     pdl_trigger();      // (before the wait: the attention of the step, which may follow, does not depend on the head)
-    pdl_wait();
-    if (SAMPLE && step_dev && blockIdx.x == 0 && threadIdx.x == 0) *step_dev += 1;   // (as in lmhead_merge_kernel)
     const int b = blockIdx.x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;      // warp = block position (blockDim = 32 L)
-    // What a warp needs first is requested together: its token, the number of live rows, the row list.  Compacted rows
+    // The tokens, the number of live rows and the row list are as they were when the head, which still runs, started: it lets
+    // its successor in behind its own wait and writes none of them.  So all that follows from them stands in front of the wait
+    // (past L1, which may hold a line from before).  Compacted rows
     // that belong to earlier rollouts = entries of the ascending list below b * L.  (A binary search by one thread, nine
     // dependent loads at 512 rows, was half of this kernel's 8 us.)
     int32_t* row = sel.tokens_block + static_cast<int64_t>(b) * sel.row_stride;
-    const int32_t tok = row[warp];
+    const int32_t tok = __ldcg(row + warp);
     const bool masked = tok == mask_id;
-    const int Mc = live_rows ? *live_rows : M;              // (NULL: the rows were evaluated where they lie)
+    const int Mc = live_rows ? __ldcg(live_rows) : M;       // (NULL: the rows were evaluated where they lie)
     if (lane == 0) s_flag[warp] = masked ? 1 : 0;
     int before = 0;
     for (int i0 = 0; live_rows && i0 < b * L; i0 += blockDim.x) {   // (rows of earlier rollouts: at most b * L of them)
         const int i = i0 + threadIdx.x;
-        const int32_t v = i < b * L ? idx[i] : 0;           // (entries from Mc on hold anything)
+        const int32_t v = i < b * L ? __ldcg(idx + i) : 0;  // (entries from Mc on hold anything)
         before += __syncthreads_count(i < b * L && i < Mc && v < b * L);
     }
     __syncthreads();
+    int c = b * L + warp;
+    if (live_rows) {
+        c = before;
+        for (int i = 0; i < warp; ++i) c += s_flag[i];
+    }
+    const int groups = masked ? lm_row_partials(allow_pair, grid_gemm, Mc, n_tiles, c, SAMPLE) : 0;
+    pdl_wait();
+    if (SAMPLE && step_dev && blockIdx.x == 0 && threadIdx.x == 0) *step_dev += 1;   // (as in lmhead_merge_kernel)
     if (masked) {
-        int c = b * L + warp;
-        if (live_rows) {
-            c = before;
-            for (int i = 0; i < warp; ++i) c += s_flag[i];
-        }
-        const int groups = lm_row_partials(allow_pair, grid_gemm, Mc, n_tiles, c, SAMPLE);
         int a;
         float cf;
         merge_row_partials<SAMPLE>(parts, static_cast<size_t>(c) * (parts_stride < 0 ? groups : parts_stride), groups, lane, a, cf);
@@ -1509,11 +1557,12 @@ static int launch_head(const dare_ctx* ctx, int grid, bool pairs, const void* x_
         parts_stride = static_cast<int>(parts_max);
         constexpr int SMEM = SW_SMEM_BYTES;
         static_assert(SMEM >= LM_PAIR_SMEM_BYTES && SMEM >= LM_SMEM_BYTES, "shared memory");
-        static std::atomic<uint64_t> smem_set{0};
-        if (ensure_dynamic_smem(smem_set, lmhead_head_kernel<MODE>, SMEM) != DARE_OK) return DARE_ERR_CUDA;
-        rc = launch_kernel(lmhead_head_kernel<MODE>, dim3(static_cast<unsigned>(grid_gemm)), LM_THREADS, SMEM, stream, 2, tmap_w,
-                           xm, M, live_rows, D, V, mask_col, n_tiles, part_max, part_sum, part_arg, ctx->dev_status, parts_stride,
-                           smp, direct);
+        static std::atomic<uint64_t> smem_set[2] = {};
+        const bool in_place = direct.tokens != nullptr;
+        const auto kernel = in_place ? lmhead_head_kernel<MODE, true> : lmhead_head_kernel<MODE, false>;
+        if (ensure_dynamic_smem(smem_set[in_place], kernel, SMEM) != DARE_OK) return DARE_ERR_CUDA;
+        rc = launch_kernel(kernel, dim3(static_cast<unsigned>(grid_gemm)), LM_THREADS, SMEM, stream, 2, tmap_w, xm, M, live_rows, D, V,
+                           mask_col, n_tiles, part_max, part_sum, part_arg, ctx->dev_status, parts_stride, smp, direct);
         if (rc != DARE_OK) return rc;
     } else {
         CUtensorMap tmap_x;
