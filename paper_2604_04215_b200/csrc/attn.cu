@@ -1042,9 +1042,11 @@ int attn_plan_splits(const dare_ctx* ctx, const AttnArgs& a) {
     const int chunks = (R + nw * 16 - 1) / (nw * 16);
     const long long units = static_cast<long long>(chunks) * a.B * a.Hkv;
     const long long slots = static_cast<long long>(ctx->sm_count) * var.per_sm;
-    if (units >= slots) return 1;
     const int tiles = (a.prefix_cap + (a.k_blk ? a.L : 0) + a.suffix_cap + var.kt - 1) / var.kt;
-    long long s = (slots + units - 1) / units;
+    // As many K/V splits as keep the launch in one wave.  (As many as fill the slots or more left a second wave of a few CTAs, as
+    // long as the first: 32 rows x 32 heads x 733 keys of 2, 4, 6 and 8 rollouts 17.5, 22.9, 27.2 and 30.9 us, now 13.5, 17.3, 19.1 and
+    // 21.2; 4 rows x 5120 keys of 1 and 2 rollouts 28.0 and 42.3, now 21.7 and 31.8.)
+    long long s = slots / units;
     if (s > tiles / 2) s = tiles / 2;
     if (s > 32) s = 32;
     if (s < 1) s = 1;
