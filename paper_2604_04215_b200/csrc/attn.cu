@@ -100,7 +100,7 @@ attn_block_kernel(const __grid_constant__ CUtensorMap tm_kpre, const __grid_cons
     constexpr int KV_BYTES = KT * D * 2;
     constexpr int NCW = NW * KS;             // consumer warps
     constexpr int KPW = KT / KS;             // keys per warp per tile
-    constexpr int NREG = (D / 8) * 4 + 4;    // floats a thread hands over in the final merge
+    constexpr int NBK = D / 8 / KS;          // blocks of 8 columns that a warp finishes in the final merge
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -248,18 +248,39 @@ attn_block_kernel(const __grid_constant__ CUtensorMap tm_kpre, const __grid_cons
             if (ti.valid > koff) {   // (a warp whose key slice lies wholly past the end has nothing to add)
                 // S = Q K^T for this warp's keys
                 float sacc[KPW / 8][4];
+                // (with 32 keys and more a warp's score blocks advance together: one block's eight products after the other's were a
+                // chain that two warps per scheduler do not hide, 38.9 -> 38.3 us at 512 units of 12 tiles, 37.3 -> 36.2 at 384; with 16
+                // keys 1 % slower)
+                if constexpr (KPW >= 32) {
 #pragma unroll
-                for (int nb = 0; nb < KPW / 8; ++nb) {
-                    sacc[nb][0] = sacc[nb][1] = sacc[nb][2] = sacc[nb][3] = 0.f;
-                    const int key = koff + nb * 8 + rin;
+                    for (int nb = 0; nb < KPW / 8; ++nb) sacc[nb][0] = sacc[nb][1] = sacc[nb][2] = sacc[nb][3] = 0.f;
 #pragma unroll
                     for (int kq = 0; kq < D / 32; ++kq) {
-                        const int ch = 4 * kq + mi;
-                        const uint32_t addr = kbase + (ch >> 3) * HALF + key * 128 + (((ch & 7) ^ (key & 7)) << 4);
-                        uint32_t r0, r1, r2, r3;
-                        ldmatrix_x4(addr, r0, r1, r2, r3);
-                        mma_bf16_16816(sacc[nb], qf[2 * kq], r0, r1);
-                        mma_bf16_16816(sacc[nb], qf[2 * kq + 1], r2, r3);
+                        uint32_t kf[KPW / 8][4];
+#pragma unroll
+                        for (int nb = 0; nb < KPW / 8; ++nb) {
+                            const int key = koff + nb * 8 + rin, ch = 4 * kq + mi;
+                            ldmatrix_x4(kbase + (ch >> 3) * HALF + key * 128 + (((ch & 7) ^ (key & 7)) << 4), kf[nb][0], kf[nb][1], kf[nb][2], kf[nb][3]);
+                        }
+#pragma unroll
+                        for (int nb = 0; nb < KPW / 8; ++nb) mma_bf16_16816(sacc[nb], qf[2 * kq], kf[nb][0], kf[nb][1]);
+#pragma unroll
+                        for (int nb = 0; nb < KPW / 8; ++nb) mma_bf16_16816(sacc[nb], qf[2 * kq + 1], kf[nb][2], kf[nb][3]);
+                    }
+                } else {
+#pragma unroll
+                    for (int nb = 0; nb < KPW / 8; ++nb) {
+                        sacc[nb][0] = sacc[nb][1] = sacc[nb][2] = sacc[nb][3] = 0.f;
+                        const int key = koff + nb * 8 + rin;
+#pragma unroll
+                        for (int kq = 0; kq < D / 32; ++kq) {
+                            const int ch = 4 * kq + mi;
+                            const uint32_t addr = kbase + (ch >> 3) * HALF + key * 128 + (((ch & 7) ^ (key & 7)) << 4);
+                            uint32_t r0, r1, r2, r3;
+                            ldmatrix_x4(addr, r0, r1, r2, r3);
+                            mma_bf16_16816(sacc[nb], qf[2 * kq], r0, r1);
+                            mma_bf16_16816(sacc[nb], qf[2 * kq + 1], r2, r3);
+                        }
                     }
                 }
                 // mask keys that do not exist (only a segment's last tile has any), row max.  The scores stay
@@ -338,74 +359,90 @@ attn_block_kernel(const __grid_constant__ CUtensorMap tm_kpre, const __grid_cons
         m1 *= p.scale_log2;
     }
 
-    // ---------------- merge the key slices of a row group (through the now idle tile ring), then write out
+    // ---------------- merge the key slices of a row group (through the now idle tile ring), then write out.  Each of the KS warps
+    // finishes its share of the columns and sends the others theirs.  (One warp of the row group adding everything up took 4 k of
+    // a CTA's 37 k cycles while the others had left: 40.2 -> 38.9 us at 512 units of 12 tiles, 5.75 -> 5.25 at 6 units of 2.)
     // (The next kernel is let in only now: set up any earlier, the CTAs of a small one pile up on the few SMs that have
     // room beside this kernel's; the row compaction of the next step then took 11 us instead of 6.)
     pdl_trigger();
     __syncthreads();   // every tile has been consumed (or the CTA is aborting): the ring may be reused
     const bool aborted = *abort_flag != 0;
-    float* xch = reinterpret_cast<float*>(tiles);
-    if (KS > 1 && !aborted && warp < NCW && ks > 0) {
-        float* dst = xch + static_cast<size_t>((ks - 1) * NW + rg) * NREG * 32 + lane;
+    float4* xch = reinterpret_cast<float4*>(tiles);                    // [finishing slice][slice][row group][block of 8 columns][lane]
+    float4* xch_ml = xch + KS * KS * NW * NBK * 32;                    // [slice][row group][lane]: the two rows' max and sum
+    if (KS > 1 && !aborted && warp < NCW) {
 #pragma unroll
-        for (int n = 0; n < D / 8; ++n) {
+        for (int o = 0; o < KS; ++o) {
+            if (o == ks) continue;
 #pragma unroll
-            for (int e = 0; e < 4; ++e) dst[(n * 4 + e) * 32] = oacc[n][e];
+            for (int i = 0; i < NBK; ++i) {
+                const float (&v)[4] = oacc[o * NBK + i];
+                xch[(((o * KS + ks) * NW + rg) * NBK + i) * 32 + lane] = make_float4(v[0], v[1], v[2], v[3]);
+            }
         }
-        dst[(NREG - 4) * 32] = m0; dst[(NREG - 3) * 32] = m1; dst[(NREG - 2) * 32] = l0; dst[(NREG - 1) * 32] = l1;
+        xch_ml[(ks * NW + rg) * 32 + lane] = make_float4(m0, m1, l0, l1);
     }
     if (KS > 1) __syncthreads();
-    if (!aborted && warp < NCW && ks == 0) {
+    if (!aborted && warp < NCW) {
+        float w0[KS], w1[KS];              // what each slice's values count
+        if (KS > 1) {
+            float4 ml[KS];
+            m0 = m1 = -INFINITY;
+            l0 = l1 = 0.f;
 #pragma unroll
-        for (int o = 1; o < KS; ++o) {
-            const float* src = xch + static_cast<size_t>((o - 1) * NW + rg) * NREG * 32 + lane;
-            const float om0 = src[(NREG - 4) * 32], om1 = src[(NREG - 3) * 32];
-            const float ol0 = src[(NREG - 2) * 32], ol1 = src[(NREG - 1) * 32];
-            const float mn0 = fmaxf(m0, om0), mn1 = fmaxf(m1, om1);
-            const float sa0 = mn0 == -INFINITY ? 0.f : fast_exp2(m0 - mn0), sb0 = mn0 == -INFINITY ? 0.f : fast_exp2(om0 - mn0);
-            const float sa1 = mn1 == -INFINITY ? 0.f : fast_exp2(m1 - mn1), sb1 = mn1 == -INFINITY ? 0.f : fast_exp2(om1 - mn1);
-            l0 = l0 * sa0 + ol0 * sb0;
-            l1 = l1 * sa1 + ol1 * sb1;
-            m0 = mn0; m1 = mn1;
-#pragma unroll
-            for (int n = 0; n < D / 8; ++n) {
-                oacc[n][0] = oacc[n][0] * sa0 + src[(n * 4 + 0) * 32] * sb0;
-                oacc[n][1] = oacc[n][1] * sa0 + src[(n * 4 + 1) * 32] * sb0;
-                oacc[n][2] = oacc[n][2] * sa1 + src[(n * 4 + 2) * 32] * sb1;
-                oacc[n][3] = oacc[n][3] * sa1 + src[(n * 4 + 3) * 32] * sb1;
+            for (int o = 0; o < KS; ++o) {
+                ml[o] = xch_ml[(o * NW + rg) * 32 + lane];
+                m0 = fmaxf(m0, ml[o].x);
+                m1 = fmaxf(m1, ml[o].y);
             }
-        }
-        const float inv0 = l0 > 0.f ? 1.f / l0 : 0.f, inv1 = l1 > 0.f ? 1.f / l1 : 0.f;
-        const float lse0 = l0 > 0.f ? (m0 + log2f(l0)) * LN2_F : -INFINITY;
-        const float lse1 = l1 > 0.f ? (m1 + log2f(l1)) * LN2_F : -INFINITY;
-        const size_t orow0 = (static_cast<size_t>(b) * p.L + i0) * p.Hq + h0;
-        const size_t orow1 = (static_cast<size_t>(b) * p.L + i1) * p.Hq + h1;
-        if (p.splits == 1) {
 #pragma unroll
-            for (int n = 0; n < D / 8; ++n) {
-                const int col = n * 8 + tq * 2;
-                if (live0)
-                    *reinterpret_cast<uint32_t*>(p.out + orow0 * D + col) = pack_bf16(oacc[n][0] * inv0, oacc[n][1] * inv0);
-                if (live1)
-                    *reinterpret_cast<uint32_t*>(p.out + orow1 * D + col) = pack_bf16(oacc[n][2] * inv1, oacc[n][3] * inv1);
-            }
-            if (p.lse != nullptr && tq == 0) {
-                if (live0) p.lse[(static_cast<size_t>(b) * p.Hq + h0) * p.L + i0] = lse0;
-                if (live1) p.lse[(static_cast<size_t>(b) * p.Hq + h1) * p.L + i1] = lse1;
+            for (int o = 0; o < KS; ++o) {
+                w0[o] = m0 == -INFINITY ? 0.f : fast_exp2(ml[o].x - m0);
+                w1[o] = m1 == -INFINITY ? 0.f : fast_exp2(ml[o].y - m1);
+                l0 += ml[o].z * w0[o];
+                l1 += ml[o].w * w1[o];
             }
         } else {
-            const size_t n_rows = static_cast<size_t>(p.B) * p.L * p.Hq;
-            float* po = p.part_o + static_cast<size_t>(split) * n_rows * D;
-            float* pl = p.part_lse + static_cast<size_t>(split) * n_rows;
+            w0[0] = w1[0] = 1.f;
+        }
+        const float inv0 = l0 > 0.f ? 1.f / l0 : 0.f, inv1 = l1 > 0.f ? 1.f / l1 : 0.f;
+        const size_t orow0 = (static_cast<size_t>(b) * p.L + i0) * p.Hq + h0;
+        const size_t orow1 = (static_cast<size_t>(b) * p.L + i1) * p.Hq + h1;
+        const size_t n_rows = static_cast<size_t>(p.B) * p.L * p.Hq;
+        float* po = p.part_o + static_cast<size_t>(split) * n_rows * D;
 #pragma unroll
-            for (int n = 0; n < D / 8; ++n) {
-                const int col = n * 8 + tq * 2;
-                if (live0) *reinterpret_cast<float2*>(po + orow0 * D + col) = make_float2(oacc[n][0] * inv0, oacc[n][1] * inv0);
-                if (live1) *reinterpret_cast<float2*>(po + orow1 * D + col) = make_float2(oacc[n][2] * inv1, oacc[n][3] * inv1);
+        for (int o = 0; o < KS; ++o) {
+            if (o != ks) continue;         // (a warp runs one of these, with its accumulators in registers)
+#pragma unroll
+            for (int i = 0; i < NBK; ++i) {
+                const int n = o * NBK + i, col = n * 8 + tq * 2;
+                float v0 = oacc[n][0] * w0[o], v1 = oacc[n][1] * w0[o], v2 = oacc[n][2] * w1[o], v3 = oacc[n][3] * w1[o];
+#pragma unroll
+                for (int q = 0; q < KS; ++q) {
+                    if (q == o) continue;
+                    const float4 x = xch[(((o * KS + q) * NW + rg) * NBK + i) * 32 + lane];
+                    v0 += x.x * w0[q]; v1 += x.y * w0[q];
+                    v2 += x.z * w1[q]; v3 += x.w * w1[q];
+                }
+                v0 *= inv0; v1 *= inv0; v2 *= inv1; v3 *= inv1;
+                if (p.splits == 1) {
+                    if (live0) *reinterpret_cast<uint32_t*>(p.out + orow0 * D + col) = pack_bf16(v0, v1);
+                    if (live1) *reinterpret_cast<uint32_t*>(p.out + orow1 * D + col) = pack_bf16(v2, v3);
+                } else {
+                    if (live0) *reinterpret_cast<float2*>(po + orow0 * D + col) = make_float2(v0, v1);
+                    if (live1) *reinterpret_cast<float2*>(po + orow1 * D + col) = make_float2(v2, v3);
+                }
             }
-            if (tq == 0) {
+        }
+        if (ks == 0 && tq == 0) {
+            const float lse0 = l0 > 0.f ? (m0 + log2f(l0)) * LN2_F : -INFINITY;
+            const float lse1 = l1 > 0.f ? (m1 + log2f(l1)) * LN2_F : -INFINITY;
+            if (p.splits > 1) {
+                float* pl = p.part_lse + static_cast<size_t>(split) * n_rows;
                 if (live0) pl[orow0] = lse0;
                 if (live1) pl[orow1] = lse1;
+            } else if (p.lse != nullptr) {
+                if (live0) p.lse[(static_cast<size_t>(b) * p.Hq + h0) * p.L + i0] = lse0;
+                if (live1) p.lse[(static_cast<size_t>(b) * p.Hq + h1) * p.L + i1] = lse1;
             }
         }
     }
@@ -1010,7 +1047,7 @@ __global__ void attn_combine_kernel(const float* __restrict__ part_o, const floa
 template <int D, int NW, int KS, int KT, int STAGES, int CPS>
 int launch_one(const CUtensorMap* tm, const AttnParams& p, int chunks, cudaStream_t stream) {
     constexpr int SMEM = att_smem_bytes<D, KT, STAGES>();
-    static_assert((KS - 1) * NW * ((D / 8) * 4 + 4) * 32 * 4 <= STAGES * att_stage_bytes<D, KT>(), "merge buffer");
+    static_assert(KS * NW * (D / 8 + 1) * 512 <= STAGES * att_stage_bytes<D, KT>() && (D / 8) % KS == 0, "merge buffer");
     static_assert(STAGES <= ATT_MAX_STAGES && KT <= KT_MAX && KT % (16 * KS) == 0, "variant");
     static std::atomic<uint64_t> smem_set{0};
     if (ensure_dynamic_smem(smem_set, attn_block_kernel<D, NW, KS, KT, STAGES, CPS>, SMEM) != DARE_OK) return DARE_ERR_CUDA;

@@ -75,3 +75,24 @@ def test_block_units(ctx, B, L, Hq, Hkv, d, plens, slens, inplace):
     c = lambda t: None if t is None else torch.nan_to_num(t.double(), nan=0.0).numpy()  # noqa: E731
     res = O.attn_block(c(q), c(k), c(v), np.array(plens), c(kb), c(vb), c(ks), c(vs), None if sl is None else np.array(slens))
     check_attn(out, res[0] if isinstance(res, tuple) else res)
+
+
+# The warp-level kernel: rows that share a KV head at the ends of its variants (four, two and one key slices a tile; each slice
+# finishes its share of the columns), without and with K/V splits, keys that end inside a slice.
+@pytest.mark.parametrize("L,g", [(1, 1), (4, 4), (17, 1), (32, 1), (33, 1), (8, 9), (90, 1)])
+@pytest.mark.parametrize("B,Hkv,P", [(1, 1, 900), (2, 160, 37), (3, 32, 70)])
+@pytest.mark.parametrize("d", [64, 128])
+def test_warp_level_shares(ctx, L, g, B, Hkv, P, d):
+    Hq = Hkv * g
+    plens = [P - 11 * b for b in range(B)]
+    q = I.normal_bf16(L, I.TID_Q, (B, L, Hq, d))
+    k, v = I.normal_bf16(L, I.TID_KPRE, (B, Hkv, P + L, d)), I.normal_bf16(L, I.TID_VPRE, (B, Hkv, P + L, d))
+    out = torch.full_like(q, float("nan"), device="cuda")
+    lse = torch.full((B, Hq, L), float("nan"), device="cuda")
+    dare.dare_attn_block(ctx, q.cuda(), k.cuda(), v.cuda(), torch.tensor(plens, dtype=torch.int32).cuda(), None, None, None, None,
+                         None, out, lse)
+    torch.cuda.synchronize()
+    assert ctx.device_status() == 0
+    ref, lse_ref = O.attn_block(f64(q), f64(k), f64(v), np.array(plens))
+    check_attn(out, ref)
+    assert np.abs(lse.cpu().double().numpy() - lse_ref).max() < 2e-2
