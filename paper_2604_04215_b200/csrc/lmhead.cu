@@ -1397,7 +1397,8 @@ lmhead_merge_select_kernel(const LmParts parts, int grid_gemm, int n_tiles, int 
         } else {
             const int want = sel.mode == DARE_SELECT_TOPK ? sel.k : 1;
             int rank = 0;
-            for (int j = 0; j < L; ++j) {
+#pragma unroll 8
+            for (int j = 0; j < L; ++j) {                              // (one after the other each is a trip to shared memory)
                 const float cj = s_conf[j];
                 rank += (cj > cf || (cj == cf && j < lane)) ? 1 : 0;   // NaN (absent) compares false
             }
@@ -1605,8 +1606,14 @@ int launch_lmhead(const dare_ctx* ctx, void* scratch, const void* hidden, int M,
     const bool pairs = grid >= 2 && lm_pair_available() &&
                        lmhead_scratch_bytes(M, D, V, ctx->sm_count, row_tokens != nullptr, sample != nullptr, 2) <= ctx->workspace_bytes;
     // The swapped path wants a CTA pair per vocabulary tile also where the rows make a single tile: with half of them each took
-    // two tiles, one after the other (128 rows x 256 x 4096 23.9 us, now 17.0; the greedy epilogue is too short to show it).
-    if (pairs && sample != nullptr && m_tiles_max == 1) grid = n_tiles < ctx->sm_count / 2 ? 2 * n_tiles : ctx->sm_count;
+    // two tiles, one after the other (sampled 128 rows x 256 x 4096 23.9 us, now 17.0; a greedy step of 32 rows x 256 x 4096 10.6, now
+    // 9.3, of 128 rows 15.4 and 12.3, x 1024 x 32000 24.0 and 20.8).  Where twice the pairs need as many rounds, the greedy head is
+    // better off with half of them (32 rows x 2048 x 24000 24.4 and 23.5).
+    if (pairs && m_tiles_max == 1) {
+        const int all = n_tiles < ctx->sm_count / 2 ? 2 * n_tiles : ctx->sm_count;
+        const auto rounds = [&](int ctas) { return (n_tiles + ctas / 2 - 1) / (ctas / 2); };
+        if (sample != nullptr || rounds(all) < rounds(grid)) grid = all;
+    }
     LmTokens direct = {};
     if (row_tokens != nullptr && pairs && M <= LM_DIRECT_ROWS) {
         direct = {row_tokens, tok_L, tok_row_stride, mask_id};
