@@ -13,8 +13,9 @@
 //     of the library writes), so the stream does not stop between kernels;
 //   * the CTAs of a tile's K slices form a cluster; each sends the accumulator columns (rows of A) it does not own to their
 //     owner through distributed shared memory, the owners add the slices in order and apply the epilogue: a thread holds 8
-//     consecutive features of one row, which is what SwiGLU (a tile: 64 gate and the matching 64 up rows), RoPE (a tile
-//     holds whole heads; channel c and its partner c + d/2 are in the same slab) and coalesced stores want.
+//     consecutive features of one row (up to FEW_QUAD_ROWS rows: two features of four rows, so that four rows go in one remote
+//     store), which is what SwiGLU (a tile: 64 gate and the matching 64 up rows), RoPE (a tile holds whole heads; channel c
+//     and its partner c + d/2 are in the same slab) and coalesced stores want.
 //   warp 0 TMA producer, warp 1 MMA issuer, warps 2..5 epilogue (TMEM lane = W row).
 #include <math.h>
 
@@ -46,7 +47,14 @@ struct FewPlan {
     int splits;      // CTAs along K per tile = cluster size (1, 2, 4 or 8)
     int stages;
     int tiles;
+    int quads;       // QUADS: groups of four rows of A that a CTA of a cluster finishes (the last ones may have none)
 };
+// Up to this many rows the slices are handed over four rows at a time (QUADS): value by value the stores to the other CTAs were
+// 1.25 of the 3.8 us that a small projection of 48 rows takes behind its wait.  A stack of 3 layers of 512 / 1280 values, us, value by
+// value / four rows: 16 rows 78.8 / 78.1, 48 rows 88.9 / 85.5, 64 rows 97.2 / 94.0; 64 rows of 2 layers of 256 62.6 / 60.4, 32 rows of 2
+// LLaDA-shaped layers 205.0 / 203.9.  More rows are cut into fewer slices, and a CTA's last part is then the longer one, where
+// 16 bytes per load and store count: 72 rows 99.0 / 107.7, 128 rows 136 / 155.
+constexpr int FEW_QUAD_ROWS = 64;
 
 FewPlan few_plan(int epi, int M, int N, int K, int sm_count) {
     FewPlan p;
@@ -59,6 +67,7 @@ FewPlan few_plan(int epi, int M, int N, int K, int sm_count) {
     // exchange takes longer (128 rows, K = 1024, N = 4096: eight slices 13.0 us, two 9.6; K = 512, N = 1280: 6.7 either way)
     const int least = p.nr > 64 ? p.nr / 16 : 2;
     while (p.splits < 8 && 2LL * p.splits * p.tiles <= 2LL * sm_count && nk >= 2 * least * p.splits) p.splits *= 2;
+    p.quads = (p.nr / 4 + p.splits - 1) / p.splits;
     const int stages = FEW_RING / (FEW_W_BYTES + p.nr * FK * 2);
     p.stages = stages > FEW_MAX_STAGES ? FEW_MAX_STAGES : stages;
     return p;
@@ -87,7 +96,11 @@ __device__ __forceinline__ void st_shared_cluster_f32(uint32_t addr, uint32_t v)
     asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 
-template <int EPI>
+__device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+
+template <int EPI, bool QUADS>
 __global__ void __launch_bounds__(FEW_THREADS, 2)
 gemm_few_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_w2,
                 const __grid_constant__ CUtensorMap tmap_a, const FewArgs g) {
@@ -185,11 +198,35 @@ gemm_few_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
     }
     __syncwarp();
 
-    // Hand-over: the ring of every CTA of the cluster is idle now.  Slab of the owner: [K slice][row][128 features].
+    // Hand-over: the ring of every CTA of the cluster is idle now.  Slab of the owner: [K slice][row][128 features], or QUADS
+    // [K slice][four rows][128 features][row].
     const int per_owner = p.nr / p.splits;               // rows of A that a CTA finishes (nr is a multiple of 16)
     if (p.splits > 1) cluster_sync_all();
     else __syncthreads();
-    if (warp >= 2) {
+    if (QUADS && warp >= 2) {
+        const int f = (warp & 3) * 32 + lane;            // W row of the tile = TMEM lane
+        const uint32_t taddr = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16);
+        const uint32_t slab = smem_u32(tiles) + (static_cast<uint32_t>(split) * p.quads * FW + f) * 16;
+        int owner = 0, q = 0;
+        uint32_t addr = p.splits > 1 ? cluster_map_shared(slab, 0u) : slab;
+        for (int c0 = 0; c0 < g.M; c0 += 16) {           // (columns from M on are padding rows: stored, not read)
+            uint32_t v[16];
+            tmem_ld_16cols(taddr + c0, v);
+            tmem_ld_wait();
+#pragma unroll
+            for (int c = 0; c < 16; c += 4) {
+                if (c0 + c < g.M) {
+                    if (p.splits > 1) st_shared_cluster_v4(addr, v[c], v[c + 1], v[c + 2], v[c + 3]);
+                    else st_shared_v4(addr, v[c], v[c + 1], v[c + 2], v[c + 3]);
+                }
+                addr += FW * 16;
+                if (++q == p.quads) {
+                    q = 0;
+                    if (++owner < p.splits) addr = cluster_map_shared(slab, static_cast<uint32_t>(owner));
+                }
+            }
+        }
+    } else if (warp >= 2) {
         // (owner and row are counted, not divided out, and 16 columns are read at a time: with two divisions per column and
         // every 8 columns waited for, each row cost 68 ns, 128 rows 8.6 us)
         const int f = (warp & 3) * 32 + lane;            // W row of the tile = TMEM lane
@@ -229,7 +266,96 @@ gemm_few_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
 
     // the last part is for all warps (the first two have not waited for the predecessor with all their lanes yet)
     if (warp < 2) pdl_wait();
-    if (!*abort_flag) {
+    if (QUADS && !*abort_flag) {
+        const float4* slab = reinterpret_cast<const float4*>(tiles);
+        // features f and f + 1 of the four rows of group q, the K slices added in order
+        const auto sum = [&](int q, int f, float (&s)[2][4]) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) s[0][j] = s[1][j] = 0.f;
+            for (int k = 0; k < p.splits; ++k) {
+                const float4 a = slab[(k * p.quads + q) * FW + f], b = slab[(k * p.quads + q) * FW + f + 1];
+                s[0][0] += a.x; s[0][1] += a.y; s[0][2] += a.z; s[0][3] += a.w;
+                s[1][0] += b.x; s[1][1] += b.y; s[1][2] += b.z; s[1][3] += b.w;
+            }
+        };
+        const int t = threadIdx.x;
+        const int row0 = split * p.quads * 4;
+        const int n_rows = min(p.quads * 4, g.M - row0);   // (may be negative: nothing to do)
+        const int n_quads = (n_rows + 3) / 4;
+        if (EPI == GEMM_EPI_ROPE) {
+            const RopeArgs& r = g.rope;
+            const int pph = r.d / 4;                     // channel pairs of half a head
+            for (int i = t; i < n_quads * (FW / 4); i += FEW_THREADS) {
+                const int q = i / (FW / 4), u = i % (FW / 4);
+                const int hh = u / pph, c = (u % pph) * 2;
+                const int H = tile * (FW / r.d) + hh;
+                if (H >= r.Hq + 2 * r.Hkv) continue;
+                const bool turns = H < r.Hq + r.Hkv, k = H < r.Hq + r.Hkv;
+                int m[4], pos[4], bb[4];
+                float4 e[4];                             // (cos, sin) of the two channels
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    m[j] = min(row0 + q * 4 + j, g.M - 1);
+                    bb[j] = m[j] / r.length;
+                    pos[j] = r.start + m[j] - bb[j] * r.length;
+                    if (turns) e[j] = *reinterpret_cast<const float4*>(r.cs + (static_cast<size_t>(pos[j]) * (r.d / 2) + c) * 2);
+                }
+                float a[2][4], b[2][4];
+                sum(q, hh * r.d + c, a);
+                sum(q, hh * r.d + r.d / 2 + c, b);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (q * 4 + j >= n_rows) break;
+                    __nv_bfloat16* dst;
+                    if (H < r.Hq) {
+                        dst = static_cast<__nv_bfloat16*>(r.q_out) + (static_cast<size_t>(m[j]) * r.Hq + H) * r.d;
+                    } else {
+                        const int h = H - r.Hq - (k ? 0 : r.Hkv);
+                        dst = static_cast<__nv_bfloat16*>(k ? r.k_cache : r.v_cache) +
+                              ((static_cast<size_t>(bb[j]) * r.Hkv + h) * r.cap + pos[j]) * r.d;
+                    }
+                    if (turns) {                         // (the projection is rounded to bf16 before it turns)
+                        const float x1 = round_bf16(a[0][j]), x2 = round_bf16(b[0][j]), y1 = round_bf16(a[1][j]), y2 = round_bf16(b[1][j]);
+                        a[0][j] = x1 * e[j].x - x2 * e[j].y;
+                        b[0][j] = x2 * e[j].x + x1 * e[j].y;
+                        a[1][j] = y1 * e[j].z - y2 * e[j].w;
+                        b[1][j] = y2 * e[j].z + y1 * e[j].w;
+                    }
+                    *reinterpret_cast<uint32_t*>(dst + c) = pack_bf16(a[0][j], a[1][j]);
+                    *reinterpret_cast<uint32_t*>(dst + r.d / 2 + c) = pack_bf16(b[0][j], b[1][j]);
+                }
+            }
+        } else {
+            constexpr int pairs = (EPI == GEMM_EPI_SWIGLU ? FW / 2 : FW) / 2;
+            for (int i = t; i < n_quads * pairs; i += FEW_THREADS) {
+                const int q = i / pairs, f = (i % pairs) * 2, col = tile * p.wcols + f;
+                if (col >= g.N) continue;                // (N is a multiple of 8)
+                const size_t o = static_cast<size_t>(row0 + q * 4) * g.ldo + col;
+                uint32_t x[4];
+                if (EPI == GEMM_EPI_RESIDUAL) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        if (q * 4 + j < n_rows) x[j] = *reinterpret_cast<const uint32_t*>(g.res + o + static_cast<size_t>(j) * g.ldo);
+                }
+                float a[2][4], up[2][4];
+                sum(q, f, a);
+                if (EPI == GEMM_EPI_SWIGLU) sum(q, FW / 2 + f, up);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (q * 4 + j >= n_rows) break;
+                    float y0 = a[0][j], y1 = a[1][j];
+                    if (EPI == GEMM_EPI_SWIGLU) {        // silu(gate) * up
+                        y0 = __fdividef(y0, 1.0f + __expf(-y0)) * up[0][j];
+                        y1 = __fdividef(y1, 1.0f + __expf(-y1)) * up[1][j];
+                    } else if (EPI == GEMM_EPI_RESIDUAL) {
+                        y0 += lo_f(x[j]);
+                        y1 += hi_f(x[j]);
+                    }
+                    *reinterpret_cast<uint32_t*>(g.out + o + static_cast<size_t>(j) * g.ldo) = pack_bf16(y0, y1);
+                }
+            }
+        }
+    } else if (!*abort_flag) {
         const float* slab = reinterpret_cast<const float*>(tiles);
         // 8 features from feature c of row r, the K slices added in order
         const auto sum8 = [&](int r, int c, float (&s)[8]) {
@@ -330,11 +456,13 @@ gemm_few_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
 
 template <int EPI>
 int launch_few(const CUtensorMap& tw, const CUtensorMap& tw2, const CUtensorMap& ta, const FewArgs& g, cudaStream_t stream) {
-    static std::atomic<uint64_t> smem_set{0};
-    if (ensure_dynamic_smem(smem_set, gemm_few_kernel<EPI>, FEW_SMEM) != DARE_OK) return DARE_ERR_CUDA;
+    static std::atomic<uint64_t> smem_set[2] = {};
+    const bool quad = g.p.nr <= FEW_QUAD_ROWS;
+    const auto kernel = quad ? gemm_few_kernel<EPI, true> : gemm_few_kernel<EPI, false>;
+    if (ensure_dynamic_smem(smem_set[quad], kernel, FEW_SMEM) != DARE_OK) return DARE_ERR_CUDA;
     const long long ctas = static_cast<long long>(g.p.tiles) * g.p.splits;
     if (ctas > 0x7fffffffLL) return DARE_ERR_SHAPE;
-    return launch_kernel(gemm_few_kernel<EPI>, dim3(static_cast<unsigned>(ctas)), FEW_THREADS, FEW_SMEM, stream, g.p.splits, tw,
+    return launch_kernel(kernel, dim3(static_cast<unsigned>(ctas)), FEW_THREADS, FEW_SMEM, stream, g.p.splits, tw,
                          tw2, ta, g);
 }
 
