@@ -47,6 +47,7 @@ struct FewPlan {
     int splits;      // CTAs along K per tile = cluster size (1, 2, 4 or 8)
     int stages;
     int tiles;
+    int slab;        // QUADS: where the slices are added: its offset in the ring, behind the stages in use (0: over them)
     int quads;       // QUADS: groups of four rows of A that a CTA of a cluster finishes (the last ones may have none)
 };
 // Up to this many rows the slices are handed over four rows at a time (QUADS): value by value the stores to the other CTAs were
@@ -70,6 +71,10 @@ FewPlan few_plan(int epi, int M, int N, int K, int sm_count) {
     p.quads = (p.nr / 4 + p.splits - 1) / p.splits;
     const int stages = FEW_RING / (FEW_W_BYTES + p.nr * FK * 2);
     p.stages = stages > FEW_MAX_STAGES ? FEW_MAX_STAGES : stages;
+    // With so few K blocks per CTA that the slab has room behind their stages, the CTAs of a cluster need not wait for one another's
+    // last MMAs before they send (48 rows through three layers of 512 / 1280 values 86.7 us, now 84.8).
+    const int kbs = (nk + p.splits - 1) / p.splits, used = (kbs < p.stages ? kbs : p.stages) * (FEW_W_BYTES + p.nr * FK * 2);
+    p.slab = p.nr <= FEW_QUAD_ROWS && p.splits > 1 && used + p.splits * p.quads * FW * 16 <= FEW_RING ? used : 0;
     return p;
 }
 
@@ -138,6 +143,7 @@ gemm_few_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem_base = bars->tmem_base;
+    if (QUADS && p.slab) cluster_arrive();               // (waited for before the hand-over: every CTA of the cluster has started)
 
     if (warp == 0) {
         if (lane == 0) {
@@ -198,15 +204,21 @@ gemm_few_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
     }
     __syncwarp();
 
-    // Hand-over: the ring of every CTA of the cluster is idle now.  Slab of the owner: [K slice][row][128 features], or QUADS
-    // [K slice][four rows][128 features][row].
+    // Hand-over: the ring of every CTA of the cluster is idle now (or the slab lies behind it).  Slab of the owner:
+    // [K slice][row][128 features], or QUADS [K slice][four rows][128 features][row].
     const int per_owner = p.nr / p.splits;               // rows of A that a CTA finishes (nr is a multiple of 16)
-    if (p.splits > 1) cluster_sync_all();
-    else __syncthreads();
+    if (QUADS && p.splits > 1) {
+        if (!p.slab) cluster_arrive();
+        cluster_wait();
+    } else if (p.splits > 1) {
+        cluster_sync_all();
+    } else {
+        __syncthreads();
+    }
     if (QUADS && warp >= 2) {
         const int f = (warp & 3) * 32 + lane;            // W row of the tile = TMEM lane
         const uint32_t taddr = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16);
-        const uint32_t slab = smem_u32(tiles) + (static_cast<uint32_t>(split) * p.quads * FW + f) * 16;
+        const uint32_t slab = smem_u32(tiles) + p.slab + (static_cast<uint32_t>(split) * p.quads * FW + f) * 16;
         int owner = 0, q = 0;
         uint32_t addr = p.splits > 1 ? cluster_map_shared(slab, 0u) : slab;
         for (int c0 = 0; c0 < g.M; c0 += 16) {           // (columns from M on are padding rows: stored, not read)
@@ -267,7 +279,7 @@ gemm_few_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
     // the last part is for all warps (the first two have not waited for the predecessor with all their lanes yet)
     if (warp < 2) pdl_wait();
     if (QUADS && !*abort_flag) {
-        const float4* slab = reinterpret_cast<const float4*>(tiles);
+        const float4* slab = reinterpret_cast<const float4*>(tiles + p.slab);
         // features f and f + 1 of the four rows of group q, the K slices added in order
         const auto sum = [&](int q, int f, float (&s)[2][4]) {
 #pragma unroll

@@ -128,9 +128,11 @@ __device__ __forceinline__ uint32_t cluster_cta_rank() {
 }
 // Barrier over every thread of every CTA of the cluster (release / acquire: shared-memory writes made before
 // the arrive, also those into a peer's shared memory, are visible after the wait).  All threads must call it.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync_all() {
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    cluster_arrive();
+    cluster_wait();
 }
 // Address of this CTA's shared-memory location `smem_addr` in CTA `rank` of the cluster (shared::cluster window).
 __device__ __forceinline__ uint32_t cluster_map_shared(uint32_t smem_addr, uint32_t rank) {
