@@ -13,7 +13,7 @@
 //     of the library writes), so the stream does not stop between kernels;
 //   * the CTAs of a tile's K slices form a cluster; each sends the accumulator columns (rows of A) it does not own to their
 //     owner through distributed shared memory, the owners add the slices in order and apply the epilogue: a thread holds 8
-//     consecutive features of one row (up to FEW_QUAD_ROWS rows: two features of four rows, so that four rows go in one remote
+//     consecutive features of one row (several slices of up to FEW_QUAD_ROWS rows: two features of four rows, so that four rows go in one remote
 //     store), which is what SwiGLU (a tile: 64 gate and the matching 64 up rows), RoPE (a tile holds whole heads; channel c
 //     and its partner c + d/2 are in the same slab) and coalesced stores want.
 //   warp 0 TMA producer, warp 1 MMA issuer, warps 2..5 epilogue (TMEM lane = W row).
@@ -48,13 +48,14 @@ struct FewPlan {
     int stages;
     int tiles;
     int slab;        // QUADS: where the slices are added: its offset in the ring, behind the stages in use (0: over them)
-    int quads;       // QUADS: groups of four rows of A that a CTA of a cluster finishes (the last ones may have none)
+    int quads;       // QUADS: groups of four rows of A that a CTA of a cluster finishes, the last CTAs maybe none (0: not QUADS)
 };
 // Up to this many rows the slices are handed over four rows at a time (QUADS): value by value the stores to the other CTAs were
 // 1.25 of the 3.8 us that a small projection of 48 rows takes behind its wait.  A stack of 3 layers of 512 / 1280 values, us, value by
 // value / four rows: 16 rows 78.8 / 78.1, 48 rows 88.9 / 85.5, 64 rows 97.2 / 94.0; 64 rows of 2 layers of 256 62.6 / 60.4, 32 rows of 2
 // LLaDA-shaped layers 205.0 / 203.9.  More rows are cut into fewer slices, and a CTA's last part is then the longer one, where
-// 16 bytes per load and store count: 72 rows 99.0 / 107.7, 128 rows 136 / 155.
+// 16 bytes per load and store count: 72 rows 99.0 / 107.7, 128 rows 136 / 155.  So it is with a single slice, which sends nothing
+// (48 rows of 4 LLaDA-shaped layers 421.6 with it, 419.3 without).
 constexpr int FEW_QUAD_ROWS = 64;
 
 FewPlan few_plan(int epi, int M, int N, int K, int sm_count) {
@@ -68,13 +69,13 @@ FewPlan few_plan(int epi, int M, int N, int K, int sm_count) {
     // exchange takes longer (128 rows, K = 1024, N = 4096: eight slices 13.0 us, two 9.6; K = 512, N = 1280: 6.7 either way)
     const int least = p.nr > 64 ? p.nr / 16 : 2;
     while (p.splits < 8 && 2LL * p.splits * p.tiles <= 2LL * sm_count && nk >= 2 * least * p.splits) p.splits *= 2;
-    p.quads = (p.nr / 4 + p.splits - 1) / p.splits;
+    p.quads = p.splits > 1 && p.nr <= FEW_QUAD_ROWS ? (p.nr / 4 + p.splits - 1) / p.splits : 0;
     const int stages = FEW_RING / (FEW_W_BYTES + p.nr * FK * 2);
     p.stages = stages > FEW_MAX_STAGES ? FEW_MAX_STAGES : stages;
     // With so few K blocks per CTA that the slab has room behind their stages, the CTAs of a cluster need not wait for one another's
     // last MMAs before they send (48 rows through three layers of 512 / 1280 values 86.7 us, now 84.8).
     const int kbs = (nk + p.splits - 1) / p.splits, used = (kbs < p.stages ? kbs : p.stages) * (FEW_W_BYTES + p.nr * FK * 2);
-    p.slab = p.nr <= FEW_QUAD_ROWS && p.splits > 1 && used + p.splits * p.quads * FW * 16 <= FEW_RING ? used : 0;
+    p.slab = p.quads > 0 && used + p.splits * p.quads * FW * 16 <= FEW_RING ? used : 0;
     return p;
 }
 
@@ -99,10 +100,6 @@ __device__ __forceinline__ void st_shared_f32(uint32_t addr, uint32_t v) {
 }
 __device__ __forceinline__ void st_shared_cluster_f32(uint32_t addr, uint32_t v) {
     asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
-}
-
-__device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
 
 template <int EPI, bool QUADS>
@@ -207,7 +204,7 @@ gemm_few_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
     // Hand-over: the ring of every CTA of the cluster is idle now (or the slab lies behind it).  Slab of the owner:
     // [K slice][row][128 features], or QUADS [K slice][four rows][128 features][row].
     const int per_owner = p.nr / p.splits;               // rows of A that a CTA finishes (nr is a multiple of 16)
-    if (QUADS && p.splits > 1) {
+    if (QUADS) {
         if (!p.slab) cluster_arrive();
         cluster_wait();
     } else if (p.splits > 1) {
@@ -220,17 +217,14 @@ gemm_few_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
         const uint32_t taddr = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16);
         const uint32_t slab = smem_u32(tiles) + p.slab + (static_cast<uint32_t>(split) * p.quads * FW + f) * 16;
         int owner = 0, q = 0;
-        uint32_t addr = p.splits > 1 ? cluster_map_shared(slab, 0u) : slab;
+        uint32_t addr = cluster_map_shared(slab, 0u);
         for (int c0 = 0; c0 < g.M; c0 += 16) {           // (columns from M on are padding rows: stored, not read)
             uint32_t v[16];
             tmem_ld_16cols(taddr + c0, v);
             tmem_ld_wait();
 #pragma unroll
             for (int c = 0; c < 16; c += 4) {
-                if (c0 + c < g.M) {
-                    if (p.splits > 1) st_shared_cluster_v4(addr, v[c], v[c + 1], v[c + 2], v[c + 3]);
-                    else st_shared_v4(addr, v[c], v[c + 1], v[c + 2], v[c + 3]);
-                }
+                if (c0 + c < g.M) st_shared_cluster_v4(addr, v[c], v[c + 1], v[c + 2], v[c + 3]);
                 addr += FW * 16;
                 if (++q == p.quads) {
                     q = 0;
@@ -469,7 +463,7 @@ gemm_few_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constan
 template <int EPI>
 int launch_few(const CUtensorMap& tw, const CUtensorMap& tw2, const CUtensorMap& ta, const FewArgs& g, cudaStream_t stream) {
     static std::atomic<uint64_t> smem_set[2] = {};
-    const bool quad = g.p.nr <= FEW_QUAD_ROWS;
+    const bool quad = g.p.quads > 0;
     const auto kernel = quad ? gemm_few_kernel<EPI, true> : gemm_few_kernel<EPI, false>;
     if (ensure_dynamic_smem(smem_set[quad], kernel, FEW_SMEM) != DARE_OK) return DARE_ERR_CUDA;
     const long long ctas = static_cast<long long>(g.p.tiles) * g.p.splits;
