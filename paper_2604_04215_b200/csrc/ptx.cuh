@@ -82,7 +82,8 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 // triggers behind its wait (that one included: behind a merge, its head; behind a step, its head, merge, selection and
 // attention), and may touch only what no kernel of the library writes: launch parameters, the rotary table, weights the caller
 // declares constant (w_static); the step's attention also its inputs, which the head, the merge and the selection do not
-// write.  A kernel that takes tensor memory calls pdl_trigger behind the allocation: a successor that takes tensor memory
+// write; lmhead_merge_select_kernel also the tokens, the row list and the row count, which the head found complete behind its own
+// wait and does not write.  A kernel that takes tensor memory calls pdl_trigger behind the allocation: a successor that takes tensor memory
 // on the same SM can then only wait for a CTA that has its share and will give it back.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
