@@ -93,6 +93,7 @@ __device__ __forceinline__ int32_t row_token(const int32_t* row_tokens, int tok_
 // front of it with 3 to 5 us.  What is left of it: the GEMM does nothing if no row is masked, and the merge kernels answer
 // committed rows.
 constexpr int LM_DIRECT_ROWS = 128;
+constexpr int LM_EARLY_SAMPLED_ROWS = 32;      // sampled: up to this many by the kernel that sets itself up in front of its wait
 // Token of row m = tokens[(m / L) * stride + m % L]; tokens == NULL: no direct launch
 struct LmTokens { const int32_t* tokens; int L; int64_t stride; int32_t mask_id; };
 
@@ -1179,7 +1180,7 @@ lmhead_head_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
         }
     }
     pdl_wait();
-    if (DIRECT && !any_masked(direct, M, threadIdx.x & 31)) return;      // (every warp of every CTA alike)
+    if (direct.tokens && !any_masked(direct, M, threadIdx.x & 31)) return;      // (every warp of every CTA alike)
     const int Mc = live_rows ? *live_rows : M;          // rows that need logits (uniform over the grid)
     if constexpr (MODE == LM_GREEDY && !DIRECT) {
         if (lm_joint(Mc, n_tiles, gridDim.x >> 1, D >= SW_DEEP, false)) {
@@ -1559,7 +1560,9 @@ static int launch_head(const dare_ctx* ctx, int grid, bool pairs, const void* x_
         constexpr int SMEM = SW_SMEM_BYTES;
         static_assert(SMEM >= LM_PAIR_SMEM_BYTES && SMEM >= LM_SMEM_BYTES, "shared memory");
         static std::atomic<uint64_t> smem_set[2] = {};
-        const bool in_place = direct.tokens != nullptr;
+        // (more sampled rows pay for their epilogue's code there: 64 rows 168.3 / 169.3 us, 96 183.0 / 187.7, 128 195.0 / 199.3; 32 rows
+        // 161.5 / 159.6)
+        const bool in_place = direct.tokens != nullptr && (!SAMPLE || M <= LM_EARLY_SAMPLED_ROWS);
         const auto kernel = in_place ? lmhead_head_kernel<MODE, true> : lmhead_head_kernel<MODE, false>;
         if (ensure_dynamic_smem(smem_set[in_place], kernel, SMEM) != DARE_OK) return DARE_ERR_CUDA;
         rc = launch_kernel(kernel, dim3(static_cast<unsigned>(grid_gemm)), LM_THREADS, SMEM, stream, 2, tmap_w, xm, M, live_rows, D, V,
