@@ -848,6 +848,22 @@ attn_block_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                 t1 = max3(__float_as_uint(t1), s1[30], s1[31]);
                 t0 = fmaxf(t0, t2);
                 t1 = fmaxf(t1, t3);
+                if (t == 0 && w.n_tiles > 1) {
+                    // The first reference is the largest score of 128 keys (the second tile's are on their way already): the oftener a
+                    // row's largest weight is 1, the less its rounding to bf16 costs (sharp rows are 3 % further off otherwise).
+                    const int valid1 = tile_info<TC_KT>(1, n_pre, n_blk, w.len_pre, w.len_blk, w.len_suf, 0, 0, 0).valid;
+                    if (!mbar_wait(&bars->s_full[j][buf ^ 1], ((n + 1) >> 1) & 1, abort_flag)) { ok = false; break; }
+                    tc_fence_after_sync();
+#pragma unroll 1
+                    for (int c = 0; c < TC_KT; c += 16) {
+                        uint32_t v[16];
+                        tmem_ld_16cols(tmem_base + S::s_col(j, buf ^ 1) + lane_off + c, v);
+                        tmem_ld_wait();
+#pragma unroll
+                        for (int k = 0; k < 16; ++k)
+                            if (c + k < valid1) t0 = fmaxf(t0, __uint_as_float(v[k]));
+                    }
+                }
                 const float tmax = fmaxf(t0, t1) * c2;     // log2 domain (the scale is > 0); finite: every tile has a key
                 // move the reference only when the true max has run away from it (decided per warp, so that the
                 // TMEM loads and stores below are executed by whole warps)
