@@ -77,6 +77,35 @@ def test_block_units(ctx, B, L, Hq, Hkv, d, plens, slens, inplace):
     check_attn(out, res[0] if isinstance(res, tuple) else res)
 
 
+
+# Behind a sequence's or a rollout's last query a tile holds the next one's queries.  With scores this sharp the references of most
+# rows lag behind their maxima, so a reference that moves shows in the bits of a row's result.
+@pytest.mark.parametrize("n,Hq,Hkv,d", [(300, 2, 2, 128), (129, 4, 2, 64), (37, 7, 1, 128), (250, 1, 1, 64)])
+@pytest.mark.parametrize("packed", [True, False])
+def test_neighbour_does_not_matter(ctx, n, Hq, Hkv, d, packed):
+    P = 200                                                     # block form: cached keys in front of the block
+    keys = n if packed else P + n
+    q = I.normal_bf16(n, I.TID_Q, (2, n, Hq, d), 5.0)
+    k, v = I.normal_bf16(n, I.TID_KPRE, (2, Hkv, keys, d)).cuda(), I.normal_bf16(n, I.TID_VPRE, (2, Hkv, keys, d)).cuda()
+    got = []
+    for scale in (1.0, 40.0):
+        qs = torch.stack((q[0], q[1] * scale)).cuda()
+        if packed:
+            flat = lambda t: t.transpose(1, 2).reshape(2 * n, Hkv, d).contiguous()  # noqa: E731
+            lse = torch.empty(Hq, 2 * n, device="cuda")
+            out = dare.dare_attn_varlen(ctx, qs.view(2 * n, Hq, d), flat(k), flat(v),
+                                        torch.tensor([0, n, 2 * n], dtype=torch.int32, device="cuda"), n, None, lse)
+            got.append((out[:n].clone(), lse[:, :n].clone()))
+        else:
+            out, lse = torch.empty_like(qs), torch.empty(2, Hq, n, device="cuda")
+            dare.dare_attn_block(ctx, qs, k, v, torch.tensor([P, P], dtype=torch.int32, device="cuda"), None, None, None, None, None,
+                                 out, lse)
+            got.append((out[0].clone(), lse[0].clone()))
+    torch.cuda.synchronize()
+    assert ctx.device_status() == 0
+    assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
+
+
 # The warp-level kernel: rows that share a KV head at the ends of its variants (four, two and one key slices a tile; each slice
 # finishes its share of the columns), without and with K/V splits, keys that end inside a slice.
 @pytest.mark.parametrize("L,g", [(1, 1), (4, 4), (17, 1), (32, 1), (33, 1), (8, 9), (90, 1)])
