@@ -872,7 +872,8 @@ attn_block_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                 // depends on what lies behind the rollout or the sequence)
                 if (__any_sync(0xffffffffu, live && tmax > m_ref + TC_RESCALE_GAP)) {
                     const float m_new = fmaxf(m_ref, tmax);
-                    const float factor = fast_exp2(m_ref - m_new);   // exp2(-inf) = 0 on the first tile
+                    // (0 with a row's first finite score; a row that has seen only -inf stays as it is)
+                    const float factor = m_new == -INFINITY ? 1.f : fast_exp2(m_ref - m_new);
                     m_ref = m_new;
                     l *= factor;
                     if (t >= 1) {

@@ -106,6 +106,28 @@ def test_neighbour_does_not_matter(ctx, n, Hq, Hkv, d, packed):
     assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
 
 
+
+# Rows whose first `blind` scores are -inf (the products overflow fp32), in warps whose other rows have finite scores and move
+# their references in the first and in later tiles.
+@pytest.mark.parametrize("blind", [64, 128, 192])
+@pytest.mark.parametrize("d", [64, 128])
+def test_rows_that_see_nothing_at_first(ctx, blind, d):
+    n, H = 400, 2
+    q, k, v = (I.normal_bf16(blind + d, t, (n, H, d), s) for t, s in ((I.TID_Q, 4.0), (I.TID_KPRE, 1.0), (I.TID_VPRE, 1.0)))
+    for t in (q, k):
+        t[:, :, 0] = 0
+    q[::3, :, 0] = 1e30
+    k[:blind, :, 0] = -1e30
+    k[300:, :, 1:] *= 4                                       # larger scores later on: references move
+    ref, lse_ref = O.attn_varlen(f64(q), f64(k), f64(v), np.array([0, n]))
+    lse = torch.empty(H, n, device="cuda")
+    out = dare.dare_attn_varlen(ctx, q.cuda(), k.cuda(), v.cuda(), torch.tensor([0, n], dtype=torch.int32, device="cuda"), n, None, lse)
+    torch.cuda.synchronize()
+    assert ctx.device_status() == 0
+    check_attn(out, ref)
+    assert np.abs(lse.cpu().double().numpy() - lse_ref).max() < 2e-2
+
+
 # The warp-level kernel: rows that share a KV head at the ends of its variants (four, two and one key slices a tile; each slice
 # finishes its share of the columns), without and with K/V splits, keys that end inside a slice.
 @pytest.mark.parametrize("L,g", [(1, 1), (4, 4), (17, 1), (32, 1), (33, 1), (8, 9), (90, 1)])
