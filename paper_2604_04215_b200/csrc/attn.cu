@@ -483,12 +483,16 @@ attn_block_kernel(const __grid_constant__ CUtensorMap tm_kpre, const __grid_cons
 // 128-key tiles with one S / P buffer, P handed over in halves: 16 x 2048 904 and 16 x 512 77, but 282 on the packed batch
 // (its ragged ends) and 30.8 on the step.
 // O stays in TMEM, so it cannot be rescaled for free when a row's max grows.  The exponentials are therefore
-// taken relative to a reference max that is only moved when the true max has run more than 2^8 ahead of it;
+// taken relative to a reference max that is only moved when the true max has run more than 2^4 ahead of it;
 // then (rarely, mostly in the first tiles) the warp waits for the MMAs in flight, multiplies its rows of O by
 // the correction factor in place and moves the reference.  The sum uses the same reference, so O / l is exact.
 // A tile holds floor(128 / g) block positions x g heads so that a position's heads never straddle two tiles.
 constexpr int TC_KT = 64;                 // keys per tile
-constexpr float TC_RESCALE_GAP = 8.0f;    // log2 units the true max may run ahead of the reference
+// log2 units the true max may run ahead of the reference.  The fewer, the oftener a row's largest weight is exactly 1 in bf16.  Distance
+// from 64 bits (rel-L2, x 1e-3; 1.5 of it the result's own rounding) for q of standard deviation 1, 2, 4, 8, 16 on 28 + 4 heads of 128:
+// 8 units 2.301, 2.223, 2.110, 1.851, 1.525; 4 units 2.300, 2.102, 1.865, 1.707, 1.469; 2 units 2.274, 1.944, 1.761, 1.669, 1.457, but the
+// ordinary scores of deviation 1 then move too (32 sequences of 256 to 1024 tokens 264 -> 283 us; 8 to 4 units: no difference).
+constexpr float TC_RESCALE_GAP = 4.0f;
 
 template <int D, int QT>
 struct TcShape {

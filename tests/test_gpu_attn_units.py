@@ -128,6 +128,21 @@ def test_rows_that_see_nothing_at_first(ctx, blind, d):
     assert np.abs(lse.cpu().double().numpy() - lse_ref).max() < 2e-2
 
 
+
+# Sharp rows: a few weights make up the result, and what rounding them to bf16 costs depends on how far a row's reference lags
+# behind its maximum.  The result's own rounding is 1.5e-3 of its norm (2^-7 / sqrt(12) of the binade, log-uniform mantissas); a single weight
+# rounded like that would double the variance (2.15e-3), one that is exact adds nothing.  The bounds allow the weights half and a third of it.
+@pytest.mark.parametrize("sharp,bar", [(4.0, 1.95e-3), (8.0, 1.77e-3)])
+@pytest.mark.parametrize("d", [64, 128])
+def test_sharp_rows(ctx, sharp, bar, d):
+    n, H = 1000, 8
+    q, k, v = (I.normal_bf16(d, t, (n, H, d), s).cuda() for t, s in ((I.TID_Q, sharp), (I.TID_KPRE, 1.0), (I.TID_VPRE, 1.0)))
+    out = dare.dare_attn_varlen(ctx, q, k, v, torch.tensor([0, n], dtype=torch.int32, device="cuda"), n).double()
+    p = torch.softmax(torch.einsum("ihd,jhd->hij", q.double(), k.double()) / d ** 0.5, -1)
+    ref = torch.einsum("hij,jhd->ihd", p, v.double())
+    assert ((out - ref).norm() / ref.norm()).item() < bar
+
+
 # The warp-level kernel: rows that share a KV head at the ends of its variants (four, two and one key slices a tile; each slice
 # finishes its share of the columns), without and with K/V splits, keys that end inside a slice.
 @pytest.mark.parametrize("L,g", [(1, 1), (4, 4), (17, 1), (32, 1), (33, 1), (8, 9), (90, 1)])
