@@ -818,10 +818,11 @@ attn_block_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             if (lane == 0) mbar_arrive(&bars->unit_empty[slot]);
             if (w.n_tiles == 0) break;
             if (j >= w.n_q) { n_kv += w.n_tiles; continue; }
-            // (the rows behind a rollout's or a sequence's last position are the next one's queries, see the producer)
-            const bool live = r < rows_in_tile && w.pos0 + j * pos_per_tile + ri < w.L_eff;
             const int n_pre = (w.len_pre + TC_KT - 1) / TC_KT, n_blk = (w.len_blk + TC_KT - 1) / TC_KT;
-            float m_ref = -INFINITY, l = 0.f;              // reference max (log2 domain) and sum of exp2(s - m_ref)
+            // Reference max (log2 domain) and sum of exp2(s - m_ref).  The rows behind a rollout's or a sequence's last position are the
+            // next one's queries (see the producer): an infinite reference, all weights 0.  (A flag of their own, alive through
+            // the loop, spilled: 243 -> 256 us on 32 sequences of 256 to 1024 tokens.)
+            float m_ref = r < rows_in_tile && w.pos0 + j * pos_per_tile + ri < w.L_eff ? -INFINITY : INFINITY, l = 0.f;
             bool ok = true;
             for (int t = 0; t < w.n_tiles; ++t) {
                 const int valid = tile_info<TC_KT>(t, n_pre, n_blk, w.len_pre, w.len_blk, w.len_suf, 0, 0, 0).valid;
@@ -872,9 +873,9 @@ attn_block_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                 }
                 const float tmax = fmaxf(t0, t1) * c2;     // log2 domain (the scale is > 0); finite: every tile has a key
                 // move the reference only when the true max has run away from it (decided per warp, so that the
-                // TMEM loads and stores below are executed by whole warps; by its live rows, so that nobody's rounding
-                // depends on what lies behind the rollout or the sequence)
-                if (__any_sync(0xffffffffu, live && tmax > m_ref + TC_RESCALE_GAP)) {
+                // TMEM loads and stores below are executed by whole warps; rows that are not live never ask for it, so that
+                // nobody's rounding depends on what lies behind the rollout or the sequence)
+                if (__any_sync(0xffffffffu, tmax > m_ref + TC_RESCALE_GAP)) {
                     const float m_new = fmaxf(m_ref, tmax);
                     // (0 with a row's first finite score; a row that has seen only -inf stays as it is)
                     const float factor = m_new == -INFINITY ? 1.f : fast_exp2(m_ref - m_new);
@@ -991,7 +992,7 @@ attn_block_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             }
             __syncwarp();
             tc_fence_before_sync();                          // (O has been read: the next unit's first P V may overwrite it)
-            if (p.lse != nullptr && live) {
+            if (p.lse != nullptr && r < rows_in_tile && pos0 + ri < w.L_eff) {
                 const int i = pos0 + ri, h = w.kvh * p.g + rh;
                 p.lse[packed ? static_cast<size_t>(h) * p.total_tokens + w.token0 + i
                              : (static_cast<size_t>(w.b) * p.Hq + h) * p.L + i] = l > 0.f ? (m_ref + log2f(l)) * LN2_F : -INFINITY;
