@@ -97,14 +97,12 @@ constexpr int LM_EARLY_SAMPLED_ROWS = 32;      // sampled: up to this many by th
 // Token of row m = tokens[(m / L) * stride + m % L]; tokens == NULL: no direct launch
 struct LmTokens { const int32_t* tokens; int L; int64_t stride; int32_t mask_id; };
 
-// Whether any of the rows is masked (a warp; all lanes get the answer).
+// Whether any of the rows is masked (a warp; all lanes get the answer).  The loads do not hang on one another's rows: behind a
+// test of each row they went one after the other, 0.15 us apiece (the sampled head of 128 rows x 256 x 1000 17.9 us, 17.0 now).
 __device__ __forceinline__ bool any_masked(const LmTokens& t, int M, int lane) {
     bool any = false;
 #pragma unroll
-    for (int u = 0; u < LM_DIRECT_ROWS / 32; ++u) {
-        const int m = lane + u * 32;
-        any |= m < M && row_token(t.tokens, t.L, t.stride, m) == t.mask_id;
-    }
+    for (int u = 0; u < LM_DIRECT_ROWS / 32; ++u) any |= row_token(t.tokens, t.L, t.stride, min(lane + u * 32, M - 1)) == t.mask_id;
     return __any_sync(0xffffffffu, any);
 }
 
