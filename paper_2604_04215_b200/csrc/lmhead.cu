@@ -719,11 +719,14 @@ __host__ __device__ constexpr int sw_smem_bytes(int mode, bool joint) {
 static_assert(sw_smem_bytes(LM_SAMPLE, false) <= SW_SMEM_BYTES && sw_smem_bytes(LM_GREEDY, false) <= SW_SMEM_BYTES &&
               sw_smem_bytes(LM_GREEDY, true) <= SW_SMEM_BYTES, "shared memory");
 static_assert(SW_SMEM_BYTES + 1024 + 3 * (1024 + 512) <= 228 * 1024, "room for three CTAs of a merge kernel beside the head's");
+// LATE: stages requested before it is known that a row is masked (their slots are not waited for)
+constexpr int SW_UNSEEN = 4;
+static_assert(SW_UNSEEN <= SW_MAX_STAGES && SW_UNSEEN * (SW_W_BYTES + LM_DIRECT_ROWS / 2 * 128) <= sw_ring_bytes(LM_GREEDY, false) &&
+              SW_UNSEEN * (SW_W_BYTES + LM_DIRECT_ROWS / 2 * 128) <= sw_ring_bytes(LM_SAMPLE, false), "slots for them at LM_DIRECT_ROWS rows");
 // X tiles of 128, 64, 32, 16 and 8 rows: a CTA's share of a chunk (a multiple of 8 rows) is covered by one or two
 // of them, stacked in shared memory (each a whole number of 1 KB swizzle atoms); a few rows too many may be loaded,
 // the MMA reads only its own.  (Exact covers of up to four boxes were measured slower: 432 us for 480 rows, where
 // each CTA loaded 64 + 32 + 16 + 8 rows per stage, against 350 us for 512 rows with one box.)
-constexpr int SW_UNSEEN = 4;                             // stages requested before it is known that a row is masked
 struct SwXMaps { CUtensorMap m[5]; };
 struct SwBoxes { int i1, i2, rows; };      // indices into SwXMaps::m (i2 < 0: one box), rows loaded in all
 __device__ __forceinline__ SwBoxes sw_boxes(int rows_half) {
@@ -837,8 +840,7 @@ lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, 
     const uint32_t tmem_base = bars->tmem_base;
     const int num_k = (D + BK - 1) / BK;
     bool any = true;                                     // is any row masked?
-    const bool late = LATE && tokens.tokens != nullptr;      // (a run-time value: as a constant W came 1 % slower, 168.9 / 167.1 us)
-    if (late) {
+    if (LATE) {
         pdl_wait();
         pdl_trigger();
         if (warp != 0) any = any_masked(tokens, Mc, lane);
@@ -867,8 +869,8 @@ lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, 
             for (int i = 0; i < 5; ++i) prefetch_tensormap(&xmaps.m[i]);
         }
         // LATE: the first stages are on their way while the tokens are looked at; if no row is masked after all, they are waited for.
-        int ahead = late ? min(SW_UNSEEN, num_k) : 0;
-        if (late) {
+        int ahead = LATE ? min(SW_UNSEEN, num_k) : 0;
+        if (LATE) {
             if (lane == 0)
                 for (int kb = 0; kb < ahead; ++kb) load(unit, unit / item_chunks, kb, kb);
             __syncwarp();
@@ -1153,45 +1155,25 @@ lm_joint_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, in
                                             parts_stride, smp, LmTokens{});
 }
 
-// The greedy (or sampled) head, one launch on CTA pairs whatever the number of live rows (known only on the device when rows are
-// skipped): the swapped-operand path for the counts lm_swapped names (up to SW_NMAX rows, and counts that
-// cut into long chunks); otherwise row-major tiles of 128 rows, on CTA pairs when the tiles come in twos, and for
-// an odd count on pairs plus single CTAs for the last tile (see above).  The W
-// tile box is 128 rows for all of them.  A row's partials start at row * parts_stride; how many there are follows
-// from the same rules in lm_row_partials.
-template <int MODE, bool DIRECT>
-__global__ void __launch_bounds__(LM_THREADS, 1)
-lmhead_head_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ SwXMaps xmaps, int M,
-                     const int32_t* __restrict__ live_rows, int D, int V, int mask_col, int n_tiles,
-                     float* __restrict__ part_max, float* __restrict__ part_sum, int32_t* __restrict__ part_arg,
-                     uint32_t* __restrict__ dev_status, int parts_stride, const LmSampling smp, const LmTokens direct) {
-    // DIRECT: rows evaluated where they lie.  How many is known before the predecessor is done, so the swapped path sets itself
-    // up beside it and waits in its place.  With what lmhead_merge_select_kernel does in front of its wait, a replayed step of 32
-    // rows x 512 x 4096 takes 12.0 us for 14.0, 128 rows x 256 x 1000 14.9 for 16.6, 32 rows x 4096 x 126464 165.6 for 167.5; one
-    // that finds no masked row 1 us more (its SW_UNSEEN stages).  (In one kernel with the other launches it slowed the sampled
-    // head of 416 rows by 1.4 %.)
-    if constexpr (DIRECT) {
-        if (lm_swapped(M, n_tiles, gridDim.x >> 1, D >= SW_DEEP, MODE == LM_SAMPLE)) {
-            lm_swapped_body<MODE, false, true>(tmap_w, xmaps, M, D, V, mask_col, n_tiles, part_max, part_sum, part_arg, dev_status,
-                                               parts_stride, smp, direct);
-            return;
-        }
-    }
+// lmhead_head_kernel behind its wait, on the path that the number of live rows asks for.
+template <int MODE>
+__device__ __forceinline__ void
+lm_head_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int M, const int32_t* __restrict__ live_rows, int D, int V, int mask_col,
+             int n_tiles, float* __restrict__ part_max, float* __restrict__ part_sum, int32_t* __restrict__ part_arg,
+             uint32_t* __restrict__ dev_status, int parts_stride, const LmSampling& smp, const LmTokens& direct) {
     pdl_wait();
     if (direct.tokens && !any_masked(direct, M, threadIdx.x & 31)) return;      // (every warp of every CTA alike)
     const int Mc = live_rows ? *live_rows : M;          // rows that need logits (uniform over the grid)
-    if constexpr (MODE == LM_GREEDY && !DIRECT) {
+    if constexpr (MODE == LM_GREEDY) {
         if (lm_joint(Mc, n_tiles, gridDim.x >> 1, D >= SW_DEEP, false)) {
             lm_joint_body(tmap_w, xmaps, Mc, D, V, mask_col, n_tiles, part_max, part_sum, part_arg, dev_status, parts_stride, smp);
             return;
         }
     }
-    if constexpr (!DIRECT) {
-        if (lm_swapped(Mc, n_tiles, gridDim.x >> 1, D >= SW_DEEP, MODE == LM_SAMPLE)) {
-            lm_swapped_body<MODE, false, false>(tmap_w, xmaps, Mc, D, V, mask_col, n_tiles, part_max, part_sum, part_arg, dev_status,
-                                                parts_stride, smp, direct);
-            return;
-        }
+    if (lm_swapped(Mc, n_tiles, gridDim.x >> 1, D >= SW_DEEP, MODE == LM_SAMPLE)) {
+        lm_swapped_body<MODE, false, false>(tmap_w, xmaps, Mc, D, V, mask_col, n_tiles, part_max, part_sum, part_arg, dev_status,
+                                            parts_stride, smp, direct);
+        return;
     }
     const int m_tiles = (Mc + BM - 1) / BM;
     const int cluster = blockIdx.x >> 1, n_clusters = gridDim.x >> 1;
@@ -1216,6 +1198,32 @@ lmhead_head_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
             lm_rowmajor_body<MODE, false, true>(xmaps.m[0], tmap_w, Mc, D, V, mask_col, n_tiles, part_max, part_sum,
                                                      part_arg, dev_status, smp, u);
         }
+    }
+}
+
+// The greedy (or sampled) head, one launch on CTA pairs whatever the number of live rows (known only on the device when rows are
+// skipped): the swapped-operand path for the counts lm_swapped names (up to SW_NMAX rows, and counts that
+// cut into long chunks); otherwise row-major tiles of 128 rows, on CTA pairs when the tiles come in twos, and for
+// an odd count on pairs plus single CTAs for the last tile (see above).  The W
+// tile box is 128 rows for all of them.  A row's partials start at row * parts_stride; how many there are follows
+// from the same rules in lm_row_partials.
+template <int MODE, bool DIRECT>
+__global__ void __launch_bounds__(LM_THREADS, 1)
+lmhead_head_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ SwXMaps xmaps, int M,
+                     const int32_t* __restrict__ live_rows, int D, int V, int mask_col, int n_tiles,
+                     float* __restrict__ part_max, float* __restrict__ part_sum, int32_t* __restrict__ part_arg,
+                     uint32_t* __restrict__ dev_status, int parts_stride, const LmSampling smp, const LmTokens direct) {
+    // DIRECT: rows evaluated where they lie, and by the swapped path (the launcher sees to it).  How many is known before the predecessor
+    // is done, so it sets itself up beside it and waits in its place.  With what lmhead_merge_select_kernel does in front of its
+    // wait, a replayed step of 32 rows x 512 x 4096 takes 12.0 us for 14.0, 128 rows x 256 x 1000 14.9 for 16.6, 32 rows x 4096 x 126464
+    // 165.6 for 167.5; one that finds no masked row 0.5 to 2 us more (its SW_UNSEEN stages, and a kernel to take down).  (In one kernel
+    // with the other launches it slowed the sampled head of 416 rows by 1.4 %.)
+    if constexpr (DIRECT) {
+        lm_swapped_body<MODE, false, true>(tmap_w, xmaps, M, D, V, mask_col, n_tiles, part_max, part_sum, part_arg, dev_status,
+                                           parts_stride, smp, direct);
+    } else {
+        lm_head_body<MODE>(tmap_w, xmaps, M, live_rows, D, V, mask_col, n_tiles, part_max, part_sum, part_arg, dev_status, parts_stride, smp,
+                           direct);
     }
 }
 
@@ -1560,7 +1568,8 @@ static int launch_head(const dare_ctx* ctx, int grid, bool pairs, const void* x_
         static std::atomic<uint64_t> smem_set[2] = {};
         // (more sampled rows pay for their epilogue's code there: 64 rows 168.3 / 169.3 us, 96 183.0 / 187.7, 128 195.0 / 199.3; 32 rows
         // 161.5 / 159.6)
-        const bool in_place = direct.tokens != nullptr && (!SAMPLE || M <= LM_EARLY_SAMPLED_ROWS);
+        const bool in_place = direct.tokens != nullptr && (!SAMPLE || M <= LM_EARLY_SAMPLED_ROWS) &&
+                              lm_swapped(M, n_tiles, grid_gemm >> 1, D >= SW_DEEP, SAMPLE);
         const auto kernel = in_place ? lmhead_head_kernel<MODE, true> : lmhead_head_kernel<MODE, false>;
         if (ensure_dynamic_smem(smem_set[in_place], kernel, SMEM) != DARE_OK) return DARE_ERR_CUDA;
         rc = launch_kernel(kernel, dim3(static_cast<unsigned>(grid_gemm)), LM_THREADS, SMEM, stream, 2, tmap_w, xm, M, live_rows, D, V,
