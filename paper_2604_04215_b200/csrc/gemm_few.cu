@@ -69,7 +69,11 @@ FewPlan few_plan(int epi, int M, int N, int K, int sm_count) {
     // exchange takes longer (128 rows, K = 1024, N = 4096: eight slices 13.0 us, two 9.6; K = 512, N = 1280: 6.7 either way)
     const int least = p.nr > 64 ? p.nr / 16 : 2;
     while (p.splits < 8 && 2LL * p.splits * p.tiles <= 2LL * sm_count && nk >= 2 * least * p.splits) p.splits *= 2;
-    p.quads = p.splits > 1 && p.nr <= FEW_QUAD_ROWS ? (p.nr / 4 + p.splits - 1) / p.splits : 0;
+    // (up to four rows all go to one CTA of the cluster, and eight slices of padded groups then take longer to arrive and to add than single
+    // values, once the launch fills the SMs: 1 row x 2048 x 2048 4.0 / 4.4 us, x 1024 x 4096 4.7 / 5.0, x 4096 x 4096 6.6 / 6.8; on fewer CTAs
+    // 1 row x 1280 x 512 3.4 / 3.0; 8 rows x 2048 x 2048 with a residual 4.3 / 4.1)
+    const bool one_owner = M <= 4 && p.splits == 8 && 4LL * p.splits * p.tiles >= 3LL * sm_count;
+    p.quads = p.splits > 1 && p.nr <= FEW_QUAD_ROWS && !one_owner ? (p.nr / 4 + p.splits - 1) / p.splits : 0;
     const int stages = FEW_RING / (FEW_W_BYTES + p.nr * FK * 2);
     p.stages = stages > FEW_MAX_STAGES ? FEW_MAX_STAGES : stages;
     // With so few K blocks per CTA that the slab has room behind their stages, the CTAs of a cluster need not wait for one another's

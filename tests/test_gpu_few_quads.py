@@ -17,7 +17,8 @@ def ctx():
 
 
 @pytest.mark.parametrize("M", [1, 3, 4, 5, 16, 31, 33, 48, 63, 64, 65])
-@pytest.mark.parametrize("K,N,slices", [(64, 136, 1), (256, 264, 2), (520, 128, 4), (1280, 512, 8), (1288, 72, 8)])
+@pytest.mark.parametrize("K,N,slices", [(64, 136, 1), (256, 264, 2), (520, 128, 4), (1280, 512, 8), (1288, 72, 8),
+                                        (1024, 1792, 8)])     # up to 4 rows: value by value
 @pytest.mark.parametrize("epilogue", [dare.LINEAR_STORE, dare.LINEAR_RESIDUAL, dare.LINEAR_SWIGLU])
 def test_projection(ctx, M, K, N, slices, epilogue):
     a, w, w2 = I.normal_bf16(M, 1, (M, K)), I.normal_bf16(K, 2, (N, K), 0.05), I.normal_bf16(K, 3, (N, K), 0.05)
