@@ -409,27 +409,38 @@ attn_block_kernel(const __grid_constant__ CUtensorMap tm_kpre, const __grid_cons
         const size_t orow1 = (static_cast<size_t>(b) * p.L + i1) * p.Hq + h1;
         const size_t n_rows = static_cast<size_t>(p.B) * p.L * p.Hq;
         float* po = p.part_o + static_cast<size_t>(split) * n_rows * D;
+        const bool whole = p.splits == 1;
 #pragma unroll
         for (int o = 0; o < KS; ++o) {
             if (o != ks) continue;         // (a warp runs one of these, with its accumulators in registers)
 #pragma unroll
             for (int i = 0; i < NBK; ++i) {
-                const int n = o * NBK + i, col = n * 8 + tq * 2;
-                float v0 = oacc[n][0] * w0[o], v1 = oacc[n][1] * w0[o], v2 = oacc[n][2] * w1[o], v3 = oacc[n][3] * w1[o];
+                float (&v)[4] = oacc[o * NBK + i];
+                if (KS > 1) { v[0] *= w0[o]; v[1] *= w0[o]; v[2] *= w1[o]; v[3] *= w1[o]; }
 #pragma unroll
                 for (int q = 0; q < KS; ++q) {
                     if (q == o) continue;
                     const float4 x = xch[(((o * KS + q) * NW + rg) * NBK + i) * 32 + lane];
-                    v0 += x.x * w0[q]; v1 += x.y * w0[q];
-                    v2 += x.z * w1[q]; v3 += x.w * w1[q];
+                    v[0] += x.x * w0[q]; v[1] += x.y * w0[q];
+                    v[2] += x.z * w1[q]; v[3] += x.w * w1[q];
                 }
-                v0 *= inv0; v1 *= inv0; v2 *= inv1; v3 *= inv1;
-                if (p.splits == 1) {
-                    if (live0) *reinterpret_cast<uint32_t*>(p.out + orow0 * D + col) = pack_bf16(v0, v1);
-                    if (live1) *reinterpret_cast<uint32_t*>(p.out + orow1 * D + col) = pack_bf16(v2, v3);
-                } else {
-                    if (live0) *reinterpret_cast<float2*>(po + orow0 * D + col) = make_float2(v0, v1);
-                    if (live1) *reinterpret_cast<float2*>(po + orow1 * D + col) = make_float2(v2, v3);
+                v[0] *= inv0; v[1] *= inv0; v[2] *= inv1; v[3] *= inv1;
+            }
+            if (whole) {
+#pragma unroll
+                for (int i = 0; i < NBK; ++i) {
+                    const float (&v)[4] = oacc[o * NBK + i];
+                    const int col = (o * NBK + i) * 8 + tq * 2;
+                    if (live0) *reinterpret_cast<uint32_t*>(p.out + orow0 * D + col) = pack_bf16(v[0], v[1]);
+                    if (live1) *reinterpret_cast<uint32_t*>(p.out + orow1 * D + col) = pack_bf16(v[2], v[3]);
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < NBK; ++i) {
+                    const float (&v)[4] = oacc[o * NBK + i];
+                    const int col = (o * NBK + i) * 8 + tq * 2;
+                    if (live0) *reinterpret_cast<float2*>(po + orow0 * D + col) = make_float2(v[0], v[1]);
+                    if (live1) *reinterpret_cast<float2*>(po + orow1 * D + col) = make_float2(v[2], v[3]);
                 }
             }
         }
