@@ -1,10 +1,17 @@
 """The head of up to 128 rows requests its first stages before it has seen the tokens: steps with and without a masked row in
-turn, with fewer, as many and more K blocks than those stages, against the head and the selection by themselves."""
+turn, with fewer, as many and more K blocks than those stages, against the head and the selection by themselves; and the head by
+itself against the fp64 oracle, with a second vocabulary tile for some CTA pairs, whose stages follow those of the first."""
+import numpy as np
 import pytest
 import torch
 
+from oracle import dare_oracle as O
+from oracle import dare_sampling_oracle as SO
 from paper_2604_04215_b200 import binding as dare
 from paper_2604_04215_b200 import inputs as I
+
+from _util import check_lmhead, f64
+from test_gpu_sampling import _check as check_sampled
 
 pytestmark = pytest.mark.gpu
 
@@ -47,4 +54,22 @@ def test_steps_with_and_without_masked_rows(B, L, D, temperature):
         for a, b in ((after, tok), (pred, p2), (conf, c2), (nc, nc2), (nr, nr2)):
             assert torch.equal(a, b)
     assert ctx.device_status() == 0
+    ctx.close()
+
+
+@pytest.mark.parametrize("M,masked", [(1, 1), (32, 5), (32, 32), (128, 40)])
+@pytest.mark.parametrize("D", [200, 264, 1024])
+def test_head_in_place_against_the_oracle(M, masked, D):
+    ctx = dare.Context(0)
+    V, mask = 75 * 256 + 1, 1000
+    x, w = I.normal_bf16(D + M, I.TID_X, (M, D)), I.normal_bf16(D, I.TID_W, (V, D), 3.0 / D ** 0.5)
+    rows = torch.full((M,), 5, dtype=torch.int32)
+    rows[M - masked:] = mask
+    args = (x.cuda(), w.cuda(), rows.cuda(), mask, True)
+    greedy, sampled = dare.dare_lmhead_confidence(ctx, *args), dare.dare_lmhead_sample(ctx, *args, 0.8, 3, 7)
+    torch.cuda.synchronize()
+    assert ctx.device_status() == 0
+    check_lmhead(*greedy, O.lmhead_confidence(f64(x), f64(w), rows.numpy(), mask, True), f64(x), f64(w), mask, True, O)
+    ref = SO.lmhead_sample(f64(x), f64(w), rows.numpy(), mask, True, 0.8, 3, 7)
+    check_sampled(*sampled, ref, f64(x), f64(w), np.arange(M), mask, True, 0.8, 3, 7)
     ctx.close()
