@@ -487,8 +487,8 @@ attn_block_kernel(const __grid_constant__ CUtensorMap tm_kpre, const __grid_cons
 // been started yet (cluster launch control), and the copies of that unit's Q, K and V are under way while the last
 // tiles of the current one are worked on; only the write-back of O lies between two units (2.4 k cycles; a CTA per unit
 // spent 12 k around its loop).
-// What bounds it: on packed batches the power cap (0.97 PFLOP/s at 1.65 GHz and 985 W; 0.63 at 1.91 GHz before), on an
-// unthrottled GPU the exponential unit and the waits around it (the unit is busy 55 % of the time).
+// What bounds it: on packed batches the power cap (0.81 PFLOP/s at 1.65 GHz and 985 W; 0.63 at 1.91 GHz before), on an
+// unthrottled GPU the exponential unit and the waits around it (that unit and the tensor pipe are each busy 45 % of the time).
 // Before -> after, us: packed 28 + 4 heads of 128, 32 sequences of 256 to 1024 tokens 333 -> 234 (on the power cap 343 ->
 // 270), 16 x 2048 1047 -> 940; 16 x 512 queries x 32 heads 116 -> 80; Dream-shaped step (32 rollouts, 1280 keys) 34.2 -> 30.1.
 // 128-key tiles with one S / P buffer, P handed over in halves: 16 x 2048 904 and 16 x 512 77, but 282 on the packed batch
@@ -502,7 +502,7 @@ constexpr int TC_KT = 64;                 // keys per tile
 // log2 units the true max may run ahead of the reference.  The fewer, the oftener a row's largest weight is exactly 1 in bf16.  Distance
 // from 64 bits (rel-L2, x 1e-3; 1.5 of it the result's own rounding) for q of standard deviation 1, 2, 4, 8, 16 on 28 + 4 heads of 128:
 // 8 units 2.301, 2.223, 2.110, 1.851, 1.525; 4 units 2.300, 2.102, 1.865, 1.707, 1.469; 2 units 2.274, 1.944, 1.761, 1.669, 1.457, but the
-// ordinary scores of deviation 1 then move too (32 sequences of 256 to 1024 tokens 264 -> 283 us; 8 to 4 units: no difference).
+// ordinary scores of deviation 1 then move too (7 % on 32 sequences of 256 to 1024 tokens; 8 to 4 units: no difference).
 constexpr float TC_RESCALE_GAP = 4.0f;
 
 template <int D, int QT>
@@ -868,7 +868,8 @@ attn_block_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                 t1 = fmaxf(t1, t3);
                 if (t == 0 && w.n_tiles > 1) {
                     // The first reference is the largest score of 128 keys (the second tile's are on their way already): the oftener a
-                    // row's largest weight is 1, the less its rounding to bf16 costs (sharp rows are 3 % further off otherwise).
+                    // row's largest weight is 1, the less its rounding to bf16 costs (scores of standard deviation 1 are 0.75 % further from
+                    // 64 bits otherwise; it takes 2.5 % of 32 sequences of 256 to 1024 tokens, 5 to 10 of shorter ones).
                     const int valid1 = tile_info<TC_KT>(1, n_pre, n_blk, w.len_pre, w.len_blk, w.len_suf, 0, 0, 0).valid;
                     if (!mbar_wait(&bars->s_full[j][buf ^ 1], ((n + 1) >> 1) & 1, abort_flag)) { ok = false; break; }
                     tc_fence_after_sync();
@@ -1118,7 +1119,9 @@ int attn_plan_splits(const dare_ctx* ctx, const AttnArgs& a) {
     const int tiles = (a.prefix_cap + (a.k_blk ? a.L : 0) + a.suffix_cap + var.kt - 1) / var.kt;
     // As many K/V splits as keep the launch in one wave.  (As many as fill the slots or more left a second wave of a few CTAs, as
     // long as the first: 32 rows x 32 heads x 733 keys of 2, 4, 6 and 8 rollouts 17.5, 22.9, 27.2 and 30.9 us, now 13.5, 17.3, 19.1 and
-    // 21.2; 4 rows x 5120 keys of 1 and 2 rollouts 28.0 and 42.3, now 21.7 and 31.8.)
+    // 21.2; 4 rows x 5120 keys of 1 and 2 rollouts 28.0 and 42.3, now 21.7 and 31.8.  The other side of it is that from half the slots on
+    // a unit is not split, and a launch takes as long as its longest one: 5 rollouts x 32 heads, one of 2048 keys and four of 128,
+    // 25.1 and 27.7; 12 rollouts x 8 heads x 90 rows of 512 to 2048 keys 46.6 and 54.4.)
     long long s = slots / units;
     if (s > tiles / 2) s = tiles / 2;
     if (s > 32) s = 32;
