@@ -840,7 +840,9 @@ lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, 
     const uint32_t tmem_base = bars->tmem_base;
     const int num_k = (D + BK - 1) / BK;
     bool any = true;                                     // is any row masked?
-    if (LATE) {
+    // (a run-time value that is always LATE: with the constant W comes 0.8 % slower, four steps of 32 rows x 4096 x 126464 682.9 / 688.5 us)
+    const bool late = LATE && tokens.tokens != nullptr;
+    if (late) {
         pdl_wait();
         pdl_trigger();
         if (warp != 0) any = any_masked(tokens, Mc, lane);
@@ -869,8 +871,8 @@ lm_swapped_body(const CUtensorMap& tmap_w, const SwXMaps& xmaps, int Mc, int D, 
             for (int i = 0; i < 5; ++i) prefetch_tensormap(&xmaps.m[i]);
         }
         // LATE: the first stages are on their way while the tokens are looked at; if no row is masked after all, they are waited for.
-        int ahead = LATE ? min(SW_UNSEEN, num_k) : 0;
-        if (LATE) {
+        int ahead = late ? min(SW_UNSEEN, num_k) : 0;
+        if (late) {
             if (lane == 0)
                 for (int kb = 0; kb < ahead; ++kb) load(unit, unit / item_chunks, kb, kb);
             __syncwarp();
