@@ -1218,7 +1218,7 @@ lmhead_head_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_cons
     // DIRECT: rows evaluated where they lie, and by the swapped path (the launcher sees to it).  How many is known before the predecessor
     // is done, so it sets itself up beside it and waits in its place.  With what lmhead_merge_select_kernel does in front of its
     // wait, a replayed step of 32 rows x 512 x 4096 takes 12.0 us for 14.0, 128 rows x 256 x 1000 14.9 for 16.6, 32 rows x 4096 x 126464
-    // 165.6 for 167.5; one that finds no masked row 0.5 to 2 us more (its SW_UNSEEN stages, and a kernel to take down).  (In one kernel
+    // 165.6 for 167.5; one that finds no masked row 0.2 to 2 us more (its SW_UNSEEN stages, and a kernel to take down).  (In one kernel
     // with the other launches it slowed the sampled head of 416 rows by 1.4 %.)
     if constexpr (DIRECT) {
         lm_swapped_body<MODE, false, true>(tmap_w, xmaps, M, D, V, mask_col, n_tiles, part_max, part_sum, part_arg, dev_status,
